@@ -19,6 +19,7 @@
 
 #include "pe_internal.h"
 #include "pe_grad.h"
+#include "pe_fx.cuh"
 #include "pe_kernels.h"
 #include "pe_measure.h"
 #include "pe_plan.h"
@@ -46,6 +47,8 @@ struct pe_detector_s {
   double* dd_dev;      // [3]
   double2* sct;        // [kSinTab] sincos table
   float4* sctw;        // [kSinTab] the same as double words
+  pe::FxCis* fcis;     // [kSinTab], [kFxSincTab] tables of the fixed-point unit
+  pe::FxSinc* fsinc;
   float2* fw;          // [nb] double words of f, pi f L, f L / 2, sin(pi f L), cos(pi f L)
   float2* aw;
   float2* atw;
@@ -53,6 +56,7 @@ struct pe_detector_s {
   float2* caw;
   float2* f13w;        // [nb] f^(1/3), f^(-7/6) as double words
   float2* fm76w;
+  float2* fm83w;       // [nb] f^(-8/3) as a double word
   float4* zw;          // [nb] z as a double-word pair
   float4* dgw;         // [3][nb] dg / dg_scale as double words
   float2* ggw;         // [3][nb] gg / gg_scale as double words
@@ -161,6 +165,49 @@ float2 host_dw(double a) {
   return make_float2(h, static_cast<float>(a - static_cast<double>(h)));
 }
 
+// hi + lo with |lo| <= ulp(hi)/2, as a multiplier of the bin's k: c = C 2^-(60 + sh), k < 2^31.
+struct hdd {
+  double h, l;
+};
+hdd hdd_div(hdd a, double b) {
+  const double q = a.h / b;
+  const double r = std::fma(-q, b, a.h);
+  return hdd{q, (r + a.l) / b};
+}
+hdd hdd_mul(hdd a, double b) {
+  const double p = a.h * b;
+  return hdd{p, std::fma(a.l, b, std::fma(a.h, b, -p))};
+}
+pe::FxConst fx_const(hdd c) {   // 0 < c < 1
+  pe::FxConst r;
+  r.sh = std::min(62, 2 - std::ilogb(c.h));   // C in [2^62, 2^63) unless c is tiny
+  const double s = std::ldexp(1.0, 60 + r.sh);
+  const double hi = std::floor(c.h * s);      // a double of 53 bits times a power of two
+  r.C = (unsigned long long)hi + (unsigned long long)(long long)std::llround((c.h * s - hi) + c.l * s);
+  r.pad_ = 0;
+  return r;
+}
+// The fixed-point unit's constants, and whether the detector meets its bounds: a = pi f L < 4 up to the last bin
+// (sinc's table), an orbital eccentricity below 0.05 (link lengths within a few per cent of L, where
+// the unit's reciprocal square root converges), k below 2^31, and a Doppler scale 2^fx_rsh >= R f of
+// at most 2^20 turns.
+void fill_fx(pe_detector_s* d) {
+  pe::DetDev& D = d->dev;
+  D.fcis = d->fcis;
+  D.fsinc = d->fsinc;
+  D.fx_iL = 1.0 / D.L;
+  const double kmax = (double)(d->k0 + d->nb);
+  const double a_max = pe::kPi * kmax / d->T * D.L, fr = kmax / d->T * D.R;
+  const bool ecc = d->cfg.orbit != PE_ORBIT_HELIO || D.L / (2.0 * std::sqrt(3.0) * D.R) < 0.05;
+  D.fx_rsh = fr < 1.0 ? 0 : std::ilogb(fr) + 1;
+  D.fx_ok = a_max < 3.999 && ecc && kmax < 2147483648.0 && D.fx_rsh <= 20 ? 1 : 0;
+  if (!D.fx_ok) return;
+  const hdd pi = {3.141592653589793, 1.2246467991473532e-16};
+  D.fx_a4 = fx_const(hdd_div(hdd_mul(pi, D.L), 4.0 * d->T));
+  D.fx_at3 = fx_const(hdd_div(hdd{D.L, 0.0}, 6.0 * d->T));
+  D.fx_fR = fx_const(hdd_div(hdd{std::ldexp(D.R, -D.fx_rsh), 0.0}, d->T));
+}
+
 void fill_dev(pe_detector_s* d) {
   pe::DetDev& D = d->dev;
   memset(&D, 0, sizeof(D));
@@ -234,12 +281,14 @@ void fill_dev(pe_detector_s* d) {
   D.sctw = d->sctw; D.fw = d->fw; D.aw = d->aw; D.atw = d->atw; D.saw = d->saw; D.caw = d->caw;
   D.zw = d->zw; D.dgw = d->dgw; D.ggw = d->ggw; D.f13w = d->f13w; D.fm76w = d->fm76w;
   const size_t nbz = (size_t)d->nb;
+  D.fm83w = d->fm83w;
   D.ff = d->f32; D.f13f = d->f32 + nbz; D.fm13f = d->f32 + 2 * nbz; D.lnf3f = d->f32 + 3 * nbz; D.fm76f = d->f32 + 4 * nbz;
   D.scaf = d->scaf; D.zf = d->zf; D.dgf = d->dgf; D.ggf = d->ggf;
   D.rate_tf = (float)D.rate_t; D.alpha0_tf = (float)D.alpha0_t; D.geo_rate_tf = (float)D.geo_rate_t;
   D.Rf = (float)D.R; D.Lf = (float)D.L;
   D.dg_scale = 1.0;
   D.gg_scale = 1.0;
+  fill_fx(d);
 }
 
 // Power of two above |x| (1 for zero or non-finite x): the double-word tables hold x / scale < 1.
@@ -304,15 +353,19 @@ pe_status pe_create_detector(const pe_detector_config* cfg, double T_obs, int64_
   const size_t nb = (size_t)nbins;
   // double2: sincos table + sca, z (2 nb) + dg (3 nb); float4: double-word sincos table, zw (nb),
   // dgw (3 nb); doubles: f, f13, fm13, lnf3, fm76 (5 nb) + fpow (3 nb) + gg (3 nb) + psd_model (3 nb) + dd (3,
-  // padded); float2: fw, aw, atw, saw, caw, f13w, fm76w (7 nb) + ggw (3 nb) + scaf, zf (2 nb) +
+  // padded); float2: fw, aw, atw, saw, caw, f13w, fm76w, fm83w (8 nb) + ggw (3 nb) + scaf, zf (2 nb) +
   // dgf (3 nb); float: five FP32 grid tables (5 nb) + ggf (3 nb)
-  const size_t n_d = 14 * nb + 8, n_d2 = 5 * nb + pe::kSinTab, n_f4 = pe::kSinTab + 4 * nb, n_f2 = 15 * nb,
+  // the fixed-point unit's tables come first (16-byte entries)
+  const size_t fx_bytes = pe::kSinTab * sizeof(pe::FxCis) + pe::kFxSincTab * sizeof(pe::FxSinc);
+  const size_t n_d = 14 * nb + 8, n_d2 = 5 * nb + pe::kSinTab, n_f4 = pe::kSinTab + 4 * nb, n_f2 = 16 * nb,
                n_f = 8 * nb;
-  const size_t bytes = n_d2 * sizeof(double2) + n_f4 * sizeof(float4) + n_d * sizeof(double) +
+  const size_t bytes = fx_bytes + n_d2 * sizeof(double2) + n_f4 * sizeof(float4) + n_d * sizeof(double) +
                        n_f2 * sizeof(float2) + n_f * sizeof(float);
   cudaError_t e = pe::dmalloc(&d->mem, bytes);
   if (e != cudaSuccess) { cudaGetLastError(); delete d; return fail(PE_ENOMEM, "pe::dmalloc(%zu) failed", bytes); }
-  double2* p2 = static_cast<double2*>(d->mem);
+  d->fcis = static_cast<pe::FxCis*>(d->mem);
+  d->fsinc = reinterpret_cast<pe::FxSinc*>(d->fcis + pe::kSinTab);
+  double2* p2 = reinterpret_cast<double2*>(d->fsinc + pe::kFxSincTab);
   d->sct = p2; p2 += pe::kSinTab;
   d->sca = p2; p2 += nb;
   d->z = p2; p2 += nb;
@@ -339,6 +392,7 @@ pe_status pe_create_detector(const pe_detector_config* cfg, double T_obs, int64_
   d->caw = pf; pf += nb;
   d->f13w = pf; pf += nb;
   d->fm76w = pf; pf += nb;
+  d->fm83w = pf; pf += nb;
   d->ggw = pf; pf += 3 * nb;
   d->scaf = pf; pf += nb;
   d->zf = pf; pf += nb;
@@ -349,12 +403,13 @@ pe_status pe_create_detector(const pe_detector_config* cfg, double T_obs, int64_
   fill_dev(d);
   const double L = det_arm_s(*cfg);
   if ((e = pe::launch_sincos_table(d->sct, 0)) != cudaSuccess ||
+      (e = pe::launch_fx_tables(d->fcis, d->fsinc, 0)) != cudaSuccess ||
       (e = pe::launch_grid_tables(T_obs, k0, d->nb, L, d->f, d->f13, d->fm13, d->lnf3, d->fm76, d->fpow, d->sca,
                                   d->z, 0)) != cudaSuccess ||
       (e = pe::launch_psd_model(d->f, d->nb, L, cfg->oms_m_rtHz, cfg->acc_ms2_rtHz, cfg->psd_shaping, cfg->tdi_gen,
                                 d->psd_model, 0)) != cudaSuccess ||
-      (e = pe::launch_dw_tables(d->f, d->f13, d->fm76, d->sca, d->z, d->sct, d->nb, L, d->fw, d->aw, d->atw, d->saw,
-                                d->caw, d->f13w, d->fm76w, d->zw, d->sctw, 0)) != cudaSuccess ||
+      (e = pe::launch_dw_tables(d->f, d->f13, d->fm13, d->fm76, d->sca, d->z, d->sct, d->nb, L, d->fw, d->aw, d->atw, d->saw,
+                                d->caw, d->f13w, d->fm76w, d->fm83w, d->zw, d->sctw, 0)) != cudaSuccess ||
       (e = pe::launch_f32_tables(d->f, d->f13, d->fm13, d->lnf3, d->fm76, d->sca, d->z, d->nb, d->f32,
                                  d->f32 + nb, d->f32 + 2 * nb, d->f32 + 3 * nb, d->f32 + 4 * nb, d->scaf, d->zf, 0)) !=
           cudaSuccess ||

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "pe_device.cuh"
+#include "pe_device_fx.cuh"
 #include "pe_device_mixed.cuh"
 #include "pe_internal.h"
 #include "pe_kernels.h"
@@ -74,6 +75,23 @@ __device__ __forceinline__ void mode_brackets(const DetDev& D, const SampleCoef&
   }
 }
 
+// The same with the fixed-point unit.
+__device__ __forceinline__ void mode_brackets_fx(const DetDev& D, const SampleCoef& S, int b, unsigned mask,
+                                                 double2 o[kNModes][3], const DetDev& D0,
+                                                 const fx* __restrict__ pc, fx* col) {
+  FxBin Bn;
+  load_bin_fx(D, b, S.tc, Bn);
+  const double2 z = D.z[b];
+#pragma unroll 1
+  for (int md = 0; md < kNModes; ++md) {
+    const ModeCoef& C = S.md[md];
+    FxAcc a;
+    fx_zero(a, col);
+    if ((mask >> md) & 1u && C.active && Bn.f < C.fend) mode_bin_fx(D, S, C, Bn, a, D0.fcis, D0.fsinc, pc, md);
+    aet_from_fx(a, z, o[md]);
+  }
+}
+
 // The same with the mixed-precision unit (FP64 phase, t_f and turn reductions; double-word
 // geometry), each mode's brackets returned to FP64.
 __device__ __forceinline__ void mode_brackets_mixed(const DetDev& D, const SampleCoef& S, int b, unsigned mask,
@@ -99,14 +117,22 @@ __device__ __forceinline__ void mode_brackets_mixed(const DetDev& D, const Sampl
 }
 
 // Reference per-mode brackets on bins [0, K): out[(md*3 + c)*K + k].
+template <bool FX>
 __global__ void k_mode_brackets(DetDev D, const SampleCoef* coef, int K, unsigned mask, double2* out) {
   __shared__ double pc[kProj];
+  __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   const SampleCoef& S = coef[0];
-  proj_prologue(D, S, pc);
+  if (FX)
+    fx_proj_prologue(D, S, reinterpret_cast<fx*>(pc));
+  else
+    proj_prologue(D, S, pc);
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= K) return;
   double2 o[kNModes][3];
-  mode_brackets(D, S, k, mask, o, D.sct, pc);
+  if (FX)
+    mode_brackets_fx(D, S, k, mask, o, D, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
+  else
+    mode_brackets(D, S, k, mask, o, D.sct, pc);
   for (int md = 0; md < kNModes; ++md)
     for (int c = 0; c < 3; ++c) out[((size_t)md * 3 + c) * K + k] = o[md][c];
 }
@@ -227,7 +253,7 @@ __device__ __forceinline__ cdf mul_conj(const cdf& a, const cdf& b) {
 // the contraction in double words (Aw, Bw); the sums across bins and the block reduction stay
 // FP64. An edge with a ratio of kHetDwRatioMax or more keeps all its ratios in FP64 (flag byte
 // per edge after the ratios), and every (bin, channel) that reads it takes the FP64 contraction.
-template <bool MIX>
+template <bool MIX, bool FX>
 __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, const SampleCoef* __restrict__ coef,
                                                            double* logl, double* dhhh) {
   extern __shared__ double2 rsh[];
@@ -235,11 +261,12 @@ __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, con
   __shared__ double pc[kProj];
   __shared__ float2 pcw[MIX ? kProj : 1];
   __shared__ double sh[6][kTileBins / 32];
-  __shared__ double2 stab[MIX ? 1 : kSinTab];
+  __shared__ double2 stab[MIX || FX ? 1 : kSinTab];
+  __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   __shared__ float4 stabw[MIX ? kSinTab : 1];
   if constexpr (MIX) {
     for (int i = threadIdx.x; i < kSinTab; i += blockDim.x) stabw[i] = hs.h[0].det.sctw[i];
-  } else {
+  } else if constexpr (!FX) {
     for (int i = threadIdx.x; i < kSinTab; i += blockDim.x) stab[i] = hs.h[0].det.sct[i];
   }
   const int s = blockIdx.x;
@@ -248,7 +275,11 @@ __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, con
   for (int I = 0; I < hs.n; ++I) {
     const HetDev& H = hs.h[I];
     const DetDev& D = H.det;
-    proj_prologue(D, S, pc);   // its barriers also order the table staging and the previous detector
+    // its barriers also order the table staging and the previous detector
+    if constexpr (FX)
+      fx_proj_prologue(D, S, reinterpret_cast<fx*>(pc));
+    else
+      proj_prologue(D, S, pc);
     if constexpr (MIX) {
       if (threadIdx.x < kProj) pcw[threadIdx.x] = to_dw(pc[threadIdx.x]);
       __syncthreads();
@@ -260,6 +291,8 @@ __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, con
       double2 o[kNModes][3];
       if constexpr (MIX)
         mode_brackets_mixed(D, S, H.edge[e], H.mask, o, stabw, pcw);
+      else if constexpr (FX)
+        mode_brackets_fx(D, S, H.edge[e], H.mask, o, hs.h[0].det, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
       else
         mode_brackets(D, S, H.edge[e], H.mask, o, stab, pc);
       // ratios in place of the brackets; in the mixed kernel, flag the edge if one of them is out
@@ -523,7 +556,8 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   if (e == cudaSuccess) e = pe::upload(d_fe, hfe.data(), ne * sizeof(double));
   if (e == cudaSuccess) e = pe::launch_prep(th0, 1, mode_mask, ds, coef, nend, nullptr, 0);
   if (e == cudaSuccess) {
-    pe::k_mode_brackets<<<(K + pe::kTileBins - 1) / pe::kTileBins, pe::kTileBins>>>(D, coef, K, mode_mask, hb);
+    auto kb = D.fx_ok ? pe::k_mode_brackets<true> : pe::k_mode_brackets<false>;
+    kb<<<(K + pe::kTileBins - 1) / pe::kTileBins, pe::kTileBins>>>(D, coef, K, mode_mask, hb);
     e = pe::launch_status();
   }
   // reference brackets at the edges, and the carry-forward sources
@@ -659,7 +693,8 @@ pe_status pe_hetero_loglike_batch(const pe_hetero* hets, int ndet, const double*
                         static_cast<int*>(stt), st);
   const bool mix = (hets[0]->dev.mask & PE_PREC_MIXED) != 0u;
   const size_t smem = (size_t)nemax * pe::kNModes * 3 * sizeof(double2) + (mix ? (size_t)nemax : 0);
-  auto kern = mix ? pe::k_het_loglike<true> : pe::k_het_loglike<false>;
+  auto kern = mix ? pe::k_het_loglike<true, false>
+                  : (pe::fx_all_ok(ds) ? pe::k_het_loglike<false, true> : pe::k_het_loglike<false, false>);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) {
     kern<<<B, pe::kTileBins, smem, st>>>(hs, B, static_cast<const pe::SampleCoef*>(coef), static_cast<double*>(ll),

@@ -22,6 +22,8 @@ constexpr int kMaxDet = 8;
 constexpr int kTileBins = 128;  // frequency bins per (sub-)tile = threads per CTA of the hot kernels
 // Arithmetic of the forward path (mode-mask flags PE_PREC_MIXED, PE_PREC_FP32).
 constexpr int kPrecFP64 = 0, kPrecMixed = 1, kPrecFP32 = 2;
+// FP64 with the response geometry in fixed point (pe_device_fx.cuh): what kPrecFP64 takes where fx_ok holds
+constexpr int kPrecFx = 3;
 // Work items of the log-likelihood kernels are R consecutive 128-bin sub-tiles of one (detector,
 // sample) pair, R in {1, 2, 4, 8} picked by the autotuner. The default (no tuned choice) keeps
 // one sub-tile per item in FP64 (most CTAs for small batches) and four in the other precisions,
@@ -109,6 +111,15 @@ struct SampleGrad {
   ModeGrad md[kNModes];
 };
 
+// A constant c of the fixed-point unit as C 2^-(60 + sh), so that k c in units of 2^-60 is (k C) >> sh.
+struct FxConst {
+  unsigned long long C;
+  int sh;
+  int pad_;
+};
+struct FxCis;    // entries of the fixed-point unit's tables (pe_fx.cuh)
+struct FxSinc;
+
 // Device view of one detector: grid, orbit constants and per-bin SoA tables.
 struct DetDev {
   double T;          // observation time = 1/df [s]
@@ -152,6 +163,7 @@ struct DetDev {
   const float2* caw;
   const float2* f13w;   // f^(1/3) and f^(-7/6) as double words
   const float2* fm76w;
+  const float2* fm83w;  // f^(-8/3) as a double word
   const float4* zw;     // z as (re hi, re lo, im hi, im lo)
   const float4* dgw;    // [3][nb]: dg / dg_scale as (re hi, re lo, im hi, im lo)
   const float2* ggw;    // [3][nb]: gg / gg_scale
@@ -176,6 +188,13 @@ struct DetDev {
   float2 Rw;            // R as a double word
   float2 ratew, alpha0w, geo_ratew;   // rate_t, alpha0_t, geo_rate_t as double words
   float tfw_max;        // |t_f| below which the mixed unit forms t_f and the orbit angles in double words
+  // fixed-point unit of the FP64 path (pe_device_fx.cuh): 1 where the detector takes it, 1/L, and
+  // pi L / (4 T), L / (6 T), R / T 2^-fx_rsh as multipliers of the bin's k
+  int fx_ok, fx_rsh;
+  double fx_iL;
+  FxConst fx_a4, fx_at3, fx_fR;
+  const FxCis* fcis;    // [kSinTab]
+  const FxSinc* fsinc;  // [kFxSincTab]
   // Q = TDI factor(z) (-i a) e^{-i a}; n_A = 1/sqrt2, n_E = 1/sqrt6, n_T = 1/sqrt3
 };
 

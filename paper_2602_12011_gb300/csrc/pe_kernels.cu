@@ -14,8 +14,11 @@
 //   k_inject         data = signal + noise scaled by the PSD (Eq. eq_diag_Sigma_to_Sn)
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "pe_device.cuh"
 #include "pe_device_f32.cuh"
+#include "pe_device_fx.cuh"
 #include "pe_device_mixed.cuh"
 #include "pe_kernels.h"
 #include "pe_fault.h"
@@ -58,6 +61,87 @@ __global__ void k_sincos_table(double2* tab) {
   tab[j] = make_double2(c, s);
 }
 
+// Tables of the fixed-point unit (pe_fx.cuh), in double-double arithmetic (about 2^-104): the sines and cosines
+// by their series below pi/4 and the octants' symmetries, sinc's Taylor coefficients about each table
+// point, f^(k)(u)/k! = sum_n (-1)^n C(2n, k) u^(2n-k) / (2n+1)!.
+struct dd {
+  double h, l;
+};
+__device__ __forceinline__ dd dd_norm(double h, double l) {
+  const double s = __dadd_rn(h, l);
+  return dd{s, __dsub_rn(l, __dsub_rn(s, h))};
+}
+__device__ __forceinline__ dd dd_add(dd a, dd b) {
+  const double s = __dadd_rn(a.h, b.h), v = __dsub_rn(s, a.h);
+  const double e = __dadd_rn(__dsub_rn(a.h, __dsub_rn(s, v)), __dsub_rn(b.h, v));
+  return dd_norm(s, __dadd_rn(e, __dadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ dd dd_mul(dd a, dd b) {
+  const double p = __dmul_rn(a.h, b.h);
+  return dd_norm(p, __dadd_rn(__fma_rn(a.h, b.h, -p), __dadd_rn(__dmul_rn(a.h, b.l), __dmul_rn(a.l, b.h))));
+}
+__device__ __forceinline__ dd dd_div(dd a, double b) {   // b exact
+  const double q = __ddiv_rn(a.h, b);
+  return dd_norm(q, __ddiv_rn(__dadd_rn(__fma_rn(-q, b, a.h), a.l), b));
+}
+__device__ __forceinline__ fx dd_to_fx(dd a) {           // |a| <= 1
+  const double x = a.h * 0x1p60;
+  const fx n = __double2ll_rn(x);
+  return n + __double2ll_rn((x - __ll2double_rn(n)) + a.l * 0x1p60);
+}
+__device__ __forceinline__ df dd_to_dw(dd a) {
+  const float h = __double2float_rn(a.h);
+  return df_make(h, __double2float_rn((a.h - (double)h) + a.l));
+}
+// One thread per angle (the first kSinTab) and per (sinc entry, order).
+constexpr int kFxSincOrders = 7;
+__global__ void k_fx_tables(FxCis* cis, FxSinc* snc) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < kSinTab) {
+    const int oct = i / (kSinTab / 8), r = i % (kSinTab / 8);
+    const int m = (oct & 1) ? kSinTab / 8 - r : r;        // angle 2 pi m / kSinTab <= pi/4
+    const dd x = dd_mul(dd{6.283185307179586, 2.4492935982947064e-16}, dd{(double)m / kSinTab, 0.0});
+    const dd x2 = dd_mul(x, x);
+    dd c = {1.0, 0.0}, s = {1.0, 0.0};
+    for (int k = 26; k >= 2; k -= 2) {                     // Horner: 1 - x2/((k-1) k) (...) and 1 - x2/(k (k+1)) (...)
+      dd t = dd_div(dd_mul(x2, c), -(double)(k - 1) * k);
+      c = dd_add(dd{1.0, 0.0}, t);
+      t = dd_div(dd_mul(x2, s), -(double)k * (k + 1));
+      s = dd_add(dd{1.0, 0.0}, t);
+    }
+    s = dd_mul(s, x);
+    if (((oct + 1) >> 1) & 1) { const dd t = c; c = s; s = t; }   // octants 1, 2, 5, 6 swap
+    if (oct >= 2 && oct <= 5) { c.h = -c.h; c.l = -c.l; }
+    if (oct >= 4) { s.h = -s.h; s.l = -s.l; }
+    const df cw = dd_to_dw(c), sw = dd_to_dw(s);
+    cis[i] = FxCis{dd_to_fx(c), dd_to_fx(s), make_float4(cw.x, cw.y, sw.x, sw.y)};
+    return;
+  }
+  const int e = (i - kSinTab) / kFxSincOrders, k = (i - kSinTab) % kFxSincOrders;
+  if (e >= kFxSincTab) return;
+  const dd u = {(double)e / kFxSincPerUnit, 0.0}, u2 = dd_mul(u, u);
+  // first term n0 = ceil(k/2): (-1)^n0 C(2 n0, k) u^(2 n0 - k) / (2 n0 + 1)!; the ratio of term n + 1 to term n is
+  // -u^2 (2n + 1) / ((2n + 2 - k) (2n + 1 - k) (2n + 3)). Terms fall below 1e-34 of the largest before the end.
+  const int n0 = (k + 1) / 2;
+  double fac = 1.0;
+  for (int j = 2; j <= 2 * n0 + 1; ++j) fac *= j;                // exact
+  dd t = dd_div(dd{(n0 & 1) ? -1.0 : 1.0, 0.0}, fac);
+  if (2 * n0 - k == 1) t = dd_mul(dd_mul(t, u), dd{(double)(2 * n0), 0.0});   // C(2 n0, 2 n0 - 1) u
+  dd sum = t;
+  for (int n = n0; n < 27 && fabs(t.h) > 1e-34; ++n) {
+    t = dd_div(dd_mul(dd_mul(t, u2), dd{-(double)(2 * n + 1), 0.0}), (double)((2 * n + 2 - k) * (2 * n + 1 - k) * (2 * n + 3)));
+    sum = dd_add(sum, t);
+  }
+  FxSinc& o = snc[e];
+  if (k == 0) o.s0 = dd_to_fx(sum);
+  else if (k == 1) o.s1 = dd_to_dw(sum);
+  else if (k == 2) o.s2 = dd_to_dw(sum);
+  else if (k == 3) o.s3 = dd_to_dw(sum);
+  else if (k == 4) o.s4 = (float)sum.h;
+  else if (k == 5) o.s5 = (float)sum.h;
+  else o.s6 = (float)sum.h;
+}
+
 // Double words of the mixed-precision path: per bin f, a = pi f L, a/(2 pi), sin a, cos a,
 // f^(1/3), f^(-7/6) and z (from the FP64 tables), and the sincos table as (cos hi, cos lo, sin hi,
 // sin lo).
@@ -65,9 +149,10 @@ __device__ __forceinline__ float2 dw_of(double a) {
   const float h = __double2float_rn(a);
   return make_float2(h, __double2float_rn(a - (double)h));
 }
-__global__ void k_dw_tables(const double* f, const double* f13, const double* fm76, const double2* sca, const double2* z,
+__global__ void k_dw_tables(const double* f, const double* f13, const double* fm13, const double* fm76, const double2* sca,
+                            const double2* z,
                             const double2* tab, int nb, double L, float2* fw, float2* aw, float2* atw, float2* saw,
-                            float2* caw, float2* f13w, float2* fm76w, float4* zw, float4* tabw) {
+                            float2* caw, float2* f13w, float2* fm76w, float2* fm83w, float4* zw, float4* tabw) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < kSinTab) {
     const float2 c = dw_of(tab[b].x), s = dw_of(tab[b].y);
@@ -81,6 +166,8 @@ __global__ void k_dw_tables(const double* f, const double* f13, const double* fm
   caw[b] = dw_of(sca[b].y);
   f13w[b] = dw_of(f13[b]);
   fm76w[b] = dw_of(fm76[b]);
+  const double m2 = fm13[b] * fm13[b], m4 = m2 * m2;
+  fm83w[b] = dw_of(m4 * m4);
   const float2 zr = dw_of(z[b].x), zi = dw_of(z[b].y);
   zw[b] = make_float4(zr.x, zr.y, zi.x, zi.y);
 }
@@ -321,10 +408,11 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
                                                                  const long long* __restrict__ offi, int R,
                                                                  double* part) {
   __shared__ double red[6][kTileBins + kRedPad];   // block_sum6 staging (as float2 or float rows)
-  __shared__ double pc[kProj];    // the item's projection forms (proj_coef)
+  __shared__ double pc[kProj];    // the item's projection forms (proj_coef; fx_proj_prologue's words)
   __shared__ float2 pcw[kProj];   // the same as double words (mixed) or floats (.x, FP32)
   __shared__ SampleF sf;          // the item's sample coefficients in FP32 (FP32 path)
-  __shared__ double2 stab[kSinTab];   // the sincos table (as float4 double words in the mixed path)
+  __shared__ fx fxcol[PREC == kPrecFx ? kFxSums : 1][kTileBins];   // the fixed-point unit's sums, a column per thread
+  __shared__ double2 stab[PREC == kPrecFx ? 1 : kSinTab];   // the sincos table (as float4 double words in the mixed path)
   if (PREC == kPrecMixed) {
     float4* t4 = reinterpret_cast<float4*>(stab);
     for (int i = threadIdx.x; i < kSinTab; i += blockDim.x) t4[i] = ds.d[0].sctw[i];
@@ -346,7 +434,10 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
     const DetDev& D = ds.d[I];
     if (!PE_CHK(ne <= D.nb, 4)) continue;
     const SampleCoef& S = coef[s];
-    proj_prologue(D, S, pc);
+    if constexpr (PREC == kPrecFx)
+      fx_proj_prologue(D, S, reinterpret_cast<fx*>(pc));
+    else
+      proj_prologue(D, S, pc);
     if constexpr (PREC == kPrecMixed) {
       if (threadIdx.x < kProj) pcw[threadIdx.x] = to_dw(pc[threadIdx.x]);
       __syncthreads();
@@ -407,9 +498,14 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
         const int b = int(j0 + (q - q0)) * kTileBins + threadIdx.x;
         double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         if (b < ne) {
-          double2 x[3], o[3];
-          bin_xyz(D, S, b, x, stab, pc);
-          aet_from_xyz(x, o);
+          double2 o[3];
+          if constexpr (PREC == kPrecFx) {
+            bin_aet_fx(D, S, b, o, ds.d[0], reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
+          } else {
+            double2 x[3];
+            bin_xyz(D, S, b, x, stab, pc);
+            aet_from_xyz(x, o);
+          }
           accum_bin(D, b, o, v);
         }
         double r;
@@ -460,8 +556,12 @@ __global__ void k_signal(DetDev D, const SampleCoef* coef, double2* out) {
   __shared__ double pc[kProj];
   __shared__ float2 pcw[kProj];
   __shared__ SampleF sf;
+  __shared__ fx fxcol[PREC == kPrecFx ? kFxSums : 1][kTileBins];
   const SampleCoef& S = coef[0];
-  proj_prologue(D, S, pc);
+  if (PREC == kPrecFx)
+    fx_proj_prologue(D, S, reinterpret_cast<fx*>(pc));
+  else
+    proj_prologue(D, S, pc);
   if (PREC == kPrecMixed && threadIdx.x < kProj) pcw[threadIdx.x] = to_dw(pc[threadIdx.x]);
   if (PREC == kPrecFP32) {
     if (threadIdx.x < kProj) reinterpret_cast<float*>(pcw)[threadIdx.x] = (float)pc[threadIdx.x];
@@ -480,6 +580,8 @@ __global__ void k_signal(DetDev D, const SampleCoef* coef, double2* out) {
     float2 of[3];
     bin_aet_f32(D, sf, b, of, reinterpret_cast<const float*>(pcw));
     for (int i = 0; i < 3; ++i) o[i] = make_double2((double)of[i].x * S.ihsc, (double)of[i].y * S.ihsc);
+  } else if (PREC == kPrecFx) {
+    bin_aet_fx(D, S, b, o, D, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
   } else {
     bin_xyz(D, S, b, x, D.sct, pc);
     aet_from_xyz(x, o);
@@ -507,6 +609,10 @@ cudaError_t launch_grid_tables(double T, long long k0, int nb, double L, double*
 }
 cudaError_t launch_sincos_table(double2* tab, cudaStream_t st) {
   k_sincos_table<<<(kSinTab + 127) / 128, 128, 0, st>>>(tab);
+  return pe::launch_status();
+}
+cudaError_t launch_fx_tables(FxCis* cis, FxSinc* snc, cudaStream_t st) {
+  k_fx_tables<<<(kSinTab + kFxSincTab * kFxSincOrders + 31) / 32, 32, 0, st>>>(cis, snc);
   return pe::launch_status();
 }
 cudaError_t launch_psd_model(const double* f, int nb, double L, double oms, double acc, int shaping, int tdi_gen,
@@ -546,13 +652,13 @@ cudaError_t launch_fwd_offsets(const int* nend, int P, long long* off, long long
   if (e == cudaSuccess && R > 1) e = launch_scan_tiles(nend, P, offi, R * kTileBins, st);
   return e;
 }
-cudaError_t launch_dw_tables(const double* f, const double* f13, const double* fm76, const double2* sca,
+cudaError_t launch_dw_tables(const double* f, const double* f13, const double* fm13, const double* fm76, const double2* sca,
                              const double2* z, const double2* tab, int nb, double L, float2* fw, float2* aw,
-                             float2* atw, float2* saw, float2* caw, float2* f13w, float2* fm76w, float4* zw,
-                             float4* tabw, cudaStream_t st) {
+                             float2* atw, float2* saw, float2* caw, float2* f13w, float2* fm76w, float2* fm83w,
+                             float4* zw, float4* tabw, cudaStream_t st) {
   const int n = nb > kSinTab ? nb : kSinTab;
-  k_dw_tables<<<(n + 127) / 128, 128, 0, st>>>(f, f13, fm76, sca, z, tab, nb, L, fw, aw, atw, saw, caw, f13w, fm76w, zw,
-                                               tabw);
+  k_dw_tables<<<(n + 127) / 128, 128, 0, st>>>(f, f13, fm13, fm76, sca, z, tab, nb, L, fw, aw, atw, saw, caw, f13w, fm76w,
+                                               fm83w, zw, tabw);
   return pe::launch_status();
 }
 cudaError_t launch_table_max(const double2* dg, const double* gg, int n, double* mx_part, double* out, cudaStream_t st) {
@@ -579,53 +685,52 @@ cudaError_t launch_loglike_fwd(const DetSet& ds, int B, const SampleCoef* coef, 
 }
 
 namespace {
+// CTAs stride over the items statically, so a grid of one and a fraction times the resident CTAs runs its last
+// round nearly empty (1024 LISA samples: 8.5 ms with 8 CTAs per SM where 6 are resident, 6.4 ms with
+// 6): the grid is cut to the resident CTAs, a count kept per kernel and device.
 template <int MINB, int PREC>
 cudaError_t fwd_one(const DetSet& ds, int B, const SampleCoef* coef, const int* nend, const long long* off,
-                    const long long* offi, int R, double* part, int grid, cudaStream_t st) {
-  k_loglike_fwd<MINB, PREC><<<grid, kTileBins, 0, st>>>(ds, B, coef, nend, off, R > 1 ? offi : off, R, part);
-  return pe::launch_status();
-}
-template <int MINB, int PREC>
-int fwd_occ() {
-  int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_loglike_fwd<MINB, PREC>, kTileBins, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
+                    const long long* offi, int R, double* part, int grid, bool items, cudaStream_t st) {
+  static std::atomic<int> resident[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+    int r = resident[dev].load(std::memory_order_relaxed);
+    if (r == 0) {
+      int occ = 0, nsm = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_loglike_fwd<MINB, PREC>, kTileBins, 0) == cudaSuccess &&
+          cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && occ > 0 && nsm > 0)
+        resident[dev].store(r = occ * nsm, std::memory_order_relaxed);
+      else
+        cudaGetLastError();
+    }
+    if (r > 0 && grid > r) grid = r;
   }
-  return n;
+  k_loglike_fwd<MINB, PREC><<<grid, kTileBins, 0, st>>>(ds, B, coef, nend, off, items ? offi : off, R, part);
+  return pe::launch_status();
 }
 }  // namespace
 
 cudaError_t launch_loglike_fwd_variant(int variant, int prec, const DetSet& ds, int B, const SampleCoef* coef,
                                        const int* nend, const long long* off, const long long* offi, int R,
-                                       double* part, int grid, cudaStream_t st) {
+                                       double* part, int grid, cudaStream_t st, bool items) {
+  items |= R > 1;
   if (R != 1 && R != 2 && R != 4 && R != 8) return cudaErrorInvalidValue;
-  switch (variant * 3 + prec) {
-    case 0: return fwd_one<2, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 1: return fwd_one<2, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 2: return fwd_one<2, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 3: return fwd_one<3, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 4: return fwd_one<3, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 5: return fwd_one<3, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 6: return fwd_one<4, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 7: return fwd_one<4, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, st);
-    case 8: return fwd_one<4, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, st);
+  // FP64: the fixed-point unit where every detector meets its bounds
+  if (prec == kPrecFP64 && fx_all_ok(ds)) prec = kPrecFx;
+  switch (variant * 4 + prec) {
+    case 0: return fwd_one<2, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 1: return fwd_one<2, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 2: return fwd_one<2, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 3: return fwd_one<4, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 4: return fwd_one<3, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 5: return fwd_one<3, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 6: return fwd_one<3, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 7: return fwd_one<6, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 8: return fwd_one<4, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 9: return fwd_one<4, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 10: return fwd_one<4, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 11: return fwd_one<5, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
     default: return cudaErrorInvalidValue;
-  }
-}
-int fwd_variant_min_blocks(int variant) { return variant == 0 ? 2 : variant == 1 ? 3 : 4; }
-int fwd_variant_max_blocks_per_sm(int variant, int prec) {
-  switch (variant * 3 + prec) {
-    case 0: return fwd_occ<2, kPrecFP64>();
-    case 1: return fwd_occ<2, kPrecMixed>();
-    case 2: return fwd_occ<2, kPrecFP32>();
-    case 3: return fwd_occ<3, kPrecFP64>();
-    case 4: return fwd_occ<3, kPrecMixed>();
-    case 5: return fwd_occ<3, kPrecFP32>();
-    case 6: return fwd_occ<4, kPrecFP64>();
-    case 7: return fwd_occ<4, kPrecMixed>();
-    case 8: return fwd_occ<4, kPrecFP32>();
-    default: return 0;
   }
 }
 cudaError_t launch_reduce(const DetSet& ds, int B, const long long* off, const double* part, const SampleCoef* coef,
@@ -642,6 +747,8 @@ cudaError_t launch_signal(const DetDev& D, const SampleCoef* coef, double2* out,
     k_signal<kPrecMixed><<<g, kTileBins, 0, st>>>(D, coef, out);
   else if (prec == kPrecFP32)
     k_signal<kPrecFP32><<<g, kTileBins, 0, st>>>(D, coef, out);
+  else if (D.fx_ok)
+    k_signal<kPrecFx><<<g, kTileBins, 0, st>>>(D, coef, out);
   else
     k_signal<kPrecFP64><<<g, kTileBins, 0, st>>>(D, coef, out);
   return pe::launch_status();

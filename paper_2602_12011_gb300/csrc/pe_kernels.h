@@ -9,6 +9,8 @@ namespace pe {
 cudaError_t launch_grid_tables(double T, long long k0, int nb, double L, double* f, double* f13, double* fm13,
                                double* lnf3, double* fm76, double* fpow, double2* sca, double2* z, cudaStream_t st);
 cudaError_t launch_sincos_table(double2* tab, cudaStream_t st);
+// The fixed-point unit's tables (pe_fx.cuh).
+cudaError_t launch_fx_tables(FxCis* cis, FxSinc* snc, cudaStream_t st);
 cudaError_t launch_psd_model(const double* f, int nb, double L, double oms, double acc, int shaping, int tdi_gen,
                              double* out, cudaStream_t st);
 cudaError_t launch_data_tables(const double* f, const double2* sca, const double2* z, int nb, double T, double L,
@@ -24,10 +26,10 @@ cudaError_t launch_scan_tiles(const int* nend, int P, long long* off, int tile_b
 // items of R sub-tiles (not written when R == 1: the kernel then takes off for both).
 cudaError_t launch_fwd_offsets(const int* nend, int P, long long* off, long long* offi, int R, cudaStream_t st);
 inline long long tiles_of(int nb, int tile_bins) { return (nb + tile_bins - 1) / tile_bins; }
-cudaError_t launch_dw_tables(const double* f, const double* f13, const double* fm76, const double2* sca,
+cudaError_t launch_dw_tables(const double* f, const double* f13, const double* fm13, const double* fm76, const double2* sca,
                              const double2* z, const double2* tab, int nb, double L, float2* fw, float2* aw,
-                             float2* atw, float2* saw, float2* caw, float2* f13w, float2* fm76w, float4* zw,
-                             float4* tabw, cudaStream_t st);
+                             float2* atw, float2* saw, float2* caw, float2* f13w, float2* fm76w, float2* fm83w,
+                             float4* zw, float4* tabw, cudaStream_t st);
 // max over n entries of max(|Re dg|, |Im dg|) and gg -> out[2]; mx_part: [ceil(n/128)][2] scratch
 cudaError_t launch_table_max(const double2* dg, const double* gg, int n, double* mx_part, double* out, cudaStream_t st);
 cudaError_t launch_dw_data(const double2* dg, const double* gg, int n, double inv_dgs, double inv_ggs, float4* dgw,
@@ -39,14 +41,13 @@ cudaError_t launch_f32_tables(const double* f, const double* f13, const double* 
 // prec: kPrecFP64, kPrecMixed or kPrecFP32 forward kernel; R: sub-tiles per work item (1, 2, 4, 8)
 cudaError_t launch_loglike_fwd(const DetSet& ds, int B, const SampleCoef* coef, const int* nend, const long long* off,
                                const long long* offi, int R, double* part, int grid, int prec, cudaStream_t st);
+// items: offi is the list of work items even where R == 1 (a list of some pairs only).
 // Register-budget variants of the forward kernel (min resident CTAs per SM 2, 3, 4), per precision.
 constexpr int kFwdVariants = 3;
 constexpr int kFwdDefaultVariant = 1;
 cudaError_t launch_loglike_fwd_variant(int variant, int prec, const DetSet& ds, int B, const SampleCoef* coef,
                                        const int* nend, const long long* off, const long long* offi, int R,
-                                       double* part, int grid, cudaStream_t st);
-int fwd_variant_min_blocks(int variant);
-int fwd_variant_max_blocks_per_sm(int variant, int prec);
+                                       double* part, int grid, cudaStream_t st, bool items = false);
 cudaError_t launch_reduce(const DetSet& ds, int B, const long long* off, const double* part, const SampleCoef* coef,
                           double* logl, double* dhhh, cudaStream_t st);
 cudaError_t launch_signal(const DetDev& D, const SampleCoef* coef, double2* out, int prec, cudaStream_t st);
@@ -59,6 +60,13 @@ inline bool fwd_mask_ok(unsigned m) {
 }
 inline int mask_prec(unsigned m) {
   return (m & PE_PREC_MIXED) ? kPrecMixed : ((m & PE_PREC_FP32) ? kPrecFP32 : kPrecFP64);
+}
+
+// True where every detector of the set takes the FP64 path's fixed-point unit (pe_device_fx.cuh).
+inline bool fx_all_ok(const DetSet& ds) {
+  for (int i = 0; i < ds.ndet; ++i)
+    if (!ds.d[i].fx_ok) return false;
+  return true;
 }
 
 // CTAs per SM the persistent forward kernel can keep resident (occupancy query).

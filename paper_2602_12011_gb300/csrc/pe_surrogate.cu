@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "pe_device.cuh"
+#include "pe_device_fx.cuh"
 #include "pe_device_mixed.cuh"
 #include "pe_kernels.h"
 #include "pe_mlp.h"
@@ -134,8 +135,10 @@ __device__ __forceinline__ double psi_of(const SampleCoef& S, double v, double l
 
 // Plain-generator node values (raw): out[s][(md*2 + kind)*kNodes + j], for the samples whose mass
 // ratio exceeds q_above (all of them for q_above < 1; the others' rows are left as they are).
+// nv (nullable): k_node_h's tables, from which f's powers and ln v come without exp, cbrt and log (1024 samples: 0.62 ms
+// with them, the FP64 log-likelihood's path)
 __global__ void k_targets(const double* theta, int B, const SampleCoef* S, const SampleCoef* S0, float* out,
-                          double q_above) {
+                          double q_above, const double2* nv) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)B * kNModes * kNodes) return;
   const int j = (int)(i % kNodes);
@@ -144,10 +147,20 @@ __global__ void k_targets(const double* theta, int B, const SampleCoef* S, const
   const double* t = theta + (size_t)s * PE_NPARAM;
   if (!(t[1] > q_above)) return;
   const int mm = (md == 0) ? 2 : (md == 1) ? 1 : (md == 2) ? 3 : (md == 3) ? 2 : 4;
-  const double M = t[0] * kMsunS;
-  const double f = kFmin * exp(j * node_h(M, mm));
-  const double v = cbrt(2.0 * kPi * M * f / mm);
-  const double lnv = log(v);
+  double v, lnv;
+  if (nv) {
+    const double2* tab = nv + ((size_t)s * kNModes + md) * kNodeTab;
+    v = tab[0].x;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if ((j >> k) & 1) v *= tab[2 + k].x;
+    lnv = fma((double)j, tab[1].y, tab[0].y);
+  } else {
+    const double M = t[0] * kMsunS;
+    const double f = kFmin * exp(j * node_h(M, mm));
+    v = cbrt(2.0 * kPi * M * f / mm);
+    lnv = log(v);
+  }
   const double r = 0.5 * mm * (psi_of(S[s], v, lnv, nullptr) - psi_of(S0[s], v, lnv, nullptr));
   const int p = S[s].md[md].p;
   const double a = hmag_of(md, t[1]) * (p >= 1 ? v : 1.0) * (p >= 2 ? v : 1.0);
@@ -294,10 +307,17 @@ __device__ __forceinline__ void node_links_f32(const DetDev& D, const SampleCoef
 // MIX: the phase, t_f, the orbit angle and the centre Doppler term stay FP64 as above; the link
 // transfer functions are FP32 (node_links_f32), and quantities 1..6 are written as floats into the
 // first half of their rows (k_spline's mixed path reads them so).
-template <bool MIX>
+// kNodesFp64, kNodesMixed: as the call's precision; kNodesFx: FP64 with the links' transfer functions from the fixed-point
+// unit where a = pi f L < 4 (1024 samples: 1.17 ms with the FP64 geometry).
+constexpr int kNodesFp64 = 0, kNodesMixed = 1, kNodesFx = 2;
+template <int KIND>
 __global__ void k_sur_nodes(DetSet ds, int B, const SampleCoef* S, const SampleCoef* S0, const float* Y,
                             const double* theta, SurBox bx, const double* hs, const double2* nv,
                             const float4* __restrict__ nvw, double* nodes) {
+  static_assert(kNodes % kTileBins == 0, "a CTA's nodes belong to one (detector, sample, mode)");
+  constexpr bool MIX = KIND == kNodesMixed, FX = KIND == kNodesFx;
+  __shared__ fx pc[FX ? kProj : 1];
+  __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long total = (long long)ds.ndet * B * kNModes * kNodes;
   if (i >= total) return;
@@ -394,6 +414,33 @@ __global__ void k_sur_nodes(DetSet ds, int B, const SampleCoef* S, const SampleC
   else drdu = y[j + 1] - y[j - 1];
   drdu *= 0.5 / h;
   const double tf = fma(invf, fma(C.tffac, D0, drdu * (0.5 / kPi)), Sa.tc);
+  if constexpr (FX) {
+    fx_proj_prologue(D, Sa, pc);
+    const double a4 = 0.25 * kPi * f * D.L;
+    if (a4 < 0.999) {
+      const fxc ca = fx_cis(fx_turns(fma(tf, D.rate_t, D.alpha0_t)), ds.d[0].fcis);
+      const double kx = D.R * fma(Sa.k[0], fx_to_double(ca.c, -60), Sa.k[1] * fx_to_double(ca.s, -60));
+      FxAcc acc;
+      fx_zero(acc, &fxcol[0][threadIdx.x]);
+      acc.E = max(fx_expo(C.Pp), fx_expo(C.Pc2));
+      const int ash = 1079 - acc.E;
+      fxs ob[4];
+      fx_basis(ca, true, ob);   // heliocentric (geocentric nodes are skipped)
+      fx_links(fx_split(fx_from_bits(f * D.L * (1.0 / 6.0), 60)), fx_from_bits(a4, 60), 0,
+               fx_split(fx_from_bits(C.Pp, ash)), fx_split(fx_from_bits(C.Pc2, ash)), nullptr, 0.0, ash, ob, true, acc,
+               ds.d[0].fcis, ds.d[0].fsinc, pc);
+      const fxc z = fx_cis(0 - fx_turns(f * D.L), ds.d[0].fcis);   // e^{-2 i a}
+      fx xr[3], xi[3];
+      xyz_from_fx(acc, fx_split(z.c), fx_split(z.s), xr, xi);
+      q[0 * kNodes] = C.ph0 - (0.5 * mm * psi0 + r) * (0.5 / kPi) - f * kx;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        q[(1 + 2 * c) * kNodes] = fx_to_double(xr[c], acc.E - 1078) * amp_ratio;
+        q[(2 + 2 * c) * kNodes] = fx_to_double(xi[c], acc.E - 1078) * amp_ratio;
+      }
+      return;
+    }
+  }
   double xc[3], dl[3][3];
   orbit_offsets(D, tf, xc, dl, D.sct);
   const double kxc = Sa.k[0] * xc[0] + Sa.k[1] * xc[1] + Sa.k[2] * xc[2];
@@ -767,38 +814,53 @@ __global__ void k_node_h(const double* theta, int B, double* hs, double2* nv, fl
 // spline (cf, quantity 0; ~1e5 turns) is evaluated in FP64; the transfer functions T (cft, FP32
 // copies of quantities 1..6, smooth and of order one relative to their own scale) and their
 // products with H in FP32, with H carried times the sample's power of two hsc.
-// h, ih: the mode's node spacing in ln f and its inverse (formed once per tile).
-__device__ __forceinline__ void mode_bin_sur(const ModeCoef& C, double ampN, double hsc, const BinIn& B, double u,
-                                             const double* cf, const float* cft, double h, double ih, float2 acc[3],
-                                             const double2* __restrict__ tab) {
-  const double uj = (u - kLnFmin) * ih;
-  int j = (int)floor(uj);
+// The phase's sine and cosine come from the fixed-point table (pe_fx.cuh, 2^-56), their products with the amplitude
+// are formed in fixed point and rounded to FP32 once: 6 FP64 operations per unit instead of 35, which bound
+// the kernel (1024 in-box samples, 2^22 s).
+// u0 = ln f - ln kFmin, u0f the same in FP32 (a bin within rounding of a node may take the neighbouring segment,
+// whose cubic agrees there to the spline's C2 continuity), fm76 = f^(-7/6), frc = f t_c modulo one turn (per bin);
+// ampN: the Newtonian amplitude times hsc, h, ihf: the node spacing in ln f and its inverse (per tile).
+__device__ __forceinline__ void mode_bin_sur(const ModeCoef& C, double ampN, double f, double fm76, double u0, float u0f,
+                                             fxu frc, const double* cf, const float* cft, double h, float ihf,
+                                             float2 acc[3], const FxCis* __restrict__ tab) {
+  int j = (int)floorf(u0f * ihf);
   j = j < 0 ? 0 : (j > kNodes - 2 ? kNodes - 2 : j);
-  const double t = (uj - j) * h;
+  const double t = fma(-h, (double)j, u0);
   const double* c0 = cf + (size_t)j * 4;
   const double ph = fma(fma(fma(c0[3], t, c0[2]), t, c0[1]), t, c0[0]);
-  const float tf = (float)t;
+  const float tf = trunc_to_float((unsigned long long)__double_as_longlong(t));
   float val[kQ - 1];
 #pragma unroll
   for (int k = 0; k < kQ - 1; ++k) {
     const float4 c = *reinterpret_cast<const float4*>(cft + ((size_t)k * (kNodes - 1) + j) * 4);
     val[k] = fmaf(fmaf(fmaf(c.w, tf, c.z), tf, c.y), tf, c.x);
   }
-  double w = 1.0;
-  if (B.f > C.ftap) {
+  double amp = ampN * fm76;   // Newtonian power law; the mode factor |H_lm| is in T
+  if (dlt_pos(C.ftap, f)) {
     const double span = C.fend - C.ftap;
-    const double zt = span / (C.fend - B.f) - span / (B.f - C.ftap);
-    w = (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
+    const double zt = span / (C.fend - f) - span / (f - C.ftap);
+    amp *= (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
   }
-  double sph, cph;
-  sincos_turns(ph - B.frc, tab, &sph, &cph);
-  const double amp = ampN * hsc * B.fm76 * w;  // Newtonian power law; the mode factor |H_lm| is in T
-  const float hr = (float)(amp * cph), hi = (float)(amp * sph);
+  // amp = A 2^(E - 1022 - 60), A in [2^59, 2^60); hr, hi = amp cos, amp sin
+  const int E = fx_expo(amp);
+  const fxs A = fx_split(fx_from_bits(amp, 1082 - E));
+  const fxc e = fx_cis(fx_turns(ph) - frc, tab);
+  const float sc = E > 935 ? __int_as_float((E - 925) << 23) : 0.f;   // 2^(E - 1022 - 30)
+  const float hr = (float)(int)(fx_mul(A, fx_split(e.c)) >> 30) * sc;
+  const float hi = (float)(int)(fx_mul(A, fx_split(e.s)) >> 30) * sc;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     acc[c].x = fmaf(hr, val[2 * c], fmaf(-hi, val[2 * c + 1], acc[c].x));
     acc[c].y = fmaf(hr, val[2 * c + 1], fmaf(hi, val[2 * c], acc[c].y));
   }
+}
+// x p2 in FP64 for a power of two p2 (exact; through the exponent fields, x = 0 or below FP32's normal range gives 0)
+__device__ __forceinline__ double scale_up(float x, double p2) {
+  const unsigned u = (unsigned)__float_as_int(x);
+  const int e = (int)((u >> 23) & 0xff);
+  if (e == 0) return 0.0;
+  return __hiloint2double((int)((u & 0x80000000u) | ((u & 0x7fffffu) >> 3)) + ((e + 896 + fx_expo(p2) - 1023) << 20),
+                          (int)(u << 29));
 }
 
 // mode_bin_sur on the FP32 pipe. The phase spline (up to ~1e5 turns) is evaluated in double words
@@ -861,29 +923,27 @@ __device__ __forceinline__ int find_pair_s(const long long* off, int P, long lon
   return lo;
 }
 
-// Persistent kernel over the same tile list as the FP64 k_loglike_fwd (kTileBins bins per tile,
-// one bin per thread, the same order of the sums), FP64 unit. mode 0: surrogate path (in-box
-// samples on heliocentric detectors) or plain path (the others), partials [tile][6] as the plain
-// kernel; mode 1: mismatch sums of the surrogate against the plain signal, partials [tile][6] =
-// (<s|p>, <s|s>, <p|p>, 0, 0, 0). The mixed-precision variant is k_sur_inbox (in-box tiles) plus
-// k_loglike_fwd itself (the other tiles).
+// Mismatch sums of the surrogate against the plain per-bin signal, FP64, over the same tile list as k_loglike_fwd
+// (kTileBins bins per tile, one bin per thread): partials [tile][6] = (<s|p>, <s|s>, <p|p>, 0, 0, 0), with the plain
+// signal itself as s where the pair takes no spline path. (log L: k_sur_inbox or k_sur_in64 on the in-box tiles and
+// k_loglike_fwd itself on the others.)
 constexpr int kSurInboxCtas = 8;    // resident CTAs per SM asked of the in-box kernel (k_sur_inbox)
 // consecutive tiles (bins per thread) k_sur_inbox takes at a time; measured on 1024 in-box samples,
 // whole call: 1 tile 1.16 ms, 2 tiles 1.29 ms (64 registers, 8 CTAs per SM), 1.45 ms (6 CTAs per SM)
 constexpr int kSurInboxBins = 1;
+template <bool FX>
 __global__ void __launch_bounds__(kTileBins, 3) k_sur_fwd(DetSet ds, int B, const SampleCoef* __restrict__ coef,
                                                         const SampleCoef* __restrict__ coefN,
                                                         const double* __restrict__ theta, SurBox bx,
                                                         const double* __restrict__ spl, const float* __restrict__ splt,
                                                         const double* __restrict__ hs,
                                                         const int* __restrict__ nend, const long long* __restrict__ off,
-                                                        double* part, int mode) {
+                                                        double* part) {
   __shared__ double red[6][kTileBins + kRedPad];   // block_sum6 staging
   __shared__ double pc[kProj];
-  __shared__ double ihs[kNModes];
-  __shared__ double2 stab[kSinTab];
-  for (int i = threadIdx.x; i < kSinTab; i += blockDim.x) stab[i] = ds.d[0].sct[i];
-  __syncthreads();
+  __shared__ double ampn[kNModes];
+  __shared__ float ihs[kNModes];
+  __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   const int P = ds.ndet * B;
   const long long total = off[P];
   int p = 0;
@@ -895,47 +955,62 @@ __global__ void __launch_bounds__(kTileBins, 3) k_sur_fwd(DetSet ds, int B, cons
     const int ne = nend[p];
     const DetDev& D = ds.d[I];
     const SampleCoef& S = coef[s];
-    proj_prologue(D, S, pc);
-    if (threadIdx.x < kNModes) ihs[threadIdx.x] = 1.0 / hs[(size_t)s * kNModes + threadIdx.x];
+    if (FX)
+      fx_proj_prologue(D, S, reinterpret_cast<fx*>(pc));
+    else
+      proj_prologue(D, S, pc);
+    if (threadIdx.x < kNModes) {
+      ihs[threadIdx.x] = (float)(1.0 / hs[(size_t)s * kNModes + threadIdx.x]);
+      ampn[threadIdx.x] = coefN[s].md[threadIdx.x].amp * S.hsc;
+    }
     __syncthreads();
     {
       double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
       for (int b = b0; b < b0 + kTileBins && b < ne; b += kTileBins) {
-        BinIn Bn;
-        load_bin(D, b, S.tc, Bn);
         float2 xs[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        XYZAcc xpa;
-        xyz_zero(xpa);
-        const double u = 3.0 * Bn.lnf3;
         if (sur) {
+          const double f = D.f[b], fm76 = D.fm76[b], u0 = fma(3.0, D.lnf3[b], -kLnFmin);
+          const float u0f = trunc_to_float((unsigned long long)__double_as_longlong(u0));
+          const fxu frc = fx_cycles(f, S.tc);
 #pragma unroll 1
           for (int md = 0; md < kNModes; ++md) {
             const ModeCoef& C = S.md[md];
-            if (!C.active || !(Bn.f < C.fend)) continue;
+            if (!C.active || !dlt_pos(f, C.fend)) continue;
             const size_t sys = ((size_t)I * B + s) * kNModes + md;
-            mode_bin_sur(C, coefN[s].md[md].amp, S.hsc, Bn, u, spl + sys * kQ * (kNodes - 1) * 4,
-                         splt + sys * (kQ - 1) * (kNodes - 1) * 4, hs[(size_t)s * kNModes + md], ihs[md], xs, stab);
+            mode_bin_sur(C, ampn[md], f, fm76, u0, u0f, frc, spl + sys * kQ * (kNodes - 1) * 4,
+                         splt + sys * (kQ - 1) * (kNodes - 1) * 4, hs[(size_t)s * kNModes + md], ihs[md], xs,
+                         ds.d[0].fcis);
           }
         }
-        if (!sur || mode == 1) bin_modes(D, S, Bn, xpa, stab, pc);   // the plain path, as k_loglike_fwd
-        double2 xp[3], xsd[3];
-        xyz_final(xpa, Bn.z, xp);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) xsd[c] = make_double2((double)xs[c].x * S.ihsc, (double)xs[c].y * S.ihsc);
         double2 os[3], op[3];
-        aet_from_xyz(sur ? xsd : xp, os);
-        if (mode == 0) {
-          accum_bin(D, b, os, v);
+        if (FX) {
+          bin_aet_fx(D, S, b, op, ds.d[0], reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
         } else {
+          XYZAcc xpa;
+          double2 xp[3];
+          xyz_zero(xpa);
+          BinIn Bn;
+          load_bin(D, b, S.tc, Bn);
+          bin_modes(D, S, Bn, xpa, D.sct, pc);
+          xyz_final(xpa, Bn.z, xp);
           aet_from_xyz(xp, op);
+        }
+        if (sur) {
+          double2 xsd[3];
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const double w = D.gg[c * D.nb + b];
-            v[0] += w * (os[c].x * op[c].x + os[c].y * op[c].y);
-            v[1] += w * (os[c].x * os[c].x + os[c].y * os[c].y);
-            v[2] += w * (op[c].x * op[c].x + op[c].y * op[c].y);
-          }
+          for (int c = 0; c < 3; ++c) xsd[c] = make_double2(scale_up(xs[c].x, S.ihsc), scale_up(xs[c].y, S.ihsc));
+          aet_from_xyz(xsd, os);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) os[c] = op[c];
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const double w = D.gg[c * D.nb + b];
+          v[0] += w * (os[c].x * op[c].x + os[c].y * op[c].y);
+          v[1] += w * (os[c].x * os[c].x + os[c].y * os[c].y);
+          v[2] += w * (op[c].x * op[c].x + op[c].y * op[c].y);
         }
       }
       double a;
@@ -973,6 +1048,70 @@ __device__ __forceinline__ bool tile_sum6(const df v[6], float2 (*red)[kTileBins
   for (int g = 1; g < 16; ++g) s = dfl_add(s, red[threadIdx.x][g]);
   *out = s;
   return true;
+}
+
+// The FP64 surrogate's in-box tiles (mode 0): mode_bin_sur per (mode, bin), A/E/T, the weighted products and the tile's
+// sum in FP64 as k_loglike_fwd. A CTA walks a contiguous run of the in-box list, as k_sur_inbox, at six CTAs
+// per SM: inside k_sur_fwd, whose register count the per-bin path sets (three CTAs per SM), the same unit left the
+// warps waiting on its coefficient loads (1024 in-box samples, whole call: 5.5 ms there).
+constexpr int kSurIn64Ctas = 6;
+__global__ void __launch_bounds__(kTileBins, kSurIn64Ctas) k_sur_in64(DetSet ds, int B, const SampleCoef* __restrict__ coef,
+                                                                    const SampleCoef* __restrict__ coefN,
+                                                                    const double* __restrict__ spl,
+                                                                    const float* __restrict__ splt,
+                                                                    const double* __restrict__ hs,
+                                                                    const int* __restrict__ nend,
+                                                                    const long long* __restrict__ off,
+                                                                    const long long* __restrict__ offk, double* part) {
+  __shared__ double red[6][kTileBins + kRedPad];
+  __shared__ double ampn[kNModes], hm[kNModes];   // Newtonian amplitude times hsc; node spacing in ln f
+  __shared__ float ihf[kNModes];                  // 1/h
+  const int P = ds.ndet * B;
+  const long long total = offk[P];
+  const long long chunk = (total + gridDim.x - 1) / gridDim.x;
+  const long long tk0 = blockIdx.x * chunk;
+  const long long tk1 = tk0 + chunk < total ? tk0 + chunk : total;
+  int p = 0, pcur = -1;
+  for (long long tk = tk0; tk < tk1; ++tk) {
+    p = find_pair_s(offk, P, tk, p);
+    const int I = p / B, s = p - I * B;
+    const DetDev& D = ds.d[I];
+    const SampleCoef& S = coef[s];
+    if (p != pcur) {     // the pair's per-sample values, staged once per run of its tiles
+      __syncthreads();   // the previous pair's readers are done
+      if (threadIdx.x < kNModes) {
+        const double h = hs[(size_t)s * kNModes + threadIdx.x];
+        ampn[threadIdx.x] = coefN[s].md[threadIdx.x].amp * S.hsc;
+        hm[threadIdx.x] = h;
+        ihf[threadIdx.x] = (float)(1.0 / h);
+      }
+      __syncthreads();
+      pcur = p;
+    }
+    const int b = int(tk - offk[p]) * kTileBins + threadIdx.x;
+    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    if (b < nend[p]) {
+      const double f = D.f[b], fm76 = D.fm76[b], u0 = fma(3.0, D.lnf3[b], -kLnFmin);
+      const float u0f = trunc_to_float((unsigned long long)__double_as_longlong(u0));
+      const fxu frc = fx_cycles(f, S.tc);
+      float2 xs[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 1
+      for (int md = 0; md < kNModes; ++md) {
+        const ModeCoef& C = S.md[md];
+        if (!C.active || !dlt_pos(f, C.fend)) continue;
+        const size_t sys = ((size_t)I * B + s) * kNModes + md;
+        mode_bin_sur(C, ampn[md], f, fm76, u0, u0f, frc, spl + sys * kQ * (kNodes - 1) * 4,
+                     splt + sys * (kQ - 1) * (kNodes - 1) * 4, hm[md], ihf[md], xs, ds.d[0].fcis);
+      }
+      double2 x[3], o[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) x[c] = make_double2(scale_up(xs[c].x, S.ihsc), scale_up(xs[c].y, S.ihsc));
+      aet_from_xyz(x, o);
+      accum_bin(D, b, o, v);
+    }
+    double r;
+    if (block_sum6(v, [](double x, double y) { return x + y; }, red, &r)) part[(off[p] + (tk - offk[p])) * 6 + threadIdx.x] = r;
+  }
 }
 
 template <int NB>
@@ -1391,7 +1530,7 @@ pe_status pe_surrogate_targets(const double* theta_dev, int B, float* out_dev) {
   if (e == cudaSuccess) {
     pe::k_sur_prep<<<(B + 63) / 64, 64>>>(theta_dev, B, PE_MODE_ALL, S, S0);
     const long long n = (long long)B * pe::kNModes * pe::kNodes;
-    pe::k_targets<<<(unsigned)((n + 255) / 256), 256>>>(theta_dev, B, S, S0, out_dev, 0.0);
+    pe::k_targets<<<(unsigned)((n + 255) / 256), 256>>>(theta_dev, B, S, S0, out_dev, 0.0, nullptr);
     e = pe::launch_status();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
@@ -1577,7 +1716,8 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   aalloc(&off, P + 1);
   int *nin = nullptr, *nout = nullptr;
   long long *offin = nullptr, *offout = nullptr;
-  if (mix) {
+  const bool split = mode == 0;   // log L: the spline path's tiles and the per-bin path's in their own kernels
+  if (split) {
     aalloc(&nin, P);
     aalloc(&nout, P);
     aalloc(&offin, P + 1);
@@ -1601,24 +1741,28 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   if (e == cudaSuccess) {
     const long long n = (long long)B * pe::kNout;
     pe::k_sur_prep<<<(B + 63) / 64, 64, 0, st>>>(theta_dev, B, mode_mask, S, S0);
+    pe::k_node_h<<<(B * pe::kNModes + 127) / 128, 128, 0, st>>>(theta_dev, B, hs, nv, nvw);
     // node values: the network's, with the plain generator's own above the network's mass-ratio
     // bound (or everywhere for node source 1)
     const long long nt = (long long)B * pe::kNModes * pe::kNodes;
     if (s->node_source == 0) {
       pe::k_destd<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s->Y, B, s->mean, s->stdv, Yd);
       if (s->box.qnet < s->box.qmax)
-        pe::k_targets<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(theta_dev, B, S, S0, Yd, s->box.qnet);
+        pe::k_targets<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(theta_dev, B, S, S0, Yd, s->box.qnet,
+                                                                       mix ? nullptr : nv);
     } else {
-      pe::k_targets<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(theta_dev, B, S, S0, Yd, 0.0);
+      pe::k_targets<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(theta_dev, B, S, S0, Yd, 0.0, mix ? nullptr : nv);
     }
-    pe::k_node_h<<<(B * pe::kNModes + 127) / 128, 128, 0, st>>>(theta_dev, B, hs, nv, nvw);
     const long long nn = (long long)nsys * pe::kNodes;
     if (mix)
-      pe::k_sur_nodes<true><<<(unsigned)((nn + 127) / 128), 128, 0, st>>>(ds, B, S, S0, Yd, theta_dev, s->box, hs,
+      pe::k_sur_nodes<pe::kNodesMixed><<<(unsigned)((nn + 127) / 128), 128, 0, st>>>(ds, B, S, S0, Yd, theta_dev, s->box, hs,
                                                                           nv, nvw, nodes);
     else
-      pe::k_sur_nodes<false><<<(unsigned)((nn + 127) / 128), 128, 0, st>>>(ds, B, S, S0, Yd, theta_dev, s->box, hs,
-                                                                           nv, nvw, nodes);
+    {
+      auto kern = pe::fx_all_ok(ds) ? pe::k_sur_nodes<pe::kNodesFx> : pe::k_sur_nodes<pe::kNodesFp64>;
+      kern<<<(unsigned)((nn + pe::kTileBins - 1) / pe::kTileBins), pe::kTileBins, 0, st>>>(ds, B, S, S0, Yd, theta_dev,
+                                                                                           s->box, hs, nv, nvw, nodes);
+    }
     e = pe::launch_status();
     // the spline kernel reads the node spacing per system (I, s, md): replicate per detector
     for (int I = 0; I < ndet && e == cudaSuccess; ++I)
@@ -1633,16 +1777,17 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   }
   if (e == cudaSuccess) e = pe::launch_prep(theta_dev, B, mode_mask, ds, S, nend, nullptr, st);
   if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, P, off, pe::kTileBins, st);
-  pe::TuneChoice tcm = pe::default_choice(pe::kPrecMixed);
-  if (mix) pe::lookup_tuned(ds, B, mode_mask | PE_PREC_MIXED, &tcm);
-  if (e == cudaSuccess && mix) {
+  const int prec = mix ? pe::kPrecMixed : pe::kPrecFP64;
+  pe::TuneChoice tcm = pe::default_choice(prec);
+  if (split) pe::lookup_tuned(ds, B, mode_mask | (mix ? PE_PREC_MIXED : 0u), &tcm);
+  if (e == cudaSuccess && split) {
     unsigned geo_mask = 0;
     for (int I = 0; I < ndet; ++I)
       if (ds.d[I].orbit != 0) geo_mask |= 1u << I;
     pe::k_split_nend<<<(P + 127) / 128, 128, 0, st>>>(theta_dev, ndet, B, s->box, geo_mask, nend, nin, nout);
     e = pe::launch_status();
     if (e == cudaSuccess) e = pe::launch_scan_tiles(nin, P, offin, pe::kTileBins, st);
-    // the fallback pairs' work items for the tuned mixed-precision forward kernel
+    // the fallback pairs' work items for the forward kernel of pe_loglike_batch
     if (e == cudaSuccess) e = pe::launch_scan_tiles(nout, P, offout, tcm.subtiles * pe::kTileBins, st);
   }
   if (e == cudaSuccess) {
@@ -1650,20 +1795,24 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const long long g = std::max<long long>(1, std::min<long long>(max_tiles, (long long)nsm * 8));
-    if (mix) {
-      const long long g1 = std::max<long long>(1, std::min<long long>(max_tiles, (long long)nsm * pe::kSurInboxCtas));
-      pe::k_sur_inbox<pe::kSurInboxBins><<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend,
-                                                                                off, offin, part);
+    if (split) {
+      const long long g1 = std::max<long long>(
+          1, std::min<long long>(max_tiles, (long long)nsm * (mix ? pe::kSurInboxCtas : pe::kSurIn64Ctas)));
+      if (mix)
+        pe::k_sur_inbox<pe::kSurInboxBins><<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend,
+                                                                                  off, offin, part);
+      else
+        pe::k_sur_in64<<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend, off, offin, part);
       e = pe::launch_status();
-      // fallback tiles: the mixed-precision forward kernel of pe_loglike_batch with its tuned (or
-      // default) choice, over the fallback pairs' work items; it writes each sub-tile's partial at
+      // fallback tiles: the forward kernel of pe_loglike_batch in the call's precision with its tuned
+      // (or default) choice, over the fallback pairs' work items; it writes each sub-tile's partial at
       // off[p] + its index, the same place as in the full list
       if (e == cudaSuccess)
-        e = pe::launch_loglike_fwd_variant(tcm.variant, pe::kPrecMixed, ds, B, S, nend, off, offout, tcm.subtiles,
-                                           part, pe::grid_for(tcm, max_tiles), st);
+        e = pe::launch_loglike_fwd_variant(tcm.variant, prec, ds, B, S, nend, off, offout, tcm.subtiles, part,
+                                           pe::grid_for(tcm, max_tiles), st, true);
     } else {
-      pe::k_sur_fwd<<<(unsigned)g, pe::kTileBins, 0, st>>>(ds, B, S, S0, theta_dev, s->box, spl, splt, hs, nend, off,
-                                                           part, mode);
+      auto kern = pe::fx_all_ok(ds) ? pe::k_sur_fwd<true> : pe::k_sur_fwd<false>;
+      kern<<<(unsigned)g, pe::kTileBins, 0, st>>>(ds, B, S, S0, theta_dev, s->box, spl, splt, hs, nend, off, part);
       e = pe::launch_status();
     }
   }

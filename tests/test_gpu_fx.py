@@ -1,0 +1,70 @@
+"""GPU tests of the FP64 path's fixed-point unit (pe_device_fx.cuh) where it can go wrong: both sides of the
+rule that picks it (a = pi f L against 4, the arm's eccentricity), both orbits, merger times on either side
+of zero, samples whose lowest mode is alone or vanishes inside a tile, and edges of 128-bin tiles.
+
+Tolerances: the FP64 parity bars of tests/_helpers.py (1e-10 of each quantity's scale plus the rounding
+floor both sides compute in); the unit's own errors are a few 2^-56 of unit-sized quantities, far below.
+"""
+import numpy as np
+import pytest
+
+import tests._helpers as H
+from paper_2602_12011_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def Lb():
+    from paper_2602_12011_gb300 import _lib
+    _lib.lib()
+    return _lib
+
+
+@pytest.fixture(scope="module")
+def oracle_mod():
+    from oracle import oracle as O
+    O.build()
+    return O
+
+
+# (detector, span, first bin, bins): a = pi f L at the last bin just below and above 4 for the LISA and
+# TianQin arms (the general unit takes over), an arm whose eccentricity is above the unit's bound, one-bin
+# and tile-edge grids
+GRIDS = {
+    "lisa_a_below_4": (W.LISA, 2.0 ** 14, 2300, 190),
+    "lisa_a_above_4": (W.LISA, 2.0 ** 14, 2300, 300),
+    "tianqin_a_below_4": (W.TIANQIN, 2.0 ** 11, 4450, 140),
+    "tianqin_a_above_4": (W.TIANQIN, 2.0 ** 11, 4450, 250),
+    "long_arm": (dict(W.LISA, arm_m=3.0e10), 2.0 ** 16, 7, 400),
+    "tdi15_odd_span": (dict(W.TAIJI, tdi_gen=15), 65536.0 - 321.7, 7, 129),
+    "one_bin": (W.LISA, 2.0 ** 16, 200, 1),
+    "tile_edge": (W.TAIJI, 2.0 ** 16, 7, 128),
+}
+
+
+def _samples(T, fmax):
+    """Masses whose modes end inside and beyond the grid, the single odd and even modes' corners (q = 1
+    drops the odd modes), merger times before, inside and after the span."""
+    fisco1 = 6.0 ** -1.5 / (2.0 * np.pi * 4.925490947641267e-6)     # of one solar mass
+    th = W.draw_prior(8, 17, T)
+    th[:, 0] = np.clip(fisco1 * np.array([0.6, 1.3, 1.9, 2.2, 3.1, 3.9, 4.2, 9.0]) / fmax, 1e3, 1e9)
+    th[2, 1] = 1.0
+    th[3, 10] = -0.3 * T
+    th[4, 10] = 0.0
+    th[5, 10] = 1.7 * T
+    return th
+
+
+@pytest.mark.parametrize("mask", [W.MODE_ALL, 0x10, 0x09])
+@pytest.mark.parametrize("name", sorted(GRIDS))
+def test_fixed_point_unit_parity(oracle_mod, Lb, name, mask):
+    det, T, k0, nb = GRIDS[name]
+    fmax = (k0 + nb - 1) / T
+    th = _samples(T, fmax)
+    od = H.oracle_detector(oracle_mod, det, T, k0, nb, th[0], mask, 23)
+    gd = H.library_detector(Lb, od)
+    g = Lb.loglike([gd], th, mask, dhhh=True)
+    ll, dhhh = oracle_mod.loglike_batch([od], th, mask)
+    dd = np.array([oracle_mod.loglike([od], th[0], 0)["dd"][0]])
+    H.assert_loglike_parity(g, ll, dhhh, dd, H.floor_terms(oracle_mod, [od], th, mask))

@@ -40,7 +40,7 @@ __device__ __forceinline__ double dsinc(double u, double cosu, double sincu) {
 
 // Reverse sweep of one unit. sX, sY, sZ: cotangents of this bin's brackets X', Y', Z'. md2 >= 0
 // adds a second mode with the same m through this unit (complex polarisation weights
-// Pp + kappa Pp2, Pc + kappa Pc2, kappa = k32 v^2; see SampleCoefT::k32), as the forward unit does.
+// Pp + kappa Pp2, Pc + kappa Pc2, kappa = k32 v^2; see SampleCoef::k32), as the forward unit does.
 __device__ __forceinline__ void mode_bwd(const DetDev& D, const SampleCoef& S, const SampleGrad& SG, int md,
                                          const BinIn& B, double2 sX, double2 sY, double2 sZ, GradAcc& g,
                                          const double2* __restrict__ tab, int md2 = -1) {

@@ -4,7 +4,6 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include "pe_dual.cuh"
 #include "pe_internal.h"
 
 namespace pe {
@@ -48,8 +47,7 @@ __device__ __forceinline__ void sincos_turns_r(double r, const double2* __restri
 
 // -2Y_lm(iota, 0) closed forms for the ten (l, +-m) the five modes need; ci, si: cos, sin of iota;
 // c2, s2: cos, sin of iota/2.
-template <class T>
-__device__ inline void sylm_pair(int l, int m, const T& ci, const T& si, const T& c2, const T& s2, T* ypos, T* yneg) {
+__device__ inline void sylm_pair(int l, int m, double ci, double si, double c2, double s2, double* ypos, double* yneg) {
   const double pi = kPi;
   if (l == 2 && m == 2) {
     *ypos = sqrt(5.0 / (64.0 * pi)) * (1.0 + ci) * (1.0 + ci);
@@ -58,15 +56,15 @@ __device__ inline void sylm_pair(int l, int m, const T& ci, const T& si, const T
     *ypos = sqrt(5.0 / (16.0 * pi)) * si * (1.0 + ci);
     *yneg = sqrt(5.0 / (16.0 * pi)) * si * (1.0 - ci);
   } else if (l == 3 && m == 3) {
-    const T c4 = c2 * c2 * c2 * c2, s4 = s2 * s2 * s2 * s2;
+    const double c4 = c2 * c2 * c2 * c2, s4 = s2 * s2 * s2 * s2;
     *ypos = -sqrt(21.0 / (2.0 * pi)) * c4 * c2 * s2;
     *yneg = sqrt(21.0 / (2.0 * pi)) * c2 * s4 * s2;
   } else if (l == 3 && m == 2) {
-    const T c4 = c2 * c2 * c2 * c2, s4 = s2 * s2 * s2 * s2;
+    const double c4 = c2 * c2 * c2 * c2, s4 = s2 * s2 * s2 * s2;
     *ypos = 0.5 * sqrt(7.0 / pi) * c4 * (3.0 * ci - 2.0);
     *yneg = sqrt(7.0 / (4.0 * pi)) * (3.0 * ci + 2.0) * s4;
   } else {  // (4, 4)
-    const T cc = c2 * c2, ss = s2 * s2;
+    const double cc = c2 * c2, ss = s2 * s2;
     *ypos = 3.0 * sqrt(7.0 / pi) * cc * cc * cc * ss;
     *yneg = 3.0 * sqrt(7.0 / pi) * cc * ss * ss * ss;
   }
@@ -96,30 +94,30 @@ __device__ inline bool theta_valid(const double* th) {
 //  TaylorF2 phase (Buonanno et al. 2009 3.5PN; 1.5PN spin-orbit, 2PN aligned spin-spin),
 //  SPA amplitudes of the leading-order spherical modes (Blanchet 2014), C-infinity taper
 //  on the orbital frequency between 0.9 F_isco and F_isco, -2Y_lm polarisation weights
-//  (h_{l,-m} = (-1)^l h*_lm), sky frame. T = double, or Dn for derivatives with respect to theta.
+//  (h_{l,-m} = (-1)^l h*_lm), sky frame. One thread per sample: the surrogate's node preparation (pe_prep.cuh: the likelihood's).
 // ln 6, ln 4, 6^(3/2); m^(-1/3) and ln(m)/3 for m = 0..4 (index m)
 constexpr double kLn6 = 1.791759469228055, kLn4 = 1.3862943611198906, k6Pow15 = 14.696938456699069;
 __device__ constexpr double kCbrtInv[5] = {0.0, 1.0, 0.7937005259840998, 0.6933612743506348, 0.6299605249474366};
 __device__ constexpr double kLnM3[5] = {0.0, 0.0, 0.23104906018664842, 0.3662040962227033, 0.46209812037329684};
 
-template <class T>
-__device__ inline void sample_prep_t(const T* th, bool valid, unsigned mask, SampleCoefT<T>& S) {
+__device__ inline void sample_prep(const double* th, unsigned mask, SampleCoef& S) {
+  const bool valid = theta_valid(th);
   S.valid = valid ? 1 : 0;
-  const T Mtot = th[0], q = th[1], chi1 = th[2], chi2 = th[3], dL = th[4], iota = th[5];
-  const T phic = th[6], lam = th[7], bet = th[8], psi = th[9], tc = th[10];
-  const T M = Mtot * kMsunS;
-  const T D = dL * kGpcS;
-  const T eta = q / ((1.0 + q) * (1.0 + q));
-  const T m1 = q / (1.0 + q), m2 = 1.0 / (1.0 + q);
-  const T delta = (q - 1.0) / (q + 1.0);
+  const double Mtot = th[0], q = th[1], chi1 = th[2], chi2 = th[3], dL = th[4], iota = th[5];
+  const double phic = th[6], lam = th[7], bet = th[8], psi = th[9], tc = th[10];
+  const double M = Mtot * kMsunS;
+  const double D = dL * kGpcS;
+  const double eta = q / ((1.0 + q) * (1.0 + q));
+  const double m1 = q / (1.0 + q), m2 = 1.0 / (1.0 + q);
+  const double delta = (q - 1.0) / (q + 1.0);
   const double pi = kPi;
-  const T bso = chi1 * (113.0 / 12.0 * m1 * m1 + 25.0 / 4.0 * eta) + chi2 * (113.0 / 12.0 * m2 * m2 + 25.0 / 4.0 * eta);
-  const T sss = 79.0 / 8.0 * eta * chi1 * chi2;
-  const T a5c = pi * (38645.0 / 756.0 - 65.0 / 9.0 * eta);
-  const T a6c = 11583231236531.0 / 4694215680.0 - 640.0 / 3.0 * pi * pi - 6848.0 / 21.0 * kEulerGamma +
+  const double bso = chi1 * (113.0 / 12.0 * m1 * m1 + 25.0 / 4.0 * eta) + chi2 * (113.0 / 12.0 * m2 * m2 + 25.0 / 4.0 * eta);
+  const double sss = 79.0 / 8.0 * eta * chi1 * chi2;
+  const double a5c = pi * (38645.0 / 756.0 - 65.0 / 9.0 * eta);
+  const double a6c = 11583231236531.0 / 4694215680.0 - 640.0 / 3.0 * pi * pi - 6848.0 / 21.0 * kEulerGamma +
                 (-15737765635.0 / 3048192.0 + 2255.0 / 12.0 * pi * pi) * eta + 76055.0 / 1728.0 * eta * eta -
                 127825.0 / 1296.0 * eta * eta * eta;
-  const T n = 3.0 / (128.0 * eta);
+  const double n = 3.0 / (128.0 * eta);
   S.tc = tc;
   S.P[0] = n;
   S.P[1] = 0.0 * n;
@@ -134,32 +132,32 @@ __device__ inline void sample_prep_t(const T* th, bool valid, unsigned mask, Sam
   S.Q5 = n * 3.0 * a5c;
   S.Q6 = n * (-6848.0 / 21.0);
   // sky frame
-  T sl, cl, sb, cb, sp, cp;
+  double sl, cl, sb, cb, sp, cp;
   sincos(lam, &sl, &cl);
   sincos(bet, &sb, &cb);
   sincos(psi, &sp, &cp);
   S.k[0] = -(cb * cl); S.k[1] = -(cb * sl); S.k[2] = -sb;
-  const T u[3] = {sl, -cl, 0.0 * sl};
-  const T v[3] = {-(sb * cl), -(sb * sl), cb};
+  const double u[3] = {sl, -cl, 0.0 * sl};
+  const double v[3] = {-(sb * cl), -(sb * sl), cb};
   for (int i = 0; i < 3; ++i) { S.p[i] = cp * u[i] + sp * v[i]; S.q[i] = -(sp * u[i]) + cp * v[i]; }
-  for (int i = 0; i < 3; ++i) S.kw[i] = to_dw(val(S.k[i]));
-  for (int k = 0; k < 8; ++k) S.Pdw[k] = to_dw(val(S.Pd[k]));
-  for (int k = 0; k < 8; ++k) S.Pw[k] = to_dw(val(S.P[k]));
-  S.Q5w = to_dw(val(S.Q5));
-  S.Q6w = to_dw(val(S.Q6));
-  S.tcw = to_dw(val(S.tc));
+  for (int i = 0; i < 3; ++i) S.kw[i] = to_dw((S.k[i]));
+  for (int k = 0; k < 8; ++k) S.Pdw[k] = to_dw((S.Pd[k]));
+  for (int k = 0; k < 8; ++k) S.Pw[k] = to_dw((S.P[k]));
+  S.Q5w = to_dw((S.Q5));
+  S.Q6w = to_dw((S.Q6));
+  S.tcw = to_dw((S.tc));
   // modes: (2 pi M / m)^(1/3) = (2 pi M)^(1/3) m^(-1/3) and its log from one cube root and one
   // log per sample; the spin-weighted harmonics share the sines and cosines of iota and iota/2
-  const T Fisco = 1.0 / (k6Pow15 * 2.0 * pi * M);
-  const T cm1 = cbrt(2.0 * pi * M);
-  const T lncm1 = log(cm1);
-  T ci, si, c2h, s2h;
+  const double Fisco = 1.0 / (k6Pow15 * 2.0 * pi * M);
+  const double cm1 = cbrt(2.0 * pi * M);
+  const double lncm1 = log(cm1);
+  double ci, si, c2h, s2h;
   sincos(iota, &si, &ci);
   sincos(0.5 * iota, &s2h, &c2h);
   for (int md = 0; md < kNModes; ++md) {
-    ModeCoefT<T>& C = S.md[md];
+    ModeCoef& C = S.md[md];
     const int l = kModeL[md], m = kModeM[md];
-    T hmag;          // |H_lm| / x^(p/2)
+    double hmag;          // |H_lm| / x^(p/2)
     double argt;     // arg(conj H_lm) in turns
     int p;
     if (md == 0) { hmag = 1.0 + 0.0 * q; argt = 0.0; p = 0; }
@@ -171,14 +169,14 @@ __device__ inline void sample_prep_t(const T* th, bool valid, unsigned mask, Sam
     C.icm = 1.0 / C.cm;
     C.lncm = lncm1 - kLnM3[m];
     C.amp = 2.0 * pi * M * M / D * sqrt(eta / (3.0 * m)) * hmag * (C.icm * C.icm * C.icm / sqrt(C.cm));
-    const T icm2 = C.icm * C.icm;
+    const double icm2 = C.icm * C.icm;
     C.icm5 = icm2 * icm2 * C.icm;
     C.ampp = p == 0 ? C.amp : (p == 1 ? C.amp * C.cm : C.amp * C.cm * C.cm);
-    const T ph = m * phic / (2.0 * pi) + (0.125 + argt);
+    const double ph = m * phic / (2.0 * pi) + (0.125 + argt);
     C.ph0 = ph - rint(ph);
     C.mfac = 0.0 * q + m / (4.0 * pi);
     C.tffac = 0.0 * q + m / (12.0 * pi);
-    T yp, yn;
+    double yp, yn;
     sylm_pair(l, m, ci, si, c2h, s2h, &yp, &yn);
     const double sgn = (l % 2) ? -1.0 : 1.0;
     C.Pp = 0.5 * (yp + sgn * yn);
@@ -186,35 +184,31 @@ __device__ inline void sample_prep_t(const T* th, bool valid, unsigned mask, Sam
     C.Pc2 = sgn * yn - yp;
     C.fend = double(m) * Fisco;
     C.ftap = 0.9 * double(m) * Fisco;
-    C.Ppw = to_dw(val(C.Pp));
-    C.Pcw = to_dw(val(C.Pc));
-    C.tffacw = to_dw(val(C.tffac));
-    C.ph0w = to_dw(val(C.ph0));
+    C.Ppw = to_dw((C.Pp));
+    C.Pcw = to_dw((C.Pc));
+    C.tffacw = to_dw((C.tffac));
+    C.ph0w = to_dw((C.ph0));
     C.p = p;
-    C.active = (valid && (mask & (1u << md)) && val(hmag) != 0.0) ? 1 : 0;
+    C.active = (valid && (mask & (1u << md)) && (hmag) != 0.0) ? 1 : 0;
   }
-  const double a0 = val(S.md[0].amp);
+  const double a0 = (S.md[0].amp);
   const int e0 = (a0 > 0.0 && isfinite(a0)) ? ilogb(a0) : 0;
   S.hsc = scalbn(1.0, -e0);
   S.ihsc = scalbn(1.0, e0);
   for (int md = 0; md < kNModes; ++md) {
-    S.md[md].cmw = to_dw(val(S.md[md].cm));
-    S.md[md].ampw = to_dw(val(S.md[md].amp) * S.hsc);
+    S.md[md].cmw = to_dw((S.md[md].cm));
+    S.md[md].ampw = to_dw((S.md[md].amp) * S.hsc);
   }
   S.pair32 = (S.md[0].active && S.md[3].active) ? 1 : 0;
   S.k32 = make_double2(0.0, 0.0);
   if (S.pair32) {
     double sd, cd;
-    sincospi(2.0 * (val(S.md[3].ph0) - val(S.md[0].ph0)), &sd, &cd);
-    const double r = val(S.md[3].amp) / val(S.md[0].amp);
+    sincospi(2.0 * ((S.md[3].ph0) - (S.md[0].ph0)), &sd, &cd);
+    const double r = (S.md[3].amp) / (S.md[0].amp);
     S.k32 = make_double2(r * cd, r * sd);
   }
   S.k32w[0] = to_dw(S.k32.x);
   S.k32w[1] = to_dw(S.k32.y);
-}
-
-__device__ inline void sample_prep(const double* th, unsigned mask, SampleCoef& S) {
-  sample_prep_t<double>(th, theta_valid(th), mask, S);
 }
 
 // Spacecraft offsets delta_i from the constellation centre and the centre x_c, at time t.

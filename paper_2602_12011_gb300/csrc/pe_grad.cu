@@ -1,8 +1,7 @@
 // pe_grad.cu -- kernels of the gradient (row G1) and Fisher matrix (row G2) of the Whittle
 // log-likelihood (arXiv:2602.12011 Sec. 2.2 and the automatic-differentiation discussion of
 // Sec. 2.3), built on the hand-written reverse sweep in pe_adjoint.cuh:
-//   k_prep_grad     per-sample coefficients (values) plus their derivatives in theta, the
-//                   latter by device dual numbers over the 11 parameters
+//   k_prep          per-sample coefficients and their derivatives in theta (pe_prep.cuh)
 //   k_grad_fwd_tape FP64, persistent, two 128-thread CTAs per SM (mixed: three): per bin the forward mode sum
 //                   writing each unit's tape (the CTA's region of global memory), the cotangents of the A/E/T
 //                   sums dL/dB_c = conj(dg_c) - gg_c B_c, one reverse sweep per mode from the
@@ -21,6 +20,7 @@
 #include "pe_adjoint_tape_mixed.cuh"
 #include "pe_grad.h"
 #include "pe_fault.h"
+#include "pe_prep.cuh"
 
 namespace pe {
 
@@ -28,64 +28,6 @@ constexpr int kGradW = 23;   // per-tile partials: dh[3], hh[3], M q c1 c2 dL io
 constexpr int kGradV = 14;   // of which reduced by shuffles: dh[3], hh[3], M q c1 c2 dL io ph tc
 constexpr int kFisherW = 66; // unique entries of the symmetric 11 x 11 matrix
 constexpr int kFisherThreads = 32;
-
-__global__ void k_prep_grad(const double* theta, int B, unsigned mask, DetSet ds, SampleCoef* coef,
-                            SampleGrad* sgrad, int* nend, int* status) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= B) return;
-  const double* th = theta + (size_t)s * PE_NPARAM;
-  const bool valid = theta_valid(th);
-  SampleCoef S;
-  sample_prep_t<double>(th, valid, mask, S);
-  coef[s] = S;
-  SampleGrad G;
-  {
-    Dn td[PE_NPARAM];
-    for (int i = 0; i < PE_NPARAM; ++i) td[i] = dvar(th[i], i);
-    SampleCoefT<Dn> SD;
-    sample_prep_t<Dn>(td, valid, mask, SD);
-    for (int k = 0; k < 8; ++k) G.dP_dq[k] = SD.P[k].d[1];
-    for (int k = 0; k < 8; ++k) G.dPd_dq[k] = double(k - 5) * G.dP_dq[k];
-    G.dQ5_dq = SD.Q5.d[1];
-    G.dQ6_dq = SD.Q6.d[1];
-    G.dP3_dc1 = SD.P[3].d[2];
-    G.dP4_dc1 = SD.P[4].d[2];
-    G.dP3_dc2 = SD.P[3].d[3];
-    G.dP4_dc2 = SD.P[4].d[3];
-    G.dlnA_ddL = -1.0 / th[4];
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) {
-        G.dk[i][j] = SD.k[i].d[7 + j];
-        G.dp[i][j] = SD.p[i].d[7 + j];
-        G.dq[i][j] = SD.q[i].d[7 + j];
-      }
-    for (int md = 0; md < kNModes; ++md) {
-      const ModeCoefT<Dn>& C = SD.md[md];
-      ModeGrad& M = G.md[md];
-      const double a = C.amp.v;
-      M.dlnA_dM = (a != 0.0) ? C.amp.d[0] / a : 0.0;
-      M.dlnA_dq = (a != 0.0) ? C.amp.d[1] / a : 0.0;
-      M.dcm_dM = C.cm.d[0];
-      M.dfend_dM = C.fend.d[0];
-      M.dPp_di = C.Pp.d[5];
-      M.dPc_di = C.Pc.d[5];
-    }
-  }
-  sgrad[s] = G;
-  double fmax = 0.0;
-  for (int md = 0; md < kNModes; ++md)
-    if (S.md[md].active) fmax = fmax > S.md[md].fend ? fmax : S.md[md].fend;
-  for (int I = 0; I < ds.ndet; ++I) {
-    const DetDev& D = ds.d[I];
-    int n = 0;
-    if (fmax > 0.0) {
-      const double kx = ceil(fmax * D.T) - double(D.k0) + 1.0;
-      n = kx <= 0.0 ? 0 : (kx >= double(D.nb) ? D.nb : int(kx));
-    }
-    nend[I * B + s] = n;
-  }
-  if (status) status[s] = valid ? 0 : 1;
-}
 
 __device__ __forceinline__ int find_pair_g(const long long* off, int P, long long t) {
   int lo = 0, hi = P;
@@ -367,8 +309,23 @@ __global__ void __launch_bounds__(kTileBins, 2) k_grad_fwd_tape(DetSet ds, int B
   }
 }
 
-// One warp per sample: fixed-order sums over each detector's tiles, then logL and grad[11].
-__global__ void k_grad_reduce(DetSet ds, int B, const long long* off, const double* part, const SampleCoef* coef,
+// logL and the gradient from the per-component sums over every detector's tiles.
+__device__ __forceinline__ void grad_write(int s, double L, const double acc[kGradW], const SampleCoef* coef,
+                                           const SampleGrad* sgrad, double* logl, double* grad) {
+  const bool valid = coef[s].valid != 0;
+  if (logl) logl[s] = valid ? L : -INFINITY;
+  GradAcc g;
+  g.M = acc[6]; g.q = acc[7]; g.c1 = acc[8]; g.c2 = acc[9]; g.dL = acc[10]; g.io = acc[11]; g.ph = acc[12];
+  g.tc = acc[13];
+  for (int i = 0; i < 3; ++i) { g.k[i] = acc[14 + i]; g.p[i] = acc[17 + i]; g.qv[i] = acc[20 + i]; }
+  double out[PE_NPARAM];
+  gacc_to_theta(g, sgrad[s], out);
+  for (int i = 0; i < PE_NPARAM; ++i) grad[(size_t)s * PE_NPARAM + i] = valid ? out[i] : 0.0;
+}
+
+// Small grids (at most kGradWarpTiles tiles a detector): one warp per sample, fixed-order sums over each detector's tiles.
+constexpr int kGradWarpTiles = 64;
+__global__ void k_grad_reduce_warp(DetSet ds, int B, const long long* off, const double* part, const SampleCoef* coef,
                               const SampleGrad* sgrad, double* logl, double* grad) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -391,16 +348,42 @@ __global__ void k_grad_reduce(DetSet ds, int B, const long long* off, const doub
       for (int i = 6; i < kGradW; ++i) acc[i] += v[i];
     }
   }
-  if (lane != 0) return;
-  const bool valid = coef[s].valid != 0;
-  if (logl) logl[s] = valid ? L : -INFINITY;
-  GradAcc g;
-  g.M = acc[6]; g.q = acc[7]; g.c1 = acc[8]; g.c2 = acc[9]; g.dL = acc[10]; g.io = acc[11]; g.ph = acc[12];
-  g.tc = acc[13];
-  for (int i = 0; i < 3; ++i) { g.k[i] = acc[14 + i]; g.p[i] = acc[17 + i]; g.qv[i] = acc[20 + i]; }
-  double out[PE_NPARAM];
-  gacc_to_theta(g, sgrad[s], out);
-  for (int i = 0; i < PE_NPARAM; ++i) grad[(size_t)s * PE_NPARAM + i] = valid ? out[i] : 0.0;
+  if (lane == 0) grad_write(s, L, acc, coef, sgrad, logl, grad);
+}
+// Larger grids: one CTA per sample, thread (r, i) adds component i of the tiles r, r + 32, ... (coalesced, four loads in flight),
+// warp i adds the 32 rows (64 samples, LISA 2^22 s: 83 us with one warp per sample).
+__global__ void __launch_bounds__(kGradW * 32) k_grad_reduce(DetSet ds, int B, const long long* off, const double* part,
+                                                             const SampleCoef* coef, const SampleGrad* sgrad,
+                                                             double* logl, double* grad) {
+  __shared__ double red[kGradW][33];
+  __shared__ double v[kGradW];
+  const int s = blockIdx.x, i = threadIdx.x % kGradW, r = threadIdx.x / kGradW;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double acc[kGradW];
+  for (int k = 0; k < kGradW; ++k) acc[k] = 0.0;
+  double L = 0.0;
+  for (int I = 0; I < ds.ndet; ++I) {
+    const int p = I * B + s;
+    long long t0 = off[p], t1 = off[p + 1];
+    if (!PE_CHK(t0 >= 0 && t1 <= off[ds.ndet * B], 32)) t0 = t1;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (long long t = t0 + r; t < t1; t += 128) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (t + 32 * k < t1) a[k] += part[(t + 32 * k) * kGradW + i];
+    }
+    red[i][r] = (a[0] + a[1]) + (a[2] + a[3]);
+    __syncthreads();
+    double x = red[w][lane];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) v[w] = x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int c = 0; c < 3; ++c) L += v[c] - 0.5 * v[3 + c] - 0.5 * ds.d[I].dd[c];
+      for (int k = 6; k < kGradW; ++k) acc[k] += v[k];
+    }
+  }
+  if (threadIdx.x == 0) grad_write(s, L, acc, coef, sgrad, logl, grad);
 }
 
 // Fisher: one warp per 128-bin tile (four 32-bin passes). Per bin and per seed (Re/Im of X',
@@ -493,8 +476,7 @@ __global__ void k_fisher_reduce(DetSet ds, int B, const long long* off, const do
 
 cudaError_t launch_prep_grad(const double* theta, int B, unsigned mask, const DetSet& ds, SampleCoef* coef,
                              SampleGrad* sgrad, int* nend, int* status, cudaStream_t st) {
-  k_prep_grad<<<(B + 31) / 32, 32, 0, st>>>(theta, B, mask, ds, coef, sgrad, nend, status);
-  return pe::launch_status();
+  return prep_launch<true>(theta, B, mask, ds, coef, sgrad, nend, status, st);
 }
 cudaError_t launch_grad_fwd(const DetSet& ds, int B, const SampleCoef* coef, const SampleGrad* sgrad, const int* nend,
                             const long long* off, double* part, int grid, bool mixed, double* tape, cudaStream_t st) {
@@ -507,9 +489,12 @@ cudaError_t launch_grad_fwd(const DetSet& ds, int B, const SampleCoef* coef, con
 cudaError_t launch_grad_reduce(const DetSet& ds, int B, const long long* off, const double* part,
                                const SampleCoef* coef, const SampleGrad* sgrad, double* logl, double* grad,
                                cudaStream_t st) {
-  const int threads = 128;
-  const int grid = int(((long long)B * 32 + threads - 1) / threads);
-  k_grad_reduce<<<grid, threads, 0, st>>>(ds, B, off, part, coef, sgrad, logl, grad);
+  bool small = true;
+  for (int i = 0; i < ds.ndet; ++i) small &= (ds.d[i].nb + kTileBins - 1) / kTileBins <= kGradWarpTiles;
+  if (small)
+    k_grad_reduce_warp<<<(unsigned)(((long long)B * 32 + 127) / 128), 128, 0, st>>>(ds, B, off, part, coef, sgrad, logl, grad);
+  else
+    k_grad_reduce<<<B, kGradW * 32, 0, st>>>(ds, B, off, part, coef, sgrad, logl, grad);
   return pe::launch_status();
 }
 cudaError_t launch_fisher_fwd(const DetSet& ds, int B, const SampleCoef* coef, const SampleGrad* sgrad,

@@ -38,20 +38,17 @@ constexpr int kSinTab = 1024;   // entries of the (cos, sin) table used by sinco
 //   |H~_lm(f)| = amp f^(-7/6) v^p w(f)   (w: Planck taper, 1 for f <= ftap, 0 for f >= fend),
 //   arg H~_lm(f) = 2 pi [ ph0 - f t_c - (m/4pi) Psi_PN(v) ] (turns, before the orbit's
 //   centre Doppler term), and the mode's tensor is H~ (Pp e+ + i Pc ex).
-// Templated on the scalar so that the same code gives values (double) and, with device dual
-// numbers, their derivatives with respect to theta.
-template <class T>
-struct ModeCoefT {
-  T cm, icm, lncm;
-  T icm5;       // icm^5 (v^-5 = icm5 f^(-5/3))
-  T amp;
-  T ampp;       // amp cm^p (amp v^p = ampp f^(p/3))
-  T ph0;
-  T mfac;       // m / (4 pi)
-  T tffac;      // m / (12 pi)
-  T Pp, Pc;
-  T Pc2;        // 2 Pc (the FP64 unit folds the 2 of Fx = 2 (n.p)(n.q) into it)
-  T fend, ftap;
+struct ModeCoef {
+  double cm, icm, lncm;
+  double icm5;       // icm^5 (v^-5 = icm5 f^(-5/3))
+  double amp;
+  double ampp;       // amp cm^p (amp v^p = ampp f^(p/3))
+  double ph0;
+  double mfac;       // m / (4 pi)
+  double tffac;      // m / (12 pi)
+  double Pp, Pc;
+  double Pc2;        // 2 Pc (the FP64 unit folds the 2 of Fx = 2 (n.p)(n.q) into it)
+  double fend, ftap;
   float2 Ppw, Pcw;   // Pp, Pc as double words (FP32 pairs) for the mixed-precision path
   float2 cmw;        // cm as a double word
   float2 ampw;       // amp times the sample's hsc as a double word
@@ -63,14 +60,13 @@ struct ModeCoefT {
 
 // Per-sample coefficients. Psi_PN(v) = v^-5 sum_k P[k] v^k + ln v (Q5 + Q6 v) (TaylorF2 3.5PN,
 // already multiplied by 3/(128 eta)).
-template <class T>
-struct SampleCoefT {
-  T tc;
-  T P[8];
-  T Pd[8];              // (k - 5) P[k]: coefficients of v dPsi_PN/dv
-  T Pdd[8];             // (k - 5)^2 P[k]: coefficients of v d(v dPsi_PN/dv)/dv (reverse sweeps)
-  T Q5, Q6;
-  T k[3], p[3], q[3];   // propagation direction and polarisation frame
+struct SampleCoef {
+  double tc;
+  double P[8];
+  double Pd[8];              // (k - 5) P[k]: coefficients of v dPsi_PN/dv
+  double Pdd[8];             // (k - 5)^2 P[k]: coefficients of v d(v dPsi_PN/dv)/dv (reverse sweeps)
+  double Q5, Q6;
+  double k[3], p[3], q[3];   // propagation direction and polarisation frame
   float2 kw[3];         // k as double words
   float2 Pdw[8];        // Pd, Q6 and tc as double words (the mixed path's t_f)
   float2 Q6w, tcw;
@@ -78,7 +74,7 @@ struct SampleCoefT {
   double hsc, ihsc;     // power of two near 1/amp of the (2,2) mode and its inverse: the mixed-
                         // precision path carries amplitudes times hsc, keeping them far from the
                         // FP32 range limits
-  ModeCoefT<T> md[kNModes];
+  ModeCoef md[kNModes];
   // (3,2) shares m = 2 with (2,2), hence v, t_f, the taper and every geometric factor; its signal
   // is k32 v^2 times that of (2,2) with its own polarisation weights, k32 = (amp_32 / amp_22)
   // e^{2 pi i (ph0_32 - ph0_22)}. pair32 = 1 when both are active, and the units evaluate them
@@ -88,9 +84,6 @@ struct SampleCoefT {
   int valid;
   int pair32;
 };
-
-using ModeCoef = ModeCoefT<double>;
-using SampleCoef = SampleCoefT<double>;
 
 // Derivatives of the per-sample coefficients with respect to theta that the adjoint needs
 // (the sparsity of the map theta -> coefficients is built in: P and Q depend on q, chi1, chi2;

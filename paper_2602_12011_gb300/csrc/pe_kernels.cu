@@ -22,6 +22,7 @@
 #include "pe_device_mixed.cuh"
 #include "pe_kernels.h"
 #include "pe_fault.h"
+#include "pe_prep.cuh"
 
 namespace pe {
 
@@ -330,53 +331,40 @@ __global__ void k_sum_parts(const double* part, int n, int w, double* out) {
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// Row A1: per-sample coefficients; active bins per (detector, sample): the bins below the
-// largest active mode's taper end m F_isco (one extra bin guards the rounding of the bound;
-// every unit still checks f < fend of its own mode).
-// ------------------------------------------------------------------------------------------
-__global__ void k_prep(const double* theta, int B, unsigned mask, DetSet ds, SampleCoef* coef, int* nend,
-                       int* status) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= B) return;
-  SampleCoef S;
-  sample_prep(theta + (size_t)s * PE_NPARAM, mask, S);
-  coef[s] = S;
-  double fmax = 0.0;
-  for (int md = 0; md < kNModes; ++md)
-    if (S.md[md].active) fmax = fmax > S.md[md].fend ? fmax : S.md[md].fend;
-  for (int I = 0; I < ds.ndet; ++I) {
-    const DetDev& D = ds.d[I];
-    int n = 0;
-    if (fmax > 0.0) {
-      const double kx = ceil(fmax * D.T) - double(D.k0) + 1.0;
-      n = kx <= 0.0 ? 0 : (kx >= double(D.nb) ? D.nb : int(kx));
-    }
-    nend[I * B + s] = n;
-  }
-  if (status) status[s] = S.valid ? 0 : 1;
-}
-
-// Exclusive prefix sum of tiles (TILE bins each) per (detector, sample) pair; off[P] = total tiles.
-// One CTA.
-template <int TILE>
-__global__ void k_scan_tiles(const int* nend, int P, long long* off) {
-  __shared__ long long part[1024];
-  const int t = threadIdx.x;
+// Exclusive prefix sums of tiles per (detector, sample) pair, for tiles of 2^sa bins (off) and, if offb is not NULL, of
+// 2^sb bins (offb); off[P], offb[P] = totals. One CTA: each thread adds a run of pairs, a warp shuffle scan
+// and one over the warps join the runs (a serial pass over 1,024 partials by one thread took 8 us).
+__global__ void k_scan_tiles(const int* nend, int P, int sa, long long* off, int sb, long long* offb) {
+  __shared__ long long wsum[2][32];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int chunk = (P + blockDim.x - 1) / blockDim.x;
-  const int lo = t * chunk, hi = min(P, lo + chunk);
-  long long s = 0;
-  for (int i = lo; i < hi; ++i) s += (nend[i] + TILE - 1) / TILE;
-  part[t] = s;
-  __syncthreads();
-  if (t == 0) {
-    long long run = 0;
-    for (int i = 0; i < (int)blockDim.x; ++i) { long long v = part[i]; part[i] = run; run += v; }
-    off[P] = run;
+  const int lo = min(P, t * chunk), hi = min(P, lo + chunk);
+  long long a = 0, b = 0;
+  for (int i = lo; i < hi; ++i) {
+    const int n = nend[i];
+    a += (n + (1 << sa) - 1) >> sa;
+    b += (n + (1 << sb) - 1) >> sb;
   }
+  long long ia = a, ib = b;   // inclusive sums over the warp, then exclusive over the block
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long xa = __shfl_up_sync(0xffffffffu, ia, o), xb = __shfl_up_sync(0xffffffffu, ib, o);
+    if (lane >= o) { ia += xa; ib += xb; }
+  }
+  if (lane == 31) { wsum[0][w] = ia; wsum[1][w] = ib; }
   __syncthreads();
-  long long run = part[t];
-  for (int i = lo; i < hi; ++i) { off[i] = run; run += (nend[i] + TILE - 1) / TILE; }
+  long long ra = ia - a, rb = ib - b;
+  for (int k = 0; k < w; ++k) { ra += wsum[0][k]; rb += wsum[1][k]; }
+  for (int i = lo; i < hi; ++i) {
+    const int n = nend[i];
+    off[i] = ra;
+    if (offb) offb[i] = rb;
+    ra += (n + (1 << sa) - 1) >> sa;
+    rb += (n + (1 << sb) - 1) >> sb;
+  }
+  if (t == (int)blockDim.x - 1) {
+    off[P] = ra;
+    if (offb) offb[P] = rb;
+  }
 }
 
 // pair index p with off[p] <= t < off[p+1]
@@ -515,10 +503,10 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
   }
 }
 
-// Row A7: one warp per sample; for each detector a lane-strided, shuffle-tree sum of that
+// Row A7, small grids (at most kReduceWarpTiles tiles a detector): one warp per sample; for each detector a lane-strided, shuffle-tree sum of that
 // pair's tile partials (fixed order), then logL = sum_{I,c} (<d|h> - <h|h>/2 - <d|d>/2).
 // dhhh: [B][ndet][3][2] or NULL.
-__global__ void k_reduce(DetSet ds, int B, const long long* off, const double* part, const SampleCoef* coef,
+__global__ void k_reduce_warp(DetSet ds, int B, const long long* off, const double* part, const SampleCoef* coef,
                          double* logl, double* dhhh) {
   const int ndet = ds.ndet;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -548,6 +536,47 @@ __global__ void k_reduce(DetSet ds, int B, const long long* off, const double* p
     }
   }
   if (lane == 0) logl[s] = coef[s].valid ? L : -INFINITY;
+}
+
+// Row A7, larger grids: one CTA per sample, thread (r, i) adds component i of the tiles r, r + 32, ... in four interleaved
+// sums (coalesced reads, four loads in flight), then warp i adds the 32 rows by a shuffle tree. One warp per sample
+// waited on 50 dependent rounds of loads per detector (57 us on the three-detector network, 10 us on LISA,
+// 2^22 s). Which of the two runs depends on the grids alone, so a sample's bits do not depend on the batch.
+constexpr int kReduceWarpTiles = 64;
+__global__ void __launch_bounds__(192) k_reduce(DetSet ds, int B, const long long* off, const double* part,
+                                                const SampleCoef* coef, double* logl, double* dhhh) {
+  __shared__ double red[6][33];
+  __shared__ double v[6];
+  const int s = blockIdx.x, i = threadIdx.x % 6, r = threadIdx.x / 6;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double L = 0.0;
+  for (int I = 0; I < ds.ndet; ++I) {
+    const int p = I * B + s;
+    long long t0 = off[p], t1 = off[p + 1];
+    if (!PE_CHK(t0 >= 0 && t1 <= off[ds.ndet * B], 8)) t0 = t1;   // checked build: uniform over the CTA
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (long long t = t0 + r; t < t1; t += 128) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (t + 32 * k < t1) a[k] += part[(t + 32 * k) * 6 + i];
+    }
+    red[i][r] = (a[0] + a[1]) + (a[2] + a[3]);
+    __syncthreads();
+    double x = red[w][lane];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) v[w] = x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int c = 0; c < 3; ++c) {
+        L += v[c] - 0.5 * v[3 + c] - 0.5 * ds.d[I].dd[c];
+        if (dhhh) {
+          dhhh[(((size_t)s * ds.ndet + I) * 3 + c) * 2 + 0] = v[c];
+          dhhh[(((size_t)s * ds.ndet + I) * 3 + c) * 2 + 1] = v[3 + c];
+        }
+      }
+    }
+  }
+  if (threadIdx.x == 0) logl[s] = coef[s].valid ? L : -INFINITY;
 }
 
 // Noise-free A/E/T signal of one sample on the whole grid: h_c = Q n_c B_c. out: [3][nb].
@@ -634,23 +663,28 @@ cudaError_t launch_sum_parts(const double* part, int n, int w, double* out, cuda
 }
 cudaError_t launch_prep(const double* theta, int B, unsigned mask, const DetSet& ds, SampleCoef* coef, int* nend,
                         int* status, cudaStream_t st) {
-  k_prep<<<(B + 63) / 64, 64, 0, st>>>(theta, B, mask, ds, coef, nend, status);
-  return pe::launch_status();
+  return prep_launch<false>(theta, B, mask, ds, coef, nullptr, nend, status, st);
 }
+namespace {
+int tile_shift(int tile_bins) {   // log2 of kTileBins times 1, 2, 4 or 8; -1 otherwise
+  for (int k = 0; k < 4; ++k)
+    if (tile_bins == kTileBins << k) return 7 + k;
+  return -1;
+}
+static_assert(kTileBins == 128, "tile_shift counts from 2^7");
+int scan_threads(int P) { return P >= 1024 ? 1024 : (P + 31) / 32 * 32; }
+}  // namespace
 cudaError_t launch_scan_tiles(const int* nend, int P, long long* off, int tile_bins, cudaStream_t st) {
-  switch (tile_bins) {
-    case kTileBins: k_scan_tiles<kTileBins><<<1, 1024, 0, st>>>(nend, P, off); break;
-    case 2 * kTileBins: k_scan_tiles<2 * kTileBins><<<1, 1024, 0, st>>>(nend, P, off); break;
-    case 4 * kTileBins: k_scan_tiles<4 * kTileBins><<<1, 1024, 0, st>>>(nend, P, off); break;
-    case 8 * kTileBins: k_scan_tiles<8 * kTileBins><<<1, 1024, 0, st>>>(nend, P, off); break;
-    default: return cudaErrorInvalidValue;
-  }
+  const int sa = tile_shift(tile_bins);
+  if (sa < 0 || P < 1) return cudaErrorInvalidValue;
+  k_scan_tiles<<<1, scan_threads(P), 0, st>>>(nend, P, sa, off, sa, nullptr);
   return pe::launch_status();
 }
 cudaError_t launch_fwd_offsets(const int* nend, int P, long long* off, long long* offi, int R, cudaStream_t st) {
-  cudaError_t e = launch_scan_tiles(nend, P, off, kTileBins, st);
-  if (e == cudaSuccess && R > 1) e = launch_scan_tiles(nend, P, offi, R * kTileBins, st);
-  return e;
+  const int sb = tile_shift(R * kTileBins);
+  if (sb < 0 || P < 1) return cudaErrorInvalidValue;
+  k_scan_tiles<<<1, scan_threads(P), 0, st>>>(nend, P, 7, off, sb, R > 1 ? offi : nullptr);
+  return pe::launch_status();
 }
 cudaError_t launch_dw_tables(const double* f, const double* f13, const double* fm13, const double* fm76, const double2* sca,
                              const double2* z, const double2* tab, int nb, double L, float2* fw, float2* aw,
@@ -735,10 +769,12 @@ cudaError_t launch_loglike_fwd_variant(int variant, int prec, const DetSet& ds, 
 }
 cudaError_t launch_reduce(const DetSet& ds, int B, const long long* off, const double* part, const SampleCoef* coef,
                           double* logl, double* dhhh, cudaStream_t st) {
-  const int threads = 128;
-  const long long warps = B;
-  const int grid = int((warps * 32 + threads - 1) / threads);
-  k_reduce<<<grid, threads, 0, st>>>(ds, B, off, part, coef, logl, dhhh);
+  bool small = true;
+  for (int i = 0; i < ds.ndet; ++i) small &= tiles_of(ds.d[i].nb, kTileBins) <= kReduceWarpTiles;
+  if (small)
+    k_reduce_warp<<<(unsigned)(((long long)B * 32 + 127) / 128), 128, 0, st>>>(ds, B, off, part, coef, logl, dhhh);
+  else
+    k_reduce<<<B, 192, 0, st>>>(ds, B, off, part, coef, logl, dhhh);
   return pe::launch_status();
 }
 cudaError_t launch_signal(const DetDev& D, const SampleCoef* coef, double2* out, int prec, cudaStream_t st) {

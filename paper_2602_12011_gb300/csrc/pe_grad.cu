@@ -27,7 +27,6 @@ namespace pe {
 constexpr int kGradW = 23;   // per-tile partials: dh[3], hh[3], M q c1 c2 dL io ph tc, k[3] p[3] q[3]
 constexpr int kGradV = 14;   // of which reduced by shuffles: dh[3], hh[3], M q c1 c2 dL io ph tc
 constexpr int kFisherW = 66; // unique entries of the symmetric 11 x 11 matrix
-constexpr int kFisherThreads = 32;
 
 __device__ __forceinline__ int find_pair_g(const long long* off, int P, long long t) {
   int lo = 0, hi = P;
@@ -386,18 +385,20 @@ __global__ void __launch_bounds__(kGradW * 32) k_grad_reduce(DetSet ds, int B, c
   if (threadIdx.x == 0) grad_write(s, L, acc, coef, sgrad, logl, grad);
 }
 
-// Fisher: one warp per 128-bin tile (four 32-bin passes). Per bin and per seed (Re/Im of X',
-// Y', Z') one reverse sweep over the modes gives a Jacobian row; the rows are combined into
-// A/E/T and accumulated into the thread's 66 unique entries (kept in shared memory).
-__global__ void __launch_bounds__(kFisherThreads) k_fisher_fwd(DetSet ds, int B, const SampleCoef* __restrict__ coef,
-                                                              const SampleGrad* __restrict__ sgrad,
-                                                              const int* __restrict__ nend,
-                                                              const long long* __restrict__ off, double* part) {
-  __shared__ double Fs[kFisherW][kFisherThreads];
-  __shared__ double Js[6][PE_NPARAM][kFisherThreads];
+// Fisher: six warps per 128-bin tile, in four 32-bin passes. Per pass warp j runs the reverse sweeps of seed j (Re/Im of X',
+// Y', Z') over its lanes' bins, giving row j of the Jacobian; the warps then form the six A/E/T rows and each
+// accumulates eleven of the 66 entries. A few points give a few hundred tiles: with one warp per tile, three warps
+// an SM each ran 24 dependent sweeps of every mode (3.1 ms for three points on LISA, 2^21 s; 1.5 ms now, 1.7 at two CTAs per SM, whose 168 registers spill).
+constexpr int kFisherWarps = 6;
+__global__ void __launch_bounds__(32 * kFisherWarps, 1) k_fisher_fwd(DetSet ds, int B, const SampleCoef* __restrict__ coef,
+                                                                    const SampleGrad* __restrict__ sgrad,
+                                                                    const int* __restrict__ nend,
+                                                                    const long long* __restrict__ off, double* part) {
+  __shared__ double Js[kFisherWarps][PE_NPARAM][32];   // rows 0 Re X', 1 Im X', 2 Re Y', 3 Im Y', 4 Re Z', 5 Im Z'
+  __shared__ double Ja[kFisherWarps][PE_NPARAM][32];   // rows Re/Im of B_A, B_E, B_T
   const int P = ds.ndet * B;
   const long long total = off[P];
-  const int tid = threadIdx.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (long long t = blockIdx.x; t < total; t += gridDim.x) {
     const int p = find_pair_g(off, P, t);
     if (!PE_CHK(p >= 0 && p < P && off[p + 1] <= total && nend[p] <= ds.d[p / B].nb, 64)) continue;
@@ -405,67 +406,83 @@ __global__ void __launch_bounds__(kFisherThreads) k_fisher_fwd(DetSet ds, int B,
     const DetDev& D = ds.d[I];
     const SampleCoef& S = coef[s];
     const SampleGrad& SG = sgrad[s];
-    for (int i = 0; i < kFisherW; ++i) Fs[i][tid] = 0.0;
-    for (int sub = 0; sub < kTileBins / kFisherThreads; ++sub) {
-      const int b = int(t - off[p]) * kTileBins + sub * kFisherThreads + tid;
-      if (b >= nend[p]) continue;
-      BinIn Bn;
-      load_bin(D, b, S.tc, Bn);
-      for (int j = 0; j < 6; ++j) {
-        const double2 one = make_double2((j & 1) ? 0.0 : 1.0, (j & 1) ? 1.0 : 0.0);
+    double F[kFisherW / kFisherWarps];
+#pragma unroll
+    for (int e = 0; e < kFisherW / kFisherWarps; ++e) F[e] = 0.0;
+#pragma unroll 1
+    for (int sub = 0; sub < kTileBins / 32; ++sub) {
+      const int b = int(t - off[p]) * kTileBins + sub * 32 + lane;
+      const bool on = b < nend[p];
+      double row[PE_NPARAM];
+      if (on) {
+        BinIn Bn;
+        load_bin(D, b, S.tc, Bn);
+        const double2 one = make_double2((w & 1) ? 0.0 : 1.0, (w & 1) ? 1.0 : 0.0);
         const double2 zero = make_double2(0.0, 0.0);
-        const double2 sX = (j / 2 == 0) ? one : zero;
-        const double2 sY = (j / 2 == 1) ? one : zero;
-        const double2 sZ = (j / 2 == 2) ? one : zero;
         GradAcc g;
         gacc_zero(g);
 #pragma unroll 1
         for (int md = 0; md < kNModes; ++md) {
           if (md == 3 && S.pair32) continue;
-          if (S.md[md].active && Bn.f < S.md[md].fend)
-            mode_bwd(D, S, SG, md, Bn, sX, sY, sZ, g, D.sct, (md == 0 && S.pair32) ? 3 : -1);
+          if (S.md[md].active && dlt_pos(Bn.f, S.md[md].fend))
+            mode_bwd(D, S, SG, md, Bn, w / 2 == 0 ? one : zero, w / 2 == 1 ? one : zero, w / 2 == 2 ? one : zero, g, D.sct,
+                     (md == 0 && S.pair32) ? 3 : -1);
         }
-        double row[PE_NPARAM];
         gacc_to_theta(g, SG, row);
-        for (int i = 0; i < PE_NPARAM; ++i) Js[j][i][tid] = row[i];
+      } else {
+#pragma unroll
+        for (int i = 0; i < PE_NPARAM; ++i) row[i] = 0.0;
       }
-      // rows j: 0 Re X', 1 Im X', 2 Re Y', 3 Im Y', 4 Re Z', 5 Im Z'
-      for (int c = 0; c < 3; ++c) {
-        const double w = D.gg[c * D.nb + b];
-        for (int ri = 0; ri < 2; ++ri) {  // real and imaginary part of B_c
-          double jr[PE_NPARAM];
-          for (int i = 0; i < PE_NPARAM; ++i) {
-            const double X = Js[0 + ri][i][tid], Y = Js[2 + ri][i][tid], Z = Js[4 + ri][i][tid];
-            jr[i] = (c == 0) ? (Z - X) : (c == 1) ? (X - 2.0 * Y + Z) : (X + Y + Z);
-          }
-          int e = 0;
-          for (int i = 0; i < PE_NPARAM; ++i)
-            for (int k = i; k < PE_NPARAM; ++k, ++e) Fs[e][tid] = fma(w * jr[i], jr[k], Fs[e][tid]);
+#pragma unroll
+      for (int i = 0; i < PE_NPARAM; ++i) Js[w][i][lane] = row[i];
+      __syncthreads();
+      const int c = w >> 1, ri = w & 1;
+#pragma unroll
+      for (int i = 0; i < PE_NPARAM; ++i) {
+        const double X = Js[ri][i][lane], Y = Js[2 + ri][i][lane], Z = Js[4 + ri][i][lane];
+        Ja[w][i][lane] = (c == 0) ? (Z - X) : (c == 1) ? (X - 2.0 * Y + Z) : (X + Y + Z);
+      }
+      __syncthreads();   // the next pass writes Js and, past its barrier, Ja
+      // entries e = w, w + 6, ... of the upper triangle, row by row
+#pragma unroll 1
+      for (int r = 0; r < kFisherWarps; ++r) {
+        const double g = on ? D.gg[(r >> 1) * D.nb + b] : 0.0;
+        int i = 0, k = w;
+        while (k >= PE_NPARAM - i) { k -= PE_NPARAM - i; ++i; }
+#pragma unroll
+        for (int e = 0; e < kFisherW / kFisherWarps; ++e) {
+          F[e] = fma(g * Ja[r][i][lane], Ja[r][i + k][lane], F[e]);
+          k += kFisherWarps;
+          while (i < PE_NPARAM && k >= PE_NPARAM - i) { k -= PE_NPARAM - i; ++i; }
         }
       }
     }
-    __syncwarp();
-    // fixed-order sum over the 32 threads of each entry
-    for (int e = tid; e < kFisherW; e += kFisherThreads) {
-      double a = 0.0;
-      for (int k = 0; k < kFisherThreads; ++k) a += Fs[e][k];
-      part[t * kFisherW + e] = a;
+    // fixed-order sums over the lanes
+#pragma unroll
+    for (int e = 0; e < kFisherW / kFisherWarps; ++e) {
+      for (int o = 16; o > 0; o >>= 1) F[e] += __shfl_down_sync(0xffffffffu, F[e], o);
+      if (lane == 0) part[t * kFisherW + w + kFisherWarps * e] = F[e];
     }
-    __syncwarp();
   }
 }
 
-__global__ void k_fisher_reduce(DetSet ds, int B, const long long* off, const double* part, const SampleCoef* coef,
-                                double* F) {
+// Per point: thread (r, e) adds entry e of the tiles r, r + 8, ... over the detectors, then thread e its eight rows.
+constexpr int kFisherRows = 8;
+__global__ void __launch_bounds__(kFisherW * kFisherRows) k_fisher_reduce(DetSet ds, int B, const long long* off, const double* part,
+                                                                        const SampleCoef* coef, double* F) {
+  __shared__ double red[kFisherRows][kFisherW];
   const int s = blockIdx.x;
-  const int e = threadIdx.x;
-  if (s >= B || e >= kFisherW) return;
+  const int e = threadIdx.x % kFisherW, r = threadIdx.x / kFisherW;
   double a = 0.0;
   for (int I = 0; I < ds.ndet; ++I) {
     const int p = I * B + s;
     if (!PE_CHK(off[p] >= 0 && off[p + 1] <= off[ds.ndet * B], 128)) continue;
-    for (long long t = off[p]; t < off[p + 1]; ++t) a += part[t * kFisherW + e];
+    for (long long t = off[p] + r; t < off[p + 1]; t += kFisherRows) a += part[t * kFisherW + e];
   }
+  red[r][e] = a;
+  __syncthreads();
+  if (r != 0) return;
+  for (int k = 1; k < kFisherRows; ++k) a += red[k][e];
   if (!coef[s].valid) a = 0.0;
   int i = 0, k = 0, idx = e;
   while (idx >= PE_NPARAM - i) { idx -= PE_NPARAM - i; ++i; }
@@ -499,12 +516,12 @@ cudaError_t launch_grad_reduce(const DetSet& ds, int B, const long long* off, co
 }
 cudaError_t launch_fisher_fwd(const DetSet& ds, int B, const SampleCoef* coef, const SampleGrad* sgrad,
                               const int* nend, const long long* off, double* part, int grid, cudaStream_t st) {
-  k_fisher_fwd<<<grid, kFisherThreads, 0, st>>>(ds, B, coef, sgrad, nend, off, part);
+  k_fisher_fwd<<<grid, 32 * kFisherWarps, 0, st>>>(ds, B, coef, sgrad, nend, off, part);
   return pe::launch_status();
 }
 cudaError_t launch_fisher_reduce(const DetSet& ds, int B, const long long* off, const double* part,
                                  const SampleCoef* coef, double* F, cudaStream_t st) {
-  k_fisher_reduce<<<B, 96, 0, st>>>(ds, B, off, part, coef, F);
+  k_fisher_reduce<<<B, kFisherW * kFisherRows, 0, st>>>(ds, B, off, part, coef, F);
   return pe::launch_status();
 }
 int grad_partial_width() { return kGradW; }

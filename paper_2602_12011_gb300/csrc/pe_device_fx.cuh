@@ -92,14 +92,18 @@ __device__ __forceinline__ void load_bin_fx(const DetDev& D, int b, double tc, F
 // stay in the thread's column of shared memory, which frees 24 registers and lets the link loop stay
 // rolled.
 constexpr int kFxSums = 12;
-struct FxAcc {
-  volatile fx* s;      // entry i at s[i * kTileBins]
+template <int STRIDE>
+struct FxAccT {
+  static constexpr int kStride = STRIDE;
+  volatile fx* s;      // entry i at s[i * kStride]
   int E;
 };
-__device__ __forceinline__ void fx_zero(FxAcc& a, fx* col) {
+using FxAcc = FxAccT<kTileBins>;
+template <class Acc>
+__device__ __forceinline__ void fx_zero(Acc& a, fx* col) {
   a.s = col;
 #pragma unroll
-  for (int i = 0; i < kFxSums; ++i) a.s[i * kTileBins] = 0;
+  for (int i = 0; i < kFxSums; ++i) a.s[i * Acc::kStride] = 0;
   a.E = 0;
 }
 constexpr float kFxTauMax = 8192.f;
@@ -126,8 +130,9 @@ __device__ __forceinline__ void fx_basis(fxc g, bool helio, fxs ob[4]) {
 // One unit's link products, added to the bin's sums: phu the mode's phase (turns), Apx, Acx the polarisation weights
 // times the amplitude; for a paired second mode Ap (its imaginary part read) and Acyd complete them, scaled by
 // 2^ash.
+template <class Acc>
 __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs Acx, const double2* Ap, double Acyd, int ash,
-                                         const fxs ob[4], bool helio, FxAcc& acc, const FxCis* __restrict__ tab,
+                                         const fxs ob[4], bool helio, Acc& acc, const FxCis* __restrict__ tab,
                                          const FxSinc* __restrict__ stab, const fx* __restrict__ pc) {
   const fxs a4s = fx_split(a4);
   // --- links (row A5): projections of the link vectors over the nominal arm; the three sum to zero.
@@ -177,19 +182,20 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
     fx_mac(gi, gy, ec);
     const fxs Gi = fx_split(fx_val(gi));
     // --- sinc(a (1 +- k.n)) and the link's products for the TDI brackets (row A6; see XYZAcc)
-    volatile fx* as = acc.s + 4 * l * kTileBins;
+    volatile fx* as = acc.s + 4 * l * Acc::kStride;
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
       const fxs sc = fx_split(fx_sinc(h == 0 ? a4 + w4 : a4 - w4, stab));
       as[0] = as[0] + fx_mul(Gr, sc);
-      as[kTileBins] = as[kTileBins] + fx_mul(Gi, sc);
-      as += 2 * kTileBins;
+      as[Acc::kStride] = as[Acc::kStride] + fx_mul(Gi, sc);
+      as += 2 * Acc::kStride;
     }
   }
 }
 
+template <class Acc>
 __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S, const ModeCoef& C, const FxBin& B,
-                                            FxAcc& acc, const FxCis* __restrict__ tab, const FxSinc* __restrict__ stab,
+                                            Acc& acc, const FxCis* __restrict__ tab, const FxSinc* __restrict__ stab,
                                             const fx* __restrict__ pc, int md, const ModeCoef* C2 = nullptr) {
   // --- waveform and time-frequency map (rows A2, A3), as mode_bin
   const double v = C.cm * B.f13;
@@ -255,7 +261,7 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
     if (acc.E > 0) {
       const int sh = min(63, E - acc.E);
 #pragma unroll 1
-      for (int i = 0; i < kFxSums; ++i) acc.s[i * kTileBins] = acc.s[i * kTileBins] >> sh;
+      for (int i = 0; i < kFxSums; ++i) acc.s[i * Acc::kStride] = acc.s[i * Acc::kStride] >> sh;
     }
     acc.E = E;
   }
@@ -283,19 +289,21 @@ __device__ __forceinline__ double fx_to_double(fx n, int e) {
 // Half the brackets X', Y', Z' of one bin's sums (xyz_final), and A/E/T from them (aet_from_xyz). Each unit's |G| is below
 // 0.2 and a bin has four at most, so the brackets P and Q stay below 1.6, X', Y', Z' below 3.2 and
 // the half sums of A/E/T below 6.4.
-__device__ __forceinline__ void xyz_from_fx(const FxAcc& a, fxs zr, fxs zi, fx xr[3], fx xi[3]) {
+template <class Acc>
+__device__ __forceinline__ void xyz_from_fx(const Acc& a, fxs zr, fxs zi, fx xr[3], fx xi[3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const volatile fx* ac = a.s + 4 * c * kTileBins;                  // S_r, S_i, M_r, M_i of link c
-    const volatile fx* al = a.s + 4 * ((c + 2) % 3) * kTileBins;      // and of link c + 2
-    const fxs qr = fx_split(al[2 * kTileBins] - ac[0]), qi = fx_split(al[3 * kTileBins] - ac[kTileBins]);
-    xr[c] = ((al[0] - ac[2 * kTileBins]) + fx_sub2(fx_prod(zr, qr), fx_prod(zi, qi))) >> 1;
+    const volatile fx* ac = a.s + 4 * c * Acc::kStride;                  // S_r, S_i, M_r, M_i of link c
+    const volatile fx* al = a.s + 4 * ((c + 2) % 3) * Acc::kStride;      // and of link c + 2
+    const fxs qr = fx_split(al[2 * Acc::kStride] - ac[0]), qi = fx_split(al[3 * Acc::kStride] - ac[Acc::kStride]);
+    xr[c] = ((al[0] - ac[2 * Acc::kStride]) + fx_sub2(fx_prod(zr, qr), fx_prod(zi, qi))) >> 1;
     fxa t = fx_prod(zr, qi);
     fx_mac(t, zi, qr);
-    xi[c] = ((al[kTileBins] - ac[3 * kTileBins]) + fx_val(t)) >> 1;
+    xi[c] = ((al[Acc::kStride] - ac[3 * Acc::kStride]) + fx_val(t)) >> 1;
   }
 }
-__device__ __forceinline__ void aet_from_fx(const FxAcc& a, double2 z, double2 o[3]) {
+template <class Acc>
+__device__ __forceinline__ void aet_from_fx(const Acc& a, double2 z, double2 o[3]) {
   fx xr[3], xi[3];
   xyz_from_fx(a, fx_split(fx_from_bits(z.x, 60)), fx_split(fx_from_bits(z.y, 60)), xr, xi);
   const int e = a.E - 1078;   // one unit of the halved sums is 2^e

@@ -30,6 +30,7 @@
 namespace pe {
 
 constexpr int kHetMaxEdges = 640;
+constexpr int kHetThreads = 320;   // most threads of a CTA of k_het_loglike
 constexpr int kPairs = kNModes * (kNModes + 1) / 2;   // unordered mode pairs (md <= md2)
 
 __host__ __device__ constexpr int pair_index(int a, int b) {   // a <= b
@@ -42,8 +43,8 @@ struct HetDev {
   const double* fe;      // [ne] edge frequencies
   const double2* ih0e;   // [ne][5][3] inverses 1/h0 of the reference brackets at the edges (0 where h0 = 0)
   const int* src;        // [ne][5][3] edge whose ratio applies (carry-forward), -1 for none
-  const double2* A;      // [ne-1][5][3][2]
-  const double2* Bs;     // [ne-1][kPairs][3][3]
+  const double2* A;      // [5][3][2][ne-1]: consecutive bins are consecutive, for the contraction's loads
+  const double2* Bs;     // [kPairs][3][3][ne-1]
   const float4* Aw;      // A and Bs as double words (re hi, re lo, im hi, im lo), for the mixed kernel
   const float4* Bw;
   int ne;
@@ -75,7 +76,8 @@ __device__ __forceinline__ void mode_brackets(const DetDev& D, const SampleCoef&
   }
 }
 
-// The same with the fixed-point unit.
+// The same with the fixed-point unit (STRIDE: threads of the CTA, between the entries of a column).
+template <int STRIDE>
 __device__ __forceinline__ void mode_brackets_fx(const DetDev& D, const SampleCoef& S, int b, unsigned mask,
                                                  double2 o[kNModes][3], const DetDev& D0,
                                                  const fx* __restrict__ pc, fx* col) {
@@ -85,7 +87,7 @@ __device__ __forceinline__ void mode_brackets_fx(const DetDev& D, const SampleCo
 #pragma unroll 1
   for (int md = 0; md < kNModes; ++md) {
     const ModeCoef& C = S.md[md];
-    FxAcc a;
+    FxAccT<STRIDE> a;
     fx_zero(a, col);
     if ((mask >> md) & 1u && C.active && Bn.f < C.fend) mode_bin_fx(D, S, C, Bn, a, D0.fcis, D0.fsinc, pc, md);
     aet_from_fx(a, z, o[md]);
@@ -130,7 +132,7 @@ __global__ void k_mode_brackets(DetDev D, const SampleCoef* coef, int K, unsigne
   if (k >= K) return;
   double2 o[kNModes][3];
   if (FX)
-    mode_brackets_fx(D, S, k, mask, o, D, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
+    mode_brackets_fx<kTileBins>(D, S, k, mask, o, D, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
   else
     mode_brackets(D, S, k, mask, o, D.sct, pc);
   for (int md = 0; md < kNModes; ++md)
@@ -176,7 +178,7 @@ __global__ void k_het_summary(DetDev D, const int* edge, const double* fe, int n
       acc.x = fma(t.x, s, acc.x);
       acc.y = fma(t.y, s, acc.y);
     }
-    A[(((size_t)b * kNModes + md) * 3 + c) * 2 + o] = acc;
+    A[(size_t)((md * 3 + c) * 2 + o) * nbin + b] = acc;
   } else {
     const int r = q - nA;
     const int p = r / 9, c = (r / 3) % 3, o = r % 3;
@@ -193,7 +195,7 @@ __global__ void k_het_summary(DetDev D, const int* edge, const double* fe, int n
       acc.x = fma(t.x, s, acc.x);
       acc.y = fma(t.y, s, acc.y);
     }
-    Bs[(((size_t)b * kPairs + p) * 3 + c) * 3 + o] = acc;
+    Bs[(size_t)((p * 3 + c) * 3 + o) * nbin + b] = acc;
   }
 }
 
@@ -226,20 +228,31 @@ __device__ __forceinline__ void het_bin_fp64(const HetDev& H, int b, int c, Ld l
     r0[md] = ra;
     r1[md] = make_double2((rb.x - ra.x) * idf, (rb.y - ra.y) * idf);
   }
+  // <h|h> = Re sum_i [ r0_i sum_j (B0_ij r0_j* + B1_ij r1_j*) + r1_i sum_j (B1_ij r0_j* + B2_ij r1_j*) ], off-diagonal pairs
+  // (j > i) twice: 16 FMAs a pair and 4 a mode, against 26 a pair for the products t0, t1, t2 of the ratios
+  const int nbin = H.ne - 1;
   dh = 0.0;
   hh = 0.0;
+#pragma unroll
   for (int md = 0; md < kNModes; ++md) {
-    const double2 a0 = H.A[(((size_t)b * kNModes + md) * 3 + c) * 2 + 0];
-    const double2 a1 = H.A[(((size_t)b * kNModes + md) * 3 + c) * 2 + 1];
-    dh += cmul(a0, r0[md]).x + cmul(a1, r1[md]).x;
-    for (int m2 = md; m2 < kNModes; ++m2) {
-      const double2* q = H.Bs + (((size_t)b * kPairs + pair_index(md, m2)) * 3 + c) * 3;
-      const double2 t0 = cmul(r0[md], cconj(r0[m2]));
-      const double2 t1 = cadd(cmul(r1[md], cconj(r0[m2])), cmul(r0[md], cconj(r1[m2])));
-      const double2 t2 = cmul(r1[md], cconj(r1[m2]));
-      const double x = cmul(q[0], t0).x + cmul(q[1], t1).x + cmul(q[2], t2).x;
-      hh += (md == m2) ? x : 2.0 * x;
+    const double2* a = H.A + (size_t)(md * 3 + c) * 2 * nbin + b;
+    const double2 a0 = a[0], a1 = a[nbin];
+    dh = fma(a0.x, r0[md].x, fma(-a0.y, r0[md].y, fma(a1.x, r1[md].x, fma(-a1.y, r1[md].y, dh))));
+    double2 y = make_double2(0.0, 0.0), w = y;
+#pragma unroll
+    for (int k = 1; k <= kNModes; ++k) {
+      const int m2 = k < kNModes ? (md + k) : md;   // the off-diagonal pairs first, doubled, then the diagonal one
+      if (m2 >= kNModes) continue;
+      if (k == kNModes) { y.x *= 2.0; y.y *= 2.0; w.x *= 2.0; w.y *= 2.0; }
+      const double2* q = H.Bs + (size_t)(pair_index(md, m2) * 3 + c) * 3 * nbin + b;
+      const double2 q0 = q[0], q1 = q[nbin], q2 = q[2 * nbin];
+      const double2 s0 = r0[m2], s1 = r1[m2];
+      y.x = fma(q0.x, s0.x, fma(q0.y, s0.y, fma(q1.x, s1.x, fma(q1.y, s1.y, y.x))));
+      y.y = fma(q0.y, s0.x, fma(-q0.x, s0.y, fma(q1.y, s1.x, fma(-q1.x, s1.y, y.y))));
+      w.x = fma(q1.x, s0.x, fma(q1.y, s0.y, fma(q2.x, s1.x, fma(q2.y, s1.y, w.x))));
+      w.y = fma(q1.y, s0.x, fma(-q1.x, s0.y, fma(q2.y, s1.x, fma(-q2.x, s1.y, w.y))));
     }
+    hh = fma(r0[md].x, y.x, fma(-r0[md].y, y.y, fma(r1[md].x, w.x, fma(-r1[md].y, w.y, hh))));
   }
 }
 // Re(a b) and Re(a conj(b)) in double words
@@ -248,23 +261,44 @@ __device__ __forceinline__ cdf mul_conj(const cdf& a, const cdf& b) {
   return cdf{dfl_add(dfl_mul(a.re, b.re), dfl_mul(a.im, b.im)), dfl_sub(dfl_mul(a.im, b.re), dfl_mul(a.re, b.im))};
 }
 
-// One CTA of kTileBins threads per sample. Dynamic shared memory: [max ne][5][3] double2 ratios.
-// MIX: the signal at the edges by the mixed-precision unit, the ratios kept as double words and
-// the contraction in double words (Aw, Bw); the sums across bins and the block reduction stay
-// FP64. An edge with a ratio of kHetDwRatioMax or more keeps all its ratios in FP64 (flag byte
-// per edge after the ratios), and every (bin, channel) that reads it takes the FP64 contraction.
+// Block sum of six doubles per thread in a fixed tree order (up to kHetThreads threads); result valid in thread 0.
+__device__ __forceinline__ void het_block_sum(double v[6], double (*sh)[kHetThreads / 32]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(0xffffffffu, v[i], o);
+    if (lane == 0) sh[i][wid] = v[i];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      v[i] = 0.0;
+      for (int w = 0; w < nw; ++w) v[i] += sh[i][w];
+    }
+}
+
+// One CTA per sample. Dynamic shared memory: [max ne][5][3] double2 ratios, which fits two CTAs on an SM at the default 300
+// edges; so a CTA has a thread for (nearly) every edge, up to kHetThreads: with 128 threads an SM had eight warps
+// and three rounds of edges, the last a third full (777 samples, LISA: 1.09 ms).
+// The signal at the edges comes from the fixed-point unit (FX; both precisions), or the precision's own where a detector
+// does not take that unit. MIX: the ratios are kept as double words and contracted in double words (Aw, Bw);
+// the sums across bins and the block reduction stay FP64. An edge with a ratio of kHetDwRatioMax or more
+// keeps all its ratios in FP64 (flag byte per edge after the ratios), and every (bin, channel) that reads it
+// takes the FP64 contraction.
 template <bool MIX, bool FX>
-__global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, const SampleCoef* __restrict__ coef,
-                                                           double* logl, double* dhhh) {
+__global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B, const SampleCoef* __restrict__ coef,
+                                                               double* logl, double* dhhh) {
   extern __shared__ double2 rsh[];
   unsigned char* wflag = reinterpret_cast<unsigned char*>(rsh + (size_t)hs.nemax * kNModes * 3);
+  constexpr bool DW = MIX && !FX;   // the mixed unit at the edges
   __shared__ double pc[kProj];
-  __shared__ float2 pcw[MIX ? kProj : 1];
-  __shared__ double sh[6][kTileBins / 32];
-  __shared__ double2 stab[MIX || FX ? 1 : kSinTab];
-  __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
-  __shared__ float4 stabw[MIX ? kSinTab : 1];
-  if constexpr (MIX) {
+  __shared__ float2 pcw[DW ? kProj : 1];
+  __shared__ double sh[6][kHetThreads / 32];
+  __shared__ double2 stab[DW || FX ? 1 : kSinTab];
+  __shared__ fx fxcol[FX ? kFxSums : 1][kHetThreads];
+  __shared__ float4 stabw[DW ? kSinTab : 1];
+  if constexpr (DW) {
     for (int i = threadIdx.x; i < kSinTab; i += blockDim.x) stabw[i] = hs.h[0].det.sctw[i];
   } else if constexpr (!FX) {
     for (int i = threadIdx.x; i < kSinTab; i += blockDim.x) stab[i] = hs.h[0].det.sct[i];
@@ -280,7 +314,7 @@ __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, con
       fx_proj_prologue(D, S, reinterpret_cast<fx*>(pc));
     else
       proj_prologue(D, S, pc);
-    if constexpr (MIX) {
+    if constexpr (DW) {
       if (threadIdx.x < kProj) pcw[threadIdx.x] = to_dw(pc[threadIdx.x]);
       __syncthreads();
     }
@@ -289,10 +323,10 @@ __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, con
       for (int j = 0; j < kNModes * 3; ++j) need |= (H.src[e * kNModes * 3 + j] == e);
       if (!need) continue;
       double2 o[kNModes][3];
-      if constexpr (MIX)
+      if constexpr (DW)
         mode_brackets_mixed(D, S, H.edge[e], H.mask, o, stabw, pcw);
       else if constexpr (FX)
-        mode_brackets_fx(D, S, H.edge[e], H.mask, o, hs.h[0].det, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
+        mode_brackets_fx<kHetThreads>(D, S, H.edge[e], H.mask, o, hs.h[0].det, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
       else
         mode_brackets(D, S, H.edge[e], H.mask, o, stab, pc);
       // ratios in place of the brackets; in the mixed kernel, flag the edge if one of them is out
@@ -355,22 +389,29 @@ __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, con
             v[3 + c] += hh;
             continue;
           }
+          // as het_bin_fp64, in double words
+          const int nbin = H.ne - 1;
           df dh = df_make(0.f, 0.f), hh = df_make(0.f, 0.f);
 #pragma unroll
           for (int md = 0; md < kNModes; ++md) {
-            const float4* a = H.Aw + (((size_t)b * kNModes + md) * 3 + c) * 2;
-            dh = dfl_add(dh, dfl_add(re_mul(unpack4(a[0]), r0[md]), re_mul(unpack4(a[1]), r1[md])));
+            const float4* a = H.Aw + (size_t)(md * 3 + c) * 2 * nbin + b;
+            dh = dfl_add(dh, dfl_add(re_mul(unpack4(a[0]), r0[md]), re_mul(unpack4(a[nbin]), r1[md])));
+            cdf y = zc, w = zc;
 #pragma unroll
-            for (int m2 = md; m2 < kNModes; ++m2) {
-              const float4* q = H.Bw + (((size_t)b * kPairs + pair_index(md, m2)) * 3 + c) * 3;
-              const cdf t0 = mul_conj(r0[md], r0[m2]);
-              const cdf ta = mul_conj(r1[md], r0[m2]), tb = mul_conj(r0[md], r1[m2]);
-              const cdf t1 = {dfl_add(ta.re, tb.re), dfl_add(ta.im, tb.im)};
-              const cdf t2 = mul_conj(r1[md], r1[m2]);
-              df x = dfl_add(dfl_add(re_mul(unpack4(q[0]), t0), re_mul(unpack4(q[1]), t1)), re_mul(unpack4(q[2]), t2));
-              if (md != m2) x = df_scale2(x, 2.0f);
-              hh = dfl_add(hh, x);
+            for (int k = 1; k <= kNModes; ++k) {
+              const int m2 = k < kNModes ? (md + k) : md;
+              if (m2 >= kNModes) continue;
+              if (k == kNModes) {
+                y = cdf{df_scale2(y.re, 2.f), df_scale2(y.im, 2.f)};
+                w = cdf{df_scale2(w.re, 2.f), df_scale2(w.im, 2.f)};
+              }
+              const float4* q = H.Bw + (size_t)(pair_index(md, m2) * 3 + c) * 3 * nbin + b;
+              const cdf q0 = unpack4(q[0]), q1 = unpack4(q[nbin]), q2 = unpack4(q[2 * nbin]);
+              const cdf a0 = mul_conj(q0, r0[m2]), a1 = mul_conj(q1, r1[m2]), b0 = mul_conj(q1, r0[m2]), b1 = mul_conj(q2, r1[m2]);
+              y = cdf{dfl_add(y.re, dfl_add(a0.re, a1.re)), dfl_add(y.im, dfl_add(a0.im, a1.im))};
+              w = cdf{dfl_add(w.re, dfl_add(b0.re, b1.re)), dfl_add(w.im, dfl_add(b0.im, b1.im))};
             }
+            hh = dfl_add(hh, dfl_add(re_mul(r0[md], y), re_mul(r1[md], w)));
           }
           v[c] += df_to(dh);
           v[3 + c] += df_to(hh);
@@ -386,7 +427,7 @@ __global__ void __launch_bounds__(kTileBins) k_het_loglike(HetSet hs, int B, con
         v[3 + c] += hh;
       }
     }
-    block_sum<6>(v, sh);
+    het_block_sum(v, sh);
     if (threadIdx.x == 0) {
       for (int c = 0; c < 3; ++c) {
         L += v[c] - 0.5 * v[3 + c] - 0.5 * D.dd[c];
@@ -693,11 +734,16 @@ pe_status pe_hetero_loglike_batch(const pe_hetero* hets, int ndet, const double*
                         static_cast<int*>(stt), st);
   const bool mix = (hets[0]->dev.mask & PE_PREC_MIXED) != 0u;
   const size_t smem = (size_t)nemax * pe::kNModes * 3 * sizeof(double2) + (mix ? (size_t)nemax : 0);
-  auto kern = mix ? pe::k_het_loglike<true, false>
-                  : (pe::fx_all_ok(ds) ? pe::k_het_loglike<false, true> : pe::k_het_loglike<false, false>);
+  const bool fxu = pe::fx_all_ok(ds);
+  auto kern = mix ? (fxu ? pe::k_het_loglike<true, true> : pe::k_het_loglike<true, false>)
+                  : (fxu ? pe::k_het_loglike<false, true> : pe::k_het_loglike<false, false>);
+  // equal rounds of edges over the fewest threads (at least 64, which stage the projection forms)
+  const int rounds = (nemax + pe::kHetThreads - 1) / pe::kHetThreads;
+  const int threads = std::max(64, ((nemax + rounds - 1) / rounds + 31) / 32 * 32);
+  static_assert(pe::kProj <= 64 && pe::kFxProj <= 64, "one thread per form");
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) {
-    kern<<<B, pe::kTileBins, smem, st>>>(hs, B, static_cast<const pe::SampleCoef*>(coef), static_cast<double*>(ll),
+    kern<<<B, threads, smem, st>>>(hs, B, static_cast<const pe::SampleCoef*>(coef), static_cast<double*>(ll),
                                          static_cast<double*>(dh));
     e = pe::launch_status();
   }

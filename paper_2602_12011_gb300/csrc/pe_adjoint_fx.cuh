@@ -1,0 +1,337 @@
+// pe_adjoint_fx.cuh -- reverse sweep of the fixed-point unit (pe_device_fx.cuh) for the gradient (row G1) and the Fisher
+// matrix (row G2); arXiv:2602.12011 Sec. 2.1-2.3. The forward pass writes each unit's tape (kFt* fields); given the
+// bin's link seeds (link_seeds, pe_adjoint_tape.cuh, as integers with one exponent per bin), the sweep pulls them back through
+// the link factors, polarisation weights, sincs, norms and phases in fixed point, and only the scalars it ends in (the
+// phase's, amplitude's, t_f's and weights' cotangents) return to FP64 for the PN chain rule.
+//
+// What bounds it: the FP64 sweep it replaces issued 619 FP64 instructions per unit at 1.67 per SM and clock; here about
+// 110 are left, most of them the PN series' derivatives in v and q.
+//
+// The sky frame enters through rotations: a change of (lambda, beta, psi) turns (k, p, q) rigidly, dk = w x k and so on,
+// so the frame's cotangent is three numbers, W.w = sum over links of (projections' cotangents) x (projections), summed per
+// bin in place of 42 sums per tile over the tape.
+//
+// Scales: seeds are below 1/16 at exponent Es (value = n 2^(Es - 1078)), amplitudes below 1/8 (n 2^(E - 1079)); then every
+// sum of products here stays inside the formats (|cotangent of a projection| < 0.4, sums of three below 1.2).
+#pragma once
+#include "pe_adjoint_tape.cuh"
+#include "pe_device_fx.cuh"
+
+namespace pe {
+
+// The tape of one thread: field f at p[f * kTileBins] of the CTA's region in global memory, held in L2 by the evict-last
+// hint (tape_l2_policy).
+struct FxTape {
+  static constexpr bool kOn = true;
+  double* p;
+  unsigned long long pol;
+  __device__ __forceinline__ void st(int f, fx v) const { tst(p + f * kTileBins, __longlong_as_double(v), pol); }
+  __device__ __forceinline__ fx ld(int f) const { return __double_as_longlong(tld(p + f * kTileBins, pol)); }
+};
+static_assert((int)kFtFields <= (int)kTapeF, "the regions are those of the FP64 tape");
+
+// Scalars of one unit's sweep, in FP64.
+struct FxBwd {
+  double th;        // cotangent of the phase (rad), summed over the links' angles
+  double lnA;       // of ln amplitude
+  double alpha, geo;   // of the centre's angle and the constellation's (rad), without the Doppler term
+  double W[3];      // of the frame's rotation about k, p, q, without the Doppler term
+  double2 Ap, Ac;   // of the weights times the amplitude
+  double co, so;    // cos, sin of the centre's angle
+};
+
+// seeds: the bin's P_l, Q_l (x, y each) at seeds[(4 l + i) * SST]; Ap, Ac the weights times the amplitude.
+template <int SST, class Tape>
+__device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx* seeds, int Es, double2 Ap, double2 Ac, bool pair,
+                                       bool helio, const fx* __restrict__ pc, const Tape& tape, FxBwd& o) {
+  int E = max(fx_expo(Ap.x), fx_expo(Ac.x));
+  if (pair) E = max(E, max(fx_expo(Ap.y), fx_expo(Ac.y)));
+  const int ash = 1079 - E;
+  fxs Apx = {0, 0}, Acx = {0, 0}, Apy = {0, 0}, Acy = {0, 0};
+  if (E) {   // else the weights vanish, and only their own cotangents are not zero
+    Apx = fx_split(fx_from_bits(Ap.x, ash));
+    Acx = fx_split(fx_from_bits(Ac.x, ash));
+  }
+  if (pair && E) {
+    Apy = fx_split(fx_from_bits(Ap.y, ash));
+    Acy = fx_split(fx_from_bits(Ac.y, ash));
+  }
+  const fxs a4s = fx_split(B.a4), a3s = fx_split(a3);
+  fx th0 = 0, th1 = 0, th2 = 0, lnA = 0, Wk = 0, Wp = 0, Wq = 0;
+  fx Apb[2] = {0, 0}, Acb[2] = {0, 0}, obb[4] = {0, 0, 0, 0};
+#pragma unroll 1
+  for (int l = 0; l < 3; ++l) {
+    const int tl = kFtL + kFtLink * l;
+    const fxs Px = fx_split(seeds[(4 * l) * SST]), Py = fx_split(seeds[(4 * l + 1) * SST]);
+    const fxs Qx = fx_split(seeds[(4 * l + 2) * SST]), Qy = fx_split(seeds[(4 * l + 3) * SST]);
+    const fxs kr = fx_split(tape.ld(tl + kFtK)), pr = fx_split(tape.ld(tl + kFtP)), qr = fx_split(tape.ld(tl + kFtQ));
+    const fxs inv = fx_split(tape.ld(tl + kFtInv));
+    const fxs ec = fx_split(tape.ld(tl + kFtEc)), es = fx_split(tape.ld(tl + kFtEs));
+    const fxs sp = fx_split(tape.ld(tl + kFtSp)), sm = fx_split(tape.ld(tl + kFtSm));
+    const fxs kn = fx_split(fx_mul(kr, inv));
+    const fx npq = fx_mul(pr, inv), nqq = fx_mul(qr, inv);
+    const fxs np = fx_split(npq), nq = fx_split(nqq);
+    const fxs Fp = fx_split(fx_mul(fx_split(npq - nqq), fx_split(npq + nqq))), Fc = fx_split(fx_mul(np, nq));
+    // gam = Fp Ap + i Fc Ac, G = gam E
+    fxs gx, gy;
+    if (pair) {
+      gx = fx_split(fx_msub(Apx, Fp, Acy, Fc));
+      fxa g = fx_prod<2>(Apy, Fp);
+      fx_mac(g, Acx, Fc);
+      gy = fx_split(fx_val(g));
+    } else {
+      gx = fx_split(fx_mul(Apx, Fp));
+      gy = fx_split(fx_mul(Acx, Fc));
+    }
+    const fxs Gx = fx_split(fx_msub(gx, ec, gy, es));
+    fxa t = fx_prod<2>(gx, es);
+    fx_mac(t, gy, ec);
+    const fxs Gy = fx_split(fx_val(t));
+    // Gb = s- P + s+ Q; cotangents of s-+ are Re(G conj P), Re(G conj Q)
+    t = fx_prod<2>(sm, Px);
+    fx_mac(t, sp, Qx);
+    const fxs Gbx = fx_split(fx_val(t));
+    t = fx_prod<2>(sm, Py);
+    fx_mac(t, sp, Qy);
+    const fxs Gby = fx_split(fx_val(t));
+    t = fx_prod<2>(Gx, Px);
+    fx_mac(t, Gy, Py);
+    const fxs smb = fx_split(fx_val(t));
+    t = fx_prod<2>(Gx, Qx);
+    fx_mac(t, Gy, Qy);
+    const fxs spb = fx_split(fx_val(t));
+    // d s-+/d kn = -+ a sinc'(u-+)
+    const fxs dp = fx_split(tape.ld(tl + kFtDp)), dm = fx_split(tape.ld(tl + kFtDm));
+    const fxs knb = fx_split(fx_mul(fx_split(fx_msub(spb, dp, smb, dm)), a4s) << 2);
+    // gamb = Gb conj E; the angle's cotangent Im(Gb conj G)
+    t = fx_prod<2>(Gbx, ec);
+    fx_mac(t, Gby, es);
+    const fx gbxq = fx_val(t);
+    const fx gbyq = fx_msub(Gby, ec, Gbx, es);
+    const fxs gbx = fx_split(gbxq), gby = fx_split(gbyq);
+    const fx th = fx_msub(Gby, Gx, Gbx, Gy);
+    if (l == 0) th0 = th;
+    else if (l == 1) th1 = th;
+    else th2 = th;
+    t = fx_prod<2>(gbx, gx);
+    fx_mac(t, gby, gy);
+    lnA += fx_val(t);
+    Apb[0] += fx_mul(gbx, Fp);
+    Acb[0] += fx_mul(gby, Fc);
+    fxs Fpb, Fcb;
+    if (pair) {
+      Apb[1] += fx_mul(gby, Fp);
+      Acb[1] -= fx_mul(gbx, Fc);
+      t = fx_prod<2>(gbx, Apx);
+      fx_mac(t, gby, Apy);
+      Fpb = fx_split(fx_val(t));
+      Fcb = fx_split(fx_msub(gby, Acx, gbx, Acy));
+    } else {
+      Fpb = fx_split(fx_mul(gbx, Apx));
+      Fcb = fx_split(fx_mul(gby, Acx));
+    }
+    // Fp = np^2 - nq^2, Fc = np nq
+    const fxs npb = fx_split(2 * fx_mul(np, Fpb) + fx_mul(nq, Fcb));
+    const fxs nqb = fx_split(fx_mul(np, Fcb) - 2 * fx_mul(nq, Fpb));
+    // the frame's rotation (norms do not change under it)
+    Wk += fx_msub(npb, nq, nqb, np);
+    Wp += fx_msub(nqb, kn, knb, nq);
+    Wq += fx_msub(knb, np, npb, kn);
+    // (kn, np, nq) = (kr, pr, qr) / |n'|
+    t = fx_prod<3>(knb, kn);
+    fx_mac(t, npb, np);
+    fx_mac(t, nqb, nq);
+    const fxs dot = fx_split(fx_val(t));
+    auto norm = [&](fxs xb, fxs x) {
+      const fx r = (((fx)xb.h << 30) + xb.l) - fx_mul(x, dot);
+      return fx_split(fx_mul(fx_split(r), inv));
+    };
+    const fxs krb = norm(knb, kn), prb = norm(npb, np), qrb = norm(nqb, nq);
+    const volatile fx* pl = l < 2 ? pc + 15 * l : pc + kFxProj3;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      if (m >= 2 && !helio) break;
+      t = fx_prod<3>(krb, fx_unpack(pl[m]));
+      fx_mac(t, prb, fx_unpack(pl[5 + m]));
+      fx_mac(t, qrb, fx_unpack(pl[10 + m]));
+      obb[m] += fx_val(t);
+    }
+  }
+  // the links' angles carry f k.delta_t / 2: (a / 3) (th_{l+1} - th_{l+2}) on k.n'_l (angles by link)
+#pragma unroll 1
+  for (int l = 0; l < 3; ++l) {
+    const int tl = kFtL + kFtLink * l;
+    const fx d = l == 0 ? th1 - th2 : (l == 1 ? th2 - th0 : th0 - th1);
+    const fxs kb = fx_split(fx_mul(fx_split(d), a3s));
+    Wq += fx_mul(kb, fx_split(tape.ld(tl + kFtP)));
+    Wp -= fx_mul(kb, fx_split(tape.ld(tl + kFtQ)));
+    const volatile fx* pl = l < 2 ? pc + 15 * l : pc + kFxProj3;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      if (m >= 2 && !helio) break;
+      obb[m] += fx_mul(kb, fx_unpack(pl[m]));
+    }
+  }
+  // orbit basis b = (cos 2 alpha, sin 2 alpha, cos alpha, sin alpha) or (cos phi_0, sin phi_0)
+  const int e = E + Es - 2097;
+  const fx cq = tape.ld(kFtC), sq = tape.ld(kFtS);
+  const fxs c = fx_split(cq), s = fx_split(sq);
+  o.co = fx_to_double(cq, -60);
+  o.so = fx_to_double(sq, -60);
+  if (helio) {
+    fxa q = fx_sq0<1>();
+    fx_macsq(q, s);
+    const fxs c2 = fx_split(kFxOne - 2 * fx_valsq(q)), s2 = fx_split(2 * fx_mul(s, c));
+    const fx r2 = fx_msub(c2, fx_split(obb[1]), s2, fx_split(obb[0]));
+    const fx r1 = fx_msub(c, fx_split(obb[3]), s, fx_split(obb[2]));
+    o.alpha = fx_to_double(2 * r2 + r1, e);
+    o.geo = 0.0;
+  } else {
+    const fxs gc = fx_split(tape.ld(kFtGc)), gs = fx_split(tape.ld(kFtGs));
+    o.alpha = 0.0;
+    o.geo = fx_to_double(fx_msub(gc, fx_split(obb[1]), gs, fx_split(obb[0])), e);
+  }
+  o.th = fx_to_double(th0 + th1 + th2, e);
+  o.lnA = fx_to_double(lnA, e);
+  o.W[0] = fx_to_double(Wk, e);
+  o.W[1] = fx_to_double(Wp, e);
+  o.W[2] = fx_to_double(Wq, e);
+  if (E == 0) o.th = o.lnA = o.alpha = o.geo = o.W[0] = o.W[1] = o.W[2] = 0.0;   // not the sums' rounding
+  o.Ap = make_double2(fx_to_double(Apb[0], Es - 1078), 0.0);
+  o.Ac = make_double2(fx_to_double(Acb[0], Es - 1078), 0.0);
+  if (pair) {
+    o.Ap.y = fx_to_double(Apb[1], Es - 1078);
+    o.Ac.y = fx_to_double(Acb[1], Es - 1078);
+  }
+}
+
+// Sums of one bin's sweeps over its modes; the factors common to the modes are applied once per bin (fx_bin_grad).
+struct FxBinAcc {
+  double lnA, vM, q, io, ph, tc;   // ln amplitude; v d/dv of phase and t_f chains; q, iota, phi_c, t_c
+  double x3, x4;                   // psib v^-2 - 2 Db v^-2, psib v^-1 - Db v^-1 (chi1, chi2 enter P3 and P4 alone)
+  double W[3], dc, ds;             // rotation; Doppler f R-weighted cos and sin
+  double Mx;                       // Mtot through the taper and the paired mode
+};
+__device__ __forceinline__ void fx_bin_zero(FxBinAcc& g) {
+  g.lnA = g.vM = g.q = g.io = g.ph = g.tc = g.x3 = g.x4 = g.dc = g.ds = g.Mx = 0.0;
+  g.W[0] = g.W[1] = g.W[2] = 0.0;
+}
+// Reverse sweep of one unit, added to the bin's sums; the PN chain in FP64. fm13 = f^(-1/3), invf = 1/f, fR = 2 pi f R. (t_f's part of the
+// chain in double words saved 14 FP64 FMAs a unit and no time: the kernel waits on dependent operations.)
+template <int SST, class Tape>
+__device__ __forceinline__ void mode_bwd_fx(const DetDev& D, const SampleCoef& S, const SampleGrad& SG, int md, int md2, const FxBin& B,
+                                            double fm13, double invf, double fR, fx a3, const volatile fx* seeds, int Es, FxBinAcc& g,
+                                            const fx* __restrict__ pc, const Tape& tape) {
+  const ModeCoef& C = S.md[md];
+  const ModeGrad& CG = SG.md[md];
+  const double v = C.cm * B.f13, lnv = C.lncm + B.lnf3, iv5 = C.icm5 * D.fm53[B.b];
+  const double amp0 = __longlong_as_double(tape.ld(kFtAmp0)), w = __longlong_as_double(tape.ld(kFtW)), amp = amp0 * w;
+  if (fx_expo(amp) == 0) return;
+  double2 kap = make_double2(0.0, 0.0);
+  double Pp2 = 0.0, Pc22 = 0.0;
+  double2 Ap = make_double2(amp * C.Pp, 0.0), Ac = make_double2(amp * C.Pc2, 0.0);
+  if (md2 >= 0) {
+    const double v2 = v * v;
+    kap = make_double2(S.k32.x * v2, S.k32.y * v2);
+    Pp2 = S.md[md2].Pp;
+    Pc22 = S.md[md2].Pc2;
+    Ap = make_double2(amp * fma(kap.x, Pp2, C.Pp), amp * (kap.y * Pp2));
+    Ac = make_double2(amp * fma(kap.x, Pc22, C.Pc2), amp * (kap.y * Pc22));
+  }
+  FxBwd o;
+  fx_bwd<SST>(B, a3, seeds, Es, Ap, Ac, md2 >= 0, D.orbit == 0, pc, tape, o);
+  // phase: ph0 = m phi_c / 2 pi + ..., -f t_c, -(m / 4 pi) Psi, -f k.x_c (turns)
+  const double mh = md == 1 ? -0.5 : (md == 2 ? -1.5 : (md == 4 ? -2.0 : -1.0));   // -m/2
+  const double psib = mh * o.th;                 // - mfac 2 pi th
+  g.ph = fma(-2.0, psib, g.ph);
+  g.tc = fma(-2.0 * kPi * B.f, o.th, g.tc);
+  // centre's Doppler term -f k.x_c, x_c = R (cos alpha, sin alpha, 0)
+  const double fc = -fR * o.th * o.co, fs = -fR * o.th * o.so;
+  g.dc += fc;
+  g.ds += fs;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) g.W[i] += o.W[i];
+  const double alphab = fma(S.k[1], fc, fma(-S.k[0], fs, o.alpha));
+  const double tfb = fma(alphab, 2.0 * kPi * D.rate_t, o.geo * (2.0 * kPi * D.geo_rate_t));
+  g.tc += tfb;                                   // t_f = t_c + (m/(12 pi f)) D(v)
+  const double Db = tfb * (C.tffac * invf);
+  // amplitude ~ M^(5/6) ... f^(-7/6 + p/3) cm^p: dlnA_dM without the mode's own v is common to the modes
+  g.lnA += o.lnA;
+  g.q = fma(o.lnA, CG.dlnA_dq, g.q);
+  if (dlt_pos(C.ftap, B.f)) {
+    const double zb = -o.lnA * (1.0 - w);
+    const double fe = C.fend, ft = C.ftap, A = fe - ft;
+    const double dz = 0.1 / (fe - B.f) - A / ((fe - B.f) * (fe - B.f)) - 0.1 / (B.f - ft) -
+                      0.9 * A / ((B.f - ft) * (B.f - ft));
+    g.Mx = fma(zb * dz, CG.dfend_dM, g.Mx);
+  }
+  // Psi_PN(v), D(v): v dPsi/dv = D, v dD/dv = v^-5 ddpol + Q6 v (2 + ln v); v ~ M^(1/3)
+  double dpol = S.Pd[7], ddpol = S.Pdd[7], pq = SG.dP_dq[7], dq = SG.dPd_dq[7];
+#pragma unroll
+  for (int k = 6; k >= 0; --k) {
+    dpol = fma(dpol, v, S.Pd[k]);
+    ddpol = fma(ddpol, v, S.Pdd[k]);
+    pq = fma(pq, v, SG.dP_dq[k]);
+    dq = fma(dq, v, SG.dPd_dq[k]);
+  }
+  const double q6v = S.Q6 * v, dq6v = SG.dQ6_dq * v;
+  const double dv = fma(iv5, dpol, fma(q6v, 1.0 + lnv, S.Q5));
+  g.vM = fma(psib, dv, fma(Db, fma(iv5, ddpol, q6v * (2.0 + lnv)), fma(o.lnA, double(C.p), g.vM)));
+  g.q = fma(psib, fma(iv5, pq, lnv * (dq6v + SG.dQ5_dq)), fma(Db, fma(iv5, dq, fma(dq6v, 1.0 + lnv, SG.dQ5_dq)), g.q));
+  const double iv = C.icm * fm13;
+  g.x4 = fma(iv, psib - Db, g.x4);
+  g.x3 = fma(iv * iv, fma(-2.0, Db, psib), g.x3);
+  // polarisation weights: Ac carries 2 Pc
+  const double2 apb = make_double2(amp * o.Ap.x, amp * o.Ap.y), acb = make_double2(amp * o.Ac.x, amp * o.Ac.y);
+  g.io = fma(apb.x, CG.dPp_di, fma(2.0 * acb.x, CG.dPc_di, g.io));
+  if (md2 >= 0) {
+    const ModeGrad& CG2 = SG.md[md2];
+    g.io += (apb.x * kap.x + apb.y * kap.y) * CG2.dPp_di + 2.0 * (acb.x * kap.x + acb.y * kap.y) * CG2.dPc_di;
+    const double2 kb = make_double2(apb.x * Pp2 + acb.x * Pc22, apb.y * Pp2 + acb.y * Pc22);   // kappa-bar
+    // kappa = k32 v^2; only ln(amp2 / amp1) varies with theta (M, q), see mode_bwd
+    const double lnrb = v * v * (kb.x * S.k32.x + kb.y * S.k32.y);
+    g.Mx = fma(lnrb, CG2.dlnA_dM - CG.dlnA_dM, g.Mx);
+    g.q = fma(lnrb, CG2.dlnA_dq - CG.dlnA_dq, g.q);
+    g.vM = fma(2.0, lnrb, g.vM);
+  }
+}
+
+// The bin's theta components from its sums, with the rotation cotangents in g.k. th: the sample's parameters enter through
+// SampleGrad alone: d ln v / d Mtot = 1 / (3 Mtot) = dcm_dM / cm.
+__device__ __forceinline__ void fx_bin_grad(const SampleCoef& S, const SampleGrad& SG, const FxBinAcc& a, GradAcc& g) {
+  const double m3 = SG.md[0].dcm_dM / S.md[0].cm;    // 1 / (3 Mtot)
+  g.M = fma(a.vM, m3, fma(a.lnA, 2.5 * m3, a.Mx));   // dlnA_dM = 5 / (6 Mtot)
+  g.q = a.q;
+  g.c1 = fma(SG.dP3_dc1, a.x3, SG.dP4_dc1 * a.x4);
+  g.c2 = fma(SG.dP3_dc2, a.x3, SG.dP4_dc2 * a.x4);
+  g.dL = a.lnA * SG.dlnA_ddL;
+  g.io = a.io;
+  g.ph = a.ph;
+  g.tc = a.tc;
+  g.k[0] = a.W[0];
+  g.k[1] = a.W[1] - fma(S.q[0], a.dc, S.q[1] * a.ds);
+  g.k[2] = a.W[2] + fma(S.p[0], a.dc, S.p[1] * a.ds);
+}
+
+// Component c of the frame vectors' cotangents (vec 0 k, 1 p, 2 q) that stand for the rotation cotangents W: with
+// dk = w x k = w_q p - w_p q and dp . q = w_k, kbar = W_q p - W_p q and pbar = W_k q give W.w for every rotation w.
+__device__ __forceinline__ double rotation_to_frame(const SampleCoef& S, const double W[3], int vec, int c) {
+  return vec == 0 ? W[2] * S.p[c] - W[1] * S.q[c] : (vec == 1 ? W[0] * S.q[c] : 0.0);
+}
+
+// The bin's link seeds as integers: exponent Es of the largest (0: all vanish, and so does the bin's gradient), n = value 2^(1078 - Es) below 1/16.
+template <int SST>
+__device__ __forceinline__ int fx_seeds(const double2 pq[6], volatile fx* seeds) {
+  int Es = 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) Es = max(Es, max(fx_expo(pq[i].x), fx_expo(pq[i].y)));
+  const int sh = 1078 - Es;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    seeds[2 * i * SST] = fx_from_bits(pq[i].x, sh);
+    seeds[(2 * i + 1) * SST] = fx_from_bits(pq[i].y, sh);
+  }
+  return Es;
+}
+
+}  // namespace pe

@@ -233,7 +233,8 @@ __device__ __forceinline__ void mode_fwd_tape(const DetDev& D, const SampleCoef&
 // bA + 3 bE and -2 bA: the T cotangent, which dwarfs the others at long wavelength (the T
 // channel's noise falls as a^4), cancels exactly, and with conj z - 1 = -2 sin a (sin a - i cos a)
 // P_l = (sV - sU) + sV (conj z - 1), Q_l = (sV - sU) - sU (conj z - 1). sa, ca: sin a, cos a.
-// Writes P_l, Q_l to pq[(2 l) * kTileBins], pq[(2 l + 1) * kTileBins].
+// Writes P_l, Q_l to pq[(2 l) * STRIDE], pq[(2 l + 1) * STRIDE].
+template <int STRIDE = kTileBins>
 __device__ __forceinline__ void link_seeds(const double2 bb[3], double sa, double ca, double2* pq) {
   const double2 sX = make_double2(-bb[0].x + bb[1].x + bb[2].x, -bb[0].y + bb[1].y + bb[2].y);
   const double2 sY = make_double2(-2.0 * bb[1].x + bb[2].x, -2.0 * bb[1].y + bb[2].y);
@@ -246,8 +247,8 @@ __device__ __forceinline__ void link_seeds(const double2 bb[3], double sa, doubl
     const double2 d = (l == 0) ? make_double2(bb[0].x - 3.0 * bb[1].x, bb[0].y - 3.0 * bb[1].y)
                     : (l == 1) ? make_double2(bb[0].x + 3.0 * bb[1].x, bb[0].y + 3.0 * bb[1].y)
                                : make_double2(-2.0 * bb[0].x, -2.0 * bb[0].y);
-    pq[2 * l * kTileBins] = cadd(d, cmul(sV, zm));
-    pq[(2 * l + 1) * kTileBins] = csub(d, cmul(sU, zm));
+    pq[2 * l * STRIDE] = cadd(d, cmul(sV, zm));
+    pq[(2 * l + 1) * STRIDE] = csub(d, cmul(sU, zm));
   }
 }
 

@@ -47,7 +47,7 @@ struct pe_detector_s {
   double* dd_dev;      // [3]
   double2* sct;        // [kSinTab] sincos table
   float4* sctw;        // [kSinTab] the same as double words
-  pe::FxCis* fcis;     // [kSinTab], [kFxSincTab] tables of the fixed-point unit
+  pe::FxCis* fcis;     // [kSinTab], [2][kFxSincTab] tables of the fixed-point unit
   pe::FxSinc* fsinc;
   float2* fw;          // [nb] double words of f, pi f L, f L / 2, sin(pi f L), cos(pi f L)
   float2* aw;
@@ -205,6 +205,7 @@ void fill_fx(pe_detector_s* d) {
   const hdd pi = {3.141592653589793, 1.2246467991473532e-16};
   D.fx_a4 = fx_const(hdd_div(hdd_mul(pi, D.L), 4.0 * d->T));
   D.fx_at3 = fx_const(hdd_div(hdd{D.L, 0.0}, 6.0 * d->T));
+  D.fx_a3 = fx_const(hdd_div(hdd_mul(pi, D.L), 3.0 * d->T));
   D.fx_fR = fx_const(hdd_div(hdd{std::ldexp(D.R, -D.fx_rsh), 0.0}, d->T));
 }
 
@@ -356,7 +357,7 @@ pe_status pe_create_detector(const pe_detector_config* cfg, double T_obs, int64_
   // padded); float2: fw, aw, atw, saw, caw, f13w, fm76w, fm83w (8 nb) + ggw (3 nb) + scaf, zf (2 nb) +
   // dgf (3 nb); float: five FP32 grid tables (5 nb) + ggf (3 nb)
   // the fixed-point unit's tables come first (16-byte entries)
-  const size_t fx_bytes = pe::kSinTab * sizeof(pe::FxCis) + pe::kFxSincTab * sizeof(pe::FxSinc);
+  const size_t fx_bytes = pe::kSinTab * sizeof(pe::FxCis) + 2 * pe::kFxSincTab * sizeof(pe::FxSinc);
   const size_t n_d = 14 * nb + 8, n_d2 = 5 * nb + pe::kSinTab, n_f4 = pe::kSinTab + 4 * nb, n_f2 = 16 * nb,
                n_f = 8 * nb;
   const size_t bytes = fx_bytes + n_d2 * sizeof(double2) + n_f4 * sizeof(float4) + n_d * sizeof(double) +
@@ -365,7 +366,7 @@ pe_status pe_create_detector(const pe_detector_config* cfg, double T_obs, int64_
   if (e != cudaSuccess) { cudaGetLastError(); delete d; return fail(PE_ENOMEM, "pe::dmalloc(%zu) failed", bytes); }
   d->fcis = static_cast<pe::FxCis*>(d->mem);
   d->fsinc = reinterpret_cast<pe::FxSinc*>(d->fcis + pe::kSinTab);
-  double2* p2 = reinterpret_cast<double2*>(d->fsinc + pe::kFxSincTab);
+  double2* p2 = reinterpret_cast<double2*>(d->fsinc + 2 * pe::kFxSincTab);
   d->sct = p2; p2 += pe::kSinTab;
   d->sca = p2; p2 += nb;
   d->z = p2; p2 += nb;
@@ -686,7 +687,7 @@ pe_status pe_loglike_grad_batch(const pe_detector* dets, int ndet, const double*
   PE_CUDA(pe::launch_scan_tiles(nend, P, off, pe::kTileBins, st));
   // a persistent grid of the kernel's resident CTAs per SM, each with its tape region
   const long long g = std::max<long long>(
-      1, std::min<long long>(max_tiles, (long long)sm_count() * pe::grad_tape_ctas_per_sm(mixed)));
+      1, std::min<long long>(max_tiles, (long long)sm_count() * pe::grad_tape_ctas_per_sm(ds, mixed)));
   double* tape = nullptr;
   PE_CUDA(sc.alloc(&tape, (size_t)g * pe::grad_tape_doubles_per_cta()));
   void* prof = nullptr;

@@ -32,8 +32,10 @@ __device__ __forceinline__ fx fx_times_k(unsigned k, const FxConst& c) {
 // links l = 0, 1 is proj_coef's over the nominal arm, m < 4 split for multiplication (h in the high word, l in the
 // low one) and the constant m = 4 a plain Q60; entries 30, 31 are k_x, k_y (split), 32 the centre's angle at t_c
 // (turns) and 33 + md mode md's m / (12 pi) cm^-5 as a double word.
+// Entries kFxProj3 + 5 v + m (m < 4): the third link's forms, minus the others' sum (fx_proj3; the reverse sweep's).
 constexpr int kFxProj = 33 + kNModes;
-static_assert(kFxProj <= kProj, "the forms share proj_coef's array");
+constexpr int kFxProj3 = kFxProj, kFxProjAll = kFxProj + 15;
+static_assert(kFxProjAll <= kProj, "the forms share proj_coef's array");
 __device__ __forceinline__ fx fx_pack(fxs s) { return ((fx)s.h << 32) | (unsigned)s.l; }
 __device__ __forceinline__ fxs fx_unpack(fx p) {
   fxs r;
@@ -55,11 +57,20 @@ __device__ __forceinline__ void fx_proj_prologue(const DetDev& D, const SampleCo
   }
   __syncthreads();
 }
+__device__ __forceinline__ void fx_proj3(fx* pc) {   // after fx_proj_prologue; a barrier at the end
+  const int i = threadIdx.x;
+  if (i < 15 && i % 5 < 4) {
+    const fxs a = fx_unpack(pc[i]), b = fx_unpack(pc[15 + i]);
+    pc[kFxProj3 + i] = fx_pack(fx_split(-((((fx)a.h + b.h) << 30) + a.l + b.l)));
+  }
+  __syncthreads();
+}
 // p[0..3] . b + p[4] (geocentric: b has two entries and the constant is zero)
 __device__ __forceinline__ fx fx_dot(const volatile fx* p, const fxs b[4], bool helio) {
-  fxa s = fx_prod(fx_unpack(p[0]), b[0]);
+  fxa s = fx_prod<2>(fx_unpack(p[0]), b[0]);
   fx_mac(s, fx_unpack(p[1]), b[1]);
   if (helio) {
+    s.c += 2 * kFxLL;
     fx_mac(s, fx_unpack(p[2]), b[2]);
     fx_mac(s, fx_unpack(p[3]), b[3]);
     s.h += p[4];
@@ -114,7 +125,7 @@ __device__ __forceinline__ int fx_expo(double v) { return (__double2hiint(v) >> 
 __device__ __forceinline__ void fx_basis(fxc g, bool helio, fxs ob[4]) {
   const fxs cs = fx_split(g.c), ss = fx_split(g.s);
   if (helio) {
-    fxa q = {0, 0};
+    fxa q = fx_sq0<1>();
     fx_macsq(q, ss);
     ob[0] = fx_split(kFxOne - 2 * fx_valsq(q));   // cos 2 alpha = 1 - 2 sin^2 alpha
     ob[1] = fx_split(2 * fx_mul(ss, cs));
@@ -127,13 +138,23 @@ __device__ __forceinline__ void fx_basis(fxc g, bool helio, fxs ob[4]) {
   }
 }
 
+// Fields of a unit's tape for the reverse sweep (pe_adjoint_fx.cuh): the centre's and the constellation's cosine and sine,
+// the amplitude before the taper and the taper's weight (doubles' bits), and per link l the projections of the link
+// vector over the arm, its inverse length, the factor e^{i phase}, sinc(a (1 +- k.n)) and their derivatives in u.
+enum : int { kFtC = 0, kFtS = 1, kFtGc = 2, kFtGs = 3, kFtAmp0 = 4, kFtW = 5, kFtL = 6, kFtLink = 10, kFtFields = 36 };
+enum : int { kFtK = 0, kFtP = 1, kFtQ = 2, kFtInv = 3, kFtEc = 4, kFtEs = 5, kFtSp = 6, kFtSm = 7, kFtDp = 8, kFtDm = 9 };
+struct FxNoTape {
+  static constexpr bool kOn = false;
+  __device__ __forceinline__ void st(int, fx) const {}
+};
+
 // One unit's link products, added to the bin's sums: phu the mode's phase (turns), Apx, Acx the polarisation weights
 // times the amplitude; for a paired second mode Ap (its imaginary part read) and Acyd complete them, scaled by
 // 2^ash.
-template <class Acc>
+template <class Acc, class Tape = FxNoTape>
 __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs Acx, const double2* Ap, double Acyd, int ash,
                                          const fxs ob[4], bool helio, Acc& acc, const FxCis* __restrict__ tab,
-                                         const FxSinc* __restrict__ stab, const fx* __restrict__ pc) {
+                                         const FxSinc* __restrict__ stab, const fx* __restrict__ pc, Tape tape = Tape()) {
   const fxs a4s = fx_split(a4);
   // --- links (row A5): projections of the link vectors over the nominal arm; the three sum to zero.
   // Third-spacecraft phases f k.delta_t / 2 in turns: delta_0 - delta_1, delta_1 - delta_2 and
@@ -153,11 +174,12 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
       nq -= qr;
     }
     const fxs k0 = fx_split(l == 0 ? kn0 : (l == 1 ? kn1 : kn2)), p0 = fx_split(pr), q0 = fx_split(qr);
-    fxa n2 = {0, 0};
+    fxa n2 = fx_sq0<3>();
     fx_macsq(n2, k0);
     fx_macsq(n2, p0);
     fx_macsq(n2, q0);
-    const fxs inv = fx_split(fx_rsqrt(fx_valsq(n2)));
+    const fx invq = fx_rsqrt(fx_valsq(n2));
+    const fxs inv = fx_split(invq);
     const fx w4 = fx_mul(fx_split(fx_mul(k0, inv)), a4s);
     const fx p1 = fx_mul(p0, inv), q1 = fx_mul(q0, inv);
     // F+ = (n.p)^2 - (n.q)^2, Fx / 2 = (n.p)(n.q) (the 2 is in Ac)
@@ -166,8 +188,8 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
     fxs gx, gy;
     if (Ap) {
       const fxs Apy = fx_split(fx_from_bits(Ap->y, ash)), Acy = fx_split(fx_from_bits(Acyd, ash));
-      gx = fx_split(fx_sub2(fx_prod(Apx, Fp), fx_prod(Acy, Fc)));
-      fxa g = fx_prod(Apy, Fp);
+      gx = fx_split(fx_msub(Apx, Fp, Acy, Fc));
+      fxa g = fx_prod<2>(Apy, Fp);
       fx_mac(g, Acx, Fc);
       gy = fx_split(fx_val(g));
     } else {
@@ -177,15 +199,29 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
     // the third spacecraft is 2, 0, 1 for l = 0, 1, 2
     const fxc e = fx_cis(l == 0 ? phu - (e0 + e1) : phu + (l == 1 ? e0 : e1), tab);
     const fxs ec = fx_split(e.c), es = fx_split(e.s);
-    const fxs Gr = fx_split(fx_sub2(fx_prod(gx, ec), fx_prod(gy, es)));
-    fxa gi = fx_prod(gx, es);
+    const int tl = kFtL + kFtLink * l;
+    if constexpr (Tape::kOn) {
+      tape.st(tl + kFtK, l == 0 ? kn0 : (l == 1 ? kn1 : kn2));
+      tape.st(tl + kFtP, pr);
+      tape.st(tl + kFtQ, qr);
+      tape.st(tl + kFtInv, invq);
+      tape.st(tl + kFtEc, e.c);
+      tape.st(tl + kFtEs, e.s);
+    }
+    const fxs Gr = fx_split(fx_msub(gx, ec, gy, es));
+    fxa gi = fx_prod<2>(gx, es);
     fx_mac(gi, gy, ec);
     const fxs Gi = fx_split(fx_val(gi));
     // --- sinc(a (1 +- k.n)) and the link's products for the TDI brackets (row A6; see XYZAcc)
     volatile fx* as = acc.s + 4 * l * Acc::kStride;
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
-      const fxs sc = fx_split(fx_sinc(h == 0 ? a4 + w4 : a4 - w4, stab));
+      const fx u4 = h == 0 ? a4 + w4 : a4 - w4, sv = fx_sinc(u4, stab);
+      const fxs sc = fx_split(sv);
+      if constexpr (Tape::kOn) {
+        tape.st(tl + kFtSp + h, sv);
+        tape.st(tl + kFtDp + h, fx_sinc(u4, stab + kFxSincTab));   // the derivative's table follows
+      }
       as[0] = as[0] + fx_mul(Gr, sc);
       as[Acc::kStride] = as[Acc::kStride] + fx_mul(Gi, sc);
       as += 2 * Acc::kStride;
@@ -193,10 +229,11 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
   }
 }
 
-template <class Acc>
+template <class Acc, class Tape = FxNoTape>
 __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S, const ModeCoef& C, const FxBin& B,
                                             Acc& acc, const FxCis* __restrict__ tab, const FxSinc* __restrict__ stab,
-                                            const fx* __restrict__ pc, int md, const ModeCoef* C2 = nullptr) {
+                                            const fx* __restrict__ pc, int md, const ModeCoef* C2 = nullptr,
+                                            Tape tape = Tape()) {
   // --- waveform and time-frequency map (rows A2, A3), as mode_bin
   const double v = C.cm * B.f13;
   const double lnv = C.lncm + B.lnf3;
@@ -243,7 +280,15 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
   if (dlt_pos(C.ftap, B.f)) {
     const double span = C.fend - C.ftap;
     const double zt = span / (C.fend - B.f) - span / (B.f - C.ftap);
-    amp *= (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
+    const double w = (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
+    if constexpr (Tape::kOn) {
+      tape.st(kFtAmp0, __double_as_longlong(amp));
+      tape.st(kFtW, __double_as_longlong(w));
+    }
+    amp *= w;
+  } else if constexpr (Tape::kOn) {
+    tape.st(kFtAmp0, __double_as_longlong(amp));
+    tape.st(kFtW, __double_as_longlong(1.0));
   }
   // polarisation weights times the amplitude (complex for a paired second mode), as integers below
   // 1/8 in units of 2^(E - 1079)
@@ -256,27 +301,37 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
   }
   int E = max(fx_expo(Ap.x), fx_expo(Ac.x));
   if (C2) E = max(E, max(fx_expo(Ap.y), fx_expo(Ac.y)));
-  if (E == 0) return;                      // nothing above FP64's smallest normal number
+  // E = 0: the weights vanish (the unit adds nothing; its tape still serves the weights' own derivatives)
+  if (!Tape::kOn && E == 0) return;
   if (E > acc.E) {
     if (acc.E > 0) {
-      const int sh = min(63, E - acc.E);
+      const int sh = min(62, E - acc.E);
 #pragma unroll 1
-      for (int i = 0; i < kFxSums; ++i) acc.s[i * Acc::kStride] = acc.s[i * Acc::kStride] >> sh;
+      for (int i = 0; i < kFxSums; ++i) acc.s[i * Acc::kStride] = (acc.s[i * Acc::kStride] + (1LL << (sh - 1))) >> sh;
     }
     acc.E = E;
   }
   const int ash = 1079 - acc.E;
-  const fxs Apx = fx_split(fx_from_bits(Ap.x, ash)), Acx = fx_split(fx_from_bits(Ac.x, ash));
+  const fxs Apx = E ? fx_split(fx_from_bits(Ap.x, ash)) : fxs{0, 0}, Acx = E ? fx_split(fx_from_bits(Ac.x, ash)) : fxs{0, 0};
   // --- orbit at t_f (row A4): mode phase in turns, the centre's Doppler term f k.x_c = f R (k_x cos + k_y sin)
   // included, and the offsets' basis
   const fxc ca = fx_cis(alpha, tab);
-  fxa kc = fx_prod(fx_unpack(pc[30]), fx_split(ca.c));
+  fxa kc = fx_prod<2>(fx_unpack(pc[30]), fx_split(ca.c));
   fx_mac(kc, fx_unpack(pc[31]), fx_split(ca.s));
   const fxu phu = fx_turns(fma(-C.mfac, psi_pn, C.ph0)) - B.frc -
                   ((fxu)fx_mul(fx_split(fx_val(kc)), B.fR) << (4 + D.fx_rsh));
   fxs ob[4];
-  fx_basis(helio ? ca : fx_cis(geo, tab), helio, ob);
-  fx_links(B.at3, B.a4, phu, Apx, Acx, C2 ? &Ap : nullptr, Ac.y, ash, ob, helio, acc, tab, stab, pc);
+  const fxc cg = helio ? ca : fx_cis(geo, tab);
+  fx_basis(cg, helio, ob);
+  if constexpr (Tape::kOn) {
+    tape.st(kFtC, ca.c);
+    tape.st(kFtS, ca.s);
+    if (!helio) {
+      tape.st(kFtGc, cg.c);
+      tape.st(kFtGs, cg.s);
+    }
+  }
+  fx_links(B.at3, B.a4, phu, Apx, Acx, C2 && E ? &Ap : nullptr, Ac.y, ash, ob, helio, acc, tab, stab, pc, tape);
 }
 
 // n 2^e as a double, the power of two added to the exponent field (0 where the result would lie below 2^-1020)
@@ -296,8 +351,9 @@ __device__ __forceinline__ void xyz_from_fx(const Acc& a, fxs zr, fxs zi, fx xr[
     const volatile fx* ac = a.s + 4 * c * Acc::kStride;                  // S_r, S_i, M_r, M_i of link c
     const volatile fx* al = a.s + 4 * ((c + 2) % 3) * Acc::kStride;      // and of link c + 2
     const fxs qr = fx_split(al[2 * Acc::kStride] - ac[0]), qi = fx_split(al[3 * Acc::kStride] - ac[Acc::kStride]);
-    xr[c] = ((al[0] - ac[2 * Acc::kStride]) + fx_sub2(fx_prod(zr, qr), fx_prod(zi, qi))) >> 1;
-    fxa t = fx_prod(zr, qi);
+    // halved: two more quarter units for the bit that drops
+    xr[c] = ((al[0] - ac[2 * Acc::kStride]) + fx_msub<2>(zr, qr, zi, qi)) >> 1;
+    fxa t = fx_prod<4>(zr, qi);
     fx_mac(t, zi, qr);
     xi[c] = ((al[Acc::kStride] - ac[3 * Acc::kStride]) + fx_val(t)) >> 1;
   }

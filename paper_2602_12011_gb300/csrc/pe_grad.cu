@@ -15,10 +15,12 @@
 #include <cuda_runtime.h>
 
 #include "pe_adjoint.cuh"
+#include "pe_adjoint_fx.cuh"
 #include "pe_adjoint_mixed.cuh"
 #include "pe_adjoint_tape.cuh"
 #include "pe_adjoint_tape_mixed.cuh"
 #include "pe_grad.h"
+#include "pe_kernels.h"
 #include "pe_fault.h"
 #include "pe_prep.cuh"
 
@@ -308,6 +310,105 @@ __global__ void __launch_bounds__(kTileBins, 2) k_grad_fwd_tape(DetSet ds, int B
   }
 }
 
+// The gradient on detectors that take the fixed-point unit, both precisions: per bin the forward mode sum writes each unit's
+// tape, the A/E/T cotangents and link seeds follow in FP64, and the reverse sweeps run in fixed point from the tape
+// (pe_adjoint_fx.cuh). Per tile 17 sums: the 14 of the FP64 kernel and the frame's three rotation cotangents, written as
+// the 23 partials the reduction reads. Bound by dependent integer and FP64 operations (about 6,000 thread instructions a
+// unit, FP64 pipe 60 %). 64 LISA samples of 2^22 s: FP64 4.08 -> 1.54 ms; 500 at the mixed precision, whose
+// double-word sweep was at the FP32 pipe's rate, 12.8 -> 10.8 ms; hence both precisions take it.
+constexpr int kGradFxV = 17;
+constexpr int kGradFxCtas = 4;   // resident CTAs per SM (tape 92 MB, inside L2)
+constexpr int kGradFxRow = 7;    // threads that add one row of the block sum
+__global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet ds, int B, const SampleCoef* __restrict__ coef,
+                                                                      const SampleGrad* __restrict__ sgrad,
+                                                                      const int* __restrict__ nend,
+                                                                      const long long* __restrict__ off, double* part,
+                                                                      double* tape_all) {
+  __shared__ double red[kGradFxV][kTileBins + kRedPad];
+  __shared__ fx col[kFxSums][kTileBins];   // the forward sums, then the link seeds, a column per thread
+  __shared__ fx pc[kProj];
+  __shared__ double rot[3];
+  static_assert(kGradFxV * kGradFxRow <= kTileBins, "one pass adds every row");
+  double* tape = tape_all + (size_t)blockIdx.x * kTapeDoubles + threadIdx.x;
+  const int P = ds.ndet * B;
+  const long long total = off[P];
+  const unsigned long long pol = tape_l2_policy();
+  for (long long t = blockIdx.x; t < total; t += gridDim.x) {
+    const int p = find_pair_g(off, P, t);
+    if (!PE_CHK(p >= 0 && p < P && off[p + 1] <= total && nend[p] <= ds.d[p / B].nb, 16)) continue;
+    const int I = p / B, s = p - I * B;
+    const int b = int(t - off[p]) * kTileBins + threadIdx.x;
+    const DetDev& D = ds.d[I];
+    const SampleCoef& S = coef[s];
+    fx_proj_prologue(D, S, pc);   // its first barrier: the previous tile's readers of red and rot are done
+    fx_proj3(pc);
+    double v[kGradFxV];
+#pragma unroll
+    for (int i = 0; i < kGradFxV; ++i) v[i] = 0.0;
+    if (b < nend[p]) {
+      const SampleGrad& SG = sgrad[s];
+      FxBin Bn;
+      load_bin_fx(D, b, S.tc, Bn);
+      FxAcc a;
+      fx_zero(a, &col[0][threadIdx.x]);
+#pragma unroll 1
+      for (int md = 0; md < kNModes; ++md) {
+        if (md == 3 && S.pair32) continue;
+        const ModeCoef& C = S.md[md];
+        if (!C.active || !dlt_pos(Bn.f, C.fend)) continue;
+        const FxTape tp = {tape + tape_slot(md) * kTapeF * kTileBins, pol};
+        mode_bin_fx(D, S, C, Bn, a, ds.d[0].fcis, ds.d[0].fsinc, pc, md, (md == 0 && S.pair32) ? &S.md[3] : nullptr, tp);
+      }
+      double2 o[3], bb[3], pq[6];
+      aet_from_fx(a, D.z[b], o);
+      aet_cotangents(D, b, o, v, bb);
+      const double2 sc = D.sca[b];
+      link_seeds<1>(bb, sc.x, sc.y, pq);
+      const int Es = fx_seeds<kTileBins>(pq, &col[0][threadIdx.x]);
+      const fx a3 = fx_times_k((unsigned)(D.k0 + b), D.fx_a3);
+      const double fm13 = D.fm13[b], invf = fm13 * fm13 * fm13, fR = 2.0 * kPi * D.R * Bn.f;
+      FxBinAcc ga;
+      fx_bin_zero(ga);
+#pragma unroll 1
+      for (int md = 0; md < kNModes; ++md) {
+        if (md == 3 && S.pair32) continue;
+        const ModeCoef& C = S.md[md];
+        if (Es == 0 || !C.active || !dlt_pos(Bn.f, C.fend)) continue;
+        const FxTape tp = {tape + tape_slot(md) * kTapeF * kTileBins, pol};
+        mode_bwd_fx<kTileBins>(D, S, SG, md, (md == 0 && S.pair32) ? 3 : -1, Bn, fm13, invf, fR, a3, &col[0][threadIdx.x], Es, ga, pc,
+                               tp);
+      }
+      GradAcc g;
+      fx_bin_grad(S, SG, ga, g);
+      v[6] = g.M; v[7] = g.q; v[8] = g.c1; v[9] = g.c2; v[10] = g.dL; v[11] = g.io; v[12] = g.ph; v[13] = g.tc;
+      v[14] = g.k[0]; v[15] = g.k[1]; v[16] = g.k[2];
+    }
+#pragma unroll
+    for (int i = 0; i < kGradFxV; ++i) red[i][threadIdx.x] = v[i];
+    __syncthreads();
+    // thread t adds entries g, g + 7, ... of row i = t / 7 (g = t % 7) into red[i][g]; then thread i its seven
+    if (threadIdx.x < kGradFxV * kGradFxRow) {
+      const int i = threadIdx.x / kGradFxRow, g = threadIdx.x % kGradFxRow;
+      double x = red[i][g];
+      for (int k = g + kGradFxRow; k < kTileBins; k += kGradFxRow) x += red[i][k];
+      red[i][g] = x;   // only this thread touches column g of row i in this step
+    }
+    __syncthreads();
+    if (threadIdx.x < kGradFxV) {
+      double x = red[threadIdx.x][0];
+#pragma unroll
+      for (int g = 1; g < kGradFxRow; ++g) x += red[threadIdx.x][g];
+      if (threadIdx.x < kGradV) part[t * kGradW + threadIdx.x] = x;
+      else rot[threadIdx.x - kGradV] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x >= kGradV && threadIdx.x < kGradW) {
+      const int k = threadIdx.x - kGradV;
+      part[t * kGradW + threadIdx.x] = rotation_to_frame(S, rot, k / 3, k % 3);
+    }
+  }
+}
+
 // logL and the gradient from the per-component sums over every detector's tiles.
 __device__ __forceinline__ void grad_write(int s, double L, const double acc[kGradW], const SampleCoef* coef,
                                            const SampleGrad* sgrad, double* logl, double* grad) {
@@ -497,7 +598,9 @@ cudaError_t launch_prep_grad(const double* theta, int B, unsigned mask, const De
 }
 cudaError_t launch_grad_fwd(const DetSet& ds, int B, const SampleCoef* coef, const SampleGrad* sgrad, const int* nend,
                             const long long* off, double* part, int grid, bool mixed, double* tape, cudaStream_t st) {
-  if (mixed)
+  if (fx_all_ok(ds))
+    k_grad_fwd_fx<<<grid, kTileBins, 0, st>>>(ds, B, coef, sgrad, nend, off, part, tape);
+  else if (mixed)
     k_grad_fwd_mixed<<<grid, kTileBins, 0, st>>>(ds, B, coef, sgrad, nend, off, part, tape);
   else
     k_grad_fwd_tape<<<grid, kTileBins, 0, st>>>(ds, B, coef, sgrad, nend, off, part, tape);
@@ -528,7 +631,8 @@ int grad_partial_width() { return kGradW; }
 // FP64: two CTAs per SM (230 registers, no spills; three, at 168 registers, ran 0.4 % slower);
 // mixed: three (168 registers, a few hundred bytes of spills), which its latency-bound sweep
 // prefers (33.6k against 30.9k grad evals/s with two, 33.0k with four)
-int grad_tape_ctas_per_sm(bool mixed) { return mixed ? 3 : 2; }
+// Fixed point: kGradFxCtas.
+int grad_tape_ctas_per_sm(const DetSet& ds, bool mixed) { return fx_all_ok(ds) ? kGradFxCtas : (mixed ? 3 : 2); }
 size_t grad_tape_doubles_per_cta() { return (size_t)kTapeDoubles; }
 int fisher_partial_width() { return kFisherW; }
 

@@ -182,12 +182,12 @@ struct DetDev {
   float2 ratew, alpha0w, geo_ratew;   // rate_t, alpha0_t, geo_rate_t as double words
   float tfw_max;        // |t_f| below which the mixed unit forms t_f and the orbit angles in double words
   // fixed-point unit of the FP64 path (pe_device_fx.cuh): 1 where the detector takes it, 1/L, and
-  // pi L / (4 T), L / (6 T), R / T 2^-fx_rsh as multipliers of the bin's k
+  // pi L / (4 T), L / (6 T), R / T 2^-fx_rsh, pi L / (3 T) as multipliers of the bin's k
   int fx_ok, fx_rsh;
   double fx_iL;
-  FxConst fx_a4, fx_at3, fx_fR;
+  FxConst fx_a4, fx_at3, fx_fR, fx_a3;
   const FxCis* fcis;    // [kSinTab]
-  const FxSinc* fsinc;  // [kFxSincTab]
+  const FxSinc* fsinc;  // [2][kFxSincTab]: sinc and its derivative
   // Q = TDI factor(z) (-i a) e^{-i a}; n_A = 1/sqrt2, n_E = 1/sqrt6, n_T = 1/sqrt3
 };
 

@@ -94,8 +94,9 @@ __device__ __forceinline__ df dd_to_dw(dd a) {
   const float h = __double2float_rn(a.h);
   return df_make(h, __double2float_rn((a.h - (double)h) + a.l));
 }
-// One thread per angle (the first kSinTab) and per (sinc entry, order).
-constexpr int kFxSincOrders = 7;
+// One thread per angle (the first kSinTab) and per (sinc entry, order); snc: sinc's kFxSincTab entries, then its
+// derivative's.
+constexpr int kFxSincOrders = 8;
 __global__ void k_fx_tables(FxCis* cis, FxSinc* snc) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < kSinTab) {
@@ -133,14 +134,17 @@ __global__ void k_fx_tables(FxCis* cis, FxSinc* snc) {
     t = dd_div(dd_mul(dd_mul(t, u2), dd{-(double)(2 * n + 1), 0.0}), (double)((2 * n + 2 - k) * (2 * n + 1 - k) * (2 * n + 3)));
     sum = dd_add(sum, t);
   }
-  FxSinc& o = snc[e];
-  if (k == 0) o.s0 = dd_to_fx(sum);
-  else if (k == 1) o.s1 = dd_to_dw(sum);
-  else if (k == 2) o.s2 = dd_to_dw(sum);
-  else if (k == 3) o.s3 = dd_to_dw(sum);
-  else if (k == 4) o.s4 = (float)sum.h;
-  else if (k == 5) o.s5 = (float)sum.h;
-  else o.s6 = (float)sum.h;
+  auto put = [](FxSinc& o, int order, dd v) {
+    if (order == 0) o.s0 = dd_to_fx(v);
+    else if (order == 1) o.s1 = dd_to_dw(v);
+    else if (order == 2) o.s2 = dd_to_dw(v);
+    else if (order == 3) o.s3 = dd_to_dw(v);
+    else if (order == 4) o.s4 = (float)v.h;
+    else if (order == 5) o.s5 = (float)v.h;
+    else if (order == 6) o.s6 = (float)v.h;
+  };
+  put(snc[e], k, sum);
+  if (k > 0) put(snc[kFxSincTab + e], k - 1, dd_mul(sum, dd{(double)k, 0.0}));   // sinc' about the same points
 }
 
 // Double words of the mixed-precision path: per bin f, a = pi f L, a/(2 pi), sin a, cos a,

@@ -68,3 +68,30 @@ def test_fixed_point_unit_parity(oracle_mod, Lb, name, mask):
     ll, dhhh = oracle_mod.loglike_batch([od], th, mask)
     dd = np.array([oracle_mod.loglike([od], th[0], 0)["dd"][0]])
     H.assert_loglike_parity(g, ll, dhhh, dd, H.floor_terms(oracle_mod, [od], th, mask))
+
+
+@pytest.mark.parametrize("mask", [W.MODE_ALL, 0x12, 0x08])
+@pytest.mark.parametrize("det,T", [(W.LISA, 2.0 ** 16), (W.TIANQIN, 2.0 ** 15), (dict(W.LISA, arm_m=3.0e10), 2.0 ** 14)])
+def test_gradient_where_weights_and_modes_vanish(oracle_mod, Lb, det, T, mask):
+    """The gradient's fixed-point sweep (and the general one, for the long arm) on the bars of the gradient parity
+    tests, where polarisation weights vanish but their derivatives do not (face-on, face-off), at the
+    poles, at edge-on, with equal masses, and with the merger before the data; both precisions."""
+    k0, nb = W.grid(T)
+    inj = W.theta_injection(T)
+    od = H.oracle_detector(oracle_mod, det, T, k0, nb, inj, W.MODE_ALL, 29)
+    gd = H.library_detector(Lb, od)
+    th = W.draw_prior(6, 19, T)
+    th[0, 5], th[1, 5], th[2, 5] = 0.0, np.pi, 0.5 * np.pi
+    th[0, 8], th[3, 8] = 0.5 * np.pi, -0.5 * np.pi
+    th[4, 1] = 1.0 + 1e-9
+    th[5, 10] = -0.2 * T
+    for flag in (0, Lb.PE_PREC_MIXED):
+        g = Lb.loglike_grad([gd], th, mask | flag)
+        for s in range(th.shape[0]):
+            r = oracle_mod.loglike([od], th[s], mask)
+            ll, ref = oracle_mod.grad([od], th[s], mask)
+            F = oracle_mod.fisher([od], th[s], mask)
+            assert abs(g["logl"][s] - ll) <= 1e-10 * H.scale_of(r["dh"], r["hh"], r["dd"])
+            for i in range(11):
+                tol = H.grad_tolerance(ref[i], float(np.sum(r["hh"])), F[i, i])
+                assert abs(g["grad"][s, i] - ref[i]) <= tol, (flag, s, W.PARAM_NAMES[i], g["grad"][s, i], ref[i], tol)

@@ -265,7 +265,9 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
   fxu alpha;           // the centre's angle and, for a geocentric orbit, the constellation's
   fxu geo = 0;
   if (helio && fabsf(tau.x) < kFxTauMax) {
-    alpha = (fxu)pc[32] + ((fxu)fx_from_dw(dfl_mul(tau, D.ratew)) << 4);
+    // the series' terms may cancel and leave a low word beyond fx_from_dw's bound: normalised first
+    const df a = dfl_mul(tau, D.ratew);
+    alpha = (fxu)pc[32] + ((fxu)fx_from_dw(two_sum(a.x, a.y)) << 4);
   } else {
     double dpol = S.Pd[7];
 #pragma unroll 1

@@ -99,7 +99,8 @@ __device__ __forceinline__ fxu fx_cycles(double f, double t) {
   return (fx)ut < 0 ? 0 - r : r;
 }
 
-// A double word of magnitude below 2^-8 as Q60: its high word's multiple of 2^-30 by the rounding
+// A double word of magnitude below 2^-8 and low word below 2^-30 (1.5 2^-30 in sum with the remainder's 2^-31, so
+// that the integers' sum holds) as Q60: its high word's multiple of 2^-30 by the rounding
 // constant, the rest (below 2^-30) converted to an integer.
 __device__ __forceinline__ fx fx_from_dw(df x) {
   const float kM = 0.01171875f;   // 1.5 2^-7: one unit in the last place is 2^-30

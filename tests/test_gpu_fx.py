@@ -95,3 +95,24 @@ def test_gradient_where_weights_and_modes_vanish(oracle_mod, Lb, det, T, mask):
             for i in range(11):
                 tol = H.grad_tolerance(ref[i], float(np.sum(r["hh"])), F[i, i])
                 assert abs(g["grad"][s, i] - ref[i]) <= tol, (flag, s, W.PARAM_NAMES[i], g["grad"][s, i], ref[i], tol)
+
+
+# High masses, unequal and spinning: t_f's series terms are hundreds of times their sum, whose double word is far from normalised.
+CANCELLING = np.array([
+    [9.44096895e+06, 9.11190755, -0.836978605, -0.425334183, 27.3127246, 2.56475767, 4.65730762, 2.08844287, -0.279393, 2.21142, 505558.0],
+    [9.99833e+06, 7.88270, -0.624269, -0.926790, 35.2661, 1.04696, 2.18150, 1.61548, -0.313205, 2.70229, 353475.0],
+    [9.75437e+06, 9.77584, -0.834856, -0.392306, 7.79320, 1.67881, 1.96344, 4.23071, -0.428794, 1.96235, 356152.0],
+    [9.78440e+06, 9.64430, -0.920518, 0.585617, 31.5393, 0.821924, 0.508002, 0.761395, -0.0310906, 2.33068, 317660.0]])
+
+
+@pytest.mark.parametrize("first", range(66, 600, 89))
+def test_time_far_below_its_terms(oracle_mod, Lb, first):
+    T, nb = 655360.0, 89
+    od = H.oracle_detector(oracle_mod, W.LISA, T, first, nb, CANCELLING[0], 0x10, 37)
+    gd = H.library_detector(Lb, od)
+    th = np.repeat(CANCELLING, 64, axis=0)
+    th[:, 0] *= 1.0 + 1e-4 * np.tile(np.arange(64), len(CANCELLING))
+    g = Lb.loglike([gd], th, 0x10, dhhh=True)
+    ll, dhhh = oracle_mod.loglike_batch([od], th, 0x10)
+    dd = np.array([oracle_mod.loglike([od], th[0], 0)["dd"][0]])
+    H.assert_loglike_parity(g, ll, dhhh, dd, H.floor_terms(oracle_mod, [od], th, 0x10))

@@ -611,7 +611,8 @@ pe_status pe_loglike_batch(const pe_detector* dets, int ndet, const double* thet
   pe::lookup_tuned(ds, B, mode_mask, &tc);
   PE_CUDA(sc.alloc(&coef, B));
   PE_CUDA(sc.alloc(&nend, P));
-  PE_CUDA(sc.alloc(&off, P + 1));
+  PE_CUDA(sc.alloc(&off, P + 3));   // and the work counter
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(off + P + 1);
   if (tc.subtiles > 1) PE_CUDA(sc.alloc(&offi, P + 1));
   PE_CUDA(sc.alloc(&part, (size_t)max_tiles * 6));
   const bool h_logl = !is_device_ptr(out_logl);
@@ -624,11 +625,11 @@ pe_status pe_loglike_batch(const pe_detector* dets, int ndet, const double* thet
   if (h_dhhh) PE_CUDA(sc.alloc(&dhhh, (size_t)B * ndet * 6));
   if (h_stat) PE_CUDA(sc.alloc(&stat, B));
   PE_CUDA(pe::launch_prep(th, B, mode_mask, ds, coef, nend, stat, st));
-  PE_CUDA(pe::launch_fwd_offsets(nend, P, off, offi, tc.subtiles, st));
+  PE_CUDA(pe::launch_fwd_offsets(nend, P, off, offi, tc.subtiles, ctr, st));
   void* prof = nullptr;
   pe::profile_begin(st, &prof);
   PE_CUDA(pe::launch_loglike_fwd_variant(tc.variant, pe::mask_prec(mode_mask), ds, B, coef, nend, off, offi,
-                                         tc.subtiles, part, pe::grid_for(tc, max_tiles), st));
+                                         tc.subtiles, part, pe::grid_for(tc, max_tiles), ctr, st));
   pe::profile_end(st, prof);
   PE_CUDA(pe::launch_reduce(ds, B, off, part, coef, logl, dhhh, st));
   if (h_logl) PE_CUDA(cudaMemcpyAsync(out_logl, logl, (size_t)B * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -672,7 +673,8 @@ pe_status pe_loglike_grad_batch(const pe_detector* dets, int ndet, const double*
   PE_CUDA(sc.alloc(&coef, B));
   PE_CUDA(sc.alloc(&sg, B));
   PE_CUDA(sc.alloc(&nend, P));
-  PE_CUDA(sc.alloc(&off, P + 1));
+  PE_CUDA(sc.alloc(&off, P + 3));   // and the work counter
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(off + P + 1);
   PE_CUDA(sc.alloc(&part, (size_t)max_tiles * W));
   const bool h_logl = out_logl && !is_device_ptr(out_logl);
   const bool h_grad = !is_device_ptr(out_grad);
@@ -684,7 +686,7 @@ pe_status pe_loglike_grad_batch(const pe_detector* dets, int ndet, const double*
   if (h_grad) PE_CUDA(sc.alloc(&grad, (size_t)B * PE_NPARAM));
   if (h_stat) PE_CUDA(sc.alloc(&stat, B));
   PE_CUDA(pe::launch_prep_grad(th, B, mode_mask, ds, coef, sg, nend, stat, st));
-  PE_CUDA(pe::launch_scan_tiles(nend, P, off, pe::kTileBins, st));
+  PE_CUDA(pe::launch_scan_tiles(nend, P, off, pe::kTileBins, ctr, st));
   // a persistent grid of the kernel's resident CTAs per SM, each with its tape region
   const long long g = std::max<long long>(
       1, std::min<long long>(max_tiles, (long long)sm_count() * pe::grad_tape_ctas_per_sm(ds, mixed)));
@@ -692,7 +694,7 @@ pe_status pe_loglike_grad_batch(const pe_detector* dets, int ndet, const double*
   PE_CUDA(sc.alloc(&tape, (size_t)g * pe::grad_tape_doubles_per_cta()));
   void* prof = nullptr;
   pe::profile_begin(st, &prof);
-  PE_CUDA(pe::launch_grad_fwd(ds, B, coef, sg, nend, off, part, (int)g, mixed, tape, st));
+  PE_CUDA(pe::launch_grad_fwd(ds, B, coef, sg, nend, off, part, (int)g, mixed, tape, ctr, st));
   pe::profile_end(st, prof);
   PE_CUDA(pe::launch_grad_reduce(ds, B, off, part, coef, sg, logl, grad, st));
   if (h_logl) PE_CUDA(cudaMemcpyAsync(out_logl, logl, (size_t)B * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -739,7 +741,7 @@ pe_status pe_fisher(const pe_detector* dets, int ndet, const double* theta, int 
   double* F = out_F;
   if (h_F) PE_CUDA(sc.alloc(&F, (size_t)B * 121));
   PE_CUDA(pe::launch_prep_grad(th, B, mode_mask, ds, coef, sg, nend, nullptr, st));
-  PE_CUDA(pe::launch_scan_tiles(nend, P, off, pe::kTileBins, st));
+  PE_CUDA(pe::launch_scan_tiles(nend, P, off, pe::kTileBins, nullptr, st));
   const long long g = std::min<long long>(max_tiles, (long long)sm_count() * 16);
   void* prof = nullptr;
   pe::profile_begin(st, &prof);

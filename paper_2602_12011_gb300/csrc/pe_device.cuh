@@ -362,6 +362,27 @@ __device__ __forceinline__ void xyz_final(const XYZAcc& a, double2 z, double2 x[
   }
 }
 
+// Dynamic work lists: a persistent CTA starts with item blockIdx.x; thread 0 draws its next item from ctr[0] when it starts
+// one (work_fetch; the atomic's latency hides behind the item) and hands it to the CTA at the end (work_next, a
+// barrier). The last CTA to leave clears both words for the next launch (work_done). ctr NULL: static striding.
+__device__ __forceinline__ long long work_fetch(unsigned long long* ctr, long long t) {
+  if (ctr == nullptr) return t + gridDim.x;
+  return threadIdx.x == 0 ? (long long)(gridDim.x + atomicAdd(ctr, 1ULL)) : 0;
+}
+__device__ __forceinline__ long long work_next(long long tn, long long* next) {
+  __syncthreads();   // the last item's readers of *next are done
+  if (threadIdx.x == 0) *next = tn;
+  __syncthreads();
+  return *next;
+}
+__device__ __forceinline__ void work_done(unsigned long long* ctr) {
+  if (ctr == nullptr || threadIdx.x != 0) return;
+  if (atomicAdd(ctr + 1, 1ULL) + 1 == gridDim.x) {
+    ctr[0] = 0;
+    ctr[1] = 0;
+  }
+}
+
 // Per-bin inputs shared by all modes of one bin.
 // a < b for non-negative doubles by the order of their bit patterns: an integer compare, exact
 // (GB300 runs the double compare DSETP on its narrow FP64 pipe)

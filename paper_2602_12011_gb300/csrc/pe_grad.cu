@@ -323,7 +323,8 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
                                                                       const SampleGrad* __restrict__ sgrad,
                                                                       const int* __restrict__ nend,
                                                                       const long long* __restrict__ off, double* part,
-                                                                      double* tape_all) {
+                                                                      double* tape_all, unsigned long long* ctr) {
+  __shared__ long long next;
   __shared__ double red[kGradFxV][kTileBins + kRedPad];
   __shared__ fx col[kFxSums][kTileBins];   // the forward sums, then the link seeds, a column per thread
   __shared__ fx pc[kProj];
@@ -333,7 +334,8 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
   const int P = ds.ndet * B;
   const long long total = off[P];
   const unsigned long long pol = tape_l2_policy();
-  for (long long t = blockIdx.x; t < total; t += gridDim.x) {
+  for (long long t = blockIdx.x, tn = 0; t < total; t = work_next(tn, &next)) {
+    tn = work_fetch(ctr, t);
     const int p = find_pair_g(off, P, t);
     if (!PE_CHK(p >= 0 && p < P && off[p + 1] <= total && nend[p] <= ds.d[p / B].nb, 16)) continue;
     const int I = p / B, s = p - I * B;
@@ -407,6 +409,7 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
       part[t * kGradW + threadIdx.x] = rotation_to_frame(S, rot, k / 3, k % 3);
     }
   }
+  work_done(ctr);
 }
 
 // logL and the gradient from the per-component sums over every detector's tiles.
@@ -597,9 +600,10 @@ cudaError_t launch_prep_grad(const double* theta, int B, unsigned mask, const De
   return prep_launch<true>(theta, B, mask, ds, coef, sgrad, nend, status, st);
 }
 cudaError_t launch_grad_fwd(const DetSet& ds, int B, const SampleCoef* coef, const SampleGrad* sgrad, const int* nend,
-                            const long long* off, double* part, int grid, bool mixed, double* tape, cudaStream_t st) {
+                            const long long* off, double* part, int grid, bool mixed, double* tape, unsigned long long* ctr,
+                            cudaStream_t st) {
   if (fx_all_ok(ds))
-    k_grad_fwd_fx<<<grid, kTileBins, 0, st>>>(ds, B, coef, sgrad, nend, off, part, tape);
+    k_grad_fwd_fx<<<grid, kTileBins, 0, st>>>(ds, B, coef, sgrad, nend, off, part, tape, ctr);
   else if (mixed)
     k_grad_fwd_mixed<<<grid, kTileBins, 0, st>>>(ds, B, coef, sgrad, nend, off, part, tape);
   else

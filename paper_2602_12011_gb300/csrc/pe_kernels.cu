@@ -338,7 +338,8 @@ __global__ void k_sum_parts(const double* part, int n, int w, double* out) {
 // Exclusive prefix sums of tiles per (detector, sample) pair, for tiles of 2^sa bins (off) and, if offb is not NULL, of
 // 2^sb bins (offb); off[P], offb[P] = totals. One CTA: each thread adds a run of pairs, a warp shuffle scan
 // and one over the warps join the runs (a serial pass over 1,024 partials by one thread took 8 us).
-__global__ void k_scan_tiles(const int* nend, int P, int sa, long long* off, int sb, long long* offb) {
+// ctr (nullable): the next kernel's work counter, cleared.
+__global__ void k_scan_tiles(const int* nend, int P, int sa, long long* off, int sb, long long* offb, unsigned long long* ctr) {
   __shared__ long long wsum[2][32];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int chunk = (P + blockDim.x - 1) / blockDim.x;
@@ -365,6 +366,7 @@ __global__ void k_scan_tiles(const int* nend, int P, int sa, long long* off, int
     ra += (n + (1 << sa) - 1) >> sa;
     rb += (n + (1 << sb) - 1) >> sb;
   }
+  if (t < 2 && ctr) ctr[t] = 0;
   if (t == (int)blockDim.x - 1) {
     off[P] = ra;
     if (offb) offb[P] = rb;
@@ -384,7 +386,9 @@ __device__ __forceinline__ int find_pair(const long long* off, int P, long long 
 // ------------------------------------------------------------------------------------------
 // Rows A2-A7: persistent fused kernel. The work list is every (detector, sample) pair's 128-bin
 // sub-tiles (off: their offsets per pair); a work item is R consecutive sub-tiles of one pair
-// (offi: the items' offsets), and CTAs stride over the items. Per item the CTA forms the pair's
+// (offi: the items' offsets); each CTA starts with the item of its index and draws the next ones from a
+// counter while it works (items differ by what modes reach them: striding statically left a last round
+// of unequal CTAs, 1024 LISA samples 6.4 ms on six resident CTAs per SM and 8.5 ms on a grid of eight). Per item the CTA forms the pair's
 // projection forms once; per sub-tile each thread owns one bin (coalesced), sums the modes' TDI
 // brackets in registers, forms A/E/T and the weighted products, and the CTA reduces them in a
 // fixed order into part[sub-tile][6] (<d|h>_c, <h|h>_c). The partials are per sub-tile whatever
@@ -398,7 +402,8 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
                                                                  const int* __restrict__ nend,
                                                                  const long long* __restrict__ off,
                                                                  const long long* __restrict__ offi, int R,
-                                                                 double* part) {
+                                                                 double* part, unsigned long long* ctr) {
+  __shared__ long long next;
   __shared__ double red[6][kTileBins + kRedPad];   // block_sum6 staging (as float2 or float rows)
   __shared__ double pc[kProj];    // the item's projection forms (proj_coef; fx_proj_prologue's words)
   __shared__ float2 pcw[kProj];   // the same as double words (mixed) or floats (.x, FP32)
@@ -414,7 +419,8 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
   __syncthreads();
   const int P = ds.ndet * B;
   const long long total = offi[P];
-  for (long long t = blockIdx.x; t < total; t += gridDim.x) {
+  for (long long t = blockIdx.x, tn = 0; t < total; t = work_next(tn, &next)) {
+    tn = work_fetch(ctr, t);
     const int p = find_pair(offi, P, t);
     if (!PE_CHK(p >= 0 && p < P, 1)) continue;              // checked build: uniform over the CTA
     const int I = p / B, s = p - I * B;
@@ -505,6 +511,7 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
       }
     }
   }
+  work_done(ctr);
 }
 
 // Row A7, small grids (at most kReduceWarpTiles tiles a detector): one warp per sample; for each detector a lane-strided, shuffle-tree sum of that
@@ -678,16 +685,17 @@ int tile_shift(int tile_bins) {   // log2 of kTileBins times 1, 2, 4 or 8; -1 ot
 static_assert(kTileBins == 128, "tile_shift counts from 2^7");
 int scan_threads(int P) { return P >= 1024 ? 1024 : (P + 31) / 32 * 32; }
 }  // namespace
-cudaError_t launch_scan_tiles(const int* nend, int P, long long* off, int tile_bins, cudaStream_t st) {
+cudaError_t launch_scan_tiles(const int* nend, int P, long long* off, int tile_bins, unsigned long long* ctr, cudaStream_t st) {
   const int sa = tile_shift(tile_bins);
   if (sa < 0 || P < 1) return cudaErrorInvalidValue;
-  k_scan_tiles<<<1, scan_threads(P), 0, st>>>(nend, P, sa, off, sa, nullptr);
+  k_scan_tiles<<<1, scan_threads(P), 0, st>>>(nend, P, sa, off, sa, nullptr, ctr);
   return pe::launch_status();
 }
-cudaError_t launch_fwd_offsets(const int* nend, int P, long long* off, long long* offi, int R, cudaStream_t st) {
+cudaError_t launch_fwd_offsets(const int* nend, int P, long long* off, long long* offi, int R, unsigned long long* ctr,
+                               cudaStream_t st) {
   const int sb = tile_shift(R * kTileBins);
   if (sb < 0 || P < 1) return cudaErrorInvalidValue;
-  k_scan_tiles<<<1, scan_threads(P), 0, st>>>(nend, P, 7, off, sb, R > 1 ? offi : nullptr);
+  k_scan_tiles<<<1, scan_threads(P), 0, st>>>(nend, P, 7, off, sb, R > 1 ? offi : nullptr, ctr);
   return pe::launch_status();
 }
 cudaError_t launch_dw_tables(const double* f, const double* f13, const double* fm13, const double* fm76, const double2* sca,
@@ -718,17 +726,16 @@ cudaError_t launch_f32_tables(const double* f, const double* f13, const double* 
   return pe::launch_status();
 }
 cudaError_t launch_loglike_fwd(const DetSet& ds, int B, const SampleCoef* coef, const int* nend, const long long* off,
-                               const long long* offi, int R, double* part, int grid, int prec, cudaStream_t st) {
-  return launch_loglike_fwd_variant(kFwdDefaultVariant, prec, ds, B, coef, nend, off, offi, R, part, grid, st);
+                               const long long* offi, int R, double* part, int grid, unsigned long long* ctr, int prec,
+                               cudaStream_t st) {
+  return launch_loglike_fwd_variant(kFwdDefaultVariant, prec, ds, B, coef, nend, off, offi, R, part, grid, ctr, st);
 }
 
 namespace {
-// CTAs stride over the items statically, so a grid of one and a fraction times the resident CTAs runs its last
-// round nearly empty (1024 LISA samples: 8.5 ms with 8 CTAs per SM where 6 are resident, 6.4 ms with
-// 6): the grid is cut to the resident CTAs, a count kept per kernel and device.
+// The grid is cut to the resident CTAs (a count kept per kernel and device): they draw the items, so more would only wait.
 template <int MINB, int PREC>
 cudaError_t fwd_one(const DetSet& ds, int B, const SampleCoef* coef, const int* nend, const long long* off,
-                    const long long* offi, int R, double* part, int grid, bool items, cudaStream_t st) {
+                    const long long* offi, int R, double* part, int grid, bool items, unsigned long long* ctr, cudaStream_t st) {
   static std::atomic<int> resident[64];
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
@@ -743,31 +750,31 @@ cudaError_t fwd_one(const DetSet& ds, int B, const SampleCoef* coef, const int* 
     }
     if (r > 0 && grid > r) grid = r;
   }
-  k_loglike_fwd<MINB, PREC><<<grid, kTileBins, 0, st>>>(ds, B, coef, nend, off, items ? offi : off, R, part);
+  k_loglike_fwd<MINB, PREC><<<grid, kTileBins, 0, st>>>(ds, B, coef, nend, off, items ? offi : off, R, part, ctr);
   return pe::launch_status();
 }
 }  // namespace
 
 cudaError_t launch_loglike_fwd_variant(int variant, int prec, const DetSet& ds, int B, const SampleCoef* coef,
                                        const int* nend, const long long* off, const long long* offi, int R,
-                                       double* part, int grid, cudaStream_t st, bool items) {
+                                       double* part, int grid, unsigned long long* ctr, cudaStream_t st, bool items) {
   items |= R > 1;
   if (R != 1 && R != 2 && R != 4 && R != 8) return cudaErrorInvalidValue;
   // FP64: the fixed-point unit where every detector meets its bounds
   if (prec == kPrecFP64 && fx_all_ok(ds)) prec = kPrecFx;
   switch (variant * 4 + prec) {
-    case 0: return fwd_one<2, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 1: return fwd_one<2, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 2: return fwd_one<2, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 3: return fwd_one<4, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 4: return fwd_one<3, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 5: return fwd_one<3, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 6: return fwd_one<3, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 7: return fwd_one<6, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 8: return fwd_one<4, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 9: return fwd_one<4, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 10: return fwd_one<4, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
-    case 11: return fwd_one<5, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, st);
+    case 0: return fwd_one<2, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 1: return fwd_one<2, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 2: return fwd_one<2, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 3: return fwd_one<4, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 4: return fwd_one<3, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 5: return fwd_one<3, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 6: return fwd_one<3, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 7: return fwd_one<6, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 8: return fwd_one<4, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 9: return fwd_one<4, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 10: return fwd_one<4, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 11: return fwd_one<5, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -27,7 +27,7 @@ namespace {
 
 constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + 256];   // and the work counter
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -102,6 +102,7 @@ extern "C" pe_status pe_loglike_batch_noalloc(const pe_detector* dets, int ndet,
   long long* off = reinterpret_cast<long long*>(sc + o_off);
   long long* offi = reinterpret_cast<long long*>(sc + o_offi);
   double* part = reinterpret_cast<double*>(sc + o_part);
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(sc + kNoAllocScratchBytes);   // after the scratch
   // Every scratch element a kernel reads is written earlier in the same call (coefficients and
   // active counts by the prep kernel, offsets by the scan, one partial per tile by the forward
   // kernel), so nothing is cleared between calls.
@@ -113,10 +114,10 @@ extern "C" pe_status pe_loglike_batch_noalloc(const pe_detector* dets, int ndet,
     nsm = 1;
   }
   cudaError_t e = pe::launch_prep(theta, B, mode_mask, ds, coef, nend, out_status, st);
-  if (e == cudaSuccess) e = pe::launch_fwd_offsets(nend, (int)P, off, offi, R, st);
+  if (e == cudaSuccess) e = pe::launch_fwd_offsets(nend, (int)P, off, offi, R, ctr, st);
   const size_t g = max_tiles < (size_t)nsm * pe::fwd_blocks_per_sm() ? max_tiles : (size_t)nsm * pe::fwd_blocks_per_sm();
   if (e == cudaSuccess) e = pe::launch_loglike_fwd(ds, B, coef, nend, off, offi, R, part, (int)(g > 0 ? g : 1),
-                                                     pe::mask_prec(mode_mask), st);
+                                                     ctr, pe::mask_prec(mode_mask), st);
   if (e == cudaSuccess) e = pe::launch_reduce(ds, B, off, part, coef, out_logl, out_dhhh, st);
   if (e != cudaSuccess) {
     char msg[256];

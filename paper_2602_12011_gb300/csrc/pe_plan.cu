@@ -143,8 +143,8 @@ int grid_for(const TuneChoice& c, long long max_tiles) {
 // precision's default sub-tiles per item, then every sub-tile count (1, 2, 4, 8) at the best of
 // those. Each candidate: one warm launch, the best of two timed ones.
 cudaError_t autotune_fwd(const DetSet& ds, int B, unsigned mask, const SampleCoef* coef, const int* nend,
-                         const long long* off, long long* offi, double* part, long long max_tiles, cudaStream_t st,
-                         TuneChoice* best) {
+                         const long long* off, long long* offi, double* part, long long max_tiles,
+                         unsigned long long* ctr, cudaStream_t st, TuneChoice* best) {
   static const int kCtas[] = {2, 4, 8, 16};
   static const int kSub[] = {1, 2, 4, 8};
   const int prec = mask_prec(mask);
@@ -156,13 +156,13 @@ cudaError_t autotune_fwd(const DetSet& ds, int B, unsigned mask, const SampleCoe
   auto time_one = [&](const TuneChoice& c, float* out_ms) -> cudaError_t {
     const int grid = grid_for(c, max_tiles);
     cudaError_t r = cudaSuccess;
-    if (c.subtiles > 1) r = launch_scan_tiles(nend, P, offi, c.subtiles * kTileBins, st);
+    if (c.subtiles > 1) r = launch_scan_tiles(nend, P, offi, c.subtiles * kTileBins, nullptr, st);
     if (r == cudaSuccess)
-      r = launch_loglike_fwd_variant(c.variant, prec, ds, B, coef, nend, off, offi, c.subtiles, part, grid, st);  // warm
+      r = launch_loglike_fwd_variant(c.variant, prec, ds, B, coef, nend, off, offi, c.subtiles, part, grid, ctr, st);  // warm
     float bm = 1e30f;
     for (int k = 0; k < 2 && r == cudaSuccess; ++k) {
       cudaEventRecord(e0, st);
-      r = launch_loglike_fwd_variant(c.variant, prec, ds, B, coef, nend, off, offi, c.subtiles, part, grid, st);
+      r = launch_loglike_fwd_variant(c.variant, prec, ds, B, coef, nend, off, offi, c.subtiles, part, grid, ctr, st);
       cudaEventRecord(e1, st);
       if (r == cudaSuccess) r = cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -249,7 +249,7 @@ pe_status pe_plan_create(const pe_detector* dets, int ndet, int B, unsigned mode
   for (int i = 0; i < ndet; ++i) max_tiles += (long long)B * pe::tiles_of(ds.d[i].nb, pe::kTileBins);
   const size_t o_nend = a256((size_t)B * sizeof(pe::SampleCoef));
   const size_t o_off = a256(o_nend + P * sizeof(int));
-  const size_t o_offi = a256(o_off + (P + 1) * sizeof(long long));
+  const size_t o_offi = a256(o_off + (P + 3) * sizeof(long long));   // and the work counter
   const size_t o_part = a256(o_offi + (P + 1) * sizeof(long long));
   const size_t bytes = o_part + (size_t)max_tiles * 6 * sizeof(double);
   pe_plan_s* pl = new (std::nothrow) pe_plan_s();
@@ -267,15 +267,16 @@ pe_status pe_plan_create(const pe_detector* dets, int ndet, int B, unsigned mode
   int* nend = reinterpret_cast<int*>(sc + o_nend);
   long long* off = reinterpret_cast<long long*>(sc + o_off);
   long long* offi = reinterpret_cast<long long*>(sc + o_offi);
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(off + P + 1);
   double* part = reinterpret_cast<double*>(sc + o_part);
   cudaStream_t cs = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   pl->choice = pe::default_choice(pe::mask_prec(mode_mask));
   if (e == cudaSuccess && !pe::lookup_tuned(ds, B, mode_mask, &pl->choice) && autotune) {
     e = pe::launch_prep(theta_dev, B, mode_mask, ds, coef, nend, nullptr, cs);
-    if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, (int)P, off, pe::kTileBins, cs);
+    if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, (int)P, off, pe::kTileBins, ctr, cs);
     pe::TuneChoice best;
-    if (e == cudaSuccess) e = pe::autotune_fwd(ds, B, mode_mask, coef, nend, off, offi, part, max_tiles, cs, &best);
+    if (e == cudaSuccess) e = pe::autotune_fwd(ds, B, mode_mask, coef, nend, off, offi, part, max_tiles, ctr, cs, &best);
     if (e == cudaSuccess) {
       pl->choice = best;
       pe::store_tuned(ds, B, mode_mask, best);
@@ -284,10 +285,10 @@ pe_status pe_plan_create(const pe_detector* dets, int ndet, int B, unsigned mode
   if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
     cudaError_t e1 = pe::launch_prep(theta_dev, B, mode_mask, ds, coef, nend, out_status_dev, cs);
-    if (e1 == cudaSuccess) e1 = pe::launch_fwd_offsets(nend, (int)P, off, offi, pl->choice.subtiles, cs);
+    if (e1 == cudaSuccess) e1 = pe::launch_fwd_offsets(nend, (int)P, off, offi, pl->choice.subtiles, ctr, cs);
     if (e1 == cudaSuccess)
       e1 = pe::launch_loglike_fwd_variant(pl->choice.variant, pe::mask_prec(mode_mask), ds, B, coef, nend, off, offi,
-                                          pl->choice.subtiles, part, pe::grid_for(pl->choice, max_tiles), cs);
+                                          pl->choice.subtiles, part, pe::grid_for(pl->choice, max_tiles), ctr, cs);
     if (e1 == cudaSuccess) e1 = pe::launch_reduce(ds, B, off, part, coef, out_logl_dev, out_dhhh_dev, cs);
     e = cudaStreamEndCapture(cs, &pl->graph);
     if (e == cudaSuccess && e1 != cudaSuccess) e = e1;
@@ -355,7 +356,7 @@ pe_status pe_autotune(const pe_detector* dets, int ndet, const double* theta_dev
   for (int i = 0; i < ndet; ++i) max_tiles += (long long)B * pe::tiles_of(ds.d[i].nb, pe::kTileBins);
   const size_t o_nend = a256((size_t)B * sizeof(pe::SampleCoef));
   const size_t o_off = a256(o_nend + P * sizeof(int));
-  const size_t o_offi = a256(o_off + (P + 1) * sizeof(long long));
+  const size_t o_offi = a256(o_off + (P + 3) * sizeof(long long));   // and the work counter
   const size_t o_part = a256(o_offi + (P + 1) * sizeof(long long));
   const size_t bytes = o_part + (size_t)max_tiles * 6 * sizeof(double);
   void* scratch = nullptr;
@@ -368,13 +369,14 @@ pe_status pe_autotune(const pe_detector* dets, int ndet, const double* theta_dev
   int* nend = reinterpret_cast<int*>(sc + o_nend);
   long long* off = reinterpret_cast<long long*>(sc + o_off);
   long long* offi = reinterpret_cast<long long*>(sc + o_offi);
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(off + P + 1);
   double* part = reinterpret_cast<double*>(sc + o_part);
   cudaStream_t cs = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   pe::TuneChoice best = pe::default_choice(pe::mask_prec(mode_mask));
   if (e == cudaSuccess) e = pe::launch_prep(theta_dev, B, mode_mask, ds, coef, nend, nullptr, cs);
-  if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, (int)P, off, pe::kTileBins, cs);
-  if (e == cudaSuccess) e = pe::autotune_fwd(ds, B, mode_mask, coef, nend, off, offi, part, max_tiles, cs, &best);
+  if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, (int)P, off, pe::kTileBins, ctr, cs);
+  if (e == cudaSuccess) e = pe::autotune_fwd(ds, B, mode_mask, coef, nend, off, offi, part, max_tiles, ctr, cs, &best);
   if (cs) cudaStreamDestroy(cs);
   pe::dfree(scratch);
   if (e != cudaSuccess) {

@@ -20,10 +20,11 @@ bool lookup_tuned(const DetSet& ds, int B, unsigned mask, TuneChoice* out);
 TuneChoice default_choice(int prec);
 int grid_for(const TuneChoice& c, long long max_tiles);
 // Times the candidates on the prepared work list (coefficients, active counts and sub-tile offsets
-// off on the device; offi: scratch for the work-item offsets, P + 1 entries) and returns the fastest.
+// off on the device; offi: scratch for the work-item offsets, P + 1 entries; ctr: off's
+// work counter) and returns the fastest.
 cudaError_t autotune_fwd(const DetSet& ds, int B, unsigned mask, const SampleCoef* coef, const int* nend,
-                         const long long* off, long long* offi, double* part, long long max_tiles, cudaStream_t st,
-                         TuneChoice* best);
+                         const long long* off, long long* offi, double* part, long long max_tiles,
+                         unsigned long long* ctr, cudaStream_t st, TuneChoice* best);
 void store_tuned(const DetSet& ds, int B, unsigned mask, const TuneChoice& c);
 
 }  // namespace pe

@@ -1716,12 +1716,13 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   aalloc(&off, P + 1);
   int *nin = nullptr, *nout = nullptr;
   long long *offin = nullptr, *offout = nullptr;
+  unsigned long long* ctr = nullptr;
   const bool split = mode == 0;   // log L: the spline path's tiles and the per-bin path's in their own kernels
   if (split) {
     aalloc(&nin, P);
     aalloc(&nout, P);
     aalloc(&offin, P + 1);
-    aalloc(&offout, P + 1);
+    aalloc(&offout, P + 3);   // and the work counter
   }
   aalloc(&part, (size_t)max_tiles * 6);
   aalloc(&nodes, nsys * pe::kQ * pe::kNodes);
@@ -1776,7 +1777,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
     }
   }
   if (e == cudaSuccess) e = pe::launch_prep(theta_dev, B, mode_mask, ds, S, nend, nullptr, st);
-  if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, P, off, pe::kTileBins, st);
+  if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, P, off, pe::kTileBins, nullptr, st);
   const int prec = mix ? pe::kPrecMixed : pe::kPrecFP64;
   pe::TuneChoice tcm = pe::default_choice(prec);
   if (split) pe::lookup_tuned(ds, B, mode_mask | (mix ? PE_PREC_MIXED : 0u), &tcm);
@@ -1786,9 +1787,10 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
       if (ds.d[I].orbit != 0) geo_mask |= 1u << I;
     pe::k_split_nend<<<(P + 127) / 128, 128, 0, st>>>(theta_dev, ndet, B, s->box, geo_mask, nend, nin, nout);
     e = pe::launch_status();
-    if (e == cudaSuccess) e = pe::launch_scan_tiles(nin, P, offin, pe::kTileBins, st);
+    if (e == cudaSuccess) e = pe::launch_scan_tiles(nin, P, offin, pe::kTileBins, nullptr, st);
     // the fallback pairs' work items for the forward kernel of pe_loglike_batch
-    if (e == cudaSuccess) e = pe::launch_scan_tiles(nout, P, offout, tcm.subtiles * pe::kTileBins, st);
+    ctr = reinterpret_cast<unsigned long long*>(offout + P + 1);
+    if (e == cudaSuccess) e = pe::launch_scan_tiles(nout, P, offout, tcm.subtiles * pe::kTileBins, ctr, st);
   }
   if (e == cudaSuccess) {
     int nsm = 1, dev = 0;
@@ -1809,7 +1811,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
       // off[p] + its index, the same place as in the full list
       if (e == cudaSuccess)
         e = pe::launch_loglike_fwd_variant(tcm.variant, prec, ds, B, S, nend, off, offout, tcm.subtiles, part,
-                                           pe::grid_for(tcm, max_tiles), st, true);
+                                           pe::grid_for(tcm, max_tiles), ctr, st, true);
     } else {
       auto kern = pe::fx_all_ok(ds) ? pe::k_sur_fwd<true> : pe::k_sur_fwd<false>;
       kern<<<(unsigned)g, pe::kTileBins, 0, st>>>(ds, B, S, S0, theta_dev, s->box, spl, splt, hs, nend, off, part);

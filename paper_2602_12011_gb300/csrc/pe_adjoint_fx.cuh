@@ -22,13 +22,61 @@ namespace pe {
 // The tape of one thread: field f at p[f * kTileBins] of the CTA's region in global memory, held in L2 by the evict-last
 // hint (tape_l2_policy).
 struct FxTape {
-  static constexpr bool kOn = true;
+  static constexpr bool kOn = true, kChain = false;
   double* p;
   unsigned long long pol;
   __device__ __forceinline__ void st(int f, fx v) const { tst(p + f * kTileBins, __longlong_as_double(v), pol); }
   __device__ __forceinline__ fx ld(int f) const { return __double_as_longlong(tld(p + f * kTileBins, pol)); }
 };
 static_assert((int)kFtFields <= (int)kTapeF, "the regions are those of the FP64 tape");
+
+// The seeds' common factors of one unit's chain rule (doubles): the weights times the amplitude, then v dPsi/dv, v dD/dv, dPsi/dq, dD/dq,
+// 1/v, cos and sin of the centre's angle and d(ln taper)/d Mtot. One sweep per unit forms them in place; the Fisher
+// matrix's six sweeps read them from the tape (kFtChain on).
+struct FxChain {
+  double dv, ddv, pq, dq, iv, co, so, tap;
+};
+enum : int { kFtChain = kFtFields, kFtWeights = kFtChain + 8, kFtAll = kFtWeights + 4 };
+__device__ __forceinline__ void fx_weights(const SampleCoef& S, const ModeCoef& C, const ModeCoef* C2, double amp, double v, double2& Ap,
+                                           double2& Ac) {
+  Ap = make_double2(amp * C.Pp, 0.0);
+  Ac = make_double2(amp * C.Pc2, 0.0);
+  if (C2) {
+    const double2 kap = make_double2(S.k32.x * (v * v), S.k32.y * (v * v));
+    Ap = make_double2(amp * fma(kap.x, C2->Pp, C.Pp), amp * (kap.y * C2->Pp));
+    Ac = make_double2(amp * fma(kap.x, C2->Pc2, C.Pc2), amp * (kap.y * C2->Pc2));
+  }
+}
+__device__ __forceinline__ FxChain fx_chain(const DetDev& D, const SampleCoef& S, const SampleGrad& SG, const ModeCoef& C,
+                                            const ModeGrad& CG, const FxBin& B, double fm13, double v, double w, fx cq, fx sq) {
+  FxChain h;
+  const double lnv = C.lncm + B.lnf3, iv5 = C.icm5 * D.fm53[B.b];
+  // Psi_PN(v), D(v): v dPsi/dv = D, v dD/dv = v^-5 ddpol + Q6 v (2 + ln v); v ~ M^(1/3)
+  double dpol = S.Pd[7], ddpol = S.Pdd[7], pq = SG.dP_dq[7], dq = SG.dPd_dq[7];
+#pragma unroll
+  for (int k = 6; k >= 0; --k) {
+    dpol = fma(dpol, v, S.Pd[k]);
+    ddpol = fma(ddpol, v, S.Pdd[k]);
+    pq = fma(pq, v, SG.dP_dq[k]);
+    dq = fma(dq, v, SG.dPd_dq[k]);
+  }
+  const double q6v = S.Q6 * v, dq6v = SG.dQ6_dq * v;
+  h.dv = fma(iv5, dpol, fma(q6v, 1.0 + lnv, S.Q5));
+  h.ddv = fma(iv5, ddpol, q6v * (2.0 + lnv));
+  h.pq = fma(iv5, pq, lnv * (dq6v + SG.dQ5_dq));
+  h.dq = fma(iv5, dq, fma(dq6v, 1.0 + lnv, SG.dQ5_dq));
+  h.iv = C.icm * fm13;
+  h.co = fx_to_double(cq, -60);
+  h.so = fx_to_double(sq, -60);
+  h.tap = 0.0;
+  if (dlt_pos(C.ftap, B.f)) {
+    const double fe = C.fend, ft = C.ftap, A = fe - ft;
+    const double dz = 0.1 / (fe - B.f) - A / ((fe - B.f) * (fe - B.f)) - 0.1 / (B.f - ft) -
+                      0.9 * A / ((B.f - ft) * (B.f - ft));
+    h.tap = -(1.0 - w) * dz * CG.dfend_dM;
+  }
+  return h;
+}
 
 // Scalars of one unit's sweep, in FP64.
 struct FxBwd {
@@ -37,7 +85,6 @@ struct FxBwd {
   double alpha, geo;   // of the centre's angle and the constellation's (rad), without the Doppler term
   double W[3];      // of the frame's rotation about k, p, q, without the Doppler term
   double2 Ap, Ac;   // of the weights times the amplitude
-  double co, so;    // cos, sin of the centre's angle
 };
 
 // seeds: the bin's P_l, Q_l (x, y each) at seeds[(4 l + i) * SST]; Ap, Ac the weights times the amplitude.
@@ -174,11 +221,8 @@ __device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx*
   }
   // orbit basis b = (cos 2 alpha, sin 2 alpha, cos alpha, sin alpha) or (cos phi_0, sin phi_0)
   const int e = E + Es - 2097;
-  const fx cq = tape.ld(kFtC), sq = tape.ld(kFtS);
-  const fxs c = fx_split(cq), s = fx_split(sq);
-  o.co = fx_to_double(cq, -60);
-  o.so = fx_to_double(sq, -60);
   if (helio) {
+    const fxs c = fx_split(tape.ld(kFtC)), s = fx_split(tape.ld(kFtS));
     fxa q = fx_sq0<1>();
     fx_macsq(q, s);
     const fxs c2 = fx_split(kFxOne - 2 * fx_valsq(q)), s2 = fx_split(2 * fx_mul(s, c));
@@ -224,29 +268,32 @@ __device__ __forceinline__ void mode_bwd_fx(const DetDev& D, const SampleCoef& S
                                             const fx* __restrict__ pc, const Tape& tape) {
   const ModeCoef& C = S.md[md];
   const ModeGrad& CG = SG.md[md];
-  const double v = C.cm * B.f13, lnv = C.lncm + B.lnf3, iv5 = C.icm5 * D.fm53[B.b];
-  const double amp0 = __longlong_as_double(tape.ld(kFtAmp0)), w = __longlong_as_double(tape.ld(kFtW)), amp = amp0 * w;
+  const double v = C.cm * B.f13;
+  const double w = __longlong_as_double(tape.ld(kFtW)), amp = __longlong_as_double(tape.ld(kFtAmp0)) * w;
   if (fx_expo(amp) == 0) return;
-  double2 kap = make_double2(0.0, 0.0);
-  double Pp2 = 0.0, Pc22 = 0.0;
-  double2 Ap = make_double2(amp * C.Pp, 0.0), Ac = make_double2(amp * C.Pc2, 0.0);
-  if (md2 >= 0) {
-    const double v2 = v * v;
-    kap = make_double2(S.k32.x * v2, S.k32.y * v2);
-    Pp2 = S.md[md2].Pp;
-    Pc22 = S.md[md2].Pc2;
-    Ap = make_double2(amp * fma(kap.x, Pp2, C.Pp), amp * (kap.y * Pp2));
-    Ac = make_double2(amp * fma(kap.x, Pc22, C.Pc2), amp * (kap.y * Pc22));
+  double2 Ap, Ac;
+  if constexpr (Tape::kChain) {
+    Ap = make_double2(__longlong_as_double(tape.ld(kFtWeights)), __longlong_as_double(tape.ld(kFtWeights + 1)));
+    Ac = make_double2(__longlong_as_double(tape.ld(kFtWeights + 2)), __longlong_as_double(tape.ld(kFtWeights + 3)));
+  } else {
+    fx_weights(S, C, md2 >= 0 ? &S.md[md2] : nullptr, amp, v, Ap, Ac);
   }
   FxBwd o;
   fx_bwd<SST>(B, a3, seeds, Es, Ap, Ac, md2 >= 0, D.orbit == 0, pc, tape, o);
+  FxChain h;
+  if constexpr (Tape::kChain) {
+    auto ld = [&](int i) { return __longlong_as_double(tape.ld(kFtChain + i)); };
+    h = FxChain{ld(0), ld(1), ld(2), ld(3), ld(4), ld(5), ld(6), ld(7)};
+  } else {
+    h = fx_chain(D, S, SG, C, CG, B, fm13, v, w, tape.ld(kFtC), tape.ld(kFtS));
+  }
   // phase: ph0 = m phi_c / 2 pi + ..., -f t_c, -(m / 4 pi) Psi, -f k.x_c (turns)
   const double mh = md == 1 ? -0.5 : (md == 2 ? -1.5 : (md == 4 ? -2.0 : -1.0));   // -m/2
   const double psib = mh * o.th;                 // - mfac 2 pi th
   g.ph = fma(-2.0, psib, g.ph);
   g.tc = fma(-2.0 * kPi * B.f, o.th, g.tc);
   // centre's Doppler term -f k.x_c, x_c = R (cos alpha, sin alpha, 0)
-  const double fc = -fR * o.th * o.co, fs = -fR * o.th * o.so;
+  const double fth = -fR * o.th, fc = fth * h.co, fs = fth * h.so;
   g.dc += fc;
   g.ds += fs;
 #pragma unroll
@@ -258,34 +305,18 @@ __device__ __forceinline__ void mode_bwd_fx(const DetDev& D, const SampleCoef& S
   // amplitude ~ M^(5/6) ... f^(-7/6 + p/3) cm^p: dlnA_dM without the mode's own v is common to the modes
   g.lnA += o.lnA;
   g.q = fma(o.lnA, CG.dlnA_dq, g.q);
-  if (dlt_pos(C.ftap, B.f)) {
-    const double zb = -o.lnA * (1.0 - w);
-    const double fe = C.fend, ft = C.ftap, A = fe - ft;
-    const double dz = 0.1 / (fe - B.f) - A / ((fe - B.f) * (fe - B.f)) - 0.1 / (B.f - ft) -
-                      0.9 * A / ((B.f - ft) * (B.f - ft));
-    g.Mx = fma(zb * dz, CG.dfend_dM, g.Mx);
-  }
-  // Psi_PN(v), D(v): v dPsi/dv = D, v dD/dv = v^-5 ddpol + Q6 v (2 + ln v); v ~ M^(1/3)
-  double dpol = S.Pd[7], ddpol = S.Pdd[7], pq = SG.dP_dq[7], dq = SG.dPd_dq[7];
-#pragma unroll
-  for (int k = 6; k >= 0; --k) {
-    dpol = fma(dpol, v, S.Pd[k]);
-    ddpol = fma(ddpol, v, S.Pdd[k]);
-    pq = fma(pq, v, SG.dP_dq[k]);
-    dq = fma(dq, v, SG.dPd_dq[k]);
-  }
-  const double q6v = S.Q6 * v, dq6v = SG.dQ6_dq * v;
-  const double dv = fma(iv5, dpol, fma(q6v, 1.0 + lnv, S.Q5));
-  g.vM = fma(psib, dv, fma(Db, fma(iv5, ddpol, q6v * (2.0 + lnv)), fma(o.lnA, double(C.p), g.vM)));
-  g.q = fma(psib, fma(iv5, pq, lnv * (dq6v + SG.dQ5_dq)), fma(Db, fma(iv5, dq, fma(dq6v, 1.0 + lnv, SG.dQ5_dq)), g.q));
-  const double iv = C.icm * fm13;
-  g.x4 = fma(iv, psib - Db, g.x4);
-  g.x3 = fma(iv * iv, fma(-2.0, Db, psib), g.x3);
+  g.Mx = fma(o.lnA, h.tap, g.Mx);
+  g.vM = fma(psib, h.dv, fma(Db, h.ddv, fma(o.lnA, double(C.p), g.vM)));
+  g.q = fma(psib, h.pq, fma(Db, h.dq, g.q));
+  g.x4 = fma(h.iv, psib - Db, g.x4);
+  g.x3 = fma(h.iv * h.iv, fma(-2.0, Db, psib), g.x3);
   // polarisation weights: Ac carries 2 Pc
   const double2 apb = make_double2(amp * o.Ap.x, amp * o.Ap.y), acb = make_double2(amp * o.Ac.x, amp * o.Ac.y);
   g.io = fma(apb.x, CG.dPp_di, fma(2.0 * acb.x, CG.dPc_di, g.io));
   if (md2 >= 0) {
     const ModeGrad& CG2 = SG.md[md2];
+    const double2 kap = make_double2(S.k32.x * (v * v), S.k32.y * (v * v));
+    const double Pp2 = S.md[md2].Pp, Pc22 = S.md[md2].Pc2;
     g.io += (apb.x * kap.x + apb.y * kap.y) * CG2.dPp_di + 2.0 * (acb.x * kap.x + acb.y * kap.y) * CG2.dPc_di;
     const double2 kb = make_double2(apb.x * Pp2 + acb.x * Pc22, apb.y * Pp2 + acb.y * Pc22);   // kappa-bar
     // kappa = k32 v^2; only ln(amp2 / amp1) varies with theta (M, q), see mode_bwd

@@ -731,23 +731,23 @@ pe_status pe_fisher(const pe_detector* dets, int ndet, const double* theta, int 
   int* nend = nullptr;
   long long* off = nullptr;
   double* part = nullptr;
-  const int W = pe::fisher_partial_width();
+  const int W = pe::fisher_partial_width(), split = pe::fisher_split(ds, max_tiles, sm_count());
   PE_CUDA(sc.alloc(&coef, B));
   PE_CUDA(sc.alloc(&sg, B));
   PE_CUDA(sc.alloc(&nend, P));
-  PE_CUDA(sc.alloc(&off, P + 1));
-  PE_CUDA(sc.alloc(&part, (size_t)max_tiles * W));
+  PE_CUDA(sc.alloc(&off, P + 3));   // and the work counter
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(off + P + 1);
+  PE_CUDA(sc.alloc(&part, (size_t)max_tiles * split * W));
   const bool h_F = !is_device_ptr(out_F);
   double* F = out_F;
   if (h_F) PE_CUDA(sc.alloc(&F, (size_t)B * 121));
   PE_CUDA(pe::launch_prep_grad(th, B, mode_mask, ds, coef, sg, nend, nullptr, st));
-  PE_CUDA(pe::launch_scan_tiles(nend, P, off, pe::kTileBins, nullptr, st));
-  const long long g = std::min<long long>(max_tiles, (long long)sm_count() * 16);
+  PE_CUDA(pe::launch_scan_tiles(nend, P, off, pe::kTileBins, ctr, st));
   void* prof = nullptr;
   pe::profile_begin(st, &prof);
-  PE_CUDA(pe::launch_fisher_fwd(ds, B, coef, sg, nend, off, part, (int)std::max<long long>(g, 1), st));
+  PE_CUDA(pe::launch_fisher_fwd(ds, B, coef, sg, nend, off, part, max_tiles, sm_count(), split, ctr, st));
   pe::profile_end(st, prof);
-  PE_CUDA(pe::launch_fisher_reduce(ds, B, off, part, coef, F, st));
+  PE_CUDA(pe::launch_fisher_reduce(ds, B, off, part, coef, split, F, st));
   if (h_F) {
     PE_CUDA(cudaMemcpyAsync(out_F, F, (size_t)B * 121 * sizeof(double), cudaMemcpyDeviceToHost, st));
     PE_WAIT(st);

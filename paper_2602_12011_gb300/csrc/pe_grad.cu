@@ -570,10 +570,148 @@ __global__ void __launch_bounds__(32 * kFisherWarps, 1) k_fisher_fwd(DetSet ds, 
   }
 }
 
+// Fisher on detectors that take the fixed-point unit: six warps per 32 bins. Warps 0-3 first run the forward pass of one mode
+// each (slot w) onto a tape in shared memory, with the chain factors that the seeds share; then warp j runs seed j's reverse
+// sweeps (Re/Im of A', E', T'), giving row j of the Jacobian, and each warp accumulates eleven of the 66 entries. Bound by
+// the dependent integer operations of the sweeps at 12 warps an SM and, at about 2,100 per bin, by the FP64 pipe.
+// Three points on LISA, 2^21 s: 1.60 ms with the FP64 sweeps (k_fisher_fwd), 0.42 ms now.
+constexpr int kFisherFxThreads = 32 * kFisherWarps;
+struct FisherTape {   // field f of a lane at p[32 f]
+  static constexpr bool kOn = true, kChain = true;
+  fx* p;
+  __device__ __forceinline__ void st(int f, fx v) const { p[f * 32] = v; }
+  __device__ __forceinline__ fx ld(int f) const { return p[f * 32]; }
+};
+struct FisherShared {
+  fx tape[kTapeSlots][kFtAll][32];
+  fx col[kFxSums][kFisherFxThreads];           // the forward's sums (unused), then the seeds, a column per thread
+  double J[kFisherWarps][PE_NPARAM][32];       // rows Re/Im of A', E', T'
+  double gJ[kFisherWarps][PE_NPARAM][32];      // the same times the channel's 4 / (T S)
+  fx pc[kProj];
+  double rot[3][3];                            // d(lambda, beta, psi) per rotation cotangent
+  long long next;
+};
+__global__ void __launch_bounds__(kFisherFxThreads, 2) k_fisher_fx(DetSet ds, int B, const SampleCoef* __restrict__ coef,
+                                                                   const SampleGrad* __restrict__ sgrad,
+                                                                   const int* __restrict__ nend,
+                                                                   const long long* __restrict__ off, double* part, int split,
+                                                                   unsigned long long* ctr) {
+  extern __shared__ __align__(16) unsigned char fisher_smem[];
+  FisherShared& sm = *reinterpret_cast<FisherShared*>(fisher_smem);
+  const int P = ds.ndet * B;
+  const long long total = off[P] * split;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  fx* col = &sm.col[0][threadIdx.x];
+  for (long long t = blockIdx.x, tn = 0; t < total; t = work_next(tn, &sm.next)) {
+    tn = work_fetch(ctr, t);
+    const long long tile = t / split;
+    const int p = find_pair_g(off, P, tile);
+    if (!PE_CHK(p >= 0 && p < P && off[p + 1] * split <= total && nend[p] <= ds.d[p / B].nb, 64)) continue;
+    const int I = p / B, s = p - I * B;
+    const DetDev& D = ds.d[I];
+    const SampleCoef& S = coef[s];
+    const SampleGrad& SG = sgrad[s];
+    fx_proj_prologue(D, S, sm.pc);
+    if (threadIdx.x >= 64 && threadIdx.x < 73) {
+      const int j = (threadIdx.x - 64) / 3, c = (threadIdx.x - 64) % 3;
+      const double W[3] = {c == 0 ? 1.0 : 0.0, c == 1 ? 1.0 : 0.0, c == 2 ? 1.0 : 0.0};
+      double a = 0.0;
+      for (int i = 0; i < 3; ++i)
+        a += rotation_to_frame(S, W, 0, i) * SG.dk[i][j] + rotation_to_frame(S, W, 1, i) * SG.dp[i][j];
+      sm.rot[j][c] = a;
+    }
+    fx_proj3(sm.pc);
+    double F[kFisherW / kFisherWarps];
+#pragma unroll
+    for (int e = 0; e < kFisherW / kFisherWarps; ++e) F[e] = 0.0;
+    const int subs = kTileBins / 32 / split, sub0 = int(t - tile * split) * subs;
+#pragma unroll 1
+    for (int sub = sub0; sub < sub0 + subs; ++sub) {
+      const int b = int(tile - off[p]) * kTileBins + sub * 32 + lane;
+      const bool on = b < nend[p];
+      FxBin Bn;
+      double fm13 = 0.0;
+      if (on) {
+        load_bin_fx(D, b, S.tc, Bn);
+        fm13 = D.fm13[b];
+#pragma unroll 1
+        for (int md = 0; md < kNModes; ++md) {
+          const ModeCoef& C = S.md[md];
+          if (tape_slot(md) != w || (md == 3 && S.pair32) || !C.active || !dlt_pos(Bn.f, C.fend)) continue;
+          const ModeCoef* C2 = (md == 0 && S.pair32) ? &S.md[3] : nullptr;
+          const FisherTape tp = {&sm.tape[w][0][lane]};
+          FxAccT<kFisherFxThreads> a;
+          fx_zero(a, col);
+          mode_bin_fx(D, S, C, Bn, a, ds.d[0].fcis, ds.d[0].fsinc, sm.pc, md, C2, tp);
+          const double v = C.cm * Bn.f13, tw = __longlong_as_double(tp.ld(kFtW)), amp = __longlong_as_double(tp.ld(kFtAmp0)) * tw;
+          double2 Ap, Ac;
+          fx_weights(S, C, C2, amp, v, Ap, Ac);
+          const FxChain h = fx_chain(D, S, SG, C, SG.md[md], Bn, fm13, v, tw, tp.ld(kFtC), tp.ld(kFtS));
+          const double f[12] = {h.dv, h.ddv, h.pq, h.dq, h.iv, h.co, h.so, h.tap, Ap.x, Ap.y, Ac.x, Ac.y};
+#pragma unroll
+          for (int i = 0; i < 12; ++i) tp.st(kFtChain + i, __double_as_longlong(f[i]));
+        }
+      }
+      __syncthreads();   // the tape is written; the last pass's readers of J and gJ are done
+      double row[PE_NPARAM];
+#pragma unroll
+      for (int i = 0; i < PE_NPARAM; ++i) row[i] = 0.0;
+      if (on) {
+        double2 bb[3], pq[6];
+        for (int c = 0; c < 3; ++c) bb[c] = make_double2(w == 2 * c ? 1.0 : 0.0, w == 2 * c + 1 ? 1.0 : 0.0);
+        const double2 sc = D.sca[b];
+        link_seeds<1>(bb, sc.x, sc.y, pq);
+        const int Es = fx_seeds<kFisherFxThreads>(pq, col);
+        const fx a3 = fx_times_k((unsigned)(D.k0 + b), D.fx_a3);
+        const double invf = fm13 * fm13 * fm13, fR = 2.0 * kPi * D.R * Bn.f;
+        FxBinAcc ga;
+        fx_bin_zero(ga);
+#pragma unroll 1
+        for (int md = 0; md < kNModes; ++md) {
+          if ((md == 3 && S.pair32) || Es == 0 || !S.md[md].active || !dlt_pos(Bn.f, S.md[md].fend)) continue;
+          const FisherTape tp = {&sm.tape[tape_slot(md)][0][lane]};
+          mode_bwd_fx<kFisherFxThreads>(D, S, SG, md, (md == 0 && S.pair32) ? 3 : -1, Bn, fm13, invf, fR, a3, col, Es, ga, sm.pc, tp);
+        }
+        GradAcc g;
+        fx_bin_grad(S, SG, ga, g);
+        row[0] = g.M; row[1] = g.q; row[2] = g.c1; row[3] = g.c2; row[4] = g.dL; row[5] = g.io; row[6] = g.ph; row[10] = g.tc;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) row[7 + j] = fma(sm.rot[j][0], g.k[0], fma(sm.rot[j][1], g.k[1], sm.rot[j][2] * g.k[2]));
+      }
+      const double gg = on ? D.gg[(w >> 1) * D.nb + b] : 0.0;
+#pragma unroll
+      for (int i = 0; i < PE_NPARAM; ++i) {
+        sm.J[w][i][lane] = row[i];
+        sm.gJ[w][i][lane] = gg * row[i];
+      }
+      __syncthreads();
+      // entries e = w, w + 6, ... of the upper triangle, row by row
+#pragma unroll 1
+      for (int r = 0; r < kFisherWarps; ++r) {
+        int i = 0, k = w;
+        while (k >= PE_NPARAM - i) { k -= PE_NPARAM - i; ++i; }
+#pragma unroll
+        for (int e = 0; e < kFisherW / kFisherWarps; ++e) {
+          F[e] = fma(sm.gJ[r][i][lane], sm.J[r][i + k][lane], F[e]);
+          k += kFisherWarps;
+          while (i < PE_NPARAM && k >= PE_NPARAM - i) { k -= PE_NPARAM - i; ++i; }
+        }
+      }
+    }
+    // fixed-order sums over the lanes
+#pragma unroll
+    for (int e = 0; e < kFisherW / kFisherWarps; ++e) {
+      for (int o = 16; o > 0; o >>= 1) F[e] += __shfl_down_sync(0xffffffffu, F[e], o);
+      if (lane == 0) part[t * kFisherW + w + kFisherWarps * e] = F[e];
+    }
+  }
+  work_done(ctr);
+}
+
 // Per point: thread (r, e) adds entry e of the tiles r, r + 8, ... over the detectors, then thread e its eight rows.
 constexpr int kFisherRows = 8;
 __global__ void __launch_bounds__(kFisherW * kFisherRows) k_fisher_reduce(DetSet ds, int B, const long long* off, const double* part,
-                                                                        const SampleCoef* coef, double* F) {
+                                                                        const SampleCoef* coef, int split, double* F) {
   __shared__ double red[kFisherRows][kFisherW];
   const int s = blockIdx.x;
   const int e = threadIdx.x % kFisherW, r = threadIdx.x / kFisherW;
@@ -581,7 +719,7 @@ __global__ void __launch_bounds__(kFisherW * kFisherRows) k_fisher_reduce(DetSet
   for (int I = 0; I < ds.ndet; ++I) {
     const int p = I * B + s;
     if (!PE_CHK(off[p] >= 0 && off[p + 1] <= off[ds.ndet * B], 128)) continue;
-    for (long long t = off[p] + r; t < off[p + 1]; t += kFisherRows) a += part[t * kFisherW + e];
+    for (long long t = off[p] * split + r; t < off[p + 1] * split; t += kFisherRows) a += part[t * kFisherW + e];
   }
   red[r][e] = a;
   __syncthreads();
@@ -621,14 +759,26 @@ cudaError_t launch_grad_reduce(const DetSet& ds, int B, const long long* off, co
     k_grad_reduce<<<B, kGradW * 32, 0, st>>>(ds, B, off, part, coef, sgrad, logl, grad);
   return pe::launch_status();
 }
+// Items per 128-bin tile: a few points leave the chip's SMs two or three tiles each, so up to 32 tiles per SM the fixed-point
+// kernel's items are a quarter tile; beyond, whole tiles (a quarter of the partials).
+int fisher_split(const DetSet& ds, long long max_tiles, int sms) { return fx_all_ok(ds) && max_tiles <= 32LL * sms ? 4 : 1; }
 cudaError_t launch_fisher_fwd(const DetSet& ds, int B, const SampleCoef* coef, const SampleGrad* sgrad,
-                              const int* nend, const long long* off, double* part, int grid, cudaStream_t st) {
-  k_fisher_fwd<<<grid, 32 * kFisherWarps, 0, st>>>(ds, B, coef, sgrad, nend, off, part);
+                              const int* nend, const long long* off, double* part, long long max_tiles, int sms, int split,
+                              unsigned long long* ctr, cudaStream_t st) {
+  if (fx_all_ok(ds)) {
+    cudaError_t e = cudaFuncSetAttribute(k_fisher_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FisherShared));
+    if (e != cudaSuccess) return e;
+    const int grid = (int)std::max(1LL, std::min(max_tiles * split, 2LL * sms));
+    k_fisher_fx<<<grid, kFisherFxThreads, sizeof(FisherShared), st>>>(ds, B, coef, sgrad, nend, off, part, split, ctr);
+  } else {
+    const int grid = (int)std::max(1LL, std::min(max_tiles, 16LL * sms));
+    k_fisher_fwd<<<grid, 32 * kFisherWarps, 0, st>>>(ds, B, coef, sgrad, nend, off, part);
+  }
   return pe::launch_status();
 }
 cudaError_t launch_fisher_reduce(const DetSet& ds, int B, const long long* off, const double* part,
-                                 const SampleCoef* coef, double* F, cudaStream_t st) {
-  k_fisher_reduce<<<B, kFisherW * kFisherRows, 0, st>>>(ds, B, off, part, coef, F);
+                                 const SampleCoef* coef, int split, double* F, cudaStream_t st) {
+  k_fisher_reduce<<<B, kFisherW * kFisherRows, 0, st>>>(ds, B, off, part, coef, split, F);
   return pe::launch_status();
 }
 int grad_partial_width() { return kGradW; }

@@ -116,3 +116,19 @@ def test_time_far_below_its_terms(oracle_mod, Lb, first):
     ll, dhhh = oracle_mod.loglike_batch([od], th, 0x10)
     dd = np.array([oracle_mod.loglike([od], th[0], 0)["dd"][0]])
     H.assert_loglike_parity(g, ll, dhhh, dd, H.floor_terms(oracle_mod, [od], th, 0x10))
+
+
+@pytest.mark.parametrize("nb,copies", [(1, 1), (32, 1), (33, 1), (129, 1), (160, 2000)])
+@pytest.mark.parametrize("det,mask", [(W.LISA, W.MODE_ALL), (W.TIANQIN, 0x19), (dict(W.TAIJI, tdi_gen=15), 0x08)])
+def test_fisher_at_pass_and_tile_edges(oracle_mod, Lb, det, mask, nb, copies):
+    """Grids around the 32-bin pass and the 128-bin tile, masses whose modes end inside them, whole tiles per item
+    (copies: many points) as well as quarters; on the bar of the Fisher parity test, 1e-10 of sqrt(F_ii F_kk)."""
+    T, k0 = 2.0 ** 16, 30
+    th = _samples(T, (k0 + nb - 1) / T)
+    od = H.oracle_detector(oracle_mod, det, T, k0, nb, th[0], W.MODE_ALL, 41)
+    F = Lb.fisher([H.library_detector(Lb, od)], np.tile(th, (copies, 1)), mask)
+    for s in range(len(th)):
+        Fr = oracle_mod.fisher([od], th[s], mask)
+        d = np.sqrt(np.abs(np.outer(np.diag(Fr), np.diag(Fr))))
+        assert np.all(np.abs(F[s] - Fr) <= 1e-10 * d + 1e-300), (s, np.max(np.abs(F[s] - Fr) / (d + 1e-300)))
+    np.testing.assert_array_equal(F, np.tile(F[:len(th)], (copies, 1, 1)))

@@ -383,6 +383,20 @@ __device__ __forceinline__ void work_done(unsigned long long* ctr) {
   }
 }
 
+// The pair p of [lo, P) with off[p] <= t < off[p + 1] (the last with off[p] <= t, as pairs may be empty), off[lo] <= t: a warp
+// tests 32 candidates at once, three dependent loads for 8,192 pairs where a bisection makes 13. Every lane of the warp calls it.
+__device__ __forceinline__ int find_pair_warp(const long long* __restrict__ off, int P, long long t, int lo = 0) {
+  const int lane = threadIdx.x & 31;
+  int n = P - lo;
+  while (n > 1) {
+    const int step = (n + 31) >> 5, i = lane * step;
+    const int k = __popc(__ballot_sync(0xffffffffu, i < n && off[lo + min(i, n - 1)] <= t)) - 1;
+    lo += k * step;
+    n = min(step, n - k * step);
+  }
+  return lo;
+}
+
 // Per-bin inputs shared by all modes of one bin.
 // a < b for non-negative doubles by the order of their bit patterns: an integer compare, exact
 // (GB300 runs the double compare DSETP on its narrow FP64 pipe)

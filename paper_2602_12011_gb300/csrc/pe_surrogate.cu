@@ -927,6 +927,13 @@ __device__ __forceinline__ int find_pair_s(const long long* off, int P, long lon
 // (kTileBins bins per tile, one bin per thread): partials [tile][6] = (<s|p>, <s|s>, <p|p>, 0, 0, 0), with the plain
 // signal itself as s where the pair takes no spline path. (log L: k_sur_inbox or k_sur_in64 on the in-box tiles and
 // k_loglike_fwd itself on the others.)
+// Consecutive tiles (as a power of two) of the in-box list that a CTA draws at a time: long runs reuse a pair's coefficients
+// from L1, short ones end together. Mixed, whole call, at runs of 1, 4 and 16 tiles: 8192 samples 9.83, 8.36, 8.12 ms;
+// 1024 in-box samples 1.08, 0.97, 1.00 ms; 100 samples 0.414, 0.417, 0.450 ms; hence some 24 runs per CTA, 16 tiles at most.
+__device__ __forceinline__ int sur_run(long long total) {
+  const long long r = total / (gridDim.x * 24LL);
+  return r < 2 ? 0 : (r < 4 ? 1 : (r < 8 ? 2 : (r < 16 ? 3 : 4)));
+}
 constexpr int kSurInboxCtas = 8;    // resident CTAs per SM asked of the in-box kernel (k_sur_inbox)
 // consecutive tiles (bins per thread) k_sur_inbox takes at a time; measured on 1024 in-box samples,
 // whole call: 1 tile 1.16 ms, 2 tiles 1.29 ms (64 registers, 8 CTAs per SM), 1.45 ms (6 CTAs per SM)
@@ -1021,11 +1028,25 @@ __global__ void __launch_bounds__(kTileBins, 3) k_sur_fwd(DetSet ds, int B, cons
 
 // The mixed-precision surrogate's in-box tiles (mode 0): mode_bin_sur_mix per (mode, bin), A/E/T
 // and the weighted products in double words, each 128-bin tile summed in double words (the tail of
-// k_loglike_fwd's mixed path) and scaled back to FP64 into its own partial. A CTA walks a contiguous
-// run of the in-box tile list (offk), so that consecutive tiles of a pair reuse its spline
+// k_loglike_fwd's mixed path) and scaled back to FP64 into its own partial. A CTA draws contiguous
+// runs of the in-box tile list (offk), so that consecutive tiles of a pair reuse its spline
 // coefficients from L1, and takes NB consecutive tiles of one pair at a time: each thread then
 // carries NB independent bins through one mode loop (their coefficient loads and arithmetic
 // overlap), and each tile still gets its own partial in the same fixed order.
+// aet_from_xyz_dw of FP32 brackets: its operations without those on the zero low words, the same bits in half the instructions.
+__device__ __forceinline__ df sum3_f32(float a, float b, float c) {
+  const df s1 = two_sum(a, b), s2 = two_sum(s1.x, c), t = two_sum(s1.y, s2.y), u = two_sum(s2.x, t.x);
+  return two_sum(u.x, __fadd_rn(u.y, t.y));
+}
+__device__ __forceinline__ df sub2_f32(float a, float b, float c) {   // a + c - 2 b
+  const df s = two_sum(a, c), r = two_sum(s.x, -2.0f * b);
+  return df_make(r.x, __fadd_rn(r.y, s.y));
+}
+__device__ __forceinline__ void aet_from_xyz_f32(const float2 x[3], cdf o[3]) {
+  o[0] = cdf{two_sum(x[2].x, -x[0].x), two_sum(x[2].y, -x[0].y)};
+  o[1] = cdf{sub2_f32(x[0].x, x[1].x, x[2].x), sub2_f32(x[0].y, x[1].y, x[2].y)};
+  o[2] = cdf{sum3_f32(x[0].x, x[1].x, x[2].x), sum3_f32(x[0].y, x[1].y, x[2].y)};
+}
 // block_sum6's fixed-order sum of six double words per thread with two barriers instead of
 // three: consecutive tiles alternate between two staging buffers, so a tile's writes cannot meet
 // the previous tile's final readers (those finish before the next tile's first barrier, and the
@@ -1051,7 +1072,7 @@ __device__ __forceinline__ bool tile_sum6(const df v[6], float2 (*red)[kTileBins
 }
 
 // The FP64 surrogate's in-box tiles (mode 0): mode_bin_sur per (mode, bin), A/E/T, the weighted products and the tile's
-// sum in FP64 as k_loglike_fwd. A CTA walks a contiguous run of the in-box list, as k_sur_inbox, at six CTAs
+// sum in FP64 as k_loglike_fwd. A CTA draws contiguous runs of the in-box list, as k_sur_inbox, at six CTAs
 // per SM: inside k_sur_fwd, whose register count the per-bin path sets (three CTAs per SM), the same unit left the
 // warps waiting on its coefficient loads (1024 in-box samples, whole call: 5.5 ms there).
 constexpr int kSurIn64Ctas = 6;
@@ -1062,56 +1083,62 @@ __global__ void __launch_bounds__(kTileBins, kSurIn64Ctas) k_sur_in64(DetSet ds,
                                                                     const double* __restrict__ hs,
                                                                     const int* __restrict__ nend,
                                                                     const long long* __restrict__ off,
-                                                                    const long long* __restrict__ offk, double* part) {
+                                                                    const long long* __restrict__ offk, double* part,
+                                                                    unsigned long long* ctr) {
+  __shared__ long long next;
   __shared__ double red[6][kTileBins + kRedPad];
   __shared__ double ampn[kNModes], hm[kNModes];   // Newtonian amplitude times hsc; node spacing in ln f
   __shared__ float ihf[kNModes];                  // 1/h
   const int P = ds.ndet * B;
   const long long total = offk[P];
-  const long long chunk = (total + gridDim.x - 1) / gridDim.x;
-  const long long tk0 = blockIdx.x * chunk;
-  const long long tk1 = tk0 + chunk < total ? tk0 + chunk : total;
-  int p = 0, pcur = -1;
-  for (long long tk = tk0; tk < tk1; ++tk) {
-    p = find_pair_s(offk, P, tk, p);
-    const int I = p / B, s = p - I * B;
-    const DetDev& D = ds.d[I];
-    const SampleCoef& S = coef[s];
-    if (p != pcur) {     // the pair's per-sample values, staged once per run of its tiles
-      __syncthreads();   // the previous pair's readers are done
-      if (threadIdx.x < kNModes) {
-        const double h = hs[(size_t)s * kNModes + threadIdx.x];
-        ampn[threadIdx.x] = coefN[s].md[threadIdx.x].amp * S.hsc;
-        hm[threadIdx.x] = h;
-        ihf[threadIdx.x] = (float)(1.0 / h);
+  const int rl = sur_run(total);
+  const long long nrun = (total + (1 << rl) - 1) >> rl;
+  int p = -1, pcur = -1;
+  for (long long run = blockIdx.x, rn = 0; run < nrun; run = work_next(rn, &next)) {
+    rn = work_fetch(ctr, run);
+    const long long tk1 = (run + 1) << rl < total ? (run + 1) << rl : total;
+    for (long long tk = run << rl; tk < tk1; ++tk) {
+      if (p < 0 || offk[p + 1] <= tk) p = find_pair_warp(offk, P, tk, max(p, 0));
+      const int I = p / B, s = p - I * B;
+      const DetDev& D = ds.d[I];
+      const SampleCoef& S = coef[s];
+      if (p != pcur) {     // the pair's per-sample values, staged once per run of its tiles
+        __syncthreads();   // the previous pair's readers are done
+        if (threadIdx.x < kNModes) {
+          const double h = hs[(size_t)s * kNModes + threadIdx.x];
+          ampn[threadIdx.x] = coefN[s].md[threadIdx.x].amp * S.hsc;
+          hm[threadIdx.x] = h;
+          ihf[threadIdx.x] = (float)(1.0 / h);
+        }
+        __syncthreads();
+        pcur = p;
       }
-      __syncthreads();
-      pcur = p;
-    }
-    const int b = int(tk - offk[p]) * kTileBins + threadIdx.x;
-    double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (b < nend[p]) {
-      const double f = D.f[b], fm76 = D.fm76[b], u0 = fma(3.0, D.lnf3[b], -kLnFmin);
-      const float u0f = trunc_to_float((unsigned long long)__double_as_longlong(u0));
-      const fxu frc = fx_cycles(f, S.tc);
-      float2 xs[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      const int b = int(tk - offk[p]) * kTileBins + threadIdx.x;
+      double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      if (b < nend[p]) {
+        const double f = D.f[b], fm76 = D.fm76[b], u0 = fma(3.0, D.lnf3[b], -kLnFmin);
+        const float u0f = trunc_to_float((unsigned long long)__double_as_longlong(u0));
+        const fxu frc = fx_cycles(f, S.tc);
+        float2 xs[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
-      for (int md = 0; md < kNModes; ++md) {
-        const ModeCoef& C = S.md[md];
-        if (!C.active || !dlt_pos(f, C.fend)) continue;
-        const size_t sys = ((size_t)I * B + s) * kNModes + md;
-        mode_bin_sur(C, ampn[md], f, fm76, u0, u0f, frc, spl + sys * kQ * (kNodes - 1) * 4,
-                     splt + sys * (kQ - 1) * (kNodes - 1) * 4, hm[md], ihf[md], xs, ds.d[0].fcis);
-      }
-      double2 x[3], o[3];
+        for (int md = 0; md < kNModes; ++md) {
+          const ModeCoef& C = S.md[md];
+          if (!C.active || !dlt_pos(f, C.fend)) continue;
+          const size_t sys = ((size_t)I * B + s) * kNModes + md;
+          mode_bin_sur(C, ampn[md], f, fm76, u0, u0f, frc, spl + sys * kQ * (kNodes - 1) * 4,
+                       splt + sys * (kQ - 1) * (kNodes - 1) * 4, hm[md], ihf[md], xs, ds.d[0].fcis);
+        }
+        double2 x[3], o[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) x[c] = make_double2(scale_up(xs[c].x, S.ihsc), scale_up(xs[c].y, S.ihsc));
-      aet_from_xyz(x, o);
-      accum_bin(D, b, o, v);
+        for (int c = 0; c < 3; ++c) x[c] = make_double2(scale_up(xs[c].x, S.ihsc), scale_up(xs[c].y, S.ihsc));
+        aet_from_xyz(x, o);
+        accum_bin(D, b, o, v);
+      }
+      double r;
+      if (block_sum6(v, [](double x, double y) { return x + y; }, red, &r)) part[(off[p] + (tk - offk[p])) * 6 + threadIdx.x] = r;
     }
-    double r;
-    if (block_sum6(v, [](double x, double y) { return x + y; }, red, &r)) part[(off[p] + (tk - offk[p])) * 6 + threadIdx.x] = r;
   }
+  work_done(ctr);
 }
 
 template <int NB>
@@ -1123,95 +1150,99 @@ __global__ void __launch_bounds__(kTileBins, kSurInboxCtas) k_sur_inbox(DetSet d
                                                                      const double* __restrict__ hs,
                                                                      const int* __restrict__ nend,
                                                                      const long long* __restrict__ off,
-                                                                     const long long* __restrict__ offk, double* part) {
+                                                                     const long long* __restrict__ offk, double* part,
+                                                                     unsigned long long* ctr) {
+  __shared__ long long next;
   __shared__ float2 red[2][6][kTileBins + kRedPad];   // tile sums' staging, alternating per tile
   __shared__ float ampf[kNModes];                  // a_lm hsc in FP32
   __shared__ float2 hsw[kNModes];                  // node spacing h as a double word
   __shared__ float ihsf[kNModes];                  // 1/h in FP32
   const int P = ds.ndet * B;
   const long long total = offk[P];
-  const long long chunk = (total + gridDim.x - 1) / gridDim.x;
-  const long long tk0 = blockIdx.x * chunk;
-  const long long tk1 = tk0 + chunk < total ? tk0 + chunk : total;
-  int p = 0, pcur = -1, buf = 0;
-  for (long long tk = tk0; tk < tk1;) {
-    p = find_pair_s(offk, P, tk, p);
-    const long long tend = offk[p + 1] < tk1 ? offk[p + 1] : tk1;   // this pair's tiles in the run
-    const int nt = (NB == 2 && tk + 1 < tend) ? 2 : 1;                // uniform over the CTA
-    const int I = p / B, s = p - I * B;
-    const int ne = nend[p];
-    const DetDev& D = ds.d[I];
-    const SampleCoef& S = coef[s];
-    if (p != pcur) {     // the pair's per-sample values, staged once per run of its tiles
-      __syncthreads();   // the previous pair's readers are done
-      if (threadIdx.x < kNModes) {
-        const double hm = hs[(size_t)s * kNModes + threadIdx.x];
-        ampf[threadIdx.x] = (float)(coefN[s].md[threadIdx.x].amp * S.hsc);
-        hsw[threadIdx.x] = to_dw(hm);
-        ihsf[threadIdx.x] = (float)(1.0 / hm);
-      }
-      __syncthreads();
-      pcur = p;
-    }
-    // per bin in double words, no FP64 arithmetic: u0 = 3 (ln f / 3) - ln kFmin, and frac(f t_c)
-    // from the double-word product (relative error ~2^-46: ~1e-8 turn at f t_c ~ 4e5 turns)
-    int bb[NB];
-    double f[NB];
-    df u0w[NB], frcw[NB];
-    float fm76[NB];
-    float2 xs[NB][3];
-#pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      bb[k] = int(tk - offk[p] + k) * kTileBins + threadIdx.x;
-      const int b = (k < nt && bb[k] < ne) ? bb[k] : 0;
-      f[k] = (k < nt && bb[k] < ne) ? D.f[b] : 0.0;   // 0 keeps an absent bin out of every mode
-      u0w[k] = dfl_sub(dfl_mulf(df_from_bits(D.lnf3[b]), 3.f), df_make(kLnFminHi, kLnFminLo));
-      fm76[k] = D.fm76w[b].x;
-      const df ftc = dfl_mul(D.fw[b], S.tcw);
-      frcw[k] = two_sum(__fsub_rn(ftc.x, rintf(ftc.x)), ftc.y);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) xs[k][c] = make_float2(0.f, 0.f);
-    }
-#pragma unroll   // the modes' (and the bins') coefficient loads overlap
-    for (int md = 0; md < kNModes; ++md) {
-      const ModeCoef& C = S.md[md];
-      if (!C.active) continue;
-      const size_t sys = ((size_t)I * B + s) * kNModes + md;
-#pragma unroll
-      for (int k = 0; k < NB; ++k)
-        if (dlt_pos(0.0, f[k]) && dlt_pos(f[k], C.fend))
-          mode_bin_sur_mix(C, ampf[md], f[k], fm76[k], u0w[k], frcw[k], spl + sys * kQ * (kNodes - 1) * 4,
-                           splt + sys * (kQ - 1) * (kNodes - 1) * 4, hsw[md], ihsf[md], xs[k]);
-    }
-    const double ih = S.ihsc;
-#pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      if (k >= nt) break;   // uniform
-      df v[6];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) v[i] = df_make(0.f, 0.f);
-      const int b = bb[k];
-      if (b < ne) {
-        cdf x[3], o[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) x[c] = cdf{df_make(xs[k][c].x, 0.f), df_make(xs[k][c].y, 0.f)};
-        aet_from_xyz_dw(x, o);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float4 g = D.dgw[c * D.nb + b];
-          v[c] = df_sub_s(df_mul(df_make(g.x, g.y), o[c].re), df_mul(df_make(g.z, g.w), o[c].im));
-          const df m2 = df_add_s(df_mul(o[c].re, o[c].re), df_mul(o[c].im, o[c].im));
-          v[3 + c] = df_mul(D.ggw[c * D.nb + b], m2);
+  const int rl = sur_run(total);
+  const long long nrun = (total + (1 << rl) - 1) >> rl;
+  int p = -1, pcur = -1, buf = 0;
+  for (long long run = blockIdx.x, rn = 0; run < nrun; run = work_next(rn, &next)) {
+    rn = work_fetch(ctr, run);
+    const long long tk1 = (run + 1) << rl < total ? (run + 1) << rl : total;
+    for (long long tk = run << rl; tk < tk1;) {
+      if (p < 0 || offk[p + 1] <= tk) p = find_pair_warp(offk, P, tk, max(p, 0));
+      const long long tend = offk[p + 1] < tk1 ? offk[p + 1] : tk1;   // this pair's tiles in the run
+      const int nt = (NB == 2 && tk + 1 < tend) ? 2 : 1;                // uniform over the CTA
+      const int I = p / B, s = p - I * B;
+      const int ne = nend[p];
+      const DetDev& D = ds.d[I];
+      const SampleCoef& S = coef[s];
+      if (p != pcur) {     // the pair's per-sample values, staged once per run of its tiles
+        __syncthreads();   // the previous pair's readers are done
+        if (threadIdx.x < kNModes) {
+          const double hm = hs[(size_t)s * kNModes + threadIdx.x];
+          ampf[threadIdx.x] = (float)(coefN[s].md[threadIdx.x].amp * S.hsc);
+          hsw[threadIdx.x] = to_dw(hm);
+          ihsf[threadIdx.x] = (float)(1.0 / hm);
         }
+        __syncthreads();
+        pcur = p;
       }
-      df r;
-      if (tile_sum6(v, red[buf], &r))
-        part[(off[p] + (tk - offk[p]) + k) * 6 + threadIdx.x] =
-            df_to(r) * (threadIdx.x < 3 ? D.dg_scale * ih : D.gg_scale * ih * ih);
-      buf ^= 1;
+      // per bin in double words, no FP64 arithmetic: u0 = 3 (ln f / 3) - ln kFmin, and frac(f t_c)
+      // from the double-word product (relative error ~2^-46: ~1e-8 turn at f t_c ~ 4e5 turns)
+      int bb[NB];
+      double f[NB];
+      df u0w[NB], frcw[NB];
+      float fm76[NB];
+      float2 xs[NB][3];
+#pragma unroll
+      for (int k = 0; k < NB; ++k) {
+        bb[k] = int(tk - offk[p] + k) * kTileBins + threadIdx.x;
+        const int b = (k < nt && bb[k] < ne) ? bb[k] : 0;
+        f[k] = (k < nt && bb[k] < ne) ? D.f[b] : 0.0;   // 0 keeps an absent bin out of every mode
+        u0w[k] = dfl_sub(dfl_mulf(df_from_bits(D.lnf3[b]), 3.f), df_make(kLnFminHi, kLnFminLo));
+        fm76[k] = D.fm76w[b].x;
+        const df ftc = dfl_mul(D.fw[b], S.tcw);
+        frcw[k] = two_sum(__fsub_rn(ftc.x, rintf(ftc.x)), ftc.y);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xs[k][c] = make_float2(0.f, 0.f);
+      }
+#pragma unroll   // the modes' (and the bins') coefficient loads overlap
+      for (int md = 0; md < kNModes; ++md) {
+        const ModeCoef& C = S.md[md];
+        if (!C.active) continue;
+        const size_t sys = ((size_t)I * B + s) * kNModes + md;
+#pragma unroll
+        for (int k = 0; k < NB; ++k)
+          if (dlt_pos(0.0, f[k]) && dlt_pos(f[k], C.fend))
+            mode_bin_sur_mix(C, ampf[md], f[k], fm76[k], u0w[k], frcw[k], spl + sys * kQ * (kNodes - 1) * 4,
+                             splt + sys * (kQ - 1) * (kNodes - 1) * 4, hsw[md], ihsf[md], xs[k]);
+      }
+      const double ih = S.ihsc;
+#pragma unroll
+      for (int k = 0; k < NB; ++k) {
+        if (k >= nt) break;   // uniform
+        df v[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) v[i] = df_make(0.f, 0.f);
+        const int b = bb[k];
+        if (b < ne) {
+          cdf o[3];
+          aet_from_xyz_f32(xs[k], o);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float4 g = D.dgw[c * D.nb + b];
+            v[c] = df_sub_s(df_mul(df_make(g.x, g.y), o[c].re), df_mul(df_make(g.z, g.w), o[c].im));
+            const df m2 = df_add_s(df_mul(o[c].re, o[c].re), df_mul(o[c].im, o[c].im));
+            v[3 + c] = df_mul(D.ggw[c * D.nb + b], m2);
+          }
+        }
+        df r;
+        if (tile_sum6(v, red[buf], &r))
+          part[(off[p] + (tk - offk[p]) + k) * 6 + threadIdx.x] =
+              df_to(r) * (threadIdx.x < 3 ? D.dg_scale * ih : D.gg_scale * ih * ih);
+        buf ^= 1;
+      }
+      tk += nt;
     }
-    tk += nt;
   }
+  work_done(ctr);
 }
 
 __global__ void k_mismatch_reduce(int ndet, int B, const long long* off, const double* part, const SampleCoef* coef,
@@ -1716,12 +1747,12 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   aalloc(&off, P + 1);
   int *nin = nullptr, *nout = nullptr;
   long long *offin = nullptr, *offout = nullptr;
-  unsigned long long* ctr = nullptr;
+  unsigned long long *ctr = nullptr, *ctrin = nullptr;
   const bool split = mode == 0;   // log L: the spline path's tiles and the per-bin path's in their own kernels
   if (split) {
     aalloc(&nin, P);
     aalloc(&nout, P);
-    aalloc(&offin, P + 1);
+    aalloc(&offin, P + 3);    // and the work counter
     aalloc(&offout, P + 3);   // and the work counter
   }
   aalloc(&part, (size_t)max_tiles * 6);
@@ -1787,7 +1818,8 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
       if (ds.d[I].orbit != 0) geo_mask |= 1u << I;
     pe::k_split_nend<<<(P + 127) / 128, 128, 0, st>>>(theta_dev, ndet, B, s->box, geo_mask, nend, nin, nout);
     e = pe::launch_status();
-    if (e == cudaSuccess) e = pe::launch_scan_tiles(nin, P, offin, pe::kTileBins, nullptr, st);
+    ctrin = reinterpret_cast<unsigned long long*>(offin + P + 1);
+    if (e == cudaSuccess) e = pe::launch_scan_tiles(nin, P, offin, pe::kTileBins, ctrin, st);
     // the fallback pairs' work items for the forward kernel of pe_loglike_batch
     ctr = reinterpret_cast<unsigned long long*>(offout + P + 1);
     if (e == cudaSuccess) e = pe::launch_scan_tiles(nout, P, offout, tcm.subtiles * pe::kTileBins, ctr, st);
@@ -1802,9 +1834,9 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
           1, std::min<long long>(max_tiles, (long long)nsm * (mix ? pe::kSurInboxCtas : pe::kSurIn64Ctas)));
       if (mix)
         pe::k_sur_inbox<pe::kSurInboxBins><<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend,
-                                                                                  off, offin, part);
+                                                                                  off, offin, part, ctrin);
       else
-        pe::k_sur_in64<<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend, off, offin, part);
+        pe::k_sur_in64<<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend, off, offin, part, ctrin);
       e = pe::launch_status();
       // fallback tiles: the forward kernel of pe_loglike_batch in the call's precision with its tuned
       // (or default) choice, over the fallback pairs' work items; it writes each sub-tile's partial at

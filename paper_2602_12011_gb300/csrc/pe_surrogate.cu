@@ -698,12 +698,17 @@ __device__ __forceinline__ void spline_solve_warp_dw(const df* yy, const df* piv
   __syncwarp();
 }
 
+// The FP64 phase's argument in an interval is s = t 2^m, below 1 (2 for a node spacing above 1/16)
+__device__ __forceinline__ int sur_shift(double h) { return max(1022 - fx_expo(h), 4); }
+
 // mixed: the phase (quantity 0, double-word node values from k_sur_nodes<true>) is solved in double
 // words and written as (c0, c1) and (c2, c3), two float4 per interval in the same 32 bytes (the
 // mixed-precision unit's form), and the transfer functions (quantities 1..6, used only through
 // their FP32 copies) are solved in FP32 and written to coef_t alone.
+// FP64: the phase's coefficients are written for the fixed-point evaluation (sur_phase) and its exponent to pexp (per (detector,
+// sample, mode)), the transfer functions' to coef_t alone.
 __global__ void __launch_bounds__(32 * kSplineWarps) k_spline(const double* nodes, long long nsys, const double* hs,
-                                                               double* coef, float* coef_t, int mixed) {
+                                                               double* coef, float* coef_t, int* pexp, int mixed) {
   constexpr int N = kNodes;
   __shared__ double ys[kSplineWarps][kSplineNP], Ms[kSplineWarps][kSplineNP];
   __shared__ double piv[kSplineNP];   // the pivots in shared memory: the lanes read different rows at once
@@ -725,9 +730,10 @@ __global__ void __launch_bounds__(32 * kSplineWarps) k_spline(const double* node
   const double h = hs[i / kQ];
   if (!(h > 0.0)) {
     for (int j = lane; j < 4 * (N - 1); j += 32) {
-      if (!(mixed && q > 0)) cf[j] = 0.0;
+      if (q == 0) cf[j] = 0.0;
       if (ct) ct[j] = 0.f;
     }
+    if (!mixed && q == 0 && lane == 0) pexp[i / kQ] = -4;
     return;
   }
   if (mixed && q > 0) {
@@ -772,14 +778,35 @@ __global__ void __launch_bounds__(32 * kSplineWarps) k_spline(const double* node
   __syncwarp();
   spline_solve_warp<double>(yy, piv, M, 6.0 / (h * h), lane);
   const double ih = 1.0 / h, h6 = h * (1.0 / 6.0), ih6 = ih * (1.0 / 6.0);
-  for (int j = lane; j < N - 1; j += 32) {
+  auto interval = [&](int j, double c[4]) {
     const double y0 = yy[spad(j)], y1 = yy[spad(j + 1)], m0 = M[spad(j)], m1 = M[spad(j + 1)];
-    const double c0 = y0;
-    const double c1 = (y1 - y0) * ih - h6 * (2.0 * m0 + m1);
-    const double c2 = 0.5 * m0;
-    const double c3 = (m1 - m0) * ih6;
-    *reinterpret_cast<double4*>(cf + 4 * j) = make_double4(c0, c1, c2, c3);
-    if (ct) *reinterpret_cast<float4*>(ct + 4 * j) = make_float4((float)c0, (float)c1, (float)c2, (float)c3);
+    c[0] = y0;
+    c[1] = (y1 - y0) * ih - h6 * (2.0 * m0 + m1);
+    c[2] = 0.5 * m0;
+    c[3] = (m1 - m0) * ih6;
+  };
+  double c[4];
+  if (ct) {
+    for (int j = lane; j < N - 1; j += 32) {
+      interval(j, c);
+      *reinterpret_cast<float4*>(ct + 4 * j) = make_float4((float)c[0], (float)c[1], (float)c[2], (float)c[3]);
+    }
+    return;
+  }
+  const int m = sur_shift(h);
+  const double p2 = __hiloint2double((1023 - m) << 20, 0);
+  int E = -4;                        // every interval's |a_1| + |a_2| + |a_3| is below 2^E
+  for (int j = lane; j < N - 1; j += 32) {
+    interval(j, c);
+    E = max(E, fx_expo(p2 * fma(p2, fma(p2, fabs(c[3]), fabs(c[2])), fabs(c[1]))) - 1022);
+  }
+  E = __reduce_max_sync(0xffffffffu, E);
+  if (lane == 0) pexp[i / kQ] = E;
+  for (int j = lane; j < N - 1; j += 32) {
+    interval(j, c);
+    fx* o = reinterpret_cast<fx*>(cf + 4 * j);
+    o[0] = (fx)fx_turns(c[0]);
+    for (int k = 1; k < 4; ++k) o[k] = fx_from_bits(c[k], 60 - E - m * k);
   }
 }
 
@@ -810,44 +837,95 @@ __global__ void k_node_h(const double* theta, int B, double* hs, double2* nv, fl
   }
 }
 
+// Per-mode constants of the FP64 surrogate's spline evaluation (sur_mode).
+struct SurMode {
+  fx h;        // node spacing in ln f, 2^-64
+  double hd;   // the same
+  float ihf;   // 1/h
+  int m, E;    // s = t 2^m; exponent of the phase's coefficients
+  int ampE;    // exponent of the Newtonian amplitude times hsc
+  fxs amp;     // and its significand, 2^-60
+};
+__device__ __forceinline__ SurMode sur_mode(double amp, double h, int E) {
+  const int ea = fx_expo(amp);
+  return SurMode{fx_from_bits(h, 64), h, (float)(1.0 / h), sur_shift(h), E, ea, fx_split(fx_from_bits(amp, 1082 - ea))};
+}
+// The phase spline a_0 + s (a_1 + s (a_2 + s a_3)) in turns modulo one: a_0 in 2^-64 turn, the others in 2^(E - 60); s = (u0 - j h) 2^m
+// in 2^-60, t = u0 - j h in 2^-64. A bin farther than h below the first node (extrapolated; low: below ln kFmin - 1/64) in FP64.
+__device__ __forceinline__ fxu sur_phase(const SurMode& md, const longlong4& a, double u0, bool low, fx t, int j) {
+  if (low || t < -md.h) {
+    const double x = ldexp(fma(-md.hd, (double)j, u0), md.m);
+    const double p = fma(fma((double)a.w, x, (double)a.z), x, (double)a.y) * x;
+    return (fxu)a.x + fx_turns(ldexp(p, md.E - 60));
+  }
+  const fxs s = fx_split(t << (md.m - 4));
+  fx x = a.z + fx_mul(fx_split(a.w), s);
+  x = a.y + fx_mul(fx_split(x), s);
+  return (fxu)a.x + ((fxu)fx_mul(fx_split(x), s) << (md.E + 4));
+}
 // Spline evaluation of one mode at one bin: adds hsc H T_X, hsc H T_Y, hsc H T_Z to acc. The phase
-// spline (cf, quantity 0; ~1e5 turns) is evaluated in FP64; the transfer functions T (cft, FP32
-// copies of quantities 1..6, smooth and of order one relative to their own scale) and their
-// products with H in FP32, with H carried times the sample's power of two hsc.
-// The phase's sine and cosine come from the fixed-point table (pe_fx.cuh, 2^-56), their products with the amplitude
-// are formed in fixed point and rounded to FP32 once: 6 FP64 operations per unit instead of 35, which bound
-// the kernel (1024 in-box samples, 2^22 s).
-// u0 = ln f - ln kFmin, u0f the same in FP32 (a bin within rounding of a node may take the neighbouring segment,
-// whose cubic agrees there to the spline's C2 continuity), fm76 = f^(-7/6), frc = f t_c modulo one turn (per bin);
-// ampN: the Newtonian amplitude times hsc, h, ihf: the node spacing in ln f and its inverse (per tile).
-__device__ __forceinline__ void mode_bin_sur(const ModeCoef& C, double ampN, double f, double fm76, double u0, float u0f,
-                                             fxu frc, const double* cf, const float* cft, double h, float ihf,
+// spline (cf, quantity 0; ~1e5 turns) is evaluated in fixed point (2^-60 of its largest slope; FP64 keeps 2^-53 of the phase);
+// the transfer functions T (cft, FP32 copies of quantities 1..6, smooth and of order one relative to their own scale) and their
+// products with H in FP32, with H carried times the sample's power of two hsc. Amplitude, sine and cosine are fixed
+// point (pe_fx.cuh), rounded to FP32 once. No FP64 operation per unit: the pipe was 86 % busy with 18 of them per
+// unit, the bins' included (k_sur_in64 on 1024 in-box samples, 2^22 s: 1.90 ms with five for phase and amplitude, 1.59 ms without).
+// u0 = ln f - ln kFmin, u the same in 2^-64 modulo one, u0f in FP32 (a bin within rounding of a node may take the neighbouring segment,
+// whose cubic agrees there to the spline's C2 continuity), fm, fmE: significand and exponent of f^(-7/6), frc = f t_c modulo
+// one turn (per bin).
+struct SurBin {
+  double f, u0;
+  float u0f;
+  bool low;
+  fx u;
+  fxu frc;
+  fxs fm;
+  int fmE;
+};
+__device__ __forceinline__ SurBin sur_bin(const DetDev& D, int b, double tc) {
+  SurBin n;
+  n.f = D.f[b];
+  n.u0 = fma(3.0, D.lnf3[b], -kLnFmin);
+  n.u0f = trunc_to_float((unsigned long long)__double_as_longlong(n.u0));
+  n.low = n.u0f < -0.015625f;
+  n.u = fx_from_bits(n.u0, 64);
+  n.frc = fx_cycles(n.f, tc);
+  const double fm76 = D.fm76[b];
+  n.fmE = fx_expo(fm76);
+  n.fm = fx_split(fx_from_bits(fm76, 1082 - n.fmE));
+  return n;
+}
+__device__ __forceinline__ void mode_bin_sur(const ModeCoef& C, const SurMode& md, const SurBin& n, const double* cf, const float* cft,
                                              float2 acc[3], const FxCis* __restrict__ tab) {
-  int j = (int)floorf(u0f * ihf);
+  int j = (int)floorf(n.u0f * md.ihf);
   j = j < 0 ? 0 : (j > kNodes - 2 ? kNodes - 2 : j);
-  const double t = fma(-h, (double)j, u0);
-  const double* c0 = cf + (size_t)j * 4;
-  const double ph = fma(fma(fma(c0[3], t, c0[2]), t, c0[1]), t, c0[0]);
-  const float tf = trunc_to_float((unsigned long long)__double_as_longlong(t));
+  const longlong2* c2 = reinterpret_cast<const longlong2*>(cf + (size_t)j * 4);
+  const longlong2 c01 = c2[0], c23 = c2[1];
+  const longlong4 a = {c01.x, c01.y, c23.x, c23.y};
+  const fx t = n.u - j * md.h;
+  const fxu ph = sur_phase(md, a, n.u0, n.low, t, j);
+  const float tf = n.low ? (float)fma(-md.hd, (double)j, n.u0) : (float)(int)(t >> 30) * 5.8207660913467407e-11f;   // 2^-34
   float val[kQ - 1];
 #pragma unroll
   for (int k = 0; k < kQ - 1; ++k) {
     const float4 c = *reinterpret_cast<const float4*>(cft + ((size_t)k * (kNodes - 1) + j) * 4);
     val[k] = fmaf(fmaf(fmaf(c.w, tf, c.z), tf, c.y), tf, c.x);
   }
-  double amp = ampN * fm76;   // Newtonian power law; the mode factor |H_lm| is in T
-  if (dlt_pos(C.ftap, f)) {
+  // amp = A 2^(E - 1022 - 60), A below 2^60 (Newtonian power law; the mode factor |H_lm| is in T); hr, hi = amp cos, amp sin
+  fx A = fx_mul(md.amp, n.fm);
+  int E = md.ampE + n.fmE - 1022;
+  if (dlt_pos(C.ftap, n.f)) {
     const double span = C.fend - C.ftap;
-    const double zt = span / (C.fend - f) - span / (f - C.ftap);
-    amp *= (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
+    const double zt = span / (C.fend - n.f) - span / (n.f - C.ftap);
+    const double w = (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
+    const int ew = fx_expo(w);
+    A = fx_mul(fx_split(A), fx_split(fx_from_bits(w, 1082 - ew)));
+    E += ew - 1022;
   }
-  // amp = A 2^(E - 1022 - 60), A in [2^59, 2^60); hr, hi = amp cos, amp sin
-  const int E = fx_expo(amp);
-  const fxs A = fx_split(fx_from_bits(amp, 1082 - E));
-  const fxc e = fx_cis(fx_turns(ph) - frc, tab);
-  const float sc = E > 935 ? __int_as_float((E - 925) << 23) : 0.f;   // 2^(E - 1022 - 30)
-  const float hr = (float)(int)(fx_mul(A, fx_split(e.c)) >> 30) * sc;
-  const float hi = (float)(int)(fx_mul(A, fx_split(e.s)) >> 30) * sc;
+  const fxs As = fx_split(A);
+  const fxc e = fx_cis(ph - n.frc, tab);
+  const float sc = E > 935 ? __int_as_float((E - 926) << 23) : 0.f;   // 2^(E - 1022 - 31)
+  const float hr = (float)(int)(fx_mul(As, fx_split(e.c)) >> 29) * sc;
+  const float hi = (float)(int)(fx_mul(As, fx_split(e.s)) >> 29) * sc;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     acc[c].x = fmaf(hr, val[2 * c], fmaf(-hi, val[2 * c + 1], acc[c].x));
@@ -943,13 +1021,12 @@ __global__ void __launch_bounds__(kTileBins, 3) k_sur_fwd(DetSet ds, int B, cons
                                                         const SampleCoef* __restrict__ coefN,
                                                         const double* __restrict__ theta, SurBox bx,
                                                         const double* __restrict__ spl, const float* __restrict__ splt,
-                                                        const double* __restrict__ hs,
+                                                        const double* __restrict__ hs, const int* __restrict__ pexp,
                                                         const int* __restrict__ nend, const long long* __restrict__ off,
                                                         double* part) {
   __shared__ double red[6][kTileBins + kRedPad];   // block_sum6 staging
   __shared__ double pc[kProj];
-  __shared__ double ampn[kNModes];
-  __shared__ float ihs[kNModes];
+  __shared__ SurMode sm[kNModes];
   __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   const int P = ds.ndet * B;
   const long long total = off[P];
@@ -966,10 +1043,9 @@ __global__ void __launch_bounds__(kTileBins, 3) k_sur_fwd(DetSet ds, int B, cons
       fx_proj_prologue(D, S, reinterpret_cast<fx*>(pc));
     else
       proj_prologue(D, S, pc);
-    if (threadIdx.x < kNModes) {
-      ihs[threadIdx.x] = (float)(1.0 / hs[(size_t)s * kNModes + threadIdx.x]);
-      ampn[threadIdx.x] = coefN[s].md[threadIdx.x].amp * S.hsc;
-    }
+    if (threadIdx.x < kNModes)
+      sm[threadIdx.x] = sur_mode(coefN[s].md[threadIdx.x].amp * S.hsc, hs[(size_t)s * kNModes + threadIdx.x],
+                                 pexp[((size_t)I * B + s) * kNModes + threadIdx.x]);
     __syncthreads();
     {
       double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -977,16 +1053,13 @@ __global__ void __launch_bounds__(kTileBins, 3) k_sur_fwd(DetSet ds, int B, cons
       for (int b = b0; b < b0 + kTileBins && b < ne; b += kTileBins) {
         float2 xs[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
         if (sur) {
-          const double f = D.f[b], fm76 = D.fm76[b], u0 = fma(3.0, D.lnf3[b], -kLnFmin);
-          const float u0f = trunc_to_float((unsigned long long)__double_as_longlong(u0));
-          const fxu frc = fx_cycles(f, S.tc);
+          const SurBin n = sur_bin(D, b, S.tc);
 #pragma unroll 1
           for (int md = 0; md < kNModes; ++md) {
             const ModeCoef& C = S.md[md];
-            if (!C.active || !dlt_pos(f, C.fend)) continue;
+            if (!C.active || !dlt_pos(n.f, C.fend)) continue;
             const size_t sys = ((size_t)I * B + s) * kNModes + md;
-            mode_bin_sur(C, ampn[md], f, fm76, u0, u0f, frc, spl + sys * kQ * (kNodes - 1) * 4,
-                         splt + sys * (kQ - 1) * (kNodes - 1) * 4, hs[(size_t)s * kNModes + md], ihs[md], xs,
+            mode_bin_sur(C, sm[md], n, spl + sys * kQ * (kNodes - 1) * 4, splt + sys * (kQ - 1) * (kNodes - 1) * 4, xs,
                          ds.d[0].fcis);
           }
         }
@@ -1081,14 +1154,14 @@ __global__ void __launch_bounds__(kTileBins, kSurIn64Ctas) k_sur_in64(DetSet ds,
                                                                     const double* __restrict__ spl,
                                                                     const float* __restrict__ splt,
                                                                     const double* __restrict__ hs,
+                                                                    const int* __restrict__ pexp,
                                                                     const int* __restrict__ nend,
                                                                     const long long* __restrict__ off,
                                                                     const long long* __restrict__ offk, double* part,
                                                                     unsigned long long* ctr) {
   __shared__ long long next;
   __shared__ double red[6][kTileBins + kRedPad];
-  __shared__ double ampn[kNModes], hm[kNModes];   // Newtonian amplitude times hsc; node spacing in ln f
-  __shared__ float ihf[kNModes];                  // 1/h
+  __shared__ SurMode sm[kNModes];
   const int P = ds.ndet * B;
   const long long total = offk[P];
   const int rl = sur_run(total);
@@ -1104,29 +1177,24 @@ __global__ void __launch_bounds__(kTileBins, kSurIn64Ctas) k_sur_in64(DetSet ds,
       const SampleCoef& S = coef[s];
       if (p != pcur) {     // the pair's per-sample values, staged once per run of its tiles
         __syncthreads();   // the previous pair's readers are done
-        if (threadIdx.x < kNModes) {
-          const double h = hs[(size_t)s * kNModes + threadIdx.x];
-          ampn[threadIdx.x] = coefN[s].md[threadIdx.x].amp * S.hsc;
-          hm[threadIdx.x] = h;
-          ihf[threadIdx.x] = (float)(1.0 / h);
-        }
+        if (threadIdx.x < kNModes)
+          sm[threadIdx.x] = sur_mode(coefN[s].md[threadIdx.x].amp * S.hsc, hs[(size_t)s * kNModes + threadIdx.x],
+                                     pexp[((size_t)I * B + s) * kNModes + threadIdx.x]);
         __syncthreads();
         pcur = p;
       }
       const int b = int(tk - offk[p]) * kTileBins + threadIdx.x;
       double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
       if (b < nend[p]) {
-        const double f = D.f[b], fm76 = D.fm76[b], u0 = fma(3.0, D.lnf3[b], -kLnFmin);
-        const float u0f = trunc_to_float((unsigned long long)__double_as_longlong(u0));
-        const fxu frc = fx_cycles(f, S.tc);
+        const SurBin n = sur_bin(D, b, S.tc);
         float2 xs[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
         for (int md = 0; md < kNModes; ++md) {
           const ModeCoef& C = S.md[md];
-          if (!C.active || !dlt_pos(f, C.fend)) continue;
+          if (!C.active || !dlt_pos(n.f, C.fend)) continue;
           const size_t sys = ((size_t)I * B + s) * kNModes + md;
-          mode_bin_sur(C, ampn[md], f, fm76, u0, u0f, frc, spl + sys * kQ * (kNodes - 1) * 4,
-                       splt + sys * (kQ - 1) * (kNodes - 1) * 4, hm[md], ihf[md], xs, ds.d[0].fcis);
+          mode_bin_sur(C, sm[md], n, spl + sys * kQ * (kNodes - 1) * 4, splt + sys * (kQ - 1) * (kNodes - 1) * 4, xs,
+                       ds.d[0].fcis);
         }
         double2 x[3], o[3];
 #pragma unroll
@@ -1745,7 +1813,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   aalloc(&S0, B);
   aalloc(&nend, P);
   aalloc(&off, P + 1);
-  int *nin = nullptr, *nout = nullptr;
+  int *nin = nullptr, *nout = nullptr, *pexp = nullptr;
   long long *offin = nullptr, *offout = nullptr;
   unsigned long long *ctr = nullptr, *ctrin = nullptr;
   const bool split = mode == 0;   // log L: the spline path's tiles and the per-bin path's in their own kernels
@@ -1761,6 +1829,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   aalloc(&splt, nsys * (pe::kQ - 1) * (pe::kNodes - 1) * 4);
   aalloc(&hs, (size_t)B * pe::kNModes);
   aalloc(&hs_sys, nsys);
+  if (!mix) aalloc(&pexp, nsys);
   aalloc(&nv, (size_t)B * pe::kNModes * pe::kNodeTab);
   aalloc(&nvw, (size_t)B * pe::kNModes * pe::kNodeTab);
   aalloc(&Yd, (size_t)B * pe::kNout);
@@ -1803,7 +1872,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
     if (e == cudaSuccess) {
       const long long ns = (long long)nsys * pe::kQ;
       pe::k_spline<<<(unsigned)((ns + pe::kSplineWarps - 1) / pe::kSplineWarps), 32 * pe::kSplineWarps, 0, st>>>(
-          nodes, ns, hs_sys, spl, splt, mix ? 1 : 0);
+          nodes, ns, hs_sys, spl, splt, pexp, mix ? 1 : 0);
       e = pe::launch_status();
     }
   }
@@ -1836,7 +1905,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
         pe::k_sur_inbox<pe::kSurInboxBins><<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend,
                                                                                   off, offin, part, ctrin);
       else
-        pe::k_sur_in64<<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, nend, off, offin, part, ctrin);
+        pe::k_sur_in64<<<(unsigned)g1, pe::kTileBins, 0, st>>>(ds, B, S, S0, spl, splt, hs, pexp, nend, off, offin, part, ctrin);
       e = pe::launch_status();
       // fallback tiles: the forward kernel of pe_loglike_batch in the call's precision with its tuned
       // (or default) choice, over the fallback pairs' work items; it writes each sub-tile's partial at
@@ -1846,7 +1915,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
                                            pe::grid_for(tcm, max_tiles), ctr, st, true);
     } else {
       auto kern = pe::fx_all_ok(ds) ? pe::k_sur_fwd<true> : pe::k_sur_fwd<false>;
-      kern<<<(unsigned)g, pe::kTileBins, 0, st>>>(ds, B, S, S0, theta_dev, s->box, spl, splt, hs, nend, off, part);
+      kern<<<(unsigned)g, pe::kTileBins, 0, st>>>(ds, B, S, S0, theta_dev, s->box, spl, splt, hs, pexp, nend, off, part);
       e = pe::launch_status();
     }
   }

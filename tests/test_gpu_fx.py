@@ -132,3 +132,27 @@ def test_fisher_at_pass_and_tile_edges(oracle_mod, Lb, det, mask, nb, copies):
         d = np.sqrt(np.abs(np.outer(np.diag(Fr), np.diag(Fr))))
         assert np.all(np.abs(F[s] - Fr) <= 1e-10 * d + 1e-300), (s, np.max(np.abs(F[s] - Fr) / (d + 1e-300)))
     np.testing.assert_array_equal(F, np.tile(F[:len(th)], (copies, 1, 1)))
+
+
+def test_surrogate_bins_below_the_first_node(Lb):
+    """The FP64 surrogate's fixed-point phase spline where the grid begins on the first node (1e-4 Hz), a fraction of an interval
+    below it and far below it (extrapolated in FP64), against the mixed unit's double-word spline on the same nodes;
+    bar: that pair's own, 1e-6 of the log-likelihood's terms."""
+    import torch
+    T = 2.0 ** 18
+    net = Lb.Surrogate(seed=5)
+    net.train(torch.tensor(W.draw_prior(1024, 5, T), device="cuda"), epochs=1, batch=1024)
+    net.set_node_source(1)
+    th = W.draw_prior(512, 6, T)
+    th = torch.tensor(th[(th[:, 1] <= 8.0) & (th[:, 0] >= 3e5)][:64], device="cuda")
+    rng = np.random.default_rng(7)
+    for f0 in (1e-4, 0.997e-4, 0.9e-4):
+        k0, nb = int(np.ceil(f0 * T)), 300
+        det = Lb.Detector(W.LISA, T, k0, nb)
+        det.set_data(torch.tensor(1e-21 * rng.standard_normal((3, nb, 2)), device="cuda"),
+                     torch.full((3, nb), 1e-38, dtype=torch.float64, device="cuda"))
+        a = net.loglike([det], th, W.MODE_ALL)[0].cpu().numpy()
+        b = net.loglike([det], th, W.MODE_ALL | Lb.PE_PREC_MIXED)[0].cpu().numpy()
+        r = Lb.loglike([det], th, W.MODE_ALL, dhhh=True)["dhhh"].cpu().numpy()
+        scale = 0.5 * det.data_norm().sum() + np.abs(r[..., 0].sum(axis=(1, 2))) + 0.5 * r[..., 1].sum(axis=(1, 2))
+        assert np.all(np.isfinite(a)) and np.all(np.abs(a - b) <= 1e-6 * scale), (f0, np.max(np.abs(a - b) / scale))

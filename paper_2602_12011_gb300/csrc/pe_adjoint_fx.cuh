@@ -194,13 +194,13 @@ __device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx*
       return fx_split(fx_mul(fx_split(r), inv));
     };
     const fxs krb = norm(knb, kn), prb = norm(npb, np), qrb = norm(nqb, nq);
-    const volatile fx* pl = l < 2 ? pc + 15 * l : pc + kFxProj3;
+    const volatile fx* pl = l < 2 ? pc + kFxL * l : pc + kFxProj3;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       if (m >= 2 && !helio) break;
       t = fx_prod<3>(krb, fx_unpack(pl[m]));
-      fx_mac(t, prb, fx_unpack(pl[5 + m]));
-      fx_mac(t, qrb, fx_unpack(pl[10 + m]));
+      fx_mac(t, prb, fx_unpack(pl[kFxV + m]));
+      fx_mac(t, qrb, fx_unpack(pl[2 * kFxV + m]));
       obb[m] += fx_val(t);
     }
   }
@@ -212,7 +212,7 @@ __device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx*
     const fxs kb = fx_split(fx_mul(fx_split(d), a3s));
     Wq += fx_mul(kb, fx_split(tape.ld(tl + kFtP)));
     Wp -= fx_mul(kb, fx_split(tape.ld(tl + kFtQ)));
-    const volatile fx* pl = l < 2 ? pc + 15 * l : pc + kFxProj3;
+    const volatile fx* pl = l < 2 ? pc + kFxL * l : pc + kFxProj3;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       if (m >= 2 && !helio) break;

@@ -607,7 +607,7 @@ pe_status pe_loglike_batch(const pe_detector* dets, int ndet, const double* thet
   long long* off = nullptr;
   long long* offi = nullptr;
   double* part = nullptr;
-  pe::TuneChoice tc = pe::default_choice(pe::mask_prec(mode_mask));
+  pe::TuneChoice tc = pe::default_choice(pe::mask_prec(mode_mask), ds, max_tiles);
   pe::lookup_tuned(ds, B, mode_mask, &tc);
   PE_CUDA(sc.alloc(&coef, B));
   PE_CUDA(sc.alloc(&nend, P));

@@ -2,9 +2,8 @@
 // fixed point (pe_fx.cuh): the same definitions as mode_bin (pe_device.cuh; arXiv:2602.12011 Sec. 2.1,
 // Eq. eq_tf, eq_fd_resp, FD TDI).
 //
-// On the FP64 pipe stay the TaylorF2 phase, t_f, the amplitudes, the reduction f t_c and the
-// PSD-weighted sums, which need FP64's range: about 42 of the 243 FP64 instructions that mode_bin
-// issues per unit. The orbit's sine and cosine, the link vectors' projections and norms, the
+// On the FP64 pipe stay the TaylorF2 phase, t_f far from t_c, the amplitudes and the PSD-weighted
+// sums, which need FP64's range: about 35 of the 243 FP64 instructions that mode_bin issues per unit. The orbit's sine and cosine, the link vectors' projections and norms, the
 // polarisation factors, the third-spacecraft and Doppler phases, the sincs and the TDI sums are Q60
 // integers or, where only a correction below 2^-8 is formed, double words. Their errors are those
 // of 2^-58 to 2^-56 of unit-sized quantities (root mean square), against 2^-54.5 for the FP64 ones.
@@ -12,6 +11,11 @@
 // Amplitudes span many orders of magnitude along a grid, so a bin's sums are block floating point:
 // the accumulators share one binary exponent per bin, taken from the largest amplitude so far, and
 // the mode sum's smaller modes lose only bits below 2^-60 of it.
+//
+// Bound by the latency of dependent integer and double-word operations, at half of the issue slots and 62 % of the FP64 pipe, so
+// warps count: 1024 LISA samples of 2^22 s (five modes) take 24.3 ms in FP64, 5.75 ms here with 6 CTAs of 128 per SM and one sinc
+// per call, 5.52 with pairs of them and the finer table, 4.95 with 8 CTAs (64 registers; 5.33 with 7, 5.37 with 9). The PN
+// series as fixed-point Horner chains took 9 more FP64 operations off each unit and made it 6.2 ms.
 #pragma once
 #include "pe_device.cuh"
 #include "pe_fx.cuh"
@@ -28,51 +32,73 @@ __device__ __forceinline__ fx fx_times_k(unsigned k, const FxConst& c) {
   return c.sh >= 32 ? (fx)(hi >> (c.sh - 32)) : (fx)((hi << (32 - c.sh)) | ((unsigned)lo >> c.sh));
 }
 
-// Projection forms of one (detector, sample) pair in shared memory (kFxProj words): entry 15 l + 5 v + m for the
-// links l = 0, 1 is proj_coef's over the nominal arm, m < 4 split for multiplication (h in the high word, l in the
-// low one) and the constant m = 4 a plain Q60; entries 30, 31 are k_x, k_y (split), 32 the centre's angle at t_c
-// (turns) and 33 + md mode md's m / (12 pi) cm^-5 as a double word.
-// Entries kFxProj3 + 5 v + m (m < 4): the third link's forms, minus the others' sum (fx_proj3; the reverse sweep's).
-constexpr int kFxProj = 33 + kNModes;
-constexpr int kFxProj3 = kFxProj, kFxProjAll = kFxProj + 15;
-static_assert(kFxProjAll <= kProj, "the forms share proj_coef's array");
+// What the units of one (detector, sample) pair share, in shared memory (kFxProj words, 16-byte aligned): for the links l = 0, 1
+// proj_coef's forms over the nominal arm at kFxL l + kFxV v + m, m < 4 split for multiplication (h in the high word, l in the
+// low one; read two at a time) and the constant m = 4 a plain Q60; k_x, k_y (split); the centre's angle at t_c (turns);
+// per mode m / (12 pi) cm^-5 as a double word, and the amplitude times the polarisation weights (doubles).
+// Entries kFxProj3 + kFxV v + m (m < 4): the third link's forms, minus the others' sum (fx_proj3; the reverse sweep's).
+constexpr int kFxV = 6, kFxL = 3 * kFxV;
+enum : int { kFpK = 2 * kFxL, kFpAlpha = kFpK + 2, kFpTau, kFpPp = kFpTau + kNModes, kFpPc = kFpPp + kNModes,
+             kFpEnd = kFpPc + kNModes };
+constexpr int kFxProj = ((kFpEnd > kProj ? kFpEnd : kProj) + 1) / 2 * 2;   // kernels of both units share the array
+constexpr int kFxProj3 = kFxProj, kFxProjAll = kFxProj + kFxL;
 __device__ __forceinline__ fx fx_pack(fxs s) { return ((fx)s.h << 32) | (unsigned)s.l; }
 __device__ __forceinline__ fxs fx_unpack(fx p) {
   fxs r;
   asm("mov.b64 {%0, %1}, %2;" : "=r"(r.l), "=r"(r.h) : "l"(p));
   return r;
 }
+// Two packed words at p (16-byte aligned, shared memory); volatile, so that no form stays in registers across the links
+__device__ __forceinline__ void fx_ld2(const volatile fx* p, fxs& a, fxs& b) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(a.l), "=r"(a.h), "=r"(b.l), "=r"(b.h)
+               : "r"((unsigned)__cvta_generic_to_shared(const_cast<const fx*>(p))));
+}
 __device__ __forceinline__ void fx_proj_prologue(const DetDev& D, const SampleCoef& S, fx* pc) {
   __syncthreads();
-  const int i = threadIdx.x;
-  if (i >= 33 && i < kFxProj) {
-    const float2 w = to_dw(S.md[i - 33].tffac * S.md[i - 33].icm5);
-    pc[i] = ((fx)__float_as_int(w.y) << 32) | (unsigned)__float_as_int(w.x);
-  } else if (i == 32) {
-    pc[i] = (fx)fx_turns(fma(S.tc, D.rate_t, D.alpha0_t));
-  } else if (i < 32) {
-    const double v = i < 30 ? proj_coef(D, S, i) * D.fx_iL : S.k[i - 30];
-    const fx q = fx_from_bits(v, 60);
-    pc[i] = (i < 30 && i % 5 == 4) ? q : fx_pack(fx_split(q));
+  for (int i = threadIdx.x; i < 30 + kFpEnd - kFpK; i += blockDim.x) {
+    if (i < 30) {   // proj_coef's order: 15 l + 5 v + m
+      const fx q = fx_from_bits(proj_coef(D, S, i) * D.fx_iL, 60);
+      pc[i / 5 * kFxV + i % 5] = i % 5 == 4 ? q : fx_pack(fx_split(q));
+      continue;
+    }
+    const int j = i - 30 + kFpK;
+    fx q = 0;
+    if (j < kFpAlpha) {
+      q = fx_pack(fx_split(fx_from_bits(S.k[j - kFpK], 60)));
+    } else if (j == kFpAlpha) {
+      q = (fx)fx_turns(fma(S.tc, D.rate_t, D.alpha0_t));
+    } else if (j < kFpPp) {
+      const ModeCoef& C = S.md[j - kFpTau];
+      const float2 w = to_dw(C.tffac * C.icm5);
+      q = ((fx)__float_as_int(w.y) << 32) | (unsigned)__float_as_int(w.x);
+    } else {
+      const ModeCoef& C = S.md[(j - kFpPp) % kNModes];
+      q = __double_as_longlong(C.ampp * (j < kFpPc ? C.Pp : C.Pc2));
+    }
+    pc[j] = q;
   }
   __syncthreads();
 }
 __device__ __forceinline__ void fx_proj3(fx* pc) {   // after fx_proj_prologue; a barrier at the end
   const int i = threadIdx.x;
-  if (i < 15 && i % 5 < 4) {
-    const fxs a = fx_unpack(pc[i]), b = fx_unpack(pc[15 + i]);
+  if (i < kFxL && i % kFxV < 4) {
+    const fxs a = fx_unpack(pc[i]), b = fx_unpack(pc[kFxL + i]);
     pc[kFxProj3 + i] = fx_pack(fx_split(-((((fx)a.h + b.h) << 30) + a.l + b.l)));
   }
   __syncthreads();
 }
 // p[0..3] . b + p[4] (geocentric: b has two entries and the constant is zero)
 __device__ __forceinline__ fx fx_dot(const volatile fx* p, const fxs b[4], bool helio) {
-  fxa s = fx_prod<2>(fx_unpack(p[0]), b[0]);
-  fx_mac(s, fx_unpack(p[1]), b[1]);
+  fxs c0, c1;
+  fx_ld2(p, c0, c1);
+  fxa s = fx_prod<2>(c0, b[0]);
+  fx_mac(s, c1, b[1]);
   if (helio) {
+    fx_ld2(p + 2, c0, c1);
     s.c += 2 * kFxLL;
-    fx_mac(s, fx_unpack(p[2]), b[2]);
-    fx_mac(s, fx_unpack(p[3]), b[3]);
+    fx_mac(s, c0, b[2]);
+    fx_mac(s, c1, b[3]);
     s.h += p[4];
   }
   return fx_val(s);
@@ -160,7 +186,7 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
   // Third-spacecraft phases f k.delta_t / 2 in turns: delta_0 - delta_1, delta_1 - delta_2 and
   // delta_2 - delta_0 are the link vectors and the offsets sum to zero, so delta_0 = (n_0 - n_2)/3,
   // delta_1 = (n_1 - n_0)/3 and delta_2 is minus both
-  const fx kn0 = fx_dot(pc, ob, helio), kn1 = fx_dot(pc + 15, ob, helio), kn2 = -(kn0 + kn1);
+  const fx kn0 = fx_dot(pc, ob, helio), kn1 = fx_dot(pc + kFxL, ob, helio), kn2 = -(kn0 + kn1);
   const fxu e0 = (fxu)fx_mul(fx_split(kn0 - kn2), at3) << 4;
   const fxu e1 = (fxu)fx_mul(fx_split(kn1 - kn0), at3) << 4;
   fx np = 0, nq = 0;   // minus the sums of the earlier links' projections
@@ -168,8 +194,8 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
   for (int l = 0; l < 3; ++l) {
     fx pr = np, qr = nq;
     if (l < 2) {
-      pr = fx_dot(pc + 15 * l + 5, ob, helio);
-      qr = fx_dot(pc + 15 * l + 10, ob, helio);
+      pr = fx_dot(pc + kFxL * l + kFxV, ob, helio);
+      qr = fx_dot(pc + kFxL * l + 2 * kFxV, ob, helio);
       np -= pr;
       nq -= qr;
     }
@@ -214,18 +240,19 @@ __device__ __forceinline__ void fx_links(fxs at3, fx a4, fxu phu, fxs Apx, fxs A
     const fxs Gi = fx_split(fx_val(gi));
     // --- sinc(a (1 +- k.n)) and the link's products for the TDI brackets (row A6; see XYZAcc)
     volatile fx* as = acc.s + 4 * l * Acc::kStride;
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      const fx u4 = h == 0 ? a4 + w4 : a4 - w4, sv = fx_sinc(u4, stab);
-      const fxs sc = fx_split(sv);
-      if constexpr (Tape::kOn) {
-        tape.st(tl + kFtSp + h, sv);
-        tape.st(tl + kFtDp + h, fx_sinc(u4, stab + kFxSincTab));   // the derivative's table follows
-      }
-      as[0] = as[0] + fx_mul(Gr, sc);
-      as[Acc::kStride] = as[Acc::kStride] + fx_mul(Gi, sc);
-      as += 2 * Acc::kStride;
+    const fx2 sv = fx_sinc2(a4 + w4, a4 - w4, stab);
+    const fxs sp = fx_split(sv.p), sm = fx_split(sv.m);
+    if constexpr (Tape::kOn) {
+      const fx2 dv = fx_sinc2(a4 + w4, a4 - w4, stab + kFxSincTab);   // the derivative's table follows
+      tape.st(tl + kFtSp, sv.p);
+      tape.st(tl + kFtSm, sv.m);
+      tape.st(tl + kFtDp, dv.p);
+      tape.st(tl + kFtDm, dv.m);
     }
+    as[0] = as[0] + fx_mul(Gr, sp);
+    as[Acc::kStride] = as[Acc::kStride] + fx_mul(Gi, sp);
+    as[2 * Acc::kStride] = as[2 * Acc::kStride] + fx_mul(Gr, sm);
+    as[3 * Acc::kStride] = as[3 * Acc::kStride] + fx_mul(Gi, sm);
   }
 }
 
@@ -258,7 +285,7 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
     const df q6v = dfl_mul(S.Q6w, vw);
     const df q = dfl_add(S.Q5w, dfl_add(q6v, dfl_mul(q6v, df_from_bits(lnv))));
     dpol = dfl_add(dpol, dfl_mul(dfl_mul(dfl_mul(v2, v2), vw), q));
-    const fx kw = pc[33 + md];
+    const fx kw = pc[kFpTau + md];
     tau = dfl_mul(dfl_mul(df_make(__int_as_float((int)kw), __int_as_float((int)(kw >> 32))), D.fm83w[B.b]), dpol);
   }
   const bool helio = D.orbit == 0;
@@ -267,7 +294,7 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
   if (helio && fabsf(tau.x) < kFxTauMax) {
     // the series' terms may cancel and leave a low word beyond fx_from_dw's bound: normalised first
     const df a = dfl_mul(tau, D.ratew);
-    alpha = (fxu)pc[32] + ((fxu)fx_from_dw(two_sum(a.x, a.y)) << 4);
+    alpha = (fxu)pc[kFpAlpha] + ((fxu)fx_from_dw(two_sum(a.x, a.y)) << 4);
   } else {
     double dpol = S.Pd[7];
 #pragma unroll 1
@@ -278,28 +305,30 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
     alpha = fx_turns(fma(tf, D.rate_t, D.alpha0_t));
     geo = fx_turns(tf * D.geo_rate_t);
   }
-  double amp = C.ampp * (C.p == 0 ? D.fm76[B.b] : (C.p == 1 ? D.fm56[B.b] : D.fm12[B.b]));
-  if (dlt_pos(C.ftap, B.f)) {
-    const double span = C.fend - C.ftap;
-    const double zt = span / (C.fend - B.f) - span / (B.f - C.ftap);
-    const double w = (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
-    if constexpr (Tape::kOn) {
-      tape.st(kFtAmp0, __double_as_longlong(amp));
-      tape.st(kFtW, __double_as_longlong(w));
-    }
-    amp *= w;
-  } else if constexpr (Tape::kOn) {
-    tape.st(kFtAmp0, __double_as_longlong(amp));
-    tape.st(kFtW, __double_as_longlong(1.0));
-  }
   // polarisation weights times the amplitude (complex for a paired second mode), as integers below
   // 1/8 in units of 2^(E - 1079)
-  double2 Ap = make_double2(amp * C.Pp, 0.0), Ac = make_double2(amp * C.Pc2, 0.0);
+  const double fp = C.p == 0 ? D.fm76[B.b] : (C.p == 1 ? D.fm56[B.b] : D.fm12[B.b]);
+  double2 Ap, Ac;
+  double w = 1.0;
   if (C2) {
-    const double v2 = v * v;
+    const double v2 = v * v, amp = C.ampp * fp;
     const double kr = S.k32.x * v2, ki = S.k32.y * v2;
     Ap = make_double2(amp * fma(kr, C2->Pp, C.Pp), amp * (ki * C2->Pp));
     Ac = make_double2(amp * fma(kr, C2->Pc2, C.Pc2), amp * (ki * C2->Pc2));
+  } else {
+    Ap = make_double2(fp * __longlong_as_double(pc[kFpPp + md]), 0.0);
+    Ac = make_double2(fp * __longlong_as_double(pc[kFpPc + md]), 0.0);
+  }
+  if (dlt_pos(C.ftap, B.f)) {
+    const double span = C.fend - C.ftap;
+    const double zt = span / (C.fend - B.f) - span / (B.f - C.ftap);
+    w = (zt > 700.0) ? 0.0 : 1.0 / (1.0 + exp(zt));
+    Ap = make_double2(Ap.x * w, Ap.y * w);
+    Ac = make_double2(Ac.x * w, Ac.y * w);
+  }
+  if constexpr (Tape::kOn) {
+    tape.st(kFtAmp0, __double_as_longlong(C.ampp * fp));
+    tape.st(kFtW, __double_as_longlong(w));
   }
   int E = max(fx_expo(Ap.x), fx_expo(Ac.x));
   if (C2) E = max(E, max(fx_expo(Ap.y), fx_expo(Ac.y)));
@@ -318,8 +347,10 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
   // --- orbit at t_f (row A4): mode phase in turns, the centre's Doppler term f k.x_c = f R (k_x cos + k_y sin)
   // included, and the offsets' basis
   const fxc ca = fx_cis(alpha, tab);
-  fxa kc = fx_prod<2>(fx_unpack(pc[30]), fx_split(ca.c));
-  fx_mac(kc, fx_unpack(pc[31]), fx_split(ca.s));
+  fxs kx, ky;
+  fx_ld2(pc + kFpK, kx, ky);
+  fxa kc = fx_prod<2>(kx, fx_split(ca.c));
+  fx_mac(kc, ky, fx_split(ca.s));
   const fxu phu = fx_turns(fma(-C.mfac, psi_pn, C.ph0)) - B.frc -
                   ((fxu)fx_mul(fx_split(fx_val(kc)), B.fR) << (4 + D.fx_rsh));
   fxs ob[4];

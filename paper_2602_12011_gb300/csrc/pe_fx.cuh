@@ -116,12 +116,13 @@ struct alignas(16) FxCis {       // the angle 2 pi j / kSinTab: cos and sin in Q
   fx c, s;
   float4 w;          // cos hi, cos lo, sin hi, sin lo
 };
-struct alignas(16) FxSinc {      // sinc about u_j = j / kFxSincPerUnit: value in Q60, derivatives f^(k)(u_j)/k!
+struct alignas(32) FxSinc {      // sinc about u_j = j / kFxSincPerUnit: value in Q60, derivatives f^(k)(u_j)/k!
   fx s0;
-  float2 s1, s2, s3; // double words
-  float s4, s5, s6, pad;
+  float2 s1, s2;     // double words
+  float s3, s4;
 };
-constexpr int kFxSincPerUnit = 64;
+constexpr int kFxSincBits = 9;                                  // 512 entries per unit of u
+constexpr int kFxSincPerUnit = 1 << kFxSincBits;
 constexpr int kFxSincMax = 8;                                   // u < 8 (a = pi f L < 4)
 constexpr int kFxSincTab = kFxSincPerUnit * kFxSincMax + 2;
 
@@ -150,20 +151,25 @@ static __device__ __noinline__ fxc fx_cis(fxu u, const FxCis* __restrict__ tab) 
 }
 
 // sinc(u) = sin u / u for u = 4 u4, 0 <= u < kFxSincMax (a value below 0 by rounding counts as 0): Taylor
-// series about the nearest table point, |u - u_j| <= 2^-7, through the sixth order (the seventh is
-// below 2^-63). The correction to the table's value is below 2^-8 and is formed in double words;
-// from the third order on the next coefficients enter the low word.
-static __device__ __noinline__ fx fx_sinc(fx u4, const FxSinc* __restrict__ tab) {
-  const int j = min(max((int)((u4 + (1LL << 51)) >> 52), 0), kFxSincTab - 1);
-  const fx d = u4 - ((fx)j << 52);                               // in 2^-58 of u
+// series about the nearest table point, |u - u_j| <= 2^-10, through the fourth order (the fifth is
+// below 2^-59). The correction to the table's value is below 2^-11 and is formed in double words;
+// from the second order on the next coefficients enter the low word.
+__device__ __forceinline__ fx fx_sinc(fx u4, const FxSinc* __restrict__ tab) {
+  constexpr int kS = 58 - kFxSincBits;
+  const int j = min(max((int)((u4 + (1LL << (kS - 1))) >> kS), 0), kFxSincTab - 1);
+  const fx d = u4 - ((fx)j << kS);                               // in 2^-58 of u
   const FxSinc e = tab[j];
-  const df x = df_make(__fmul_rn(__int2float_rn((int)(d >> 28)), 9.3132257461547852e-10f),           // 2^-30
-                       __fmul_rn(__int2float_rn((int)d & 0xfffffff), 3.4694469519536142e-18f));      // 2^-58
-  const float tail = __fmaf_rn(x.x, __fmaf_rn(x.x, e.s6, e.s5), e.s4);
-  df p = df_make(e.s3.x, __fmaf_rn(x.x, tail, e.s3.y));
-  p = dfl_add(e.s2, dfl_mul(x, p));
-  p = dfl_add(e.s1, dfl_mul(x, p));
+  const df x = df_make(__fmul_rn(__int2float_rn((int)(d >> 25)), 1.16415321826934814e-10f),          // 2^-33
+                       __fmul_rn(__int2float_rn((int)d & 0x1ffffff), 3.4694469519536142e-18f));      // 2^-58
+  const df p = dfl_add(e.s1, dfl_mul(x, df_make(e.s2.x, __fmaf_rn(x.x, __fmaf_rn(x.x, e.s4, e.s3), e.s2.y))));
   return e.s0 + fx_from_dw(dfl_mul(x, p));
+}
+// sinc of two arguments at once: each is a chain of dependent double-word operations, and two fill each other's gaps
+struct fx2 {
+  fx p, m;
+};
+static __device__ __noinline__ fx2 fx_sinc2(fx p, fx m, const FxSinc* __restrict__ tab) {
+  return fx2{fx_sinc(p, tab), fx_sinc(m, tab)};
 }
 
 // 1/sqrt(x) for Q60 x in [1/2, 2): a float seed y (24 bits, taken to 2^-30), then y + y (e/2 + 3 e^2/8)

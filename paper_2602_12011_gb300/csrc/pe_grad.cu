@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
   __shared__ long long next;
   __shared__ double red[kGradFxV][kTileBins + kRedPad];
   __shared__ fx col[kFxSums][kTileBins];   // the forward sums, then the link seeds, a column per thread
-  __shared__ fx pc[kProj];
+  __shared__ __align__(16) fx pc[kFxProjAll];
   __shared__ double rot[3];
   static_assert(kGradFxV * kGradFxRow <= kTileBins, "one pass adds every row");
   double* tape = tape_all + (size_t)blockIdx.x * kTapeDoubles + threadIdx.x;
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
   const unsigned long long pol = tape_l2_policy();
   for (long long t = blockIdx.x, tn = 0; t < total; t = work_next(tn, &next)) {
     tn = work_fetch(ctr, t);
-    const int p = find_pair_g(off, P, t);
+    const int p = find_pair_warp(off, P, t);
     if (!PE_CHK(p >= 0 && p < P && off[p + 1] <= total && nend[p] <= ds.d[p / B].nb, 16)) continue;
     const int I = p / B, s = p - I * B;
     const int b = int(t - off[p]) * kTileBins + threadIdx.x;
@@ -587,7 +587,7 @@ struct FisherShared {
   fx col[kFxSums][kFisherFxThreads];           // the forward's sums (unused), then the seeds, a column per thread
   double J[kFisherWarps][PE_NPARAM][32];       // rows Re/Im of A', E', T'
   double gJ[kFisherWarps][PE_NPARAM][32];      // the same times the channel's 4 / (T S)
-  fx pc[kProj];
+  alignas(16) fx pc[kFxProjAll];
   double rot[3][3];                            // d(lambda, beta, psi) per rotation cotangent
   long long next;
 };
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(kFisherFxThreads, 2) k_fisher_fx(DetSet ds, in
   for (long long t = blockIdx.x, tn = 0; t < total; t = work_next(tn, &sm.next)) {
     tn = work_fetch(ctr, t);
     const long long tile = t / split;
-    const int p = find_pair_g(off, P, tile);
+    const int p = find_pair_warp(off, P, tile);
     if (!PE_CHK(p >= 0 && p < P && off[p + 1] * split <= total && nend[p] <= ds.d[p / B].nb, 64)) continue;
     const int I = p / B, s = p - I * B;
     const DetDev& D = ds.d[I];

@@ -121,7 +121,7 @@ __device__ __forceinline__ void mode_brackets_mixed(const DetDev& D, const Sampl
 // Reference per-mode brackets on bins [0, K): out[(md*3 + c)*K + k].
 template <bool FX>
 __global__ void k_mode_brackets(DetDev D, const SampleCoef* coef, int K, unsigned mask, double2* out) {
-  __shared__ double pc[kProj];
+  __shared__ __align__(16) double pc[kFxProj];
   __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   const SampleCoef& S = coef[0];
   if (FX)
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
   extern __shared__ double2 rsh[];
   unsigned char* wflag = reinterpret_cast<unsigned char*>(rsh + (size_t)hs.nemax * kNModes * 3);
   constexpr bool DW = MIX && !FX;   // the mixed unit at the edges
-  __shared__ double pc[kProj];
+  __shared__ __align__(16) double pc[kFxProj];
   __shared__ float2 pcw[DW ? kProj : 1];
   __shared__ double sh[6][kHetThreads / 32];
   __shared__ double2 stab[DW || FX ? 1 : kSinTab];
@@ -740,7 +740,7 @@ pe_status pe_hetero_loglike_batch(const pe_hetero* hets, int ndet, const double*
   // equal rounds of edges over the fewest threads (at least 64, which stage the projection forms)
   const int rounds = (nemax + pe::kHetThreads - 1) / pe::kHetThreads;
   const int threads = std::max(64, ((nemax + rounds - 1) / rounds + 31) / 32 * 32);
-  static_assert(pe::kProj <= 64 && pe::kFxProj <= 64, "one thread per form");
+  static_assert(pe::kProj <= 64, "one thread per form");
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) {
     kern<<<B, threads, smem, st>>>(hs, B, static_cast<const pe::SampleCoef*>(coef), static_cast<double*>(ll),

@@ -26,11 +26,13 @@ constexpr int kPrecFP64 = 0, kPrecMixed = 1, kPrecFP32 = 2;
 constexpr int kPrecFx = 3;
 // Work items of the log-likelihood kernels are R consecutive 128-bin sub-tiles of one (detector,
 // sample) pair, R in {1, 2, 4, 8} picked by the autotuner. The default (no tuned choice) keeps
-// one sub-tile per item in FP64 (most CTAs for small batches) and four in the other precisions,
-// which amortise their per-item staging over more bins. Each sub-tile keeps its own partial, so R
+// one sub-tile per item in FP64 and the fixed-point unit (most CTAs for small batches) and four in the other
+// units, which amortise their per-item staging over more bins. Each sub-tile keeps its own partial, so R
 // never changes a result.
 constexpr int kFwdMaxSubtiles = 8;
-__host__ __device__ constexpr int fwd_default_subtiles(int prec) { return prec == kPrecFP64 ? 1 : 4; }
+__host__ __device__ constexpr int fwd_default_subtiles(int prec, bool fx) {
+  return prec == kPrecFP64 || (fx && prec != kPrecFP32) ? 1 : 4;
+}
 constexpr int kSinTab = 1024;   // entries of the (cos, sin) table used by sincos_turns
 
 // Per-(sample, mode) coefficients (row A1 of the path). With v = (2 pi M f/m)^(1/3):

@@ -96,7 +96,7 @@ __device__ __forceinline__ df dd_to_dw(dd a) {
 }
 // One thread per angle (the first kSinTab) and per (sinc entry, order); snc: sinc's kFxSincTab entries, then its
 // derivative's.
-constexpr int kFxSincOrders = 8;
+constexpr int kFxSincOrders = 6;
 __global__ void k_fx_tables(FxCis* cis, FxSinc* snc) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < kSinTab) {
@@ -138,10 +138,8 @@ __global__ void k_fx_tables(FxCis* cis, FxSinc* snc) {
     if (order == 0) o.s0 = dd_to_fx(v);
     else if (order == 1) o.s1 = dd_to_dw(v);
     else if (order == 2) o.s2 = dd_to_dw(v);
-    else if (order == 3) o.s3 = dd_to_dw(v);
+    else if (order == 3) o.s3 = (float)v.h;
     else if (order == 4) o.s4 = (float)v.h;
-    else if (order == 5) o.s5 = (float)v.h;
-    else if (order == 6) o.s6 = (float)v.h;
   };
   put(snc[e], k, sum);
   if (k > 0) put(snc[kFxSincTab + e], k - 1, dd_mul(sum, dd{(double)k, 0.0}));   // sinc' about the same points
@@ -373,16 +371,6 @@ __global__ void k_scan_tiles(const int* nend, int P, int sa, long long* off, int
   }
 }
 
-// pair index p with off[p] <= t < off[p+1]
-__device__ __forceinline__ int find_pair(const long long* off, int P, long long t) {
-  int lo = 0, hi = P;  // invariant off[lo] <= t < off[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (off[mid] <= t) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
 // ------------------------------------------------------------------------------------------
 // Rows A2-A7: persistent fused kernel. The work list is every (detector, sample) pair's 128-bin
 // sub-tiles (off: their offsets per pair); a work item is R consecutive sub-tiles of one pair
@@ -394,8 +382,8 @@ __device__ __forceinline__ int find_pair(const long long* off, int P, long long 
 // fixed order into part[sub-tile][6] (<d|h>_c, <h|h>_c). The partials are per sub-tile whatever
 // R, MINB (resident CTAs per SM requested from the compiler, which sets the register budget) or
 // the grid, so the autotuner's choices never change a result. PREC selects the all-FP64 unit, the
-// mixed FP64/double-word one (pe_device_mixed.cuh) or the all-FP32 one of the precision study
-// (pe_device_f32.cuh).
+// mixed FP64/double-word one (pe_device_mixed.cuh), the all-FP32 one of the precision study
+// (pe_device_f32.cuh) or, for FP64 and mixed calls on the detectors that allow it, the fixed-point one (pe_device_fx.cuh).
 // ------------------------------------------------------------------------------------------
 template <int MINB, int PREC>
 __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int B, const SampleCoef* __restrict__ coef,
@@ -405,7 +393,7 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
                                                                  double* part, unsigned long long* ctr) {
   __shared__ long long next;
   __shared__ double red[6][kTileBins + kRedPad];   // block_sum6 staging (as float2 or float rows)
-  __shared__ double pc[kProj];    // the item's projection forms (proj_coef; fx_proj_prologue's words)
+  __shared__ __align__(16) double pc[kFxProj];    // the item's projection forms (proj_coef; fx_proj_prologue's words)
   __shared__ float2 pcw[kProj];   // the same as double words (mixed) or floats (.x, FP32)
   __shared__ SampleF sf;          // the item's sample coefficients in FP32 (FP32 path)
   __shared__ fx fxcol[PREC == kPrecFx ? kFxSums : 1][kTileBins];   // the fixed-point unit's sums, a column per thread
@@ -421,7 +409,7 @@ __global__ void __launch_bounds__(kTileBins, MINB) k_loglike_fwd(DetSet ds, int 
   const long long total = offi[P];
   for (long long t = blockIdx.x, tn = 0; t < total; t = work_next(tn, &next)) {
     tn = work_fetch(ctr, t);
-    const int p = find_pair(offi, P, t);
+    const int p = find_pair_warp(offi, P, t);
     if (!PE_CHK(p >= 0 && p < P, 1)) continue;              // checked build: uniform over the CTA
     const int I = p / B, s = p - I * B;
     const long long j0 = (t - offi[p]) * R;                 // first sub-tile of the item in the pair
@@ -593,7 +581,7 @@ __global__ void __launch_bounds__(192) k_reduce(DetSet ds, int B, const long lon
 // Noise-free A/E/T signal of one sample on the whole grid: h_c = Q n_c B_c. out: [3][nb].
 template <int PREC>
 __global__ void k_signal(DetDev D, const SampleCoef* coef, double2* out) {
-  __shared__ double pc[kProj];
+  __shared__ __align__(16) double pc[kFxProj];
   __shared__ float2 pcw[kProj];
   __shared__ SampleF sf;
   __shared__ fx fxcol[PREC == kPrecFx ? kFxSums : 1][kTileBins];
@@ -760,21 +748,22 @@ cudaError_t launch_loglike_fwd_variant(int variant, int prec, const DetSet& ds, 
                                        double* part, int grid, unsigned long long* ctr, cudaStream_t st, bool items) {
   items |= R > 1;
   if (R != 1 && R != 2 && R != 4 && R != 8) return cudaErrorInvalidValue;
-  // FP64: the fixed-point unit where every detector meets its bounds
-  if (prec == kPrecFP64 && fx_all_ok(ds)) prec = kPrecFx;
+  // FP64 and mixed: the fixed-point unit where every detector meets its bounds. It overtook the double-word unit at eight
+  // CTAs per SM (1024 LISA samples of 2^22 s: 4.97 ms, double words 5.50) with errors a hundredth of it.
+  if (prec != kPrecFP32 && fx_all_ok(ds)) prec = kPrecFx;
   switch (variant * 4 + prec) {
     case 0: return fwd_one<2, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 1: return fwd_one<2, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 2: return fwd_one<2, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
-    case 3: return fwd_one<4, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 3: return fwd_one<7, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 4: return fwd_one<3, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 5: return fwd_one<3, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 6: return fwd_one<3, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
-    case 7: return fwd_one<6, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 7: return fwd_one<8, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 8: return fwd_one<4, kPrecFP64>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 9: return fwd_one<4, kPrecMixed>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     case 10: return fwd_one<4, kPrecFP32>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
-    case 11: return fwd_one<5, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
+    case 11: return fwd_one<6, kPrecFx>(ds, B, coef, nend, off, offi, R, part, grid, items, ctr, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -46,7 +46,7 @@ cudaError_t launch_loglike_fwd(const DetSet& ds, int B, const SampleCoef* coef, 
                                cudaStream_t st);
 // ctr: the list's work counter (launch_scan_tiles), left cleared; NULL: CTAs stride over the items.
 // items: offi is the list of work items even where R == 1 (a list of some pairs only).
-// Register-budget variants of the forward kernel (min resident CTAs per SM 2, 3, 4), per precision.
+// Register-budget variants of the forward kernel (min resident CTAs per SM 2, 3, 4; the fixed-point unit's 7, 8, 6).
 constexpr int kFwdVariants = 3;
 constexpr int kFwdDefaultVariant = 1;
 cudaError_t launch_loglike_fwd_variant(int variant, int prec, const DetSet& ds, int B, const SampleCoef* coef,

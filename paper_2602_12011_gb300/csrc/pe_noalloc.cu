@@ -76,7 +76,7 @@ extern "C" pe_status pe_loglike_batch_noalloc(const pe_detector* dets, int ndet,
   // [P+1], sub-tile partials [sub-tiles][6]. The work items take the precision's default number of
   // sub-tiles (no tuned choice is read here).
   const size_t P = (size_t)ndet * B;
-  const int R = pe::fwd_default_subtiles(pe::mask_prec(mode_mask));
+  const int R = pe::fwd_default_subtiles(pe::mask_prec(mode_mask), pe::fx_all_ok(ds));
   size_t max_tiles = 0;
   for (int i = 0; i < ndet; ++i) max_tiles += (size_t)B * pe::tiles_of(ds.d[i].nb, pe::kTileBins);
   const size_t o_coef = 0;

@@ -132,7 +132,12 @@ bool lookup_tuned(const DetSet& ds, int B, unsigned mask, TuneChoice* out) {
   return true;
 }
 
-TuneChoice default_choice(int prec) { return TuneChoice{kFwdDefaultVariant, 8, fwd_default_subtiles(prec), 0.0}; }
+// The fixed-point unit's items are one sub-tile, two from 2^19 possible ones on (1024 LISA samples of 2^22 s: 4.95 ms with one, 4.88 with
+// two; 45 samples on three detectors and single points are faster with one, whose last round is shorter).
+TuneChoice default_choice(int prec, const DetSet& ds, long long max_tiles) {
+  const bool fx = fx_all_ok(ds) && prec != kPrecFP32;
+  return TuneChoice{kFwdDefaultVariant, 8, fx && max_tiles >= (1LL << 19) ? 2 : fwd_default_subtiles(prec, fx), 0.0};
+}
 
 int grid_for(const TuneChoice& c, long long max_tiles) {
   const long long g = std::min<long long>(max_tiles, (long long)sm_count_now() * c.ctas_per_sm);
@@ -172,10 +177,11 @@ cudaError_t autotune_fwd(const DetSet& ds, int B, unsigned mask, const SampleCoe
     *out_ms = bm;
     return r;
   };
-  TuneChoice b{-1, 0, fwd_default_subtiles(prec), 1e30};
+  const int r1 = fwd_default_subtiles(prec, fx_all_ok(ds));
+  TuneChoice b{-1, 0, r1, 1e30};
   for (int v = 0; v < kFwdVariants && e == cudaSuccess; ++v)
     for (int ci = 0; ci < 4 && e == cudaSuccess; ++ci) {
-      TuneChoice c{v, kCtas[ci], fwd_default_subtiles(prec), 0.0};
+      TuneChoice c{v, kCtas[ci], r1, 0.0};
       float ms = 0.f;
       e = time_one(c, &ms);
       if (e == cudaSuccess && ms < b.ms) { b = c; b.ms = ms; }
@@ -271,7 +277,7 @@ pe_status pe_plan_create(const pe_detector* dets, int ndet, int B, unsigned mode
   double* part = reinterpret_cast<double*>(sc + o_part);
   cudaStream_t cs = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-  pl->choice = pe::default_choice(pe::mask_prec(mode_mask));
+  pl->choice = pe::default_choice(pe::mask_prec(mode_mask), ds, max_tiles);
   if (e == cudaSuccess && !pe::lookup_tuned(ds, B, mode_mask, &pl->choice) && autotune) {
     e = pe::launch_prep(theta_dev, B, mode_mask, ds, coef, nend, nullptr, cs);
     if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, (int)P, off, pe::kTileBins, ctr, cs);
@@ -373,7 +379,7 @@ pe_status pe_autotune(const pe_detector* dets, int ndet, const double* theta_dev
   double* part = reinterpret_cast<double*>(sc + o_part);
   cudaStream_t cs = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-  pe::TuneChoice best = pe::default_choice(pe::mask_prec(mode_mask));
+  pe::TuneChoice best = pe::default_choice(pe::mask_prec(mode_mask), ds, max_tiles);
   if (e == cudaSuccess) e = pe::launch_prep(theta_dev, B, mode_mask, ds, coef, nend, nullptr, cs);
   if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, (int)P, off, pe::kTileBins, ctr, cs);
   if (e == cudaSuccess) e = pe::autotune_fwd(ds, B, mode_mask, coef, nend, off, offi, part, max_tiles, ctr, cs, &best);

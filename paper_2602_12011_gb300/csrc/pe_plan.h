@@ -17,7 +17,7 @@ struct TuneChoice {
 
 std::string tune_key(const DetSet& ds, int B, unsigned mask);
 bool lookup_tuned(const DetSet& ds, int B, unsigned mask, TuneChoice* out);
-TuneChoice default_choice(int prec);
+TuneChoice default_choice(int prec, const DetSet& ds, long long max_tiles);
 int grid_for(const TuneChoice& c, long long max_tiles);
 // Times the candidates on the prepared work list (coefficients, active counts and sub-tile offsets
 // off on the device; offi: scratch for the work-item offsets, P + 1 entries; ctr: off's

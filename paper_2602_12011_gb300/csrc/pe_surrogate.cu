@@ -316,7 +316,7 @@ __global__ void k_sur_nodes(DetSet ds, int B, const SampleCoef* S, const SampleC
                             const float4* __restrict__ nvw, double* nodes) {
   static_assert(kNodes % kTileBins == 0, "a CTA's nodes belong to one (detector, sample, mode)");
   constexpr bool MIX = KIND == kNodesMixed, FX = KIND == kNodesFx;
-  __shared__ fx pc[FX ? kProj : 1];
+  __shared__ __align__(16) fx pc[FX ? kFxProj : 1];
   __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long total = (long long)ds.ndet * B * kNModes * kNodes;
@@ -1025,7 +1025,7 @@ __global__ void __launch_bounds__(kTileBins, 3) k_sur_fwd(DetSet ds, int B, cons
                                                         const int* __restrict__ nend, const long long* __restrict__ off,
                                                         double* part) {
   __shared__ double red[6][kTileBins + kRedPad];   // block_sum6 staging
-  __shared__ double pc[kProj];
+  __shared__ __align__(16) double pc[kFxProj];
   __shared__ SurMode sm[kNModes];
   __shared__ fx fxcol[FX ? kFxSums : 1][kTileBins];
   const int P = ds.ndet * B;
@@ -1879,7 +1879,7 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
   if (e == cudaSuccess) e = pe::launch_prep(theta_dev, B, mode_mask, ds, S, nend, nullptr, st);
   if (e == cudaSuccess) e = pe::launch_scan_tiles(nend, P, off, pe::kTileBins, nullptr, st);
   const int prec = mix ? pe::kPrecMixed : pe::kPrecFP64;
-  pe::TuneChoice tcm = pe::default_choice(prec);
+  pe::TuneChoice tcm = pe::default_choice(prec, ds, max_tiles);
   if (split) pe::lookup_tuned(ds, B, mode_mask | (mix ? PE_PREC_MIXED : 0u), &tcm);
   if (e == cudaSuccess && split) {
     unsigned geo_mask = 0;

@@ -137,16 +137,19 @@ __device__ __forceinline__ double psi_of(const SampleCoef& S, double v, double l
 // ratio exceeds q_above (all of them for q_above < 1; the others' rows are left as they are).
 // nv (nullable): k_node_h's tables, from which f's powers and ln v come without exp, cbrt and log (1024 samples: 0.62 ms
 // with them, the FP64 log-likelihood's path)
-__global__ void k_targets(const double* theta, int B, const SampleCoef* S, const SampleCoef* S0, float* out,
-                          double q_above, const double2* nv) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)B * kNModes * kNodes) return;
-  const int j = (int)(i % kNodes);
-  const int md = (int)((i / kNodes) % kNModes);
-  const int s = (int)(i / ((long long)kNodes * kNModes));
+// Bound by the FP64 pipe. A CTA's kNodes nodes belong to one (sample, mode), so one thread forms their spacing (a logarithm)
+// and mode factor (8192 samples over the prior, a fifth above the bound: 1.14 ms with every thread forming them, 0.56 ms).
+__global__ void __launch_bounds__(kNodes) k_targets(const double* theta, int B, const SampleCoef* S, const SampleCoef* S0, float* out,
+                                                    double q_above, const double2* nv) {
+  __shared__ double sh[2];
+  const int j = threadIdx.x;
+  const int md = blockIdx.x % kNModes, s = blockIdx.x / kNModes;
   const double* t = theta + (size_t)s * PE_NPARAM;
-  if (!(t[1] > q_above)) return;
+  if (!(t[1] > q_above)) return;   // uniform over the CTA
   const int mm = (md == 0) ? 2 : (md == 1) ? 1 : (md == 2) ? 3 : (md == 3) ? 2 : 4;
+  if (j == 0) sh[0] = node_h(t[0] * kMsunS, mm);
+  if (j == 32) sh[1] = hmag_of(md, t[1]);
+  __syncthreads();
   double v, lnv;
   if (nv) {
     const double2* tab = nv + ((size_t)s * kNModes + md) * kNodeTab;
@@ -157,13 +160,13 @@ __global__ void k_targets(const double* theta, int B, const SampleCoef* S, const
     lnv = fma((double)j, tab[1].y, tab[0].y);
   } else {
     const double M = t[0] * kMsunS;
-    const double f = kFmin * exp(j * node_h(M, mm));
+    const double f = kFmin * exp(j * sh[0]);
     v = cbrt(2.0 * kPi * M * f / mm);
     lnv = log(v);
   }
   const double r = 0.5 * mm * (psi_of(S[s], v, lnv, nullptr) - psi_of(S0[s], v, lnv, nullptr));
   const int p = S[s].md[md].p;
-  const double a = hmag_of(md, t[1]) * (p >= 1 ? v : 1.0) * (p >= 2 ? v : 1.0);
+  const double a = sh[1] * (p >= 1 ? v : 1.0) * (p >= 2 ? v : 1.0);
   out[(size_t)s * kNout + (md * 2 + 0) * kNodes + j] = (float)r;
   out[(size_t)s * kNout + (md * 2 + 1) * kNodes + j] = (float)a;
 }
@@ -1628,8 +1631,7 @@ pe_status pe_surrogate_targets(const double* theta_dev, int B, float* out_dev) {
   if (e == cudaSuccess) e = dalloc(&S0, B);
   if (e == cudaSuccess) {
     pe::k_sur_prep<<<(B + 63) / 64, 64>>>(theta_dev, B, PE_MODE_ALL, S, S0);
-    const long long n = (long long)B * pe::kNModes * pe::kNodes;
-    pe::k_targets<<<(unsigned)((n + 255) / 256), 256>>>(theta_dev, B, S, S0, out_dev, 0.0, nullptr);
+    pe::k_targets<<<(unsigned)(B * pe::kNModes), pe::kNodes>>>(theta_dev, B, S, S0, out_dev, 0.0, nullptr);
     e = pe::launch_status();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
@@ -1845,14 +1847,13 @@ static pe_status sur_run(pe_surrogate s, const pe_detector* dets, int ndet, cons
     pe::k_node_h<<<(B * pe::kNModes + 127) / 128, 128, 0, st>>>(theta_dev, B, hs, nv, nvw);
     // node values: the network's, with the plain generator's own above the network's mass-ratio
     // bound (or everywhere for node source 1)
-    const long long nt = (long long)B * pe::kNModes * pe::kNodes;
     if (s->node_source == 0) {
       pe::k_destd<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(s->Y, B, s->mean, s->stdv, Yd);
       if (s->box.qnet < s->box.qmax)
-        pe::k_targets<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(theta_dev, B, S, S0, Yd, s->box.qnet,
+        pe::k_targets<<<(unsigned)(B * pe::kNModes), pe::kNodes, 0, st>>>(theta_dev, B, S, S0, Yd, s->box.qnet,
                                                                        mix ? nullptr : nv);
     } else {
-      pe::k_targets<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(theta_dev, B, S, S0, Yd, 0.0, mix ? nullptr : nv);
+      pe::k_targets<<<(unsigned)(B * pe::kNModes), pe::kNodes, 0, st>>>(theta_dev, B, S, S0, Yd, 0.0, mix ? nullptr : nv);
     }
     const long long nn = (long long)nsys * pe::kNodes;
     if (mix)

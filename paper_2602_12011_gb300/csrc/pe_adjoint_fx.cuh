@@ -249,22 +249,36 @@ __device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx*
   }
 }
 
-// Sums of one bin's sweeps over its modes; the factors common to the modes are applied once per bin (fx_bin_grad).
-struct FxBinAcc {
-  double lnA, vM, q, io, ph, tc;   // ln amplitude; v d/dv of phase and t_f chains; q, iota, phi_c, t_c
-  double x3, x4;                   // psib v^-2 - 2 Db v^-2, psib v^-1 - Db v^-1 (chi1, chi2 enter P3 and P4 alone)
-  double W[3], dc, ds;             // rotation; Doppler f R-weighted cos and sin
-  double Mx;                       // Mtot through the taper and the paired mode
+// Sums of one bin's sweeps over its modes; the factors common to the modes are applied once per bin (fx_bin_grad): ln amplitude; v d/dv of
+// the phase and t_f chains; q, iota, phi_c, t_c; psib v^-2 - 2 Db v^-2 and psib v^-1 - Db v^-1 (chi1, chi2 enter P3 and P4
+// alone); rotation; Doppler, f R-weighted cos and sin; Mtot through the taper and the paired mode.
+enum : int { kGlnA, kGvM, kGq, kGio, kGph, kGtc, kGx3, kGx4, kGW, kGdc = kGW + 3, kGds, kGMx, kGSums };
+struct FxBinAcc {       // in registers
+  double v[kGSums];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < kGSums; ++i) v[i] = 0.0;
+  }
+  __device__ __forceinline__ double get(int i) const { return v[i]; }
+  __device__ __forceinline__ void add(int i, double x) { v[i] += x; }
+  __device__ __forceinline__ void mac(int i, double x, double y) { v[i] = fma(x, y, v[i]); }
 };
-__device__ __forceinline__ void fx_bin_zero(FxBinAcc& g) {
-  g.lnA = g.vM = g.q = g.io = g.ph = g.tc = g.x3 = g.x4 = g.dc = g.ds = g.Mx = 0.0;
-  g.W[0] = g.W[1] = g.W[2] = 0.0;
-}
-// Reverse sweep of one unit, added to the bin's sums; the PN chain in FP64. fm13 = f^(-1/3), invf = 1/f, fR = 2 pi f R. (t_f's part of the
+template <int STRIDE>
+struct FxBinAccShared {   // in a thread's column of shared memory: 28 registers less across the sweep
+  volatile double* v;
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < kGSums; ++i) v[i * STRIDE] = 0.0;
+  }
+  __device__ __forceinline__ double get(int i) const { return v[i * STRIDE]; }
+  __device__ __forceinline__ void add(int i, double x) { v[i * STRIDE] = v[i * STRIDE] + x; }
+  __device__ __forceinline__ void mac(int i, double x, double y) { v[i * STRIDE] = fma(x, y, v[i * STRIDE]); }
+};
+// Reverse sweep of one unit, added to the bin's sums; the PN chain in FP64. fm13 = f^(-1/3), invf = 1/f, fR = 2 pi f R, n2pif = -2 pi f. (t_f's part of the
 // chain in double words saved 14 FP64 FMAs a unit and no time: the kernel waits on dependent operations.)
-template <int SST, class Tape>
+template <int SST, class Tape, class BinAcc>
 __device__ __forceinline__ void mode_bwd_fx(const DetDev& D, const SampleCoef& S, const SampleGrad& SG, int md, int md2, const FxBin& B,
-                                            double fm13, double invf, double fR, fx a3, const volatile fx* seeds, int Es, FxBinAcc& g,
+                                            double fm13, double invf, double fR, double n2pif, fx a3, const volatile fx* seeds, int Es, BinAcc& g,
                                             const fx* __restrict__ pc, const Tape& tape) {
   const ModeCoef& C = S.md[md];
   const ModeGrad& CG = SG.md[md];
@@ -290,58 +304,63 @@ __device__ __forceinline__ void mode_bwd_fx(const DetDev& D, const SampleCoef& S
   // phase: ph0 = m phi_c / 2 pi + ..., -f t_c, -(m / 4 pi) Psi, -f k.x_c (turns)
   const double mh = md == 1 ? -0.5 : (md == 2 ? -1.5 : (md == 4 ? -2.0 : -1.0));   // -m/2
   const double psib = mh * o.th;                 // - mfac 2 pi th
-  g.ph = fma(-2.0, psib, g.ph);
-  g.tc = fma(-2.0 * kPi * B.f, o.th, g.tc);
+  g.mac(kGph, -2.0, psib);
   // centre's Doppler term -f k.x_c, x_c = R (cos alpha, sin alpha, 0)
   const double fth = -fR * o.th, fc = fth * h.co, fs = fth * h.so;
-  g.dc += fc;
-  g.ds += fs;
+  g.add(kGdc, fc);
+  g.add(kGds, fs);
 #pragma unroll
-  for (int i = 0; i < 3; ++i) g.W[i] += o.W[i];
+  for (int i = 0; i < 3; ++i) g.add(kGW + i, o.W[i]);
   const double alphab = fma(S.k[1], fc, fma(-S.k[0], fs, o.alpha));
-  const double tfb = fma(alphab, 2.0 * kPi * D.rate_t, o.geo * (2.0 * kPi * D.geo_rate_t));
-  g.tc += tfb;                                   // t_f = t_c + (m/(12 pi f)) D(v)
+  double tfb = alphab * D.rate_rad;
+  if (D.orbit != 0) tfb = fma(o.geo, D.geo_rate_rad, tfb);
+  g.add(kGtc, fma(n2pif, o.th, tfb));   // frac(f t_c); t_f = t_c + (m/(12 pi f)) D(v)
   const double Db = tfb * (C.tffac * invf);
   // amplitude ~ M^(5/6) ... f^(-7/6 + p/3) cm^p: dlnA_dM without the mode's own v is common to the modes
-  g.lnA += o.lnA;
-  g.q = fma(o.lnA, CG.dlnA_dq, g.q);
-  g.Mx = fma(o.lnA, h.tap, g.Mx);
-  g.vM = fma(psib, h.dv, fma(Db, h.ddv, fma(o.lnA, double(C.p), g.vM)));
-  g.q = fma(psib, h.pq, fma(Db, h.dq, g.q));
-  g.x4 = fma(h.iv, psib - Db, g.x4);
-  g.x3 = fma(h.iv * h.iv, fma(-2.0, Db, psib), g.x3);
+  g.add(kGlnA, o.lnA);
+  g.mac(kGMx, o.lnA, h.tap);
+  double vM = fma(psib, h.dv, Db * h.ddv);
+  if (C.p != 0) vM += C.p == 1 ? o.lnA : 2.0 * o.lnA;
+  double q = fma(psib, h.pq, fma(Db, h.dq, o.lnA * CG.dlnA_dq));
+  g.mac(kGx4, h.iv, psib - Db);
+  g.mac(kGx3, h.iv * h.iv, fma(-2.0, Db, psib));
   // polarisation weights: Ac carries 2 Pc
-  const double2 apb = make_double2(amp * o.Ap.x, amp * o.Ap.y), acb = make_double2(amp * o.Ac.x, amp * o.Ac.y);
-  g.io = fma(apb.x, CG.dPp_di, fma(2.0 * acb.x, CG.dPc_di, g.io));
+  double io = amp * fma(o.Ap.x, CG.dPp_di, o.Ac.x * (2.0 * CG.dPc_di));
   if (md2 >= 0) {
+    const double2 apb = make_double2(amp * o.Ap.x, amp * o.Ap.y), acb = make_double2(amp * o.Ac.x, amp * o.Ac.y);
     const ModeGrad& CG2 = SG.md[md2];
     const double2 kap = make_double2(S.k32.x * (v * v), S.k32.y * (v * v));
     const double Pp2 = S.md[md2].Pp, Pc22 = S.md[md2].Pc2;
-    g.io += (apb.x * kap.x + apb.y * kap.y) * CG2.dPp_di + 2.0 * (acb.x * kap.x + acb.y * kap.y) * CG2.dPc_di;
+    io += (apb.x * kap.x + apb.y * kap.y) * CG2.dPp_di + 2.0 * (acb.x * kap.x + acb.y * kap.y) * CG2.dPc_di;
     const double2 kb = make_double2(apb.x * Pp2 + acb.x * Pc22, apb.y * Pp2 + acb.y * Pc22);   // kappa-bar
     // kappa = k32 v^2; only ln(amp2 / amp1) varies with theta (M, q), see mode_bwd
     const double lnrb = v * v * (kb.x * S.k32.x + kb.y * S.k32.y);
-    g.Mx = fma(lnrb, CG2.dlnA_dM - CG.dlnA_dM, g.Mx);
-    g.q = fma(lnrb, CG2.dlnA_dq - CG.dlnA_dq, g.q);
-    g.vM = fma(2.0, lnrb, g.vM);
+    g.mac(kGMx, lnrb, CG2.dlnA_dM - CG.dlnA_dM);
+    q = fma(lnrb, CG2.dlnA_dq - CG.dlnA_dq, q);
+    vM = fma(2.0, lnrb, vM);
   }
+  g.add(kGvM, vM);
+  g.add(kGq, q);
+  g.add(kGio, io);
 }
 
 // The bin's theta components from its sums, with the rotation cotangents in g.k. th: the sample's parameters enter through
 // SampleGrad alone: d ln v / d Mtot = 1 / (3 Mtot) = dcm_dM / cm.
-__device__ __forceinline__ void fx_bin_grad(const SampleCoef& S, const SampleGrad& SG, const FxBinAcc& a, GradAcc& g) {
+template <class BinAcc>
+__device__ __forceinline__ void fx_bin_grad(const SampleCoef& S, const SampleGrad& SG, const BinAcc& a, GradAcc& g) {
   const double m3 = SG.md[0].dcm_dM / S.md[0].cm;    // 1 / (3 Mtot)
-  g.M = fma(a.vM, m3, fma(a.lnA, 2.5 * m3, a.Mx));   // dlnA_dM = 5 / (6 Mtot)
-  g.q = a.q;
-  g.c1 = fma(SG.dP3_dc1, a.x3, SG.dP4_dc1 * a.x4);
-  g.c2 = fma(SG.dP3_dc2, a.x3, SG.dP4_dc2 * a.x4);
-  g.dL = a.lnA * SG.dlnA_ddL;
-  g.io = a.io;
-  g.ph = a.ph;
-  g.tc = a.tc;
-  g.k[0] = a.W[0];
-  g.k[1] = a.W[1] - fma(S.q[0], a.dc, S.q[1] * a.ds);
-  g.k[2] = a.W[2] + fma(S.p[0], a.dc, S.p[1] * a.ds);
+  const double lnA = a.get(kGlnA), x3 = a.get(kGx3), x4 = a.get(kGx4), dc = a.get(kGdc), ds = a.get(kGds);
+  g.M = fma(a.get(kGvM), m3, fma(lnA, 2.5 * m3, a.get(kGMx)));   // dlnA_dM = 5 / (6 Mtot)
+  g.q = a.get(kGq);
+  g.c1 = fma(SG.dP3_dc1, x3, SG.dP4_dc1 * x4);
+  g.c2 = fma(SG.dP3_dc2, x3, SG.dP4_dc2 * x4);
+  g.dL = lnA * SG.dlnA_ddL;
+  g.io = a.get(kGio);
+  g.ph = a.get(kGph);
+  g.tc = a.get(kGtc);
+  g.k[0] = a.get(kGW);
+  g.k[1] = a.get(kGW + 1) - fma(S.q[0], dc, S.q[1] * ds);
+  g.k[2] = a.get(kGW + 2) + fma(S.p[0], dc, S.p[1] * ds);
 }
 
 // Component c of the frame vectors' cotangents (vec 0 k, 1 p, 2 q) that stand for the rotation cotangents W: with

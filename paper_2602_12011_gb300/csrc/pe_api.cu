@@ -270,6 +270,8 @@ void fill_dev(pe_detector_s* d) {
     for (int j = 0; j < 3; ++j)
       for (int m = 0; m < 5; ++m) D.Mof[i][j][m] = static_cast<float>(D.Mo[i][j][m]);
   D.ratew = host_dw(D.rate_t);
+  D.rate_rad = 2.0 * pe::kPi * D.rate_t;
+  D.geo_rate_rad = 2.0 * pe::kPi * D.geo_rate_t;
   D.alpha0w = host_dw(D.alpha0_t);
   D.geo_ratew = host_dw(D.geo_rate_t);
   // double-word t_f carries ~6e-14 relative error (a dozen rounded operations); below 2^23 s the

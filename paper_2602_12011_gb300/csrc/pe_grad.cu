@@ -313,10 +313,12 @@ __global__ void __launch_bounds__(kTileBins, 2) k_grad_fwd_tape(DetSet ds, int B
 // The gradient on detectors that take the fixed-point unit, both precisions: per bin the forward mode sum writes each unit's
 // tape, the A/E/T cotangents and link seeds follow in FP64, and the reverse sweeps run in fixed point from the tape
 // (pe_adjoint_fx.cuh). Per tile 17 sums: the 14 of the FP64 kernel and the frame's three rotation cotangents, written as
-// the 23 partials the reduction reads. Bound by dependent integer and FP64 operations (about 6,000 thread instructions a
-// unit, FP64 pipe 60 %). 64 LISA samples of 2^22 s: FP64 4.08 -> 1.54 ms; 500 at the mixed precision, whose
-// double-word sweep was at the FP32 pipe's rate, 12.8 -> 10.8 ms; hence both precisions take it.
+// the 23 partials the reduction reads. Bound by the FP64 pipe (about 135 operations a unit, 67 % busy of 84 %) and dependent integer operations (5,600 thread
+// instructions a unit). 64 LISA samples of 2^22 s: FP64 4.08 -> 1.54 ms; 500 at the mixed precision, whose
+// double-word sweep was at the FP32 pipe's rate, 12.8 -> 10.8 ms; hence both precisions take it. (Items drawn from a counter and the
+// bin's sums in shared memory: 1.34 and 9.9 ms; five and six CTAs per SM spill, 4 and 6 % slower.)
 constexpr int kGradFxV = 17;
+constexpr int kGradFxRows = 6 + kGSums;
 constexpr int kGradFxCtas = 4;   // resident CTAs per SM (tape 92 MB, inside L2)
 constexpr int kGradFxRow = 7;    // threads that add one row of the block sum
 __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet ds, int B, const SampleCoef* __restrict__ coef,
@@ -325,7 +327,7 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
                                                                       const long long* __restrict__ off, double* part,
                                                                       double* tape_all, unsigned long long* ctr) {
   __shared__ long long next;
-  __shared__ double red[kGradFxV][kTileBins + kRedPad];
+  __shared__ double red[kGradFxRows][kTileBins + kRedPad];   // the values of the block sums; before, from row 6 on, the bin's sums
   __shared__ fx col[kFxSums][kTileBins];   // the forward sums, then the link seeds, a column per thread
   __shared__ __align__(16) fx pc[kFxProjAll];
   __shared__ double rot[3];
@@ -344,9 +346,6 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
     const SampleCoef& S = coef[s];
     fx_proj_prologue(D, S, pc);   // its first barrier: the previous tile's readers of red and rot are done
     fx_proj3(pc);
-    double v[kGradFxV];
-#pragma unroll
-    for (int i = 0; i < kGradFxV; ++i) v[i] = 0.0;
     if (b < nend[p]) {
       const SampleGrad& SG = sgrad[s];
       FxBin Bn;
@@ -363,30 +362,35 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
       }
       double2 o[3], bb[3], pq[6];
       aet_from_fx(a, D.z[b], o);
+      double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
       aet_cotangents(D, b, o, v, bb);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) red[i][threadIdx.x] = v[i];
       const double2 sc = D.sca[b];
       link_seeds<1>(bb, sc.x, sc.y, pq);
       const int Es = fx_seeds<kTileBins>(pq, &col[0][threadIdx.x]);
       const fx a3 = fx_times_k((unsigned)(D.k0 + b), D.fx_a3);
-      const double fm13 = D.fm13[b], invf = fm13 * fm13 * fm13, fR = 2.0 * kPi * D.R * Bn.f;
-      FxBinAcc ga;
-      fx_bin_zero(ga);
+      const double fm13 = D.fm13[b], invf = fm13 * fm13 * fm13, n2pif = -2.0 * kPi * Bn.f, fR = -D.R * n2pif;
+      FxBinAccShared<kTileBins + kRedPad> ga = {&red[6][threadIdx.x]};
+      ga.zero();
 #pragma unroll 1
       for (int md = 0; md < kNModes; ++md) {
         if (md == 3 && S.pair32) continue;
         const ModeCoef& C = S.md[md];
         if (Es == 0 || !C.active || !dlt_pos(Bn.f, C.fend)) continue;
         const FxTape tp = {tape + tape_slot(md) * kTapeF * kTileBins, pol};
-        mode_bwd_fx<kTileBins>(D, S, SG, md, (md == 0 && S.pair32) ? 3 : -1, Bn, fm13, invf, fR, a3, &col[0][threadIdx.x], Es, ga, pc,
+        mode_bwd_fx<kTileBins>(D, S, SG, md, (md == 0 && S.pair32) ? 3 : -1, Bn, fm13, invf, fR, n2pif, a3, &col[0][threadIdx.x], Es, ga, pc,
                                tp);
       }
       GradAcc g;
       fx_bin_grad(S, SG, ga, g);
-      v[6] = g.M; v[7] = g.q; v[8] = g.c1; v[9] = g.c2; v[10] = g.dL; v[11] = g.io; v[12] = g.ph; v[13] = g.tc;
-      v[14] = g.k[0]; v[15] = g.k[1]; v[16] = g.k[2];
-    }
+      const double out[kGradFxV - 6] = {g.M, g.q, g.c1, g.c2, g.dL, g.io, g.ph, g.tc, g.k[0], g.k[1], g.k[2]};
 #pragma unroll
-    for (int i = 0; i < kGradFxV; ++i) red[i][threadIdx.x] = v[i];
+      for (int i = 6; i < kGradFxV; ++i) red[i][threadIdx.x] = out[i - 6];
+    } else {
+#pragma unroll
+      for (int i = 0; i < kGradFxV; ++i) red[i][threadIdx.x] = 0.0;
+    }
     __syncthreads();
     // thread t adds entries g, g + 7, ... of row i = t / 7 (g = t % 7) into red[i][g]; then thread i its seven
     if (threadIdx.x < kGradFxV * kGradFxRow) {
@@ -663,14 +667,14 @@ __global__ void __launch_bounds__(kFisherFxThreads, 2) k_fisher_fx(DetSet ds, in
         link_seeds<1>(bb, sc.x, sc.y, pq);
         const int Es = fx_seeds<kFisherFxThreads>(pq, col);
         const fx a3 = fx_times_k((unsigned)(D.k0 + b), D.fx_a3);
-        const double invf = fm13 * fm13 * fm13, fR = 2.0 * kPi * D.R * Bn.f;
+        const double invf = fm13 * fm13 * fm13, n2pif = -2.0 * kPi * Bn.f, fR = -D.R * n2pif;
         FxBinAcc ga;
-        fx_bin_zero(ga);
+        ga.zero();
 #pragma unroll 1
         for (int md = 0; md < kNModes; ++md) {
           if ((md == 3 && S.pair32) || Es == 0 || !S.md[md].active || !dlt_pos(Bn.f, S.md[md].fend)) continue;
           const FisherTape tp = {&sm.tape[tape_slot(md)][0][lane]};
-          mode_bwd_fx<kFisherFxThreads>(D, S, SG, md, (md == 0 && S.pair32) ? 3 : -1, Bn, fm13, invf, fR, a3, col, Es, ga, sm.pc, tp);
+          mode_bwd_fx<kFisherFxThreads>(D, S, SG, md, (md == 0 && S.pair32) ? 3 : -1, Bn, fm13, invf, fR, n2pif, a3, col, Es, ga, sm.pc, tp);
         }
         GradAcc g;
         fx_bin_grad(S, SG, ga, g);

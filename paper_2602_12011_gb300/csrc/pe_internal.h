@@ -133,6 +133,7 @@ struct DetDev {
   double cb[3], sb[3];
   // geocentric: offsets r (cos phi_i e1 + sin phi_i e2), phi_0 in half-turns = t * geo_rate_ht
   double rgeo, geo_rate_ht, geo_rate_t;
+  double rate_rad, geo_rate_rad;   // the rates in rad/s
   double e1[3], e2[3];
   // per-bin tables (length nb)
   const double* f;      // f_k = k / T

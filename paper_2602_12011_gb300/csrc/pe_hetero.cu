@@ -47,6 +47,9 @@ struct HetDev {
   const double2* Bs;     // [kPairs][3][3][ne-1]
   const float4* Aw;      // A and Bs as double words (re hi, re lo, im hi, im lo), for the mixed kernel
   const float4* Bw;
+  const longlong2* Ax;   // A and Bs for the fixed-point contraction (k_het_words): packed words of re, im
+  const longlong2* Bx;
+  const int2* Ex;        // [3][ne-1] their exponents
   int ne;
   unsigned mask;
 };
@@ -255,6 +258,105 @@ __device__ __forceinline__ void het_bin_fp64(const HetDev& H, int b, int c, Ld l
     hh = fma(r0[md].x, y.x, fma(-r0[md].y, y.y, fma(r1[md].x, w.x, fma(-r1[md].y, w.y, hh))));
   }
 }
+// Summary data of one (channel c, bin b) for the fixed-point contraction: over ra and d = rb - ra (the slopes' powers of
+// 1/(fe[b+1] - fe[b]) in the data), as multiples of 2^(E - 60) with E (one for A, one for Bs) above twice the sum of the magnitudes that
+// multiply components below 1, packed for multiplication (fx_pack).
+__global__ void k_het_words(const double* fe, int ne, const double2* A, const double2* Bs, longlong2* Ax, longlong2* Bx, int2* Ex) {
+  const int nbin = ne - 1, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 3 * nbin) return;
+  const int c = i / nbin, b = i % nbin;
+  const double idf = 1.0 / (fe[b + 1] - fe[b]);
+  auto at = [&](const double2* q, int row, int o) {
+    const double2 v = q[(size_t)row * nbin + b];
+    const double f = o == 0 ? 1.0 : (o == 1 ? idf : idf * idf);
+    return make_double2(v.x * f, v.y * f);
+  };
+  auto row_a = [&](int md, int o) { return (md * 3 + c) * 2 + o; };
+  auto row_b = [&](int pr, int o) { return (pr * 3 + c) * 3 + o; };
+  double sa = 0.0, sb = 0.0;
+  for (int md = 0; md < kNModes; ++md)
+    for (int o = 0; o < 2; ++o) {
+      const double2 v = at(A, row_a(md, o), o);
+      sa += fabs(v.x) + fabs(v.y);
+    }
+  for (int pr = 0; pr < kPairs; ++pr)
+    for (int o = 0; o < 3; ++o) {
+      const double2 v = at(Bs, row_b(pr, o), o);
+      sb += (o == 1 ? 4.0 : 2.0) * (fabs(v.x) + fabs(v.y));
+    }
+  auto word = [](double2 v, double sum, int E) {
+    if (sum == 0.0) return longlong2{0, 0};
+    return longlong2{fx_pack(fx_split(fx_from_bits(v.x, 60 - E))), fx_pack(fx_split(fx_from_bits(v.y, 60 - E)))};
+  };
+  const int ea = fx_expo(sa) - 1021, eb = fx_expo(sb) - 1021;
+  for (int md = 0; md < kNModes; ++md)
+    for (int o = 0; o < 2; ++o) Ax[(size_t)row_a(md, o) * nbin + b] = word(at(A, row_a(md, o), o), sa, ea);
+  for (int pr = 0; pr < kPairs; ++pr)
+    for (int o = 0; o < 3; ++o) Bx[(size_t)row_b(pr, o) * nbin + b] = word(at(Bs, row_b(pr, o), o), sb, eb);
+  Ex[i] = make_int2(ea, eb);
+}
+
+// Ratios that the fixed-point contraction takes: components below 2, held as a quarter in 2^-60. Those of a posterior's bulk are near
+// 1; an edge with a larger one is kept in FP64, and its bins take het_bin_fp64.
+constexpr double kHetFxRatioMax = 2.0;
+constexpr int kHetFxBits = 58;
+// het_bin_fp64's contraction in fixed point: ratios below 1/2, d below 1, the data's sums below 1/2, so every sum stays below 1. Bound by the
+// 32 x 32-bit products, about 900 per (bin, channel) at 16 per SM and clock where the FP64 form issues 340 operations
+// at 1.67 (777 samples, LISA, 2^22 s: 0.68 -> 0.36 ms).
+__device__ __forceinline__ void het_bin_fx(const HetDev& H, int b, int c, const longlong2* __restrict__ rx, double& dh, double& hh) {
+  const int nbin = H.ne - 1;
+  fxs rr[kNModes], ri[kNModes], dr[kNModes], di[kNModes];
+#pragma unroll
+  for (int md = 0; md < kNModes; ++md) {
+    const int s0 = H.src[(b * kNModes + md) * 3 + c], s1 = H.src[((b + 1) * kNModes + md) * 3 + c];
+    const longlong2 ra = s0 >= 0 ? rx[(s0 * kNModes + md) * 3 + c] : longlong2{0, 0};
+    const longlong2 rb = s1 >= 0 ? rx[(s1 * kNModes + md) * 3 + c] : longlong2{0, 0};
+    rr[md] = fx_split(ra.x);
+    ri[md] = fx_split(ra.y);
+    dr[md] = fx_split(rb.x - ra.x);
+    di[md] = fx_split(rb.y - ra.y);
+  }
+  fx sd = 0, sh = 0;
+#pragma unroll
+  for (int md = 0; md < kNModes; ++md) {
+    const longlong2* a = H.Ax + (size_t)(md * 3 + c) * 2 * nbin + b;
+    const longlong2 w0 = a[0], w1 = a[nbin];
+    sd += fx_msub(fx_unpack(w0.x), rr[md], fx_unpack(w0.y), ri[md]) + fx_msub(fx_unpack(w1.x), dr[md], fx_unpack(w1.y), di[md]);
+    fx yx = 0, yy = 0, wx = 0, wy = 0;
+#pragma unroll
+    for (int k = 1; k <= kNModes; ++k) {
+      const int m2 = k < kNModes ? (md + k) : md;   // the off-diagonal pairs first, doubled, then the diagonal one
+      if (m2 >= kNModes) continue;
+      if (k == kNModes) { yx *= 2; yy *= 2; wx *= 2; wy *= 2; }
+      const longlong2* q = H.Bx + (size_t)(pair_index(md, m2) * 3 + c) * 3 * nbin + b;
+      const longlong2 u0 = q[0], u1 = q[nbin], u2 = q[2 * nbin];
+      const fxs x0 = fx_unpack(u0.x), y0 = fx_unpack(u0.y), x1 = fx_unpack(u1.x), y1 = fx_unpack(u1.y), x2 = fx_unpack(u2.x), y2 = fx_unpack(u2.y);
+      // (x + i y) conj(r): (x rr + y ri) + i (y rr - x ri)
+      auto madd = [&](fxs a0, fxs b0, fxs a1, fxs b1, fxs a2, fxs b2, fxs a3, fxs b3) {
+        fxa t = fx_prod<4>(a0, b0);
+        fx_mac(t, a1, b1);
+        fx_mac(t, a2, b2);
+        fx_mac(t, a3, b3);
+        return fx_val(t);
+      };
+      auto msub = [&](fxs a0, fxs b0, fxs a1, fxs b1, fxs a2, fxs b2, fxs a3, fxs b3) {   // a0 b0 + a1 b1 - a2 b2 - a3 b3
+        fxa t = fx_prod<0>(a0, b0), n = fxa{fx_mulw(a2.h, b2.h), fx_madw(a2.h, b2.l, fx_mulw(a2.l, b2.h))};
+        fx_mac(t, a1, b1);
+        fx_mac(n, a3, b3);
+        return (t.h - n.h) + ((t.c - n.c) >> 30);
+      };
+      yx += madd(x0, rr[m2], y0, ri[m2], x1, dr[m2], y1, di[m2]);
+      yy += msub(y0, rr[m2], y1, dr[m2], x0, ri[m2], x1, di[m2]);
+      wx += madd(x1, rr[m2], y1, ri[m2], x2, dr[m2], y2, di[m2]);
+      wy += msub(y1, rr[m2], y2, dr[m2], x1, ri[m2], x2, di[m2]);
+    }
+    sh += fx_msub(rr[md], fx_split(yx), ri[md], fx_split(yy)) + fx_msub(dr[md], fx_split(wx), di[md], fx_split(wy));
+  }
+  const int2 E = H.Ex[c * nbin + b];
+  dh = fx_to_double(sd, E.x - 60 + (60 - kHetFxBits));
+  hh = fx_to_double(sh, E.y - 60 + 2 * (60 - kHetFxBits));
+}
+
 // Re(a b) and Re(a conj(b)) in double words
 __device__ __forceinline__ df re_mul(const cdf& a, const cdf& b) { return dfl_sub(dfl_mul(a.re, b.re), dfl_mul(a.im, b.im)); }
 __device__ __forceinline__ cdf mul_conj(const cdf& a, const cdf& b) {
@@ -283,7 +385,8 @@ __device__ __forceinline__ void het_block_sum(double v[6], double (*sh)[kHetThre
 // and three rounds of edges, the last a third full (777 samples, LISA: 1.09 ms).
 // The signal at the edges comes from the fixed-point unit (FX; both precisions), or the precision's own where a detector
 // does not take that unit. MIX: the ratios are kept as double words and contracted in double words (Aw, Bw);
-// the sums across bins and the block reduction stay FP64. An edge with a ratio of kHetDwRatioMax or more
+// the sums across bins and the block reduction stay FP64. FP64 on the fixed-point unit: the ratios are kept and contracted in fixed
+// point (het_bin_fx). An edge with a ratio of kHetDwRatioMax (kHetFxRatioMax) or more
 // keeps all its ratios in FP64 (flag byte per edge after the ratios), and every (bin, channel) that reads it
 // takes the FP64 contraction.
 template <bool MIX, bool FX>
@@ -292,6 +395,7 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
   extern __shared__ double2 rsh[];
   unsigned char* wflag = reinterpret_cast<unsigned char*>(rsh + (size_t)hs.nemax * kNModes * 3);
   constexpr bool DW = MIX && !FX;   // the mixed unit at the edges
+  constexpr bool XC = FX && !MIX;   // the fixed-point contraction
   __shared__ __align__(16) double pc[kFxProj];
   __shared__ float2 pcw[DW ? kProj : 1];
   __shared__ double sh[6][kHetThreads / 32];
@@ -339,9 +443,9 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
           const int j = (e * kNModes + md) * 3 + c;
           if (H.src[j] != e) continue;
           o[md][c] = cmul(o[md][c], H.ih0e[j]);
-          if constexpr (MIX) wide |= !(fmax(fabs(o[md][c].x), fabs(o[md][c].y)) < kHetDwRatioMax);
+          if constexpr (MIX || XC) wide |= !(fmax(fabs(o[md][c].x), fabs(o[md][c].y)) < (XC ? kHetFxRatioMax : kHetDwRatioMax));
         }
-      if constexpr (MIX) wflag[e] = wide ? 1 : 0;
+      if constexpr (MIX || XC) wflag[e] = wide ? 1 : 0;
 #pragma unroll
       for (int md = 0; md < kNModes; ++md)
 #pragma unroll
@@ -351,6 +455,8 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
           if (MIX && !wide) {
             const float2 re = to_dw(o[md][c].x), im = to_dw(o[md][c].y);
             reinterpret_cast<float4*>(rsh)[j] = make_float4(re.x, re.y, im.x, im.y);
+          } else if (XC && !wide) {
+            reinterpret_cast<longlong2*>(rsh)[j] = longlong2{fx_from_bits(o[md][c].x, kHetFxBits), fx_from_bits(o[md][c].y, kHetFxBits)};
           } else {
             rsh[j] = o[md][c];
           }
@@ -415,6 +521,29 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
           }
           v[c] += df_to(dh);
           v[3 + c] += df_to(hh);
+        }
+      }
+    } else if constexpr (XC) {
+      const longlong2* rx = reinterpret_cast<const longlong2*>(rsh);
+      for (int b = threadIdx.x; b < H.ne - 1; b += blockDim.x) {
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) {
+          bool wide = false;
+#pragma unroll
+          for (int md = 0; md < kNModes; ++md) {
+            const int s0 = H.src[(b * kNModes + md) * 3 + c], s1 = H.src[((b + 1) * kNModes + md) * 3 + c];
+            wide |= (s0 >= 0 && wflag[s0]) || (s1 >= 0 && wflag[s1]);
+          }
+          double dh, hh;
+          if (wide)
+            het_bin_fp64(H, b, c, [&](int e, int md) {
+              const int j = (e * kNModes + md) * 3 + c;
+              return wflag[e] ? rsh[j] : make_double2(fx_to_double(rx[j].x, -kHetFxBits), fx_to_double(rx[j].y, -kHetFxBits));
+            }, dh, hh);
+          else
+            het_bin_fx(H, b, c, rx, dh, hh);
+          v[c] += dh;
+          v[3 + c] += hh;
         }
       }
     } else
@@ -560,7 +689,10 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   const size_t o_B = a256(o_A + (size_t)nb * 30 * sizeof(double2));
   const size_t o_Aw = a256(o_B + (size_t)nb * pe::kPairs * 9 * sizeof(double2));
   const size_t o_Bw = a256(o_Aw + (size_t)nb * 30 * sizeof(float4));
-  const size_t bytes = o_Bw + (size_t)nb * pe::kPairs * 9 * sizeof(float4);
+  const size_t o_Ax = a256(o_Bw + (size_t)nb * pe::kPairs * 9 * sizeof(float4));
+  const size_t o_Bx = a256(o_Ax + (size_t)nb * 30 * sizeof(longlong2));
+  const size_t o_Ex = a256(o_Bx + (size_t)nb * pe::kPairs * 9 * sizeof(longlong2));
+  const size_t bytes = o_Ex + (size_t)nb * 3 * sizeof(int2);
   pe_hetero_s* h = new (std::nothrow) pe_hetero_s();
   if (!h) return herr(PE_ENOMEM, "pe_hetero_create: host allocation failed");
   cudaGetDevice(&h->device);
@@ -578,6 +710,9 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   double2* d_B = reinterpret_cast<double2*>(base + o_B);
   float4* d_Aw = reinterpret_cast<float4*>(base + o_Aw);
   float4* d_Bw = reinterpret_cast<float4*>(base + o_Bw);
+  longlong2* d_Ax = reinterpret_cast<longlong2*>(base + o_Ax);
+  longlong2* d_Bx = reinterpret_cast<longlong2*>(base + o_Bx);
+  int2* d_Ex = reinterpret_cast<int2*>(base + o_Ex);
   std::vector<int> he(ne);
   std::vector<double> hfe(ne);
   for (int i = 0; i < ne; ++i) {
@@ -636,10 +771,11 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
     pe::k_het_summary<<<(unsigned)((n + 127) / 128), 128>>>(D, d_edge, d_fe, ne, hb, K, d_A, d_B);
     e = pe::launch_status();
   }
-  if (e == cudaSuccess) {   // double-word copies of the summary data for the mixed-precision kernel
+  if (e == cudaSuccess) {   // double-word and fixed-point copies of the summary data
     const long long na = (long long)nb * 30, nbq = (long long)nb * pe::kPairs * 9;
     pe::k_to_dw4<<<(unsigned)((na + 255) / 256), 256>>>(d_A, na, d_Aw);
     pe::k_to_dw4<<<(unsigned)((nbq + 255) / 256), 256>>>(d_B, nbq, d_Bw);
+    pe::k_het_words<<<(3 * nb + 127) / 128, 128>>>(d_fe, ne, d_A, d_B, d_Ax, d_Bx, d_Ex);
     e = pe::launch_status();
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -664,6 +800,9 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   h->dev.Bs = d_B;
   h->dev.Aw = d_Aw;
   h->dev.Bw = d_Bw;
+  h->dev.Ax = d_Ax;
+  h->dev.Bx = d_Bx;
+  h->dev.Ex = d_Ex;
   h->dev.ne = ne;
   h->dev.mask = mode_mask;
   *out = h;
@@ -733,8 +872,8 @@ pe_status pe_hetero_loglike_batch(const pe_hetero* hets, int ndet, const double*
     e = pe::launch_prep(th, B, hets[0]->dev.mask, ds, static_cast<pe::SampleCoef*>(coef), static_cast<int*>(nend),
                         static_cast<int*>(stt), st);
   const bool mix = (hets[0]->dev.mask & PE_PREC_MIXED) != 0u;
-  const size_t smem = (size_t)nemax * pe::kNModes * 3 * sizeof(double2) + (mix ? (size_t)nemax : 0);
   const bool fxu = pe::fx_all_ok(ds);
+  const size_t smem = (size_t)nemax * pe::kNModes * 3 * sizeof(double2) + (mix || fxu ? (size_t)nemax : 0);   // and the flags
   auto kern = mix ? (fxu ? pe::k_het_loglike<true, true> : pe::k_het_loglike<true, false>)
                   : (fxu ? pe::k_het_loglike<false, true> : pe::k_het_loglike<false, false>);
   // equal rounds of edges over the fewest threads (at least 64, which stage the projection forms)

@@ -156,3 +156,30 @@ def test_surrogate_bins_below_the_first_node(Lb):
         r = Lb.loglike([det], th, W.MODE_ALL, dhhh=True)["dhhh"].cpu().numpy()
         scale = 0.5 * det.data_norm().sum() + np.abs(r[..., 0].sum(axis=(1, 2))) + 0.5 * r[..., 1].sum(axis=(1, 2))
         assert np.all(np.isfinite(a)) and np.all(np.abs(a - b) <= 1e-6 * scale), (f0, np.max(np.abs(a - b) / scale))
+
+
+@pytest.mark.parametrize("nbins,mask", [(1, 0x04), (2, W.MODE_ALL), (64, W.MODE_ALL), (300, 0x19)])
+def test_heterodyned_ratios_on_either_side_of_the_bound(oracle_mod, Lb, nbins, mask):
+    """The fixed-point contraction and its FP64 fallback: distances that put every ratio far below, just below, just above and far
+    above 2, with and without shifts in the other parameters, one to 300 coarse bins; on the bar of the
+    heterodyned parity tests, against the oracle on the same edges."""
+    from oracle import hetero as HT
+    T = 2.0 ** 19
+    k0, nb = W.grid(T)
+    th0 = W.theta_injection(T)
+    od = H.oracle_detector(oracle_mod, W.LISA, T, k0, nb, th0, mask, 47)
+    gd = H.library_detector(Lb, od)
+    edges = HT.default_edges(T, k0, nb, th0, mask, nbins)
+    oh = HT.Hetero(od, th0, mask, edges)
+    gh = Lb.Hetero(gd, th0, mask, edges=edges)
+    th = np.tile(th0, (14, 1))
+    th[:, 4] /= np.tile([0.02, 0.9, 1.9, 1.999999, 2.000001, 2.1, 40.0], 2)
+    th[7:, 0] *= 1.00003
+    th[7:, 7] += 0.004
+    th[7:, 10] += 0.7
+    g = Lb.hetero_loglike([gh], th, dhhh=True)
+    for s in range(len(th)):
+        r = oh.loglike(th[s])
+        scale = H.scale_of(r["dh"], r["hh"], r["dd"])
+        assert abs(g["logl"][s] - r["logl"]) <= 1e-10 * scale, (s, abs(g["logl"][s] - r["logl"]) / scale)
+        assert np.all(np.abs(g["dhhh"][s, 0] - np.stack([r["dh"], r["hh"]], -1)) <= 1e-10 * scale)

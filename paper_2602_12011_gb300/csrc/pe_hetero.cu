@@ -259,8 +259,8 @@ __device__ __forceinline__ void het_bin_fp64(const HetDev& H, int b, int c, Ld l
   }
 }
 // Summary data of one (channel c, bin b) for the fixed-point contraction: over ra and d = rb - ra (the slopes' powers of
-// 1/(fe[b+1] - fe[b]) in the data), as multiples of 2^(E - 60) with E (one for A, one for Bs) above twice the sum of the magnitudes that
-// multiply components below 1, packed for multiplication (fx_pack).
+// 1/(fe[b+1] - fe[b]) in the data), as multiples of 2^(E - 60) with E (one for A, one for Bs) above twice the sum of the magnitudes, B's
+// weighted by how often the contraction meets them, packed for multiplication (fx_pack).
 __global__ void k_het_words(const double* fe, int ne, const double2* A, const double2* Bs, longlong2* Ax, longlong2* Bx, int2* Ex) {
   const int nbin = ne - 1, i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * nbin) return;
@@ -286,7 +286,8 @@ __global__ void k_het_words(const double* fe, int ne, const double2* A, const do
     }
   auto word = [](double2 v, double sum, int E) {
     if (sum == 0.0) return longlong2{0, 0};
-    return longlong2{fx_pack(fx_split(fx_from_bits(v.x, 60 - E))), fx_pack(fx_split(fx_from_bits(v.y, 60 - E)))};
+    auto q = [&](double x) { return fx_pack(fx_split((fx_from_bits(x, 61 - E) + 1) >> 1)); };   // rounded
+    return longlong2{q(v.x), q(v.y)};
   };
   const int ea = fx_expo(sa) - 1021, eb = fx_expo(sb) - 1021;
   for (int md = 0; md < kNModes; ++md)
@@ -296,11 +297,11 @@ __global__ void k_het_words(const double* fe, int ne, const double2* A, const do
   Ex[i] = make_int2(ea, eb);
 }
 
-// Ratios that the fixed-point contraction takes: components below 2, held as a quarter in 2^-60. Those of a posterior's bulk are near
+// Ratios that the fixed-point contraction takes: components below 2, held as a half in 2^-60. Those of a posterior's bulk are near
 // 1; an edge with a larger one is kept in FP64, and its bins take het_bin_fp64.
 constexpr double kHetFxRatioMax = 2.0;
-constexpr int kHetFxBits = 58;
-// het_bin_fp64's contraction in fixed point: ratios below 1/2, d below 1, the data's sums below 1/2, so every sum stays below 1. Bound by the
+constexpr int kHetFxBits = 59;
+// het_bin_fp64's contraction in fixed point: ratios below 1, d below 2, the data's weighted sums below 1/2, so every sum stays below 2. Bound by the
 // 32 x 32-bit products, about 900 per (bin, channel) at 16 per SM and clock where the FP64 form issues 340 operations
 // at 1.67 (777 samples, LISA, 2^22 s: 0.68 -> 0.36 ms).
 __device__ __forceinline__ void het_bin_fx(const HetDev& H, int b, int c, const longlong2* __restrict__ rx, double& dh, double& hh) {

@@ -51,7 +51,9 @@ extern "C" {
  * in double-word arithmetic (~48-bit significands, ~1e-14 relative; t_f and the orbit angles in
  * FP64 where t_f lies more than 2^23 s, heliocentric, or 2^21 s, geocentric, from the origin).
  * It agrees with the FP64 path to far below the 1e-10 parity bar but not bit for bit; each
- * precision is bitwise batch-invariant by itself. pe_loglike_grad_batch, pe_hetero_create and
+ * precision is bitwise batch-invariant by itself. Where every detector of a call has pi f L < 4 on its
+ * grid, the likelihood and the gradient of both precisions run the same unit, whose geometry is 64-bit
+ * fixed point (2^-60), and give the same results. pe_loglike_grad_batch, pe_hetero_create and
  * pe_surrogate_loglike_batch also take the flag (see there); pe_fisher and
  * pe_surrogate_mismatch are FP64 only and reject it. */
 #define PE_PREC_MIXED 0x100u
@@ -286,7 +288,7 @@ pe_status pe_surrogate_load(pe_surrogate s, const char* path);
  * forward mode sum (which out_logl and the cotangents come from) then runs in the mixed-precision
  * unit of pe_loglike_batch, and the reverse sweeps keep FP64 for the phase, t_f, the turn
  * reductions, the PN-coefficient chain rule and the sums, with the geometry, link factors and
- * their cotangents in double words. PE_PREC_FP32 gives PE_EINVAL. */
+ * their cotangents in double words (in fixed point, for both precisions, where the detectors allow it). PE_PREC_FP32 gives PE_EINVAL. */
 pe_status pe_loglike_grad_batch(const pe_detector* dets, int ndet, const double* theta, int B, unsigned mode_mask,
                                 double* out_logl, double* out_grad, int32_t* out_status, void* stream);
 
@@ -345,7 +347,7 @@ pe_status pe_fisher_gaussian(const pe_detector* dets, int ndet, const double* th
  *   pe_hetero_create: summary data for detector det (with data set), reference theta0 [11] (host),
  *     mode_mask and edges [nedges] (host, strictly increasing, 2 <= nedges <= 640, within the grid).
  *     mode_mask may carry PE_PREC_MIXED: pe_hetero_loglike_batch then evaluates the signal at the
- *     edges with the mixed-precision unit and the per-bin contraction in double words (the
+ *     edges with the mixed-precision (or fixed-point) unit and the per-bin contraction in double words (the
  *     summary data are built in FP64, the sums across bins stay FP64). An edge where a ratio
  *     h/h0 reaches 2^24 (a reference that has almost vanished, e.g. past its taper) keeps FP64
  *     ratios, and the bins that read it are contracted in FP64. PE_PREC_FP32 gives PE_EINVAL.

@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
       for (int md = 0; md < kNModes; ++md) {
         if (md == 3 && S.pair32) continue;
         const ModeCoef& C = S.md[md];
-        if (Es == 0 || !C.active || !dlt_pos(Bn.f, C.fend)) continue;
+        if (Es == 0 || Es == 0x7ff || !C.active || !dlt_pos(Bn.f, C.fend)) continue;
         const FxTape tp = {tape + tape_slot(md) * kTapeF * kTileBins, pol};
         mode_bwd_fx<kTileBins>(D, S, SG, md, (md == 0 && S.pair32) ? 3 : -1, Bn, fm13, invf, fR, n2pif, a3, &col[0][threadIdx.x], Es, ga, pc,
                                tp);
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kTileBins, kGradFxCtas) k_grad_fwd_fx(DetSet d
       fx_bin_grad(S, SG, ga, g);
       const double out[kGradFxV - 6] = {g.M, g.q, g.c1, g.c2, g.dL, g.io, g.ph, g.tc, g.k[0], g.k[1], g.k[2]};
 #pragma unroll
-      for (int i = 6; i < kGradFxV; ++i) red[i][threadIdx.x] = out[i - 6];
+      for (int i = 6; i < kGradFxV; ++i) red[i][threadIdx.x] = Es == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL) : out[i - 6];   // seeds of inf or NaN data
     } else {
 #pragma unroll
       for (int i = 0; i < kGradFxV; ++i) red[i][threadIdx.x] = 0.0;

@@ -261,6 +261,7 @@ __device__ __forceinline__ void het_bin_fp64(const HetDev& H, int b, int c, Ld l
 // Summary data of one (channel c, bin b) for the fixed-point contraction: over ra and d = rb - ra (the slopes' powers of
 // 1/(fe[b+1] - fe[b]) in the data), as multiples of 2^(E - 60) with E (one for A, one for Bs) above twice the sum of the magnitudes, B's
 // weighted by how often the contraction meets them, packed for multiplication (fx_pack).
+constexpr int kHetNotFinite = 1 << 20;   // E of data that hold an inf or a NaN
 __global__ void k_het_words(const double* fe, int ne, const double2* A, const double2* Bs, longlong2* Ax, longlong2* Bx, int2* Ex) {
   const int nbin = ne - 1, i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * nbin) return;
@@ -294,7 +295,7 @@ __global__ void k_het_words(const double* fe, int ne, const double2* A, const do
     for (int o = 0; o < 2; ++o) Ax[(size_t)row_a(md, o) * nbin + b] = word(at(A, row_a(md, o), o), sa, ea);
   for (int pr = 0; pr < kPairs; ++pr)
     for (int o = 0; o < 3; ++o) Bx[(size_t)row_b(pr, o) * nbin + b] = word(at(Bs, row_b(pr, o), o), sb, eb);
-  Ex[i] = make_int2(ea, eb);
+  Ex[i] = make_int2(isfinite(sa) ? ea : kHetNotFinite, isfinite(sb) ? eb : kHetNotFinite);
 }
 
 // Ratios that the fixed-point contraction takes: components below 2, held as a half in 2^-60. Those of a posterior's bulk are near
@@ -356,6 +357,8 @@ __device__ __forceinline__ void het_bin_fx(const HetDev& H, int b, int c, const 
   const int2 E = H.Ex[c * nbin + b];
   dh = fx_to_double(sd, E.x - 60 + (60 - kHetFxBits));
   hh = fx_to_double(sh, E.y - 60 + 2 * (60 - kHetFxBits));
+  if (E.x == kHetNotFinite) dh = __longlong_as_double(0x7ff8000000000000LL);
+  if (E.y == kHetNotFinite) hh = __longlong_as_double(0x7ff8000000000000LL);
 }
 
 // Re(a b) and Re(a conj(b)) in double words

@@ -183,3 +183,30 @@ def test_heterodyned_ratios_on_either_side_of_the_bound(oracle_mod, Lb, nbins, m
         scale = H.scale_of(r["dh"], r["hh"], r["dd"])
         assert abs(g["logl"][s] - r["logl"]) <= 1e-10 * scale, (s, abs(g["logl"][s] - r["logl"]) / scale)
         assert np.all(np.abs(g["dhhh"][s, 0] - np.stack([r["dh"], r["hh"]], -1)) <= 1e-10 * scale)
+
+
+def test_a_bin_without_a_finite_datum(Lb):
+    """One NaN among the data: the likelihood, every gradient component and the heterodyned sums of its channel are NaN for the
+    samples that reach the bin, as in floating point, and the others' values do not change."""
+    T = 2.0 ** 17
+    k0, nb = W.grid(T)
+    th = W.draw_prior(2, 3, T)
+    th[:, 0] = [3e6, 3e5]      # the first ends below 1.5e-3 Hz * 4/2, the second well above
+    rng = np.random.default_rng(5)
+    d = 1e-21 * (rng.standard_normal((3, nb)) + 1j * rng.standard_normal((3, nb)))
+    psd = np.full((3, nb), 1e-38)
+    bad = int(0.01 * T) - k0
+    out = []
+    for value in (d[1, bad], np.nan):
+        d[1, bad] = value
+        det = Lb.Detector(W.LISA, T, k0, nb)
+        det.set_data(d, psd)
+        het = Lb.Hetero(det, th[1], W.MODE_ALL, nbins_coarse=32)
+        out.append((Lb.loglike([det], th, W.MODE_ALL, dhhh=True)["dhhh"], Lb.loglike_grad([det], th, W.MODE_ALL)["grad"],
+                    Lb.hetero_loglike([het], th[1:], dhhh=True)["dhhh"]))
+    (l0, g0, h0), (l1, g1, h1) = out
+    np.testing.assert_array_equal(l1[0], l0[0])
+    np.testing.assert_array_equal(g1[0], g0[0])
+    assert np.isnan(l1[1, 0, 1, 0]) and np.all(np.isnan(g1[1])) and np.isnan(h1[0, 0, 1, 0])
+    np.testing.assert_array_equal(l1[1, 0, [0, 2]], l0[1, 0, [0, 2]])
+    np.testing.assert_array_equal(h1[0, 0, [0, 2]], h0[0, 0, [0, 2]])

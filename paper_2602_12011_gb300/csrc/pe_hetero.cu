@@ -45,7 +45,7 @@ struct HetDev {
   const int* src;        // [ne][5][3] edge whose ratio applies (carry-forward), -1 for none
   const double2* A;      // [5][3][2][ne-1]: consecutive bins are consecutive, for the contraction's loads
   const double2* Bs;     // [kPairs][3][3][ne-1]
-  const float4* Aw;      // A and Bs as double words (re hi, re lo, im hi, im lo), for the mixed kernel
+  const float4* Aw;      // A and Bs over the edges' ratios, in double words, for the mixed kernel (k_het_dw)
   const float4* Bw;
   const longlong2* Ax;   // A and Bs for the fixed-point contraction (k_het_words): packed words of re, im
   const longlong2* Bx;
@@ -202,12 +202,32 @@ __global__ void k_het_summary(DetDev D, const int* edge, const double* fe, int n
   }
 }
 
-// double2 -> double-word complex (re hi, re lo, im hi, im lo)
-__global__ void k_to_dw4(const double2* in, long long n, float4* out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float2 re = to_dw(in[i].x), im = to_dw(in[i].y);
-  out[i] = make_float4(re.x, re.y, im.x, im.y);
+// Summary data of one (channel c, bin b) for the mixed contraction, over the ratios at the bin's two edges: with slopes
+// (rb - ra) / (fe[b+1] - fe[b]) the moments A0, A1 become A_a = A0 - A1', A_b = A1' and B0, B1, B2 become
+// B_aa = B0 - 2 B1' + B2', B_ab = B1' - B2', B_bb = B2' (primes: over the width's powers), as double words (re hi, re lo, im hi, im lo).
+__global__ void k_het_dw(const double* fe, int ne, const double2* A, const double2* Bs, float4* Aw, float4* Bw) {
+  const int nbin = ne - 1, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 3 * nbin) return;
+  const int c = i / nbin, b = i % nbin;
+  const double idf = 1.0 / (fe[b + 1] - fe[b]);
+  auto put = [](float4* o, double x, double y) {
+    const float2 re = to_dw(x), im = to_dw(y);
+    *o = make_float4(re.x, re.y, im.x, im.y);
+  };
+  for (int md = 0; md < kNModes; ++md) {
+    const size_t r = (size_t)(md * 3 + c) * 2 * nbin + b;
+    const double2 a0 = A[r], a1 = make_double2(A[r + nbin].x * idf, A[r + nbin].y * idf);
+    put(Aw + r, a0.x - a1.x, a0.y - a1.y);
+    put(Aw + r + nbin, a1.x, a1.y);
+  }
+  for (int pr = 0; pr < kPairs; ++pr) {
+    const size_t r = (size_t)(pr * 3 + c) * 3 * nbin + b;
+    const double2 b0 = Bs[r], b1 = make_double2(Bs[r + nbin].x * idf, Bs[r + nbin].y * idf);
+    const double2 b2 = make_double2(Bs[r + 2 * nbin].x * idf * idf, Bs[r + 2 * nbin].y * idf * idf);
+    put(Bw + r, (b0.x - b1.x) - (b1.x - b2.x), (b0.y - b1.y) - (b1.y - b2.y));
+    put(Bw + r + nbin, b1.x - b2.x, b1.y - b2.y);
+    put(Bw + r + 2 * nbin, b2.x, b2.y);
+  }
 }
 
 __device__ __forceinline__ cdf unpack4(float4 q) { return cdf{df_make(q.x, q.y), df_make(q.z, q.w)}; }
@@ -469,24 +489,23 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
     __syncthreads();
     double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     if constexpr (MIX) {
+      // double words over the ratios at both edges, in rolled loops that read the ratios from shared memory: unrolled over the pairs
+      // the code overran the instruction cache (3.79 -> 3.76 ms, 4096 samples on two detectors)
       const float4* rw = reinterpret_cast<const float4*>(rsh);
       const cdf zc = {df_make(0.f, 0.f), df_make(0.f, 0.f)};
-      for (int b = threadIdx.x; b < H.ne - 1; b += blockDim.x) {
-        const df idf = to_dw(1.0 / (H.fe[b + 1] - H.fe[b]));
+      const int nbin = H.ne - 1;
+      for (int b = threadIdx.x; b < nbin; b += blockDim.x) {
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) {
-          cdf r0[kNModes], r1[kNModes];
+          const int* sa = H.src + (size_t)b * kNModes * 3 + c;          // edge of mode md's ratio at sa[3 md], and at the
+          const int* sb = sa + kNModes * 3;                             // bin's other edge
           bool wide = false;
 #pragma unroll
           for (int md = 0; md < kNModes; ++md) {
-            const int s0 = H.src[(b * kNModes + md) * 3 + c], s1 = H.src[((b + 1) * kNModes + md) * 3 + c];
+            const int s0 = sa[3 * md], s1 = sb[3 * md];
             wide |= (s0 >= 0 && wflag[s0]) || (s1 >= 0 && wflag[s1]);
-            const cdf ra = s0 >= 0 ? unpack4(rw[(s0 * kNModes + md) * 3 + c]) : zc;
-            const cdf rb = s1 >= 0 ? unpack4(rw[(s1 * kNModes + md) * 3 + c]) : zc;
-            r0[md] = ra;
-            r1[md] = cdf{dfl_mul(dfl_sub(rb.re, ra.re), idf), dfl_mul(dfl_sub(rb.im, ra.im), idf)};
           }
-          if (wide) {   // an edge of this bin keeps FP64 ratios (the double words above are unused)
+          if (wide) {   // an edge of this bin keeps FP64 ratios
             auto ld = [&](int e, int md) -> double2 {
               const int j = (e * kNModes + md) * 3 + c;
               if (wflag[e]) return rsh[j];
@@ -499,29 +518,28 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
             v[3 + c] += hh;
             continue;
           }
-          // as het_bin_fp64, in double words
-          const int nbin = H.ne - 1;
+          auto ratio = [&](int e, int md) { return e >= 0 ? unpack4(rw[(e * kNModes + md) * 3 + c]) : zc; };
           df dh = df_make(0.f, 0.f), hh = df_make(0.f, 0.f);
-#pragma unroll
+#pragma unroll 1
           for (int md = 0; md < kNModes; ++md) {
+            const cdf ra = ratio(sa[3 * md], md), rb = ratio(sb[3 * md], md);
             const float4* a = H.Aw + (size_t)(md * 3 + c) * 2 * nbin + b;
-            dh = dfl_add(dh, dfl_add(re_mul(unpack4(a[0]), r0[md]), re_mul(unpack4(a[nbin]), r1[md])));
+            dh = dfl_add(dh, dfl_add(re_mul(unpack4(a[0]), ra), re_mul(unpack4(a[nbin]), rb)));
             cdf y = zc, w = zc;
-#pragma unroll
-            for (int k = 1; k <= kNModes; ++k) {
-              const int m2 = k < kNModes ? (md + k) : md;
-              if (m2 >= kNModes) continue;
-              if (k == kNModes) {
+#pragma unroll 1
+            for (int m2 = kNModes - 1; m2 >= md; --m2) {   // the off-diagonal pairs first, doubled, then the diagonal one
+              if (m2 == md) {
                 y = cdf{df_scale2(y.re, 2.f), df_scale2(y.im, 2.f)};
                 w = cdf{df_scale2(w.re, 2.f), df_scale2(w.im, 2.f)};
               }
+              const cdf la = ratio(sa[3 * m2], m2), lb = ratio(sb[3 * m2], m2);
               const float4* q = H.Bw + (size_t)(pair_index(md, m2) * 3 + c) * 3 * nbin + b;
               const cdf q0 = unpack4(q[0]), q1 = unpack4(q[nbin]), q2 = unpack4(q[2 * nbin]);
-              const cdf a0 = mul_conj(q0, r0[m2]), a1 = mul_conj(q1, r1[m2]), b0 = mul_conj(q1, r0[m2]), b1 = mul_conj(q2, r1[m2]);
+              const cdf a0 = mul_conj(q0, la), a1 = mul_conj(q1, lb), b0 = mul_conj(q1, la), b1 = mul_conj(q2, lb);
               y = cdf{dfl_add(y.re, dfl_add(a0.re, a1.re)), dfl_add(y.im, dfl_add(a0.im, a1.im))};
               w = cdf{dfl_add(w.re, dfl_add(b0.re, b1.re)), dfl_add(w.im, dfl_add(b0.im, b1.im))};
             }
-            hh = dfl_add(hh, dfl_add(re_mul(r0[md], y), re_mul(r1[md], w)));
+            hh = dfl_add(hh, dfl_add(re_mul(ra, y), re_mul(rb, w)));
           }
           v[c] += df_to(dh);
           v[3 + c] += df_to(hh);
@@ -776,9 +794,7 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
     e = pe::launch_status();
   }
   if (e == cudaSuccess) {   // double-word and fixed-point copies of the summary data
-    const long long na = (long long)nb * 30, nbq = (long long)nb * pe::kPairs * 9;
-    pe::k_to_dw4<<<(unsigned)((na + 255) / 256), 256>>>(d_A, na, d_Aw);
-    pe::k_to_dw4<<<(unsigned)((nbq + 255) / 256), 256>>>(d_B, nbq, d_Bw);
+    pe::k_het_dw<<<(3 * nb + 127) / 128, 128>>>(d_fe, ne, d_A, d_B, d_Aw, d_Bw);
     pe::k_het_words<<<(3 * nb + 127) / 128, 128>>>(d_fe, ne, d_A, d_B, d_Ax, d_Bx, d_Ex);
     e = pe::launch_status();
   }

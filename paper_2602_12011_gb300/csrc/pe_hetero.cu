@@ -49,7 +49,7 @@ struct HetDev {
   const float4* Bw;
   const longlong2* Ax;   // A and Bs for the fixed-point contraction (k_het_words): packed words of re, im
   const longlong2* Bx;
-  const int2* Ex;        // [3][ne-1] their exponents
+  const int* Gx;         // [6][3][ne-1] their exponents
   int ne;
   unsigned mask;
 };
@@ -278,11 +278,17 @@ __device__ __forceinline__ void het_bin_fp64(const HetDev& H, int b, int c, Ld l
     hh = fma(r0[md].x, y.x, fma(-r0[md].y, y.y, fma(r1[md].x, w.x, fma(-r1[md].y, w.y, hh))));
   }
 }
-// Summary data of one (channel c, bin b) for the fixed-point contraction: over ra and d = rb - ra (the slopes' powers of
-// 1/(fe[b+1] - fe[b]) in the data), as multiples of 2^(E - 60) with E (one for A, one for Bs) above twice the sum of the magnitudes, B's
-// weighted by how often the contraction meets them, packed for multiplication (fx_pack).
-constexpr int kHetNotFinite = 1 << 20;   // E of data that hold an inf or a NaN
-__global__ void k_het_words(const double* fe, int ne, const double2* A, const double2* Bs, longlong2* Ax, longlong2* Bx, int2* Ex) {
+// Summary data of one (channel c, bin b) for the fixed-point contraction (het_bin_fx), over ra and d = rb - ra (the slopes'
+// powers of 1/(fe[b+1] - fe[b]) in the data). Every mode is scaled by 2^-g, the least power of two above its
+// sqrt(B0_ii), the norm of its reference signal in the bin; with that the entries of Bs are below 1 (Cauchy-Schwarz) and are
+// words in 2^-60, and those of A are below 2^a, words in 2^(a - 60); packed for multiplication (fx_pack). Gx: rows 0..4
+// the g, row 5 a. A bin whose data the words cannot hold (an inf or NaN, a norm outside 2^+-400, entries of a
+// mode without a norm) has a = kHetGeneral and is contracted in FP64.
+constexpr int kHetGeneral = 1 << 20;
+constexpr int kHetNoMode = -(1 << 20);   // g of a mode without signal in the bin
+constexpr int kHetExpo = 450;            // bound of the exponents a and N (het_bin_fx)
+constexpr int kHetLeast = 50;            // least hh of the fixed-point form, 2^kHetLeast in 2^-60
+__global__ void k_het_words(const double* fe, int ne, const double2* A, const double2* Bs, longlong2* Ax, longlong2* Bx, int* Gx) {
   const int nbin = ne - 1, i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 3 * nbin) return;
   const int c = i / nbin, b = i % nbin;
@@ -294,49 +300,92 @@ __global__ void k_het_words(const double* fe, int ne, const double2* A, const do
   };
   auto row_a = [&](int md, int o) { return (md * 3 + c) * 2 + o; };
   auto row_b = [&](int pr, int o) { return (pr * 3 + c) * 3 + o; };
-  double sa = 0.0, sb = 0.0;
-  for (int md = 0; md < kNModes; ++md)
+  auto mag = [](double2 v) { return fabs(v.x) > fabs(v.y) || isnan(v.x) ? fabs(v.x) : fabs(v.y); };   // NaN if either is one
+  int g[kNModes], a = -kHetGeneral;
+  bool ok = true;
+  for (int md = 0; md < kNModes; ++md) {
+    const double n2 = at(Bs, row_b(pair_index(md, md), 0), 0).x;
+    const bool some = n2 > 0x1p-800 && n2 < 0x1p800;
+    g[md] = some ? (fx_expo(n2) - 1021) >> 1 : kHetNoMode;     // n2 < 2^(2 g), and >= 2^(2 g - 2)
     for (int o = 0; o < 2; ++o) {
-      const double2 v = at(A, row_a(md, o), o);
-      sa += fabs(v.x) + fabs(v.y);
+      const double m = mag(at(A, row_a(md, o), o));
+      if (some && m > 0.0) a = max(a, fx_expo(m) - 1022 - g[md]);
+      ok &= some ? m < 0x1p800 : m == 0.0;
     }
-  for (int pr = 0; pr < kPairs; ++pr)
-    for (int o = 0; o < 3; ++o) {
-      const double2 v = at(Bs, row_b(pr, o), o);
-      sb += (o == 1 ? 4.0 : 2.0) * (fabs(v.x) + fabs(v.y));
-    }
-  auto word = [](double2 v, double sum, int E) {
-    if (sum == 0.0) return longlong2{0, 0};
-    auto q = [&](double x) { return fx_pack(fx_split((fx_from_bits(x, 61 - E) + 1) >> 1)); };   // rounded
+  }
+  if (a == -kHetGeneral) a = 0;
+  ok &= a > -kHetExpo && a < kHetExpo;
+  auto word = [](double2 v, int e) {   // v 2^-e, rounded
+    auto q = [&](double x) { return fx_pack(fx_split((fx_from_bits(scalbn(x, -e), 61) + 1) >> 1)); };
     return longlong2{q(v.x), q(v.y)};
   };
-  const int ea = fx_expo(sa) - 1021, eb = fx_expo(sb) - 1021;
-  for (int md = 0; md < kNModes; ++md)
-    for (int o = 0; o < 2; ++o) Ax[(size_t)row_a(md, o) * nbin + b] = word(at(A, row_a(md, o), o), sa, ea);
-  for (int pr = 0; pr < kPairs; ++pr)
-    for (int o = 0; o < 3; ++o) Bx[(size_t)row_b(pr, o) * nbin + b] = word(at(Bs, row_b(pr, o), o), sb, eb);
-  Ex[i] = make_int2(isfinite(sa) ? ea : kHetNotFinite, isfinite(sb) ? eb : kHetNotFinite);
+  for (int m1 = 0; m1 < kNModes; ++m1)
+    for (int m2 = m1; m2 < kNModes; ++m2)
+      for (int o = 0; o < 3; ++o) {
+        const int r = row_b(pair_index(m1, m2), o);
+        const double2 v = at(Bs, r, o);
+        const bool some = g[m1] != kHetNoMode && g[m2] != kHetNoMode;
+        const int e = some ? g[m1] + g[m2] : 0;
+        const bool in = some ? mag(v) <= scalbn(1.0625, e) : mag(v) == 0.0;
+        ok &= in;
+        Bx[(size_t)r * nbin + b] = in ? word(v, e) : longlong2{0, 0};
+      }
+  for (int md = 0; md < kNModes; ++md) {
+    for (int o = 0; o < 2; ++o)
+      Ax[(size_t)row_a(md, o) * nbin + b] = ok && g[md] != kHetNoMode ? word(at(A, row_a(md, o), o), g[md] + a) : longlong2{0, 0};
+    Gx[(size_t)(md * 3 + c) * nbin + b] = g[md];
+  }
+  Gx[(size_t)(kNModes * 3 + c) * nbin + b] = ok ? a : kHetGeneral;
 }
 
-// Ratios that the fixed-point contraction takes: components below 2, held as a half in 2^-60. Those of a posterior's bulk are near
-// 1; an edge with a larger one is kept in FP64, and its bins take het_bin_fp64.
-constexpr double kHetFxRatioMax = 2.0;
-constexpr int kHetFxBits = 59;
-// het_bin_fp64's contraction in fixed point: ratios below 1, d below 2, the data's weighted sums below 1/2, so every sum stays below 2. Bound by the
-// 32 x 32-bit products, about 900 per (bin, channel) at 16 per SM and clock where the FP64 form issues 340 operations
-// at 1.67 (777 samples, LISA, 2^22 s: 0.68 -> 0.36 ms).
-__device__ __forceinline__ void het_bin_fx(const HetDev& H, int b, int c, const longlong2* __restrict__ rx, double& dh, double& hh) {
+// het_bin_fp64's contraction in fixed point, block floating per (bin, channel): with m_i the largest component of mode i's
+// ratios at the two edges, every ratio is held in 2^-60 of 2^(N - g_i), N the least power of two for which sum m_i 2^(g_i - N)
+// is below 1/2. What is lost is then below 2^-59 of the sample's own signal in the bin, whatever its distance
+// and however the modes' ratios differ (FP64 keeps 2^-53 of each ratio), and powers of two in the signal pass through exactly.
+// Bounds: d is below 1, y and w below sqrt(2) (Cauchy-Schwarz over the bin's fine bins), hh below 1/2 and, where the ratios' size is
+// the signal's, above 2^-8. False where the bin takes the FP64 form: a ratio that is not finite, exponents outside the words', or hh below
+// 2^-10 (an edge where the reference has almost vanished has ratios far above the signal in the bin, or the modes cancel).
+// Bound by the 32 x 32-bit products, about 900 per (bin, channel) at 16 per SM and clock where the FP64 form issues 340 operations
+// at 1.67 (777 samples, LISA, 2^22 s, whole call: 677 us with the FP64 form, 381 us; 363 us with the ratios held in 2^-59 of 1, which lost
+// the faint samples' bits and sent ratios above 2 to the FP64 form).
+__device__ __forceinline__ bool het_bin_fx(const HetDev& H, int b, int c, const double2* __restrict__ ratio, double& dh, double& hh) {
   const int nbin = H.ne - 1;
+  const int ea = H.Gx[(size_t)(kNModes * 3 + c) * nbin + b];
+  if (ea == kHetGeneral) return false;
+  const int *sa = H.src + (size_t)b * kNModes * 3 + c, *sb = sa + kNModes * 3;
+  auto at = [&](int e, int md) { return e >= 0 ? ratio[(e * kNModes + md) * 3 + c] : make_double2(0.0, 0.0); };
+  unsigned m[kNModes];
+  int g[kNModes], top = 2 * kHetNoMode;
+  unsigned most = 0;
+#pragma unroll
+  for (int md = 0; md < kNModes; ++md) {
+    const double2 ra = at(sa[3 * md], md), rb = at(sb[3 * md], md);
+    auto hi = [](double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
+    m[md] = max(max(hi(ra.x), hi(ra.y)), max(hi(rb.x), hi(rb.y)));
+    g[md] = H.Gx[(size_t)(md * 3 + c) * nbin + b];
+    most = max(most, m[md]);
+    if (m[md] >= 0x100000u) top = max(top, (int)(m[md] >> 20) + g[md]);
+  }
+  dh = 0.0;
+  hh = 0.0;
+  if (most < 0x100000u) return true;      // no ratio (or none above 2^-1022)
+  if (most >= 0x7ff00000u) return false;
+  unsigned sum = 0;                       // above sum m_i 2^g_i, in 2^(top - 1043)
+#pragma unroll
+  for (int md = 0; md < kNModes; ++md)
+    if (m[md] >= 0x100000u) sum += (((m[md] & 0xfffffu) | 0x100000u) >> min(top - (int)(m[md] >> 20) - g[md], 31)) + 1;
+  const int N = top - 1043 + (32 - __clz(sum)) + 1;
+  if (N < -kHetExpo || N > kHetExpo) return false;
   fxs rr[kNModes], ri[kNModes], dr[kNModes], di[kNModes];
 #pragma unroll
   for (int md = 0; md < kNModes; ++md) {
-    const int s0 = H.src[(b * kNModes + md) * 3 + c], s1 = H.src[((b + 1) * kNModes + md) * 3 + c];
-    const longlong2 ra = s0 >= 0 ? rx[(s0 * kNModes + md) * 3 + c] : longlong2{0, 0};
-    const longlong2 rb = s1 >= 0 ? rx[(s1 * kNModes + md) * 3 + c] : longlong2{0, 0};
-    rr[md] = fx_split(ra.x);
-    ri[md] = fx_split(ra.y);
-    dr[md] = fx_split(rb.x - ra.x);
-    di[md] = fx_split(rb.y - ra.y);
+    const double2 ra = at(sa[3 * md], md), rb = at(sb[3 * md], md);
+    const int k = 60 + g[md] - N;
+    const fx ax = fx_from_bits(ra.x, k), ay = fx_from_bits(ra.y, k);
+    rr[md] = fx_split(ax);
+    ri[md] = fx_split(ay);
+    dr[md] = fx_split(fx_from_bits(rb.x, k) - ax);
+    di[md] = fx_split(fx_from_bits(rb.y, k) - ay);
   }
   fx sd = 0, sh = 0;
 #pragma unroll
@@ -374,11 +423,10 @@ __device__ __forceinline__ void het_bin_fx(const HetDev& H, int b, int c, const 
     }
     sh += fx_msub(rr[md], fx_split(yx), ri[md], fx_split(yy)) + fx_msub(dr[md], fx_split(wx), di[md], fx_split(wy));
   }
-  const int2 E = H.Ex[c * nbin + b];
-  dh = fx_to_double(sd, E.x - 60 + (60 - kHetFxBits));
-  hh = fx_to_double(sh, E.y - 60 + 2 * (60 - kHetFxBits));
-  if (E.x == kHetNotFinite) dh = __longlong_as_double(0x7ff8000000000000LL);
-  if (E.y == kHetNotFinite) hh = __longlong_as_double(0x7ff8000000000000LL);
+  if (sh < (1LL << kHetLeast)) return false;
+  dh = fx_to_double(sd, ea + N - 60);
+  hh = fx_to_double(sh, 2 * N - 60);
+  return true;
 }
 
 // Re(a b) and Re(a conj(b)) in double words
@@ -409,10 +457,10 @@ __device__ __forceinline__ void het_block_sum(double v[6], double (*sh)[kHetThre
 // and three rounds of edges, the last a third full (777 samples, LISA: 1.09 ms).
 // The signal at the edges comes from the fixed-point unit (FX; both precisions), or the precision's own where a detector
 // does not take that unit. MIX: the ratios are kept as double words and contracted in double words (Aw, Bw);
-// the sums across bins and the block reduction stay FP64. FP64 on the fixed-point unit: the ratios are kept and contracted in fixed
-// point (het_bin_fx). An edge with a ratio of kHetDwRatioMax (kHetFxRatioMax) or more
+// the sums across bins and the block reduction stay FP64. An edge with a ratio of kHetDwRatioMax or more
 // keeps all its ratios in FP64 (flag byte per edge after the ratios), and every (bin, channel) that reads it
-// takes the FP64 contraction.
+// takes the FP64 contraction. FP64 on the fixed-point unit: the ratios stay FP64, and the contraction holds them in
+// fixed point relative to the bin's largest (het_bin_fx).
 template <bool MIX, bool FX>
 __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B, const SampleCoef* __restrict__ coef,
                                                                double* logl, double* dhhh) {
@@ -467,9 +515,9 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
           const int j = (e * kNModes + md) * 3 + c;
           if (H.src[j] != e) continue;
           o[md][c] = cmul(o[md][c], H.ih0e[j]);
-          if constexpr (MIX || XC) wide |= !(fmax(fabs(o[md][c].x), fabs(o[md][c].y)) < (XC ? kHetFxRatioMax : kHetDwRatioMax));
+          if constexpr (MIX) wide |= !(fmax(fabs(o[md][c].x), fabs(o[md][c].y)) < kHetDwRatioMax);
         }
-      if constexpr (MIX || XC) wflag[e] = wide ? 1 : 0;
+      if constexpr (MIX) wflag[e] = wide ? 1 : 0;
 #pragma unroll
       for (int md = 0; md < kNModes; ++md)
 #pragma unroll
@@ -479,8 +527,6 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
           if (MIX && !wide) {
             const float2 re = to_dw(o[md][c].x), im = to_dw(o[md][c].y);
             reinterpret_cast<float4*>(rsh)[j] = make_float4(re.x, re.y, im.x, im.y);
-          } else if (XC && !wide) {
-            reinterpret_cast<longlong2*>(rsh)[j] = longlong2{fx_from_bits(o[md][c].x, kHetFxBits), fx_from_bits(o[md][c].y, kHetFxBits)};
           } else {
             rsh[j] = o[md][c];
           }
@@ -545,37 +591,16 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
           v[3 + c] += df_to(hh);
         }
       }
-    } else if constexpr (XC) {
-      const longlong2* rx = reinterpret_cast<const longlong2*>(rsh);
+    } else {
       for (int b = threadIdx.x; b < H.ne - 1; b += blockDim.x) {
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) {
-          bool wide = false;
-#pragma unroll
-          for (int md = 0; md < kNModes; ++md) {
-            const int s0 = H.src[(b * kNModes + md) * 3 + c], s1 = H.src[((b + 1) * kNModes + md) * 3 + c];
-            wide |= (s0 >= 0 && wflag[s0]) || (s1 >= 0 && wflag[s1]);
-          }
           double dh, hh;
-          if (wide)
-            het_bin_fp64(H, b, c, [&](int e, int md) {
-              const int j = (e * kNModes + md) * 3 + c;
-              return wflag[e] ? rsh[j] : make_double2(fx_to_double(rx[j].x, -kHetFxBits), fx_to_double(rx[j].y, -kHetFxBits));
-            }, dh, hh);
-          else
-            het_bin_fx(H, b, c, rx, dh, hh);
+          if (!XC || !het_bin_fx(H, b, c, rsh, dh, hh))
+            het_bin_fp64(H, b, c, [&](int e, int md) { return rsh[(e * kNModes + md) * 3 + c]; }, dh, hh);
           v[c] += dh;
           v[3 + c] += hh;
         }
-      }
-    } else
-    for (int b = threadIdx.x; b < H.ne - 1; b += blockDim.x) {
-#pragma unroll 1
-      for (int c = 0; c < 3; ++c) {
-        double dh, hh;
-        het_bin_fp64(H, b, c, [&](int e, int md) { return rsh[(e * kNModes + md) * 3 + c]; }, dh, hh);
-        v[c] += dh;
-        v[3 + c] += hh;
       }
     }
     het_block_sum(v, sh);
@@ -713,8 +738,8 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   const size_t o_Bw = a256(o_Aw + (size_t)nb * 30 * sizeof(float4));
   const size_t o_Ax = a256(o_Bw + (size_t)nb * pe::kPairs * 9 * sizeof(float4));
   const size_t o_Bx = a256(o_Ax + (size_t)nb * 30 * sizeof(longlong2));
-  const size_t o_Ex = a256(o_Bx + (size_t)nb * pe::kPairs * 9 * sizeof(longlong2));
-  const size_t bytes = o_Ex + (size_t)nb * 3 * sizeof(int2);
+  const size_t o_Gx = a256(o_Bx + (size_t)nb * pe::kPairs * 9 * sizeof(longlong2));
+  const size_t bytes = o_Gx + (size_t)nb * 3 * (pe::kNModes + 1) * sizeof(int);
   pe_hetero_s* h = new (std::nothrow) pe_hetero_s();
   if (!h) return herr(PE_ENOMEM, "pe_hetero_create: host allocation failed");
   cudaGetDevice(&h->device);
@@ -734,7 +759,7 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   float4* d_Bw = reinterpret_cast<float4*>(base + o_Bw);
   longlong2* d_Ax = reinterpret_cast<longlong2*>(base + o_Ax);
   longlong2* d_Bx = reinterpret_cast<longlong2*>(base + o_Bx);
-  int2* d_Ex = reinterpret_cast<int2*>(base + o_Ex);
+  int* d_Gx = reinterpret_cast<int*>(base + o_Gx);
   std::vector<int> he(ne);
   std::vector<double> hfe(ne);
   for (int i = 0; i < ne; ++i) {
@@ -795,7 +820,7 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   }
   if (e == cudaSuccess) {   // double-word and fixed-point copies of the summary data
     pe::k_het_dw<<<(3 * nb + 127) / 128, 128>>>(d_fe, ne, d_A, d_B, d_Aw, d_Bw);
-    pe::k_het_words<<<(3 * nb + 127) / 128, 128>>>(d_fe, ne, d_A, d_B, d_Ax, d_Bx, d_Ex);
+    pe::k_het_words<<<(3 * nb + 127) / 128, 128>>>(d_fe, ne, d_A, d_B, d_Ax, d_Bx, d_Gx);
     e = pe::launch_status();
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -822,7 +847,7 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   h->dev.Bw = d_Bw;
   h->dev.Ax = d_Ax;
   h->dev.Bx = d_Bx;
-  h->dev.Ex = d_Ex;
+  h->dev.Gx = d_Gx;
   h->dev.ne = ne;
   h->dev.mask = mode_mask;
   *out = h;
@@ -893,7 +918,7 @@ pe_status pe_hetero_loglike_batch(const pe_hetero* hets, int ndet, const double*
                         static_cast<int*>(stt), st);
   const bool mix = (hets[0]->dev.mask & PE_PREC_MIXED) != 0u;
   const bool fxu = pe::fx_all_ok(ds);
-  const size_t smem = (size_t)nemax * pe::kNModes * 3 * sizeof(double2) + (mix || fxu ? (size_t)nemax : 0);   // and the flags
+  const size_t smem = (size_t)nemax * pe::kNModes * 3 * sizeof(double2) + (mix ? (size_t)nemax : 0);   // and the flags
   auto kern = mix ? (fxu ? pe::k_het_loglike<true, true> : pe::k_het_loglike<true, false>)
                   : (fxu ? pe::k_het_loglike<false, true> : pe::k_het_loglike<false, false>);
   // equal rounds of edges over the fewest threads (at least 64, which stage the projection forms)

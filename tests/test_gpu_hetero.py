@@ -145,3 +145,32 @@ def test_hetero_errors(Lb):
     with pytest.raises(Lb.PeError) as e:
         Lb.hetero_loglike([a, b], th0[None, :])
     assert e.value.status == Lb.PE_EINVAL
+
+
+def _edges_and_samples(Lb, T, nbins):
+    k0, nb = W.grid(T)
+    th0 = np.array([8e5, 2.0, 0.4, -0.2, 20.0, 0.6, 0.9, 2.0, 0.4, 1.1, 0.5 * 2.0 ** 16])
+    d = Lb.Detector(W.LISA, T, k0, nb)
+    d.inject(th0, W.MODE_ALL, W.normals(nb, 3))
+    th = _near(th0, 12, 11, 0.3)
+    th[6:, 5] += 0.7                 # another inclination: the odd modes' ratios differ from the (2,2) mode's
+    th[9:, 1] = 1.02
+    return d, th0, th, Lb.pe_hetero_default_edges(T, k0, nb, th0, W.MODE_ALL, nbins)
+
+
+@pytest.mark.parametrize("nbins", [1, 40, 300])
+def test_hetero_sums_scale_with_the_distance_exactly(Lb, nbins):
+    """The signal is proportional to 1 / d_L, and a power of two is exact in floating point: at 2^k times the distance
+    <d|h> is 2^-k and <h|h> 4^-k of its value, bit for bit, from samples much louder than the reference
+    to much fainter ones. (A ratio held to a fixed absolute step loses bits with every k.)"""
+    d, th0, th, edges = _edges_and_samples(Lb, 2.0 ** 18, nbins)
+    het = Lb.Hetero(d, th0, W.MODE_ALL, edges=edges)
+    ref = Lb.hetero_loglike([het], th, dhhh=True)["dhhh"][:, 0]
+    assert np.all(ref[..., 1] > 0.0)
+    for k in (-8, -3, -1, 1, 2, 6, 11):
+        tk = th.copy()
+        tk[:, 4] *= 2.0 ** k
+        g = Lb.hetero_loglike([het], tk, dhhh=True)["dhhh"][:, 0]
+        np.testing.assert_array_equal(g[..., 0] * 2.0 ** k, ref[..., 0])
+        np.testing.assert_array_equal(g[..., 1] * 4.0 ** k, ref[..., 1])
+    het.close()

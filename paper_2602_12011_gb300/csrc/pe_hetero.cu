@@ -31,6 +31,12 @@ namespace pe {
 
 constexpr int kHetMaxEdges = 640;
 constexpr int kHetThreads = 320;   // most threads of a CTA of k_het_loglike
+// Threads of a detector with ne edges: equal rounds of edges over the fewest threads (at least 64, which stage the projection forms). They
+// also share out its bins, so the order of its sums depends on nothing but its own edges; a CTA has those of the detector that wants the most.
+inline int het_threads(int ne) {
+  const int rounds = (ne + kHetThreads - 1) / kHetThreads, t = ((ne + rounds - 1) / rounds + 31) / 32 * 32;
+  return t < 64 ? 64 : t;
+}
 constexpr int kPairs = kNModes * (kNModes + 1) / 2;   // unordered mode pairs (md <= md2)
 
 __host__ __device__ constexpr int pair_index(int a, int b) {   // a <= b
@@ -51,6 +57,7 @@ struct HetDev {
   const longlong2* Bx;
   const int* Gx;         // [6][3][ne-1] their exponents
   int ne;
+  int nt;                // threads that share out its bins (het_threads)
   unsigned mask;
 };
 struct HetSet {
@@ -540,7 +547,7 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
       const float4* rw = reinterpret_cast<const float4*>(rsh);
       const cdf zc = {df_make(0.f, 0.f), df_make(0.f, 0.f)};
       const int nbin = H.ne - 1;
-      for (int b = threadIdx.x; b < nbin; b += blockDim.x) {
+      for (int b = threadIdx.x < H.nt ? threadIdx.x : nbin; b < nbin; b += H.nt) {
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) {
           const int* sa = H.src + (size_t)b * kNModes * 3 + c;          // edge of mode md's ratio at sa[3 md], and at the
@@ -592,7 +599,7 @@ __global__ void __launch_bounds__(kHetThreads, 2) k_het_loglike(HetSet hs, int B
         }
       }
     } else {
-      for (int b = threadIdx.x; b < H.ne - 1; b += blockDim.x) {
+      for (int b = threadIdx.x < H.nt ? threadIdx.x : H.ne; b < H.ne - 1; b += H.nt) {
 #pragma unroll 1
         for (int c = 0; c < 3; ++c) {
           double dh, hh;
@@ -849,6 +856,7 @@ pe_status pe_hetero_create(pe_detector det, const double* theta0, unsigned mode_
   h->dev.Bx = d_Bx;
   h->dev.Gx = d_Gx;
   h->dev.ne = ne;
+  h->dev.nt = pe::het_threads(ne);
   h->dev.mask = mode_mask;
   *out = h;
   return PE_OK;
@@ -921,9 +929,8 @@ pe_status pe_hetero_loglike_batch(const pe_hetero* hets, int ndet, const double*
   const size_t smem = (size_t)nemax * pe::kNModes * 3 * sizeof(double2) + (mix ? (size_t)nemax : 0);   // and the flags
   auto kern = mix ? (fxu ? pe::k_het_loglike<true, true> : pe::k_het_loglike<true, false>)
                   : (fxu ? pe::k_het_loglike<false, true> : pe::k_het_loglike<false, false>);
-  // equal rounds of edges over the fewest threads (at least 64, which stage the projection forms)
-  const int rounds = (nemax + pe::kHetThreads - 1) / pe::kHetThreads;
-  const int threads = std::max(64, ((nemax + rounds - 1) / rounds + 31) / 32 * 32);
+  int threads = 0;
+  for (int i = 0; i < ndet; ++i) threads = std::max(threads, hs.h[i].nt);
   static_assert(pe::kProj <= 64, "one thread per form");
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) {

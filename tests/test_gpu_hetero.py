@@ -174,3 +174,24 @@ def test_hetero_sums_scale_with_the_distance_exactly(Lb, nbins):
         np.testing.assert_array_equal(g[..., 0] * 2.0 ** k, ref[..., 0])
         np.testing.assert_array_equal(g[..., 1] * 4.0 ** k, ref[..., 1])
     het.close()
+
+
+@pytest.mark.parametrize("mix", [False, True], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("nbins", [1, 40, 290])
+def test_hetero_sums_do_not_depend_on_the_other_detectors(Lb, nbins, mix):
+    """A detector's <d|h> and <h|h> are the same bits alone and beside detectors with fewer and with more edges
+    (which set the threads of a CTA)."""
+    prec = Lb.PE_PREC_MIXED if mix else 0
+    d, th0, th, edges = _edges_and_samples(Lb, 2.0 ** 18, nbins)
+    het = Lb.Hetero(d, th0, W.MODE_ALL | prec, edges=edges)
+    ref = Lb.hetero_loglike([het], th, dhhh=True)["dhhh"][:, 0]
+    k0, nb = W.grid(2.0 ** 17)
+    for other in (10, 150, 330, 620):
+        o = Lb.Detector(W.TAIJI, 2.0 ** 17, k0, nb)
+        o.inject(th0, W.MODE_ALL, W.normals(nb, 4))
+        oh = Lb.Hetero(o, th0, W.MODE_ALL | prec, edges=np.unique(np.linspace(0, nb - 1, other).astype(np.int64)))
+        for hets, i in (([het, oh], 0), ([oh, het], 1)):
+            g = Lb.hetero_loglike(hets, th, dhhh=True)["dhhh"][:, i]
+            np.testing.assert_array_equal(g, ref)
+        oh.close()
+    het.close()

@@ -574,6 +574,38 @@ __global__ void __launch_bounds__(32 * kFisherWarps, 1) k_fisher_fwd(DetSet ds, 
   }
 }
 
+// Sums over the lanes of the eleven values of each lane: in five steps a lane keeps half of its values, sends the
+// other half and adds what it gets, 13 additions where eleven shuffle trees make 55. Lane l ends with the sum of value fisher_lane_entry(l)
+// (-1: with none).
+__host__ __device__ constexpr int fisher_kept(int step) { return step == 0 ? 6 : (step == 1 ? 3 : (step == 2 ? 2 : 1)); }   // of 11, 6, 3, 2, 1
+static_assert(kFisherW / kFisherWarps == 11, "fisher_kept halves eleven values");
+__device__ __forceinline__ double fisher_lane_sum(double v[kFisherW / kFisherWarps], int lane) {
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int o = 16 >> st, keep = fisher_kept(st), have = st == 0 ? kFisherW / kFisherWarps : fisher_kept(st - 1);
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < keep; ++k) {
+      const double lo = v[k], hi = k + keep < have ? v[k + keep] : 0.0;
+      v[k] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+    }
+  }
+  return v[0];
+}
+__device__ __forceinline__ int fisher_lane_entry(int lane) {
+  int first = 0, n = kFisherW / kFisherWarps;
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    if (lane & (16 >> st)) {
+      first += fisher_kept(st);
+      n -= fisher_kept(st);
+    } else {
+      n = min(n, fisher_kept(st));
+    }
+  }
+  return n > 0 ? first : -1;
+}
+
 // Fisher on detectors that take the fixed-point unit: six warps per 32 bins. Warps 0-3 first run the forward pass of one mode
 // each (slot w) onto a tape in shared memory, with the chain factors that the seeds share; then warp j runs seed j's reverse
 // sweeps (Re/Im of A', E', T'), giving row j of the Jacobian, and each warp accumulates eleven of the 66 entries. Bound by
@@ -625,9 +657,7 @@ __global__ void __launch_bounds__(kFisherFxThreads, 2) k_fisher_fx(DetSet ds, in
       sm.rot[j][c] = a;
     }
     fx_proj3(sm.pc);
-    double F[kFisherW / kFisherWarps];
-#pragma unroll
-    for (int e = 0; e < kFisherW / kFisherWarps; ++e) F[e] = 0.0;
+    double own = 0.0;   // this lane's entry (fisher_lane_entry), summed over the passes
     const int subs = kTileBins / 32 / split, sub0 = int(t - tile * split) * subs;
 #pragma unroll 1
     for (int sub = sub0; sub < sub0 + subs; ++sub) {
@@ -690,6 +720,9 @@ __global__ void __launch_bounds__(kFisherFxThreads, 2) k_fisher_fx(DetSet ds, in
       }
       __syncthreads();
       // entries e = w, w + 6, ... of the upper triangle, row by row
+      double F[kFisherW / kFisherWarps];
+#pragma unroll
+      for (int e = 0; e < kFisherW / kFisherWarps; ++e) F[e] = 0.0;
 #pragma unroll 1
       for (int r = 0; r < kFisherWarps; ++r) {
         int i = 0, k = w;
@@ -701,18 +734,16 @@ __global__ void __launch_bounds__(kFisherFxThreads, 2) k_fisher_fx(DetSet ds, in
           while (i < PE_NPARAM && k >= PE_NPARAM - i) { k -= PE_NPARAM - i; ++i; }
         }
       }
+      own += fisher_lane_sum(F, lane);
     }
-    // fixed-order sums over the lanes
-#pragma unroll
-    for (int e = 0; e < kFisherW / kFisherWarps; ++e) {
-      for (int o = 16; o > 0; o >>= 1) F[e] += __shfl_down_sync(0xffffffffu, F[e], o);
-      if (lane == 0) part[t * kFisherW + w + kFisherWarps * e] = F[e];
-    }
+    const int e = fisher_lane_entry(lane);
+    if (e >= 0) part[t * kFisherW + w + kFisherWarps * e] = own;
   }
   work_done(ctr);
 }
 
-// Per point: thread (r, e) adds entry e of the tiles r, r + 8, ... over the detectors, then thread e its eight rows.
+// Per point: thread (r, e) adds entry e of the tiles r, r + 8, ... over the detectors, then thread e its eight rows. A tile's sum is that of its
+// items (split of them) in order, as k_fisher_fx adds the passes of an undivided tile, so the bits do not depend on the split.
 constexpr int kFisherRows = 8;
 __global__ void __launch_bounds__(kFisherW * kFisherRows) k_fisher_reduce(DetSet ds, int B, const long long* off, const double* part,
                                                                         const SampleCoef* coef, int split, double* F) {
@@ -723,7 +754,11 @@ __global__ void __launch_bounds__(kFisherW * kFisherRows) k_fisher_reduce(DetSet
   for (int I = 0; I < ds.ndet; ++I) {
     const int p = I * B + s;
     if (!PE_CHK(off[p] >= 0 && off[p + 1] <= off[ds.ndet * B], 128)) continue;
-    for (long long t = off[p] * split + r; t < off[p + 1] * split; t += kFisherRows) a += part[t * kFisherW + e];
+    for (long long t = off[p] + r; t < off[p + 1]; t += kFisherRows) {
+      double x = part[t * split * kFisherW + e];
+      for (int k = 1; k < split; ++k) x += part[(t * split + k) * kFisherW + e];
+      a += x;
+    }
   }
   red[r][e] = a;
   __syncthreads();

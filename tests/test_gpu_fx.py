@@ -210,3 +210,17 @@ def test_a_bin_without_a_finite_datum(Lb):
     assert np.isnan(l1[1, 0, 1, 0]) and np.all(np.isnan(g1[1])) and np.isnan(h1[0, 0, 1, 0])
     np.testing.assert_array_equal(l1[1, 0, [0, 2]], l0[1, 0, [0, 2]])
     np.testing.assert_array_equal(h1[0, 0, [0, 2]], h0[0, 0, [0, 2]])
+
+
+@pytest.mark.parametrize("det", [W.LISA, dict(W.LISA, arm_m=3.0e10)], ids=["fixed_point", "general"])
+def test_fisher_of_a_point_does_not_depend_on_the_batch(Lb, det):
+    """A point's Fisher matrix is the same bits alone and inside batches from one tile per SM to more than a thousand tiles
+    per SM, on both sides of the rule that picks the kernel's work items."""
+    T = 2.0 ** 16
+    k0, nb = W.grid(T)
+    d = Lb.Detector(det, T, k0, nb)
+    d.inject(W.theta_injection(T), W.MODE_ALL, W.normals(nb, 2))
+    th = _samples(T, 0.02)
+    alone = np.concatenate([Lb.fisher([d], t[None, :], W.MODE_ALL) for t in th])
+    for B in (8, 72, 1200, 8000):
+        np.testing.assert_array_equal(Lb.fisher([d], np.tile(th, (B // 8, 1)), W.MODE_ALL), np.tile(alone, (B // 8, 1, 1)))

@@ -189,7 +189,7 @@ pe_status pe_loglike_batch_noalloc(const pe_detector* dets, int ndet, const doub
  * any stream; results equal pe_loglike_batch's bit for bit.
  *   The forward kernel's work items are 1, 2, 4 or 8 consecutive 128-bin sub-tiles of one
  *   (detector, sample) pair; each sub-tile keeps its own partial sum in a fixed reduction order.
- *   autotune = 1: if the tuning cache has no entry for this workload (GPU, SM count, batch size,
+ *   autotune = 1: if the tuning cache has no entry for this workload (GPU, SM count, kernels, batch size,
  *   mode mask, grids), time the forward kernel's launch choices on the theta present at
  *   creation (register-budget variant x persistent grid size, then the sub-tiles per work item)
  *   and store the fastest. The cache is a JSON file at $PE_TUNE_CACHE, else

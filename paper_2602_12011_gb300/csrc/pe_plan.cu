@@ -104,6 +104,8 @@ int sm_count_now() {
 
 }  // namespace
 
+// The unit that runs is part of the key, with the resident CTAs its variants 0, 1, 2 ask for: a choice timed on other kernels
+// (another arm on the same grid, an entry of an earlier build) does not match.
 std::string tune_key(const DetSet& ds, int B, unsigned mask) {
   int dev = 0;
   cudaGetDevice(&dev);
@@ -111,7 +113,8 @@ std::string tune_key(const DetSet& ds, int B, unsigned mask) {
   char buf[256];
   std::string k;
   if (cudaGetDeviceProperties(&prop, dev) == cudaSuccess) k = prop.name; else { cudaGetLastError(); k = "gpu"; }
-  snprintf(buf, sizeof(buf), "|sm=%d|B=%d|mask=%u|nb=", sm_count_now(), B, mask);
+  const char* unit = mask_prec(mask) != kPrecFP32 && fx_all_ok(ds) ? "fx7,8,6" : "general2,3,4";
+  snprintf(buf, sizeof(buf), "|sm=%d|unit=%s|B=%d|mask=%u|nb=", sm_count_now(), unit, B, mask);
   k += buf;
   for (int i = 0; i < ds.ndet; ++i) {
     snprintf(buf, sizeof(buf), "%s%d@%lld", i ? "," : "", ds.d[i].nb, ds.d[i].k0);

@@ -132,3 +132,22 @@ def test_network_full_size_plan_sampled(oracle_mod, Lb):
     H.assert_loglike_parity({"logl": logl[pick], "dhhh": dhhh[pick]}, ll, ref, dd,
                             H.floor_terms(oracle_mod, ods, th[pick], wl["mode_mask"]))
     plan.close()
+
+
+def test_tuned_choices_are_kept_per_unit(Lb):
+    """Two detectors on one grid whose arms put them on different kernels keep a tuned choice each."""
+    import torch
+    T = 2.0 ** 14
+    k0, nb = W.grid(T)
+    th = torch.tensor(W.draw_prior(11, 3, T), device="cuda")
+    dets, want = [], [(0, 16, 1), (2, 2, 8)]
+    for arm, c in zip((2.5e9, 3.0e10), want):
+        d = Lb.Detector(dict(W.LISA, arm_m=arm), T, k0, nb)
+        d.inject(W.theta_injection(T), W.MODE_ALL, W.normals(nb, 5))
+        Lb.pe_tune_set([d.handle], 11, W.MODE_ALL, *c)
+        dets.append(d)
+    for d, c in zip(dets, want):
+        pl = Lb.Plan([d], 11, W.MODE_ALL, theta=th, autotune=False)
+        info = pl.info()
+        assert (info["fwd_variant"], info["ctas_per_sm"], info["subtiles"]) == c
+        pl.close()

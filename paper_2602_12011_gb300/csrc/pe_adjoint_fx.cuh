@@ -95,11 +95,12 @@ __device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx*
   if (pair) E = max(E, max(fx_expo(Ap.y), fx_expo(Ac.y)));
   const int ash = 1079 - E;
   fxs Apx = {0, 0}, Acx = {0, 0}, Apy = {0, 0}, Acy = {0, 0};
-  if (E) {   // else the weights vanish, and only their own cotangents are not zero
+  const bool some = E >= kFxLeastE;
+  if (some) {   // else the weights vanish, and only their own cotangents are not zero
     Apx = fx_split(fx_from_bits(Ap.x, ash));
     Acx = fx_split(fx_from_bits(Ac.x, ash));
   }
-  if (pair && E) {
+  if (pair && some) {
     Apy = fx_split(fx_from_bits(Ap.y, ash));
     Acy = fx_split(fx_from_bits(Ac.y, ash));
   }
@@ -220,7 +221,7 @@ __device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx*
     }
   }
   // orbit basis b = (cos 2 alpha, sin 2 alpha, cos alpha, sin alpha) or (cos phi_0, sin phi_0)
-  const int e = E + Es - 2097;
+  const int e0 = E + Es - 2097, e = min(e0, kFxMostExpo), es = min(Es - 1078, kFxMostExpo);
   if (helio) {
     const fxs c = fx_split(tape.ld(kFtC)), s = fx_split(tape.ld(kFtS));
     fxa q = fx_sq0<1>();
@@ -240,12 +241,22 @@ __device__ __forceinline__ void fx_bwd(const FxBin& B, fx a3, const volatile fx*
   o.W[0] = fx_to_double(Wk, e);
   o.W[1] = fx_to_double(Wp, e);
   o.W[2] = fx_to_double(Wq, e);
-  if (E == 0) o.th = o.lnA = o.alpha = o.geo = o.W[0] = o.W[1] = o.W[2] = 0.0;   // not the sums' rounding
-  o.Ap = make_double2(fx_to_double(Apb[0], Es - 1078), 0.0);
-  o.Ac = make_double2(fx_to_double(Acb[0], Es - 1078), 0.0);
+  if (!some) o.th = o.lnA = o.alpha = o.geo = o.W[0] = o.W[1] = o.W[2] = 0.0;   // not the sums' rounding
+  o.Ap = make_double2(fx_to_double(Apb[0], es), 0.0);
+  o.Ac = make_double2(fx_to_double(Acb[0], es), 0.0);
   if (pair) {
-    o.Ap.y = fx_to_double(Apb[1], Es - 1078);
-    o.Ac.y = fx_to_double(Acb[1], Es - 1078);
+    o.Ap.y = fx_to_double(Apb[1], es);
+    o.Ac.y = fx_to_double(Acb[1], es);
+  }
+  if (max(e0, Es - 1078) > kFxMostExpo) {   // where floating point may overflow
+    const double p = __hiloint2double(min(e0 - e + 1023, 0x7ff) << 20, 0), pa = __hiloint2double((Es - 1078 - es + 1023) << 20, 0);
+    o.th *= p;
+    o.lnA *= p;
+    o.alpha *= p;
+    o.geo *= p;
+    for (int i = 0; i < 3; ++i) o.W[i] *= p;
+    o.Ap = make_double2(o.Ap.x * pa, o.Ap.y * pa);
+    o.Ac = make_double2(o.Ac.x * pa, o.Ac.y * pa);
   }
 }
 

@@ -143,6 +143,7 @@ __device__ __forceinline__ void fx_zero(Acc& a, fx* col) {
   for (int i = 0; i < kFxSums; ++i) a.s[i * Acc::kStride] = 0;
   a.E = 0;
 }
+constexpr int kFxLeastE = 64;   // amplitudes below 2^-959 count as 0: above, a zero beside them converts to 0 (fx_from_bits)
 constexpr float kFxTauMax = 8192.f;
 __device__ __forceinline__ int fx_expo(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
@@ -332,8 +333,8 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
   }
   int E = max(fx_expo(Ap.x), fx_expo(Ac.x));
   if (C2) E = max(E, max(fx_expo(Ap.y), fx_expo(Ac.y)));
-  // E = 0: the weights vanish (the unit adds nothing; its tape still serves the weights' own derivatives)
-  if (!Tape::kOn && E == 0) return;
+  // below kFxLeastE the weights vanish (the unit adds nothing; its tape still serves the weights' own derivatives)
+  if (!Tape::kOn && E < kFxLeastE) return;
   if (E > acc.E) {
     if (acc.E > 0) {
       const int sh = min(62, E - acc.E);
@@ -343,7 +344,8 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
     acc.E = E;
   }
   const int ash = 1079 - acc.E;
-  const fxs Apx = E ? fx_split(fx_from_bits(Ap.x, ash)) : fxs{0, 0}, Acx = E ? fx_split(fx_from_bits(Ac.x, ash)) : fxs{0, 0};
+  const bool some = E >= kFxLeastE;
+  const fxs Apx = some ? fx_split(fx_from_bits(Ap.x, ash)) : fxs{0, 0}, Acx = some ? fx_split(fx_from_bits(Ac.x, ash)) : fxs{0, 0};
   // --- orbit at t_f (row A4): mode phase in turns, the centre's Doppler term f k.x_c = f R (k_x cos + k_y sin)
   // included, and the offsets' basis
   const fxc ca = fx_cis(alpha, tab);
@@ -364,10 +366,11 @@ __device__ __forceinline__ void mode_bin_fx(const DetDev& D, const SampleCoef& S
       tape.st(kFtGs, cg.s);
     }
   }
-  fx_links(B.at3, B.a4, phu, Apx, Acx, C2 && E ? &Ap : nullptr, Ac.y, ash, ob, helio, acc, tab, stab, pc, tape);
+  fx_links(B.at3, B.a4, phu, Apx, Acx, C2 && some ? &Ap : nullptr, Ac.y, ash, ob, helio, acc, tab, stab, pc, tape);
 }
 
-// n 2^e as a double, the power of two added to the exponent field (0 where the result would lie below 2^-1020)
+// n 2^e as a double, the power of two added to the exponent field (0 where the result would lie below 2^-1020); e <= kFxMostExpo
+constexpr int kFxMostExpo = 960;   // n's largest power of two then still fits a double
 __device__ __forceinline__ double fx_to_double(fx n, int e) {
   const double d = __ll2double_rn(n);
   const int hi = __double2hiint(d);
@@ -395,7 +398,8 @@ template <class Acc>
 __device__ __forceinline__ void aet_from_fx(const Acc& a, double2 z, double2 o[3]) {
   fx xr[3], xi[3];
   xyz_from_fx(a, fx_split(fx_from_bits(z.x, 60)), fx_split(fx_from_bits(z.y, 60)), xr, xi);
-  const int e = a.E - 1078;   // one unit of the halved sums is 2^e
+  // one unit of the halved sums is 2^e; amplitudes beyond 2^1015 (and infinite ones) count as 2^1015, whose <h|h> overflows too
+  const int e = min(a.E - 1078, kFxMostExpo);
   o[0] = make_double2(fx_to_double(xr[2] - xr[0], e), fx_to_double(xi[2] - xi[0], e));
   o[1] = make_double2(fx_to_double(xr[0] - 2 * xr[1] + xr[2], e), fx_to_double(xi[0] - 2 * xi[1] + xi[2], e));
   o[2] = make_double2(fx_to_double(xr[0] + xr[1] + xr[2], e), fx_to_double(xi[0] + xi[1] + xi[2], e));
@@ -403,9 +407,9 @@ __device__ __forceinline__ void aet_from_fx(const Acc& a, double2 z, double2 o[3
 
 // Adds every active mode of one sample at one bin ((2,2) and (3,2) through one unit when both are
 // active), then forms A/E/T. D0: the detector whose copy of the tables is read (the set's first, so that one copy
-// stays in L1); col: the thread's column of kFxSums x kTileBins words of shared memory.
+// stays in L1); col: the thread's column of kFxSums x kTileBins words of shared memory; expo (nullable): the sums' exponent (FxAccT).
 __device__ __forceinline__ void bin_aet_fx(const DetDev& D, const SampleCoef& S, int b, double2 o[3],
-                                           const DetDev& D0, const fx* __restrict__ pc, fx* col) {
+                                           const DetDev& D0, const fx* __restrict__ pc, fx* col, int* expo = nullptr) {
   FxBin B;
   load_bin_fx(D, b, S.tc, B);
   FxAcc a;
@@ -418,6 +422,7 @@ __device__ __forceinline__ void bin_aet_fx(const DetDev& D, const SampleCoef& S,
     mode_bin_fx(D, S, C, B, a, D0.fcis, D0.fsinc, pc, md, (md == 0 && S.pair32) ? &S.md[3] : nullptr);
   }
   aet_from_fx(a, D.z[b], o);
+  if (expo) *expo = a.E;
 }
 
 }  // namespace pe

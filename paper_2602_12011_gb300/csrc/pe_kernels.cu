@@ -609,7 +609,10 @@ __global__ void k_signal(DetDev D, const SampleCoef* coef, double2* out) {
     bin_aet_f32(D, sf, b, of, reinterpret_cast<const float*>(pcw));
     for (int i = 0; i < 3; ++i) o[i] = make_double2((double)of[i].x * S.ihsc, (double)of[i].y * S.ihsc);
   } else if (PREC == kPrecFx) {
-    bin_aet_fx(D, S, b, o, D, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x]);
+    int expo;
+    bin_aet_fx(D, S, b, o, D, reinterpret_cast<const fx*>(pc), &fxcol[0][threadIdx.x], &expo);
+    if (expo == 0x7ff)   // an infinite amplitude
+      for (int i = 0; i < 3; ++i) o[i].x = o[i].y = __longlong_as_double(0x7ff8000000000000LL);
   } else {
     bin_xyz(D, S, b, x, D.sct, pc);
     aet_from_xyz(x, o);

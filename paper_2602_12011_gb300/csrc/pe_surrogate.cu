@@ -926,7 +926,7 @@ __device__ __forceinline__ void mode_bin_sur(const ModeCoef& C, const SurMode& m
   }
   const fxs As = fx_split(A);
   const fxc e = fx_cis(ph - n.frc, tab);
-  const float sc = E > 935 ? __int_as_float((E - 926) << 23) : 0.f;   // 2^(E - 1022 - 31)
+  const float sc = E > 935 ? __int_as_float(min(E - 926, 0xff) << 23) : 0.f;   // 2^(E - 1022 - 31), or an infinity
   const float hr = (float)(int)(fx_mul(As, fx_split(e.c)) >> 29) * sc;
   const float hi = (float)(int)(fx_mul(As, fx_split(e.s)) >> 29) * sc;
 #pragma unroll
@@ -935,13 +935,14 @@ __device__ __forceinline__ void mode_bin_sur(const ModeCoef& C, const SurMode& m
     acc[c].y = fmaf(hr, val[2 * c + 1], fmaf(hi, val[2 * c], acc[c].y));
   }
 }
-// x p2 in FP64 for a power of two p2 (exact; through the exponent fields, x = 0 or below FP32's normal range gives 0)
+// x p2 in FP64 for a power of two p2 (exact; through the exponent fields: x = 0 or below FP32's normal range, or a product below
+// FP64's, gives 0; an infinity, a NaN or a product above FP64's range no finite number)
 __device__ __forceinline__ double scale_up(float x, double p2) {
   const unsigned u = (unsigned)__float_as_int(x);
   const int e = (int)((u >> 23) & 0xff);
-  if (e == 0) return 0.0;
-  return __hiloint2double((int)((u & 0x80000000u) | ((u & 0x7fffffu) >> 3)) + ((e + 896 + fx_expo(p2) - 1023) << 20),
-                          (int)(u << 29));
+  const int E = e == 0xff ? 0x7ff : e + 896 + fx_expo(p2) - 1023;
+  if (e == 0 || E <= 0) return 0.0;
+  return __hiloint2double((int)((u & 0x80000000u) | ((u & 0x7fffffu) >> 3)) + (min(E, 0x7ff) << 20), (int)(u << 29));
 }
 
 // mode_bin_sur on the FP32 pipe. The phase spline (up to ~1e5 turns) is evaluated in double words

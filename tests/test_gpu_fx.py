@@ -224,3 +224,34 @@ def test_fisher_of_a_point_does_not_depend_on_the_batch(Lb, det):
     alone = np.concatenate([Lb.fisher([d], t[None, :], W.MODE_ALL) for t in th])
     for B in (8, 72, 1200, 8000):
         np.testing.assert_array_equal(Lb.fisher([d], np.tile(th, (B // 8, 1)), W.MODE_ALL), np.tile(alone, (B // 8, 1, 1)))
+
+
+@pytest.mark.parametrize("arm_m", [2.5e9, 3.0e10], ids=["fixed_point", "general"])
+def test_amplitudes_at_the_limits_of_a_double(Lb, arm_m):
+    """A distance so small that the amplitude or <h|h> overflows gives no finite log L or derivative in the distance, in every
+    unit and on the surrogate's spline path; one so large that the signal underflows gives the log L of no signal."""
+    import torch
+    T = 2.0 ** 16
+    d = Lb.Detector(dict(W.LISA, arm_m=arm_m), T, 200, 300)
+    rng = np.random.default_rng(3)
+    d.set_data(1e-21 * (rng.standard_normal((3, 300)) + 1j * rng.standard_normal((3, 300))), np.full((3, 300), 1e-38))
+    none = -0.5 * d.data_norm().sum()
+    th0 = np.array([1e6, 2.0, 0.1, -0.2, 1.0, 0.6, 0.9, 2.0, 0.4, 1.1, 100.0])
+    th = np.tile(th0, (8, 1))
+    th[:, 4] = [5e-324, 1e-312, 1e-306, 1e-290, 1e-200, 1e-160, 1e280, 1e290]
+    net = Lb.Surrogate(seed=1)
+    net.set_node_source(1)
+    for flag in (0, Lb.PE_PREC_MIXED):
+        for mask in (W.MODE_22, W.MODE_ALL):
+            ll = Lb.loglike([d], th, mask | flag)["logl"]
+            g = Lb.loglike_grad([d], th, mask | flag)
+            sur = net.loglike([d], torch.tensor(th, device="cuda"), mask | flag)[0].cpu().numpy()
+            for x in (ll, g["logl"], g["grad"][:, 4], sur):
+                assert not np.any(np.isfinite(x[:6])), (flag, mask, x)
+            assert not np.any(np.isfinite(d.signal(th[0], mask | flag)[:, :60]))    # below the (2,2) mode's end
+            for x in (ll, g["logl"], sur):
+                assert np.all(np.abs(x[6:] - none) <= 1e-12 * abs(none)), (flag, mask, x)
+            assert np.all(np.isfinite(g["grad"][6:]))
+    het = Lb.Hetero(d, th0, W.MODE_ALL, nbins_coarse=20)
+    ll = Lb.hetero_loglike([het], th)["logl"]
+    assert not np.any(np.isfinite(ll[:6])) and np.all(np.abs(ll[6:] - none) <= 1e-12 * abs(none)), ll

@@ -177,3 +177,19 @@ def test_mixed_batch_invariance_and_entry_points(oracle_mod, Lb):
     with pytest.raises(Lb.PeError) as e:
         Lb.fisher([gd], th[:2], m)
     assert e.value.status == Lb.PE_EINVAL
+
+
+@pytest.mark.parametrize("arm_m", [2.5e9, 3.0e10], ids=["fixed_point", "general"])
+def test_both_precisions_are_one_kernel_where_documented(Lb, arm_m):
+    """Where every detector takes the fixed-point unit, the likelihood and the gradient of both precisions are the same bits; on an
+    arm that does not take it they come from different kernels."""
+    T = 2.0 ** 15
+    k0, nb = W.grid(T)
+    d = Lb.Detector(dict(W.LISA, arm_m=arm_m), T, k0, nb)
+    d.inject(_th_small(T), W.MODE_ALL, W.normals(nb, 3))
+    th = W.draw_prior(9, 4, T)
+    a, b = (Lb.loglike([d], th, W.MODE_ALL | f, dhhh=True) for f in (0, MIX))
+    ga, gb = (Lb.loglike_grad([d], th, W.MODE_ALL | f) for f in (0, MIX))
+    same = [np.array_equal(a["logl"], b["logl"]), np.array_equal(a["dhhh"], b["dhhh"]),
+            np.array_equal(ga["logl"], gb["logl"]), np.array_equal(ga["grad"], gb["grad"])]
+    assert same == [arm_m < 1e10] * 4

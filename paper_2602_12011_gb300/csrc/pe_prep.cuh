@@ -8,8 +8,9 @@
 // What bounds it: one thread's chain of ~1,500 FP64 instructions (five sincos, a cube root, a log, square roots and
 // divisions, five modes) at ~50 cycles each, 38 us whatever the batch, half of a single-sample call. The pieces are
 // independent, so eight threads of a warp share a sample: its sines and cosines, modes and converted coefficients
-// are then one instruction stream each. From kPrepSerialB samples on, where every SM has work, one thread per sample
-// issues fewer instructions in all. Both run the same pieces (not inlined, exchanged through memory), so a
+// are then one instruction stream each. From kPrepSerialB samples on one thread per sample issues fewer instructions in
+// all (whole calls on a grid of four bins, eight threads against one: 4,096 samples 112 and 121 us, gradients 311 and 324; 6,144: 165 and 162,
+// gradients 435 and 426; 8,192: 186 and 173; 65,536: 1144 and 858). Both run the same pieces (not inlined, exchanged through memory), so a
 // sample's coefficients are the same bits in any batch.
 #pragma once
 #include "pe_device.cuh"
@@ -18,7 +19,7 @@ namespace pe {
 
 constexpr int kPrepThreads = 64;
 constexpr int kPrepGroup = 8;
-constexpr int kPrepSerialB = 8192;
+constexpr int kPrepSerialB = 6144;
 
 // Values shared by the pieces of one sample.
 struct PrepTmp {

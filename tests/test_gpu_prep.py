@@ -66,3 +66,8 @@ def test_reductions_at_the_rule_between_warp_and_cta(Lb, tiles):
     g = Lb.loglike_grad([d], t2, W.MODE_ALL)
     scale = 0.5 * d.data_norm().sum() + abs(dh.sum()) + hh.sum()
     assert abs(g["logl"][0] - r["logl"][0]) <= 1e-12 * scale
+
+
+@pytest.mark.parametrize("B", [6143, 6144, 6145])
+def test_batches_at_the_rule_between_eight_threads_and_one(Lb, B):
+    test_batch_sizes_give_a_sample_the_same_bits(Lb, B)

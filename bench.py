@@ -36,7 +36,7 @@ MSUN_S = 4.925490947641267e-6
 # of one launch on the 64-sample case of this workload:
 #   fp64_flops  DFMA x 2 + DMUL + DADD
 #   fp64_inst   every FP64-pipe instruction (DFMA, DMUL, DADD, DSETP, F2F, FRND)
-#   fp32_inst   FFMA + FMUL + FADD (the double-word arithmetic of the mixed path)
+#   fp32_inst   FFMA + FMUL + FADD (the double-word corrections of the fixed-point unit)
 UNIT_COUNTS = {
     # fp64 and mixed: both run the fixed-point unit on this workload (2,464 thread instructions per unit,
     # most of them integer)
@@ -83,7 +83,7 @@ def parse():
     ap.add_argument("--no-network", action="store_true")
     ap.add_argument("--no-surrogate", action="store_true")
     ap.add_argument("--precision", choices=["fp64", "mixed"], default="fp64",
-                    help="headline forward path: all FP64, or FP64 phase/t_f/sums with double-word geometry")
+                    help="headline forward path; on this detector both run the fixed-point unit")
     ap.add_argument("--no-precision-study", action="store_true")
     ap.add_argument("--no-hetero", action="store_true")
     return ap.parse_args()
@@ -445,8 +445,8 @@ def main():
                             "max_rel_dlogl_vs_fp64": rel, "max_abs_dlogl_vs_fp64": absmax, "parity_bar": 1e-10,
                             "roofline": roofline(other, units, (o_ms / max(o_n, 1)) / 1e3, peaks, n_sm, sm_max,
                                                  clk.get("sm_mhz"), bins)}
-        study["note"] = ("mixed: FP64 TaylorF2 phase, t_f, turn reductions and tile sums; response "
-                         "geometry, TDI, A/E/T and per-bin products in double-word FP32 arithmetic. "
+        study["note"] = ("mixed: on this detector the same fixed-point kernel as fp64 (deviation 0); double-word "
+                         "FP32 geometry only on detectors outside that unit's bounds. "
                          "fp32: every step in FP32 (the paper's float32 option); misses the 1e-10 bar")
 
     # ---- plain path: one call per sample (B = 1), same samples, device-timed
@@ -519,9 +519,9 @@ def main():
         gms.append(e0.elapsed_time(e1))
     grad_value = world * B * Kg / (sum(gms) / 1e3)
     grad_ok = bool(torch.isfinite(grad_dev).all().item())
-    # the same gradient in mixed precision (PE_PREC_MIXED): the forward mode sum and the reverse
-    # sweeps with double-word geometry. Its deviation from the FP64 gradient: per component, the
-    # largest |g_mixed - g_fp64| over the batch divided by the largest |g_fp64|
+    # the same gradient in mixed precision (PE_PREC_MIXED): on this detector the same fixed-point kernel, timed
+    # again. Its deviation from the FP64 gradient (0): per component, the largest |g_mixed - g_fp64| over the
+    # batch divided by the largest |g_fp64|
     grad_mx = torch.empty_like(grad_dev)
     ll_mx = torch.empty_like(ll_dev)
     L.pe_loglike_grad_batch(hs, th_dev, B, mask64 | L.PE_PREC_MIXED, ll_mx, grad_mx, None, stream)
@@ -537,8 +537,8 @@ def main():
                   "ms_per_step": sum(gms_mx) / Kg, "steps": Kg,
                   "max_rel_dgrad_vs_fp64": float(((grad_mx - grad_dev).abs().amax(dim=0)
                                                   / grad_dev.abs().amax(dim=0).clamp_min(1e-300)).max().item()),
-                  "note": ("FP64 TaylorF2 phase, t_f, turn reductions, PN chain rule and sums; "
-                           "double-word geometry, link factors and their cotangents")}
+                  "note": ("the same kernel as fp64 on this detector: FP64 TaylorF2 phase, PN chain rule and "
+                           "sums; geometry, link factors and their cotangents in 64-bit fixed point")}
 
     # ---- Fisher matrix at the injected source (5 modes, all 11 parameters), device-timed
     thf = torch.tensor(wl["inj"][None, :], device="cuda")
@@ -655,9 +655,9 @@ def main():
                "heldout_max_mismatch_no_network": float(np.max(mm_n[inbox])),
                "heldout_in_box": int(inbox.sum()),
                "note": ("network: MLP node values (3PN/3.5PN phase terms, |H_lm|) + node splines; no_network: "
-                        "the same splines from the plain generator's exact node values; plain: per-bin FP64; "
-                        "plain_mixed: per-bin FP64 phase with double-word geometry (1e-10 parity); *_mixed: "
-                        "the surrogate path with PE_PREC_MIXED (fallbacks on the mixed plain unit, in-box spline "
+                        "the same splines from the plain generator's exact node values; plain and plain_mixed: "
+                        "per bin, FP64 phase with fixed-point geometry (one kernel on this detector); *_mixed: "
+                        "the surrogate path with PE_PREC_MIXED (fallbacks on that kernel, in-box spline "
                         "sincos and transfer functions in FP32, double-word A/E/T and products)")}
         srg.close()
 
@@ -702,7 +702,7 @@ def main():
                "max_abs_dlogl_vs_exact": dl.max().item(), "median_abs_dlogl_vs_exact": dl.median().item(),
                "samples": "Fisher-Gaussian draws at 0.1 of its width around the injection (posterior bulk)",
                "dtype": "f64"}
-        # the same summary data with the signal at the edges from the mixed-precision unit
+        # the same edges with the mixed precision's contraction (double words)
         hmix = L.Hetero(gd, wl["inj"], mask64 | L.PE_PREC_MIXED, edges=hobj.edges)
         llm = torch.empty_like(llh)
         for _ in range(3):
@@ -719,7 +719,7 @@ def main():
         het["mixed"] = {"value": world * Bh / (sum(mms) / len(mms) / 1e3), "unit": UNIT,
                         "ms_per_step": sum(mms) / len(mms),
                         "max_abs_dlogl_vs_fp64_heterodyned": (llm - llh).abs().max().item(),
-                        "note": "signal at the edges from the mixed-precision unit; ratios and sums FP64"}
+                        "note": "signal at the edges from the fixed-point unit, as fp64; ratios and contraction in double words"}
         hmix.close()
         hobj.close()
 
@@ -741,7 +741,7 @@ def main():
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K,
             "warmup": max(args.warmup, 3), "ms_per_step": 1e3 * t_total / K, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": "f64" if args.precision == "fp64" else "f64+f32x2 (double-word)", "data": "synthetic",
+            "dtype": "f64", "data": "synthetic",
             "config": {"workload": wl["name"], "detectors": "LISA", "modes": "22,21,33,32,44", "T_obs_s": T,
                        "nbins": nb, "batch_per_gpu": B, "parallelism": "replicas (independent samples per GPU)",
                        "l2": "flushed before every timed step (256 MiB write)"},

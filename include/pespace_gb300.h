@@ -44,16 +44,20 @@ extern "C" {
 #define PE_MODE_44 0x10u
 #define PE_MODE_ALL 0x1Fu
 /* Precision flag, OR-ed into the mode_mask of the forward entry points (pe_loglike_batch,
- * pe_loglike_batch_noalloc, pe_plan_create, pe_autotune, pe_signal_aet). Without it every step
- * runs in FP64. With it the TaylorF2 phase, its reduction to a fraction of a turn and every sum
- * across tiles stay FP64, while t_f, the orbit angles and the response geometry (orbit offsets,
- * link vectors, projections, sincs, third-spacecraft phases, TDI brackets) run on the FP32 pipe
- * in double-word arithmetic (~48-bit significands, ~1e-14 relative; t_f and the orbit angles in
- * FP64 where t_f lies more than 2^23 s, heliocentric, or 2^21 s, geocentric, from the origin).
- * It agrees with the FP64 path to far below the 1e-10 parity bar but not bit for bit; each
- * precision is bitwise batch-invariant by itself. Where every detector of a call has pi f L < 4 on its
- * grid, the likelihood and the gradient of both precisions run the same unit, whose geometry is 64-bit
- * fixed point (2^-60), and give the same results. pe_loglike_grad_batch, pe_hetero_create and
+ * pe_loglike_batch_noalloc, pe_plan_create, pe_autotune, pe_signal_aet). Two kinds of detector:
+ *   - pi f L < 4 on the whole grid and, on a heliocentric orbit, an eccentricity L / (2 sqrt(3) R) below 0.05. Where every
+ *     detector of a call is of this kind, the likelihood and the gradient of both precisions run the same
+ *     unit and give the same results, bit for bit: the TaylorF2 phase, t_f far from t_c, the amplitudes and
+ *     the sums in FP64, the response geometry in 64-bit fixed point (2^-60). pe_signal_aet runs it without
+ *     the flag.
+ *   - otherwise every step runs in FP64 without the flag. With it the TaylorF2 phase, its reduction to a
+ *     fraction of a turn and every sum across tiles stay FP64, while t_f, the orbit angles and the
+ *     response geometry (orbit offsets, link vectors, projections, sincs, third-spacecraft phases, TDI
+ *     brackets) run on the FP32 pipe in double-word arithmetic (~48-bit significands, ~1e-14 relative; t_f
+ *     and the orbit angles in FP64 where t_f lies more than 2^23 s, heliocentric, or 2^21 s, geocentric,
+ *     from the origin). That agrees with FP64 to far below the 1e-10 parity bar but not bit for bit.
+ * One detector of the second kind sends the whole call to the second kind's kernels. Every result is bitwise
+ * independent of the batch around its sample. pe_loglike_grad_batch, pe_hetero_create and
  * pe_surrogate_loglike_batch also take the flag (see there); pe_fisher and
  * pe_surrogate_mismatch are FP64 only and reject it. */
 #define PE_PREC_MIXED 0x100u
@@ -284,11 +288,12 @@ pe_status pe_surrogate_load(pe_surrogate s, const char* path);
 
 /* Batched gradient d logL_s / d theta_s (hand-written adjoint of the same path, Sec. 2.3 on
  * automatic differentiation); arguments as pe_loglike_batch, plus out_grad [B][11]
- * (host or device). out_logl may be NULL. mode_mask may carry PE_PREC_MIXED: the per-bin
- * forward mode sum (which out_logl and the cotangents come from) then runs in the mixed-precision
- * unit of pe_loglike_batch, and the reverse sweeps keep FP64 for the phase, t_f, the turn
- * reductions, the PN-coefficient chain rule and the sums, with the geometry, link factors and
- * their cotangents in double words (in fixed point, for both precisions, where the detectors allow it). PE_PREC_FP32 gives PE_EINVAL. */
+ * (host or device). out_logl may be NULL. Where every detector takes the fixed-point unit (PE_PREC_MIXED
+ * above) both precisions run it, and the reverse sweeps' geometry, link factors and their cotangents are in
+ * fixed point too. Elsewhere mode_mask may carry PE_PREC_MIXED: the per-bin forward mode sum (which out_logl
+ * and the cotangents come from) then runs in the mixed-precision unit of pe_loglike_batch, and the reverse
+ * sweeps keep FP64 for the phase, t_f, the turn reductions, the PN-coefficient chain rule and the sums, with
+ * the geometry, link factors and their cotangents in double words. PE_PREC_FP32 gives PE_EINVAL. */
 pe_status pe_loglike_grad_batch(const pe_detector* dets, int ndet, const double* theta, int B, unsigned mode_mask,
                                 double* out_logl, double* out_grad, int32_t* out_status, void* stream);
 
@@ -346,11 +351,13 @@ pe_status pe_fisher_gaussian(const pe_detector* dets, int ndet, const double* th
  *     if too small).
  *   pe_hetero_create: summary data for detector det (with data set), reference theta0 [11] (host),
  *     mode_mask and edges [nedges] (host, strictly increasing, 2 <= nedges <= 640, within the grid).
- *     mode_mask may carry PE_PREC_MIXED: pe_hetero_loglike_batch then evaluates the signal at the
- *     edges with the mixed-precision (or fixed-point) unit and the per-bin contraction in double words (the
- *     summary data are built in FP64, the sums across bins stay FP64). An edge where a ratio
- *     h/h0 reaches 2^24 (a reference that has almost vanished, e.g. past its taper) keeps FP64
- *     ratios, and the bins that read it are contracted in FP64. PE_PREC_FP32 gives PE_EINVAL.
+ *     pe_hetero_loglike_batch evaluates the signal at the edges with the fixed-point unit (PE_PREC_MIXED
+ *     above) where every detector takes it, in both precisions. Without the flag the per-bin contraction then
+ *     runs in block fixed point (relative to the sample's signal in the bin; FP64 elsewhere). With
+ *     PE_PREC_MIXED the other detectors' edges take the mixed-precision unit, and the contraction runs in
+ *     double words (the summary data are built in FP64, the sums across bins stay FP64); an edge where a
+ *     ratio h/h0 reaches 2^24 (a reference that has almost vanished, e.g. past its taper) keeps FP64 ratios,
+ *     and the bins that read it are contracted in FP64. PE_PREC_FP32 gives PE_EINVAL.
  *     The library owns the result; det must outlive it. Synchronous.
  *   pe_hetero_loglike_batch: log L per sample for hets[ndet] (1..8 detectors sharing one mode mask),
  *     theta [B][11], out_logl [B], out_dhhh nullable [B][ndet][3][2], out_status nullable [B] (host or

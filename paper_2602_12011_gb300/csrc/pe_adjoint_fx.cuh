@@ -4,8 +4,8 @@
 // the link factors, polarisation weights, sincs, norms and phases in fixed point, and only the scalars it ends in (the
 // phase's, amplitude's, t_f's and weights' cotangents) return to FP64 for the PN chain rule.
 //
-// What bounds it: the FP64 sweep it replaces issued 619 FP64 instructions per unit at 1.67 per SM and clock; here about
-// 110 are left, most of them the PN series' derivatives in v and q.
+// What bounds it: the FP64 forward and reverse it replaces issued 619 FP64 instructions per unit at 1.67 per SM and clock; here
+// 141 are left, 34 of them the forward's, most of the others the PN series' derivatives in v and q.
 //
 // The sky frame enters through rotations: a change of (lambda, beta, psi) turns (k, p, q) rigidly, dk = w x k and so on,
 // so the frame's cotangent is three numbers, W.w = sum over links of (projections' cotangents) x (projections), summed per

@@ -120,7 +120,7 @@ __device__ inline void sample_prep(const double* th, unsigned mask, SampleCoef& 
   const double n = 3.0 / (128.0 * eta);
   S.tc = tc;
   S.P[0] = n;
-  S.P[1] = 0.0 * n;
+  S.P[1] = 0.0;
   S.P[2] = n * (3715.0 / 756.0 + 55.0 / 9.0 * eta);
   S.P[3] = n * (-16.0 * pi + 4.0 * bso);
   S.P[4] = n * (15293365.0 / 508032.0 + 27145.0 / 504.0 * eta + 3085.0 / 72.0 * eta * eta - 10.0 * sss);
@@ -137,15 +137,15 @@ __device__ inline void sample_prep(const double* th, unsigned mask, SampleCoef& 
   sincos(bet, &sb, &cb);
   sincos(psi, &sp, &cp);
   S.k[0] = -(cb * cl); S.k[1] = -(cb * sl); S.k[2] = -sb;
-  const double u[3] = {sl, -cl, 0.0 * sl};
+  const double u[3] = {sl, -cl, 0.0};
   const double v[3] = {-(sb * cl), -(sb * sl), cb};
   for (int i = 0; i < 3; ++i) { S.p[i] = cp * u[i] + sp * v[i]; S.q[i] = -(sp * u[i]) + cp * v[i]; }
-  for (int i = 0; i < 3; ++i) S.kw[i] = to_dw((S.k[i]));
-  for (int k = 0; k < 8; ++k) S.Pdw[k] = to_dw((S.Pd[k]));
-  for (int k = 0; k < 8; ++k) S.Pw[k] = to_dw((S.P[k]));
-  S.Q5w = to_dw((S.Q5));
-  S.Q6w = to_dw((S.Q6));
-  S.tcw = to_dw((S.tc));
+  for (int i = 0; i < 3; ++i) S.kw[i] = to_dw(S.k[i]);
+  for (int k = 0; k < 8; ++k) S.Pdw[k] = to_dw(S.Pd[k]);
+  for (int k = 0; k < 8; ++k) S.Pw[k] = to_dw(S.P[k]);
+  S.Q5w = to_dw(S.Q5);
+  S.Q6w = to_dw(S.Q6);
+  S.tcw = to_dw(S.tc);
   // modes: (2 pi M / m)^(1/3) = (2 pi M)^(1/3) m^(-1/3) and its log from one cube root and one
   // log per sample; the spin-weighted harmonics share the sines and cosines of iota and iota/2
   const double Fisco = 1.0 / (k6Pow15 * 2.0 * pi * M);
@@ -160,7 +160,7 @@ __device__ inline void sample_prep(const double* th, unsigned mask, SampleCoef& 
     double hmag;          // |H_lm| / x^(p/2)
     double argt;     // arg(conj H_lm) in turns
     int p;
-    if (md == 0) { hmag = 1.0 + 0.0 * q; argt = 0.0; p = 0; }
+    if (md == 0) { hmag = 1.0; argt = 0.0; p = 0; }
     else if (md == 1) { hmag = delta / 3.0; argt = -0.25; p = 1; }
     else if (md == 2) { hmag = 0.75 * ::sqrt(15.0 / 14.0) * delta; argt = 0.25; p = 1; }
     else if (md == 3) { hmag = ::sqrt(5.0 / 7.0) / 3.0 * (1.0 - 3.0 * eta); argt = 0.0; p = 2; }
@@ -174,8 +174,8 @@ __device__ inline void sample_prep(const double* th, unsigned mask, SampleCoef& 
     C.ampp = p == 0 ? C.amp : (p == 1 ? C.amp * C.cm : C.amp * C.cm * C.cm);
     const double ph = m * phic / (2.0 * pi) + (0.125 + argt);
     C.ph0 = ph - rint(ph);
-    C.mfac = 0.0 * q + m / (4.0 * pi);
-    C.tffac = 0.0 * q + m / (12.0 * pi);
+    C.mfac = m / (4.0 * pi);
+    C.tffac = m / (12.0 * pi);
     double yp, yn;
     sylm_pair(l, m, ci, si, c2h, s2h, &yp, &yn);
     const double sgn = (l % 2) ? -1.0 : 1.0;
@@ -184,27 +184,27 @@ __device__ inline void sample_prep(const double* th, unsigned mask, SampleCoef& 
     C.Pc2 = sgn * yn - yp;
     C.fend = double(m) * Fisco;
     C.ftap = 0.9 * double(m) * Fisco;
-    C.Ppw = to_dw((C.Pp));
-    C.Pcw = to_dw((C.Pc));
-    C.tffacw = to_dw((C.tffac));
-    C.ph0w = to_dw((C.ph0));
+    C.Ppw = to_dw(C.Pp);
+    C.Pcw = to_dw(C.Pc);
+    C.tffacw = to_dw(C.tffac);
+    C.ph0w = to_dw(C.ph0);
     C.p = p;
-    C.active = (valid && (mask & (1u << md)) && (hmag) != 0.0) ? 1 : 0;
+    C.active = (valid && (mask & (1u << md)) && hmag != 0.0) ? 1 : 0;
   }
-  const double a0 = (S.md[0].amp);
+  const double a0 = S.md[0].amp;
   const int e0 = (a0 > 0.0 && isfinite(a0)) ? ilogb(a0) : 0;
   S.hsc = scalbn(1.0, -e0);
   S.ihsc = scalbn(1.0, e0);
   for (int md = 0; md < kNModes; ++md) {
-    S.md[md].cmw = to_dw((S.md[md].cm));
-    S.md[md].ampw = to_dw((S.md[md].amp) * S.hsc);
+    S.md[md].cmw = to_dw(S.md[md].cm);
+    S.md[md].ampw = to_dw(S.md[md].amp * S.hsc);
   }
   S.pair32 = (S.md[0].active && S.md[3].active) ? 1 : 0;
   S.k32 = make_double2(0.0, 0.0);
   if (S.pair32) {
     double sd, cd;
-    sincospi(2.0 * ((S.md[3].ph0) - (S.md[0].ph0)), &sd, &cd);
-    const double r = (S.md[3].amp) / (S.md[0].amp);
+    sincospi(2.0 * (S.md[3].ph0 - S.md[0].ph0), &sd, &cd);
+    const double r = S.md[3].amp / S.md[0].amp;
     S.k32 = make_double2(r * cd, r * sd);
   }
   S.k32w[0] = to_dw(S.k32.x);

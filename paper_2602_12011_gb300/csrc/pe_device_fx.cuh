@@ -12,7 +12,7 @@
 // the accumulators share one binary exponent per bin, taken from the largest amplitude so far, and
 // the mode sum's smaller modes lose only bits below 2^-60 of it.
 //
-// Bound by the latency of dependent integer and double-word operations, at half of the issue slots and 62 % of the FP64 pipe, so
+// Bound by the latency of dependent integer and double-word operations, at 62 % of the issue slots and 61 % of the FP64 pipe, so
 // warps count: 1024 LISA samples of 2^22 s (five modes) take 24.3 ms in FP64, 5.75 ms here with 6 CTAs of 128 per SM and one sinc
 // per call, 5.52 with pairs of them and the finer table, 4.95 with 8 CTAs (64 registers; 5.33 with 7, 5.37 with 9). The PN
 // series as fixed-point Horner chains took 9 more FP64 operations off each unit and made it 6.2 ms.
@@ -22,7 +22,7 @@
 
 namespace pe {
 
-// A detector takes this path where the formats' bounds hold (fx_detector_ok, pe_api.cu): a = pi f L < 4 on its whole
+// A detector takes this path where the formats' bounds hold (fill_fx, pe_api.cu): a = pi f L < 4 on its whole
 // grid, an eccentricity below 0.05 (link lengths near the nominal arm), and indices below 2^31.
 
 // (k c) 2^60 for the detector constant c = C 2^-(60 + sh): see DetDev::fx_*.

@@ -1,7 +1,7 @@
 // pe_fx.cuh -- fixed-point arithmetic of the FP64 path's response geometry.
 //
 // Why: GB300's FP64 pipe retires 1.67 operations per SM and clock (measured loops, FMA, MUL and ADD
-// alike), its FP32 pipe 122, and its integer pipes 12 32x32->64-bit multiply-adds (IMAD.WIDE) and
+// alike), its FP32 pipe 122, and its integer pipes about 16 32x32->64-bit multiply-adds (IMAD.WIDE) and
 // about 80 additions or shifts. The response's quantities (sines and cosines, unit-vector
 // projections, sincs, third-spacecraft phases) are bounded by a few units, so a 64-bit fixed-point
 // number holds them to 2^-60, finer than FP64's 2^-53, and a product of two costs three IMAD.WIDE

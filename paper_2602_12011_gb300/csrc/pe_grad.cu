@@ -8,9 +8,14 @@
 //                   tape, and per tile the contraction of the form cotangents (pe_adjoint_tape.cuh)
 //   k_grad_fwd_mixed the same in mixed precision with a double-word tape
 //                   (pe_adjoint_tape_mixed.cuh)
-//   k_grad_reduce   fixed-order per-sample sums of the tile partials -> logL, grad[11]
-//   k_fisher_fwd    per bin six reverse sweeps (Re/Im of X', Y', Z') -> Jacobian J, then
+//   k_grad_fwd_fx   both precisions where every detector takes the fixed-point unit, four CTAs per SM: the same with the
+//                   sweeps in fixed point (pe_adjoint_fx.cuh); the two kernels above serve the other detectors
+//   k_grad_reduce_warp, k_grad_reduce  fixed-order per-sample sums of the tile partials -> logL, grad[11], a warp per
+//                   sample on small grids, a CTA on larger ones
+//   k_fisher_fwd    per bin six reverse sweeps (Re/Im of X', Y', Z') by six warps -> Jacobian J, then
 //                   F += sum_c gg_c (J_Re B_c^T J_Re B_c + J_Im B_c^T J_Im B_c)
+//   k_fisher_fx     the same on the fixed-point unit: one forward pass per mode onto a tape in shared memory that six
+//                   warps' sweeps (Re/Im of A', E', T') read
 //   k_fisher_reduce fixed-order per-sample sums -> F[11][11]
 #include <cuda_runtime.h>
 
@@ -313,7 +318,7 @@ __global__ void __launch_bounds__(kTileBins, 2) k_grad_fwd_tape(DetSet ds, int B
 // The gradient on detectors that take the fixed-point unit, both precisions: per bin the forward mode sum writes each unit's
 // tape, the A/E/T cotangents and link seeds follow in FP64, and the reverse sweeps run in fixed point from the tape
 // (pe_adjoint_fx.cuh). Per tile 17 sums: the 14 of the FP64 kernel and the frame's three rotation cotangents, written as
-// the 23 partials the reduction reads. Bound by the FP64 pipe (about 135 operations a unit, 67 % busy of 84 %) and dependent integer operations (5,600 thread
+// the 23 partials the reduction reads. Bound by the FP64 pipe (141 operations a unit, 67 % busy of 84 %) and dependent integer operations (5,600 thread
 // instructions a unit). 64 LISA samples of 2^22 s: FP64 4.08 -> 1.54 ms; 500 at the mixed precision, whose
 // double-word sweep was at the FP32 pipe's rate, 12.8 -> 10.8 ms; hence both precisions take it. (Items drawn from a counter and the
 // bin's sums in shared memory: 1.34 and 9.9 ms; five and six CTAs per SM spill, 4 and 6 % slower.)
@@ -430,7 +435,9 @@ __device__ __forceinline__ void grad_write(int s, double L, const double acc[kGr
   for (int i = 0; i < PE_NPARAM; ++i) grad[(size_t)s * PE_NPARAM + i] = valid ? out[i] : 0.0;
 }
 
-// Small grids (at most kGradWarpTiles tiles a detector): one warp per sample, fixed-order sums over each detector's tiles.
+// Small grids (at most kGradWarpTiles tiles a detector): one warp per sample, fixed-order sums over each detector's tiles. (Whole calls,
+// one warp and one CTA per sample: 8 tiles 87 and 86 us for one sample, 703 and 721 for 1024; 64 tiles 90 and 86, 5028 and 5053; 820 tiles
+// 197 and 176 us for one sample, 7108 and 7082 for 128.)
 constexpr int kGradWarpTiles = 64;
 __global__ void k_grad_reduce_warp(DetSet ds, int B, const long long* off, const double* part, const SampleCoef* coef,
                               const SampleGrad* sgrad, double* logl, double* grad) {
@@ -610,7 +617,7 @@ __device__ __forceinline__ int fisher_lane_entry(int lane) {
 // each (slot w) onto a tape in shared memory, with the chain factors that the seeds share; then warp j runs seed j's reverse
 // sweeps (Re/Im of A', E', T'), giving row j of the Jacobian, and each warp accumulates eleven of the 66 entries. Bound by
 // the dependent integer operations of the sweeps at 12 warps an SM and, at about 2,100 per bin, by the FP64 pipe.
-// Three points on LISA, 2^21 s: 1.60 ms with the FP64 sweeps (k_fisher_fwd), 0.42 ms now.
+// Three points on LISA, 2^21 s: 1.60 ms with the FP64 sweeps (k_fisher_fwd), 0.39 ms now.
 constexpr int kFisherFxThreads = 32 * kFisherWarps;
 struct FisherTape {   // field f of a lane at p[32 f]
   static constexpr bool kOn = true, kChain = true;
@@ -798,8 +805,10 @@ cudaError_t launch_grad_reduce(const DetSet& ds, int B, const long long* off, co
     k_grad_reduce<<<B, kGradW * 32, 0, st>>>(ds, B, off, part, coef, sgrad, logl, grad);
   return pe::launch_status();
 }
-// Items per 128-bin tile: a few points leave the chip's SMs two or three tiles each, so up to 32 tiles per SM the fixed-point
-// kernel's items are a quarter tile; beyond, whole tiles (a quarter of the partials).
+// Items per 128-bin tile: a few points leave the chip's SMs two or three tiles each, so up to 32 possible tiles per SM the fixed-point
+// kernel's items are a quarter tile; beyond, whole tiles (a quarter of the partials). Whole and quarter tiles, whole calls with every bin
+// active: 8 tiles 265 and 113 us, 128 267 and 203, 1,024 1072 and 1020, 2,048 2015 and 1971, 4,096 3783 and 3871, 8,192 7481 and 7672. Samples over
+// the prior leave most of a long grid's tiles without work, and quarters win for longer.
 int fisher_split(const DetSet& ds, long long max_tiles, int sms) { return fx_all_ok(ds) && max_tiles <= 32LL * sms ? 4 : 1; }
 cudaError_t launch_fisher_fwd(const DetSet& ds, int B, const SampleCoef* coef, const SampleGrad* sgrad,
                               const int* nend, const long long* off, double* part, long long max_tiles, int sms, int split,

@@ -135,8 +135,9 @@ bool lookup_tuned(const DetSet& ds, int B, unsigned mask, TuneChoice* out) {
   return true;
 }
 
-// The fixed-point unit's items are one sub-tile, two from 2^19 possible ones on (1024 LISA samples of 2^22 s: 4.95 ms with one, 4.88 with
-// two; 45 samples on three detectors and single points are faster with one, whose last round is shorter).
+// The fixed-point unit's items are one sub-tile, two from 2^19 possible ones on, where the two cross. With one and two, on LISA grids of
+// 2^18, 2^20 and 2^22 s: 2^18 sub-tiles 1024 and 1035, 906 and 926, 716 and 742 us; 2^19 1966 and 1951, 1665 and 1660, 1494 and 1499; 2^20 3783 and
+// 3719, 3428 and 3383, 3208 and 3178. Short lists lose more (2^12: 93 and 121 us), as their last round is longer.
 TuneChoice default_choice(int prec, const DetSet& ds, long long max_tiles) {
   const bool fx = fx_all_ok(ds) && prec != kPrecFP32;
   return TuneChoice{kFwdDefaultVariant, 8, fx && max_tiles >= (1LL << 19) ? 2 : fwd_default_subtiles(prec, fx), 0.0};

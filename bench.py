@@ -33,17 +33,17 @@ METRIC = "log-likelihood evals/s (HM, 3 TDI ch, batched) vs plain path; grad eva
 UNIT = "evals/s"
 MSUN_S = 4.925490947641267e-6
 # Work per active (sample, mode, bin) unit of the fused forward kernel, from the ncu SASS counters
-# of one launch on the 64-sample case of this workload:
+# of one launch on a 128-sample case of this workload:
 #   fp64_flops  DFMA x 2 + DMUL + DADD
 #   fp64_inst   every FP64-pipe instruction (DFMA, DMUL, DADD, DSETP, F2F, FRND)
 #   fp32_inst   FFMA + FMUL + FADD (the double-word corrections of the fixed-point unit)
 UNIT_COUNTS = {
-    # fp64 and mixed: both run the fixed-point unit on this workload (2,464 thread instructions per unit,
+    # fp64 and mixed: both run the fixed-point unit on this workload (2,471 thread instructions per unit,
     # most of them integer)
-    "fp64": {"fp64_flops": 50.8, "fp64_inst": 33.9, "fp32_inst": 532.4},
-    "mixed": {"fp64_flops": 50.8, "fp64_inst": 33.9, "fp32_inst": 532.4},
+    "fp64": {"fp64_flops": 50.8, "fp64_inst": 33.9, "fp32_inst": 534.0},
+    "mixed": {"fp64_flops": 50.8, "fp64_inst": 33.9, "fp32_inst": 534.0},
     # FP32 path: fp64_inst counts the FRND and F2F of CUDA's FP32 sincospif/sinf and conversions
-    "fp32": {"fp64_flops": 0.5, "fp64_inst": 8.9, "fp32_inst": 355.5},
+    "fp32": {"fp64_flops": 0.5, "fp64_inst": 8.9, "fp32_inst": 353.1},
 }
 # SHA-256 (first 16 hex digits) of the per-bin unit's sources the counts were taken on; the bench
 # marks the counts stale (and warns) when the sources have changed since.
@@ -52,10 +52,10 @@ UNIT_SOURCES = {
     "mixed": ("pe_device.cuh", "pe_device_fx.cuh", "pe_fx.cuh", "pe_df.cuh", "pe_kernels.cu", "pe_internal.h"),
     "fp32": ("pe_device.cuh", "pe_device_f32.cuh", "pe_kernels.cu", "pe_internal.h"),
 }
-UNIT_COUNTS_SOURCE_SHA = {"fp64": "3b8e65fcbe360bee", "mixed": "3b8e65fcbe360bee", "fp32": "75ea947647228f96"}
+UNIT_COUNTS_SOURCE_SHA = {"fp64": "5006297410eab940", "mixed": "5006297410eab940", "fp32": "e9efb17d983dc2e9"}
 # DRAM bytes (read + write) of one full-size launch (B = 1024), ncu dram__bytes_{read,write}.sum:
 # the per-bin tables, read once per launch
-TRAFFIC = {"fp64": 35.89e6 + 0.40e6, "mixed": 35.89e6 + 0.40e6, "fp32": None}
+TRAFFIC = {"fp64": 35.84e6 + 0.53e6, "mixed": 35.84e6 + 0.53e6, "fp32": None}
 # Algorithmic work of the method (oracle/flop_model.py: the oracle's own operations, counted on
 # 16 samples of this workload): add/sub/mul/div per active (sample, mode, bin) unit and per active
 # (sample, bin) for the A/E/T and likelihood terms, and math-library calls per unit.

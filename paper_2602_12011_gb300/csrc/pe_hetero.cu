@@ -349,12 +349,14 @@ __global__ void k_het_words(const double* fe, int ne, const double2* A, const do
 // ratios at the two edges, every ratio is held in 2^-60 of 2^(N - g_i), N the least power of two for which sum m_i 2^(g_i - N)
 // is below 1/2. What is lost is then below 2^-59 of the sample's own signal in the bin, whatever its distance
 // and however the modes' ratios differ (FP64 keeps 2^-53 of each ratio), and powers of two in the signal pass through exactly.
-// Bounds: d is below 1, y and w below sqrt(2) (Cauchy-Schwarz over the bin's fine bins), hh below 1/2 and, where the ratios' size is
-// the signal's, above 2^-8. False where the bin takes the FP64 form: a ratio that is not finite, exponents outside the words', or hh below
-// 2^-10 (an edge where the reference has almost vanished has ratios far above the signal in the bin, or the modes cancel).
+// Bounds: d is below 1, y and w below sqrt(2) (Cauchy-Schwarz over the bin's fine bins), hh below 1/2 and, where neither the modes nor
+// the edges cancel, above 2^-8. False where the bin takes the FP64 form: a ratio that is not finite, exponents outside the words', or an edge whose
+// ratio is far above the signal in the bin (the reference has almost vanished there): a mode's ratios differ fourfold or more and hh is
+// below 2^-10. Where hh is that small because the terms cancel, FP64 loses more. (A bin left to the FP64 form costs its CTA some 30 us: its 340
+// operations are one thread's chain. With every hh below 2^-10 left to it, a bin or two in a sample, calls took 5 to 9 % longer.)
 // Bound by the 32 x 32-bit products, about 900 per (bin, channel) at 16 per SM and clock where the FP64 form issues 340 operations
-// at 1.67 (777 samples, LISA, 2^22 s, whole call: 677 us with the FP64 form, 381 us; 363 us with the ratios held in 2^-59 of 1, which lost
-// the faint samples' bits and sent ratios above 2 to the FP64 form).
+// at 1.67 (777 samples, LISA, 2^22 s, whole call: 677 us with the FP64 form, 356 us at any distance; 363 us, and 749 at a third of the reference's distance, with the ratios
+// held in 2^-59 of 1, which lost the faint samples' bits and sent ratios above 2 to the FP64 form).
 __device__ __forceinline__ bool het_bin_fx(const HetDev& H, int b, int c, const double2* __restrict__ ratio, double& dh, double& hh) {
   const int nbin = H.ne - 1;
   const int ea = H.Gx[(size_t)(kNModes * 3 + c) * nbin + b];
@@ -364,11 +366,14 @@ __device__ __forceinline__ bool het_bin_fx(const HetDev& H, int b, int c, const 
   unsigned m[kNModes];
   int g[kNModes], top = 2 * kHetNoMode;
   unsigned most = 0;
+  bool uneven = false;                    // a mode's ratios differ fourfold or more
 #pragma unroll
   for (int md = 0; md < kNModes; ++md) {
     const double2 ra = at(sa[3 * md], md), rb = at(sb[3 * md], md);
     auto hi = [](double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
-    m[md] = max(max(hi(ra.x), hi(ra.y)), max(hi(rb.x), hi(rb.y)));
+    const unsigned ma = max(hi(ra.x), hi(ra.y)), mb = max(hi(rb.x), hi(rb.y));
+    m[md] = max(ma, mb);
+    uneven |= m[md] - min(ma, mb) >= 0x200000u;
     g[md] = H.Gx[(size_t)(md * 3 + c) * nbin + b];
     most = max(most, m[md]);
     if (m[md] >= 0x100000u) top = max(top, (int)(m[md] >> 20) + g[md]);
@@ -430,7 +435,7 @@ __device__ __forceinline__ bool het_bin_fx(const HetDev& H, int b, int c, const 
     }
     sh += fx_msub(rr[md], fx_split(yx), ri[md], fx_split(yy)) + fx_msub(dr[md], fx_split(wx), di[md], fx_split(wy));
   }
-  if (sh < (1LL << kHetLeast)) return false;
+  if (uneven && sh < (1LL << kHetLeast)) return false;
   dh = fx_to_double(sd, ea + N - 60);
   hh = fx_to_double(sh, 2 * N - 60);
   return true;
